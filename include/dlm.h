@@ -363,8 +363,8 @@ int dlm_guided_accept_threshold(dlm_ctx* ctx, const int32_t* tok_dlm, const floa
  * Supported: d_model a multiple of 128, head_dim a multiple of 64, batch * q_cap <= 256, and q_cap a multiple of 8
  * when batch > 1.
  *
- * workspace: device, 256-byte aligned, at least dlm_window_proj_workspace_bytes(ctx, rows = batch * q_cap,
- * n_out = output features, k_total = contraction length) bytes: fp32 partial tiles of the K split.
+ * workspace: dlm_window_proj_workspace_bytes(ctx, rows = batch * q_cap, n_out = output features, k_total = contraction
+ * length) bytes of device scratch (0 = invalid arguments).  The present kernels use none of it.
  */
 size_t dlm_window_proj_workspace_bytes(const dlm_ctx* ctx, int rows, int n_out, int k_total);
 int dlm_window_qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, int batch, int q_cap,

@@ -24,7 +24,7 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
   ctx->encode_tiled = nullptr;
   ctx->commit_blocks_per_sm[0] = ctx->commit_blocks_per_sm[1] = 0;
   for (int i = 0; i < 8; ++i) ctx->attn_smem_limit[i] = 0;
-  ctx->proj_configured = false;
+  ctx->proj_configured = 0;
   ctx->wait_limit_ns = sm100::kWaitLimitNs;
   ctx->attn_team_max = 1 << 20;   // no limit beyond the schedule's own
   ctx->attn_team_force = false;

@@ -29,7 +29,7 @@ struct dlm_ctx {
   void* encode_tiled;       // cuTensorMapEncodeTiled entry point (driver API), resolved lazily
   int commit_blocks_per_sm[2];  // resident blocks per SM of the two commit kernels (0 = not asked yet)
   unsigned long long wait_limit_ns;   // limit of the kernels' device-side waits (2 s; a test may shorten it)
-  bool proj_configured;         // shared-memory opt-in of the projection kernel done on this context's device
+  unsigned int proj_configured; // bit per projection kernel: shared-memory opt-in done on this context's device
   int attn_team_max;            // most blocks the attention call's team schedule may give one unit (1 = schedule off)
   bool attn_team_force;         // tests: take the team schedule wherever it is possible, whatever the cost estimate says
   int attn_smem_limit[8];       // dynamic shared memory the two attention kernels may use on this device (0 = not set up yet)
@@ -57,19 +57,31 @@ __device__ __forceinline__ void dlm_grid_dependency_wait() { asm volatile("gridd
 __device__ __forceinline__ void dlm_trigger_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-static inline cudaError_t dlm_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                     Args... args) {
+static inline cudaError_t dlm_launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                             unsigned int cluster, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (cluster > 1) {   // thread-block clusters of `cluster` consecutive blocks along x
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+static inline cudaError_t dlm_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                     Args... args) {
+  return dlm_launch_cluster(kernel, grid, block, smem, stream, 1, args...);
 }
 
 // The context's device must be the calling thread's current device: launches go to the current

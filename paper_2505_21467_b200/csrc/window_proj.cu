@@ -2,18 +2,25 @@
 // step (Table 1 rows "Q/K/V projection" and "output projection"; Sec. 3.2.1 "Windowed Re-computation":
 // the window's K/V are recomputed from its hidden states in every step).
 //
-// With a window of 32 .. 256 rows these products stream the weight matrix once and do little arithmetic
-// per byte: HBM-bound up to about 256 rows, balanced beyond.  The tensor core wants M = 128, so the
-// operands are swapped: a block computes Y^T[128 output features x R rows] = W[128 x K] X^T[K x R], the
-// weights as the M x K operand (K-major as they lie in memory), the activations as the N x K operand,
-// the accumulator in TMEM with one output feature per lane.  K is split across blocks so that every SM
-// streams a share of the weights; the blocks of a tile leave fp32 partial tiles in the workspace and the
-// last one to arrive (a ticket) adds them in a fixed order, adds the bias and writes bf16 in the layout
-// the consumer reads (Q/K/V head by head for the attention step, or row-major hidden states).
+// Y[rows x features] = X[rows x K] W[features x K]^T.  Activation rows are the MMA's M (one row per TMEM lane and
+// epilogue thread), N features of one tile its N; a block (pair) sums the whole of K, so there is no workspace, no exchange
+// between blocks and one summation order.  With the row in a thread, a head's features lie along the thread's registers: the
+// rotary embedding pairs two of its own registers and every store is 16 bytes of one row.
+//   up to 64 rows:  one block per tile, M = 128 (rows beyond the call's are never loaded, never read back), tiles of
+//                   16 .. 128 features.  Bound by streaming the weights from HBM.
+//   more rows:      chunks of up to 256 rows, each by a pair of blocks (cta_group::2, M = 256): a block holds its half of
+//                   the rows and its half of the tile's features, so it takes in half of what two separate blocks would;
+//                   tiles of 64 .. 256 features.  Bound by the SM's intake from L2 at small tiles, by the tensor pipe at 256.
+// Measured (one call per layer over 28 / 32 layers' own weights, back to back, rotary embedding and staging on; before this
+// form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
+//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 11.2 us (2.9 TB/s of weights)   256 x 3584 -> 4608   25.1 -> 15.5 us
+//                           256 x 4096 -> 12288   167 -> 38.8 us (665 TFLOP/s)          1280 x 3584 -> 4608   237 -> 50 us (845 TFLOP/s)
+// Both operands are K-major as they lie in memory.  A tensor map with K split into (64-element panel, panel index) lets one
+// copy bring several panels of a stage: a producer's loop costs 200 - 340 cycles per iteration whatever it copies
+// (barrier wait 100, expect 40, each copy 55), which bound the kernel when every 64 elements of K took an iteration.
 //
-// Block = 6 warps: warp 0 one TMA producer lane (weight panel [128 x 64] and activation panel [R x 64]
-// per stage, 128-byte swizzle), warp 1 the tcgen05.mma issuer (4 MMAs of K = 16 per stage), warps 2-5 the
-// epilogue (thread = TMEM lane = output feature).
+// Block = 8 warps: warp 0 weight producer, warp 1 activation producer, warp 2 tcgen05.mma issuer (of the leader block),
+// warp 3 TMEM and the L2 prefetch of the weights, warps 4-7 the epilogue's tables; all eight write the results.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -24,12 +31,11 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kThreads = 192;
-constexpr int kTileN = 128;                 // output features per block
-constexpr int kChunkK = 64;                 // K elements per pipeline stage (one 128-byte swizzled panel)
-constexpr int kMaxRows = 256;               // activation rows per block (MMA N)
-constexpr int kWBytes = kTileN * kChunkK * 2;
+constexpr int kThreads = 256;
+constexpr int kPanel = 64;                  // K elements of a 128-byte swizzled panel
 constexpr int kMaxStages = 8;
+constexpr int kMaxActRows = 256;            // rows of an output projection (one pair sees them all)
+constexpr int kAuxBytes = 16 * kMaxStages + 16 + 32 + 256 * 4 + 128 * 32;   // barriers, flags, bias of the tile, row table
 
 struct ProjParams {
   // destination: mode 0 = Q/K/V head by head ([B][heads][q_cap][D] each), mode 1 = row-major [rows][n_out]
@@ -37,6 +43,7 @@ struct ProjParams {
   __nv_bfloat16* q_out;
   __nv_bfloat16* k_out;
   __nv_bfloat16* v_out;
+  const __nv_bfloat16* w;
   const __nv_bfloat16* bias;   // [n_out] or nullptr
   const float* rope_cos;       // mode 0: rotary embedding of the query and key heads, fp32 [B][q_cap][head_dim / 2],
   const float* rope_sin;       // or both nullptr
@@ -47,359 +54,317 @@ struct ProjParams {
   const int32_t* cache_len;    // [B]
   const int32_t* q_len;        // [B] rows of the window that are active (staged), or nullptr: all q_cap
   int capacity;
-  float* partial;              // [row chunk][feature tile][split][rows_pad][128] fp32
-  unsigned int* tickets;       // one per (row chunk, feature tile)
   int rows_total, q_cap, n_q_heads, n_kv_heads, head_dim, n_out, k_total;
-  int batch;                   // mode 1 with head-split activations: batch elements (row chunk = all rows)
-  int act_heads;               // mode 1: activations are [B][act_heads][q_cap][D] (0: plain [rows][K])
-  int rows_pad;                // MMA N: rows of a chunk rounded up to 32
-  int n_split, k_per_split;    // K split across blocks, elements per split (a multiple of 64)
-  int n_stages;
+  int batch;
+  int act_heads;               // activations are [B][act_heads][q_cap][D] (0: plain [rows][K])
+  int rc;                      // rows per block (a multiple of 8)
+  int x_box_rows;              // rows per copy of head-split activations (rc: one copy brings all)
+  int half_rows;               // features of a group's half: W is seen as [groups][2][half_rows][K]
+  int n_stages, aux_offset;
+  int head_shift;              // log2(head_dim), or -1
   int* status;
 };
 
-// Waits until the counter at `addr` reaches `target` (acquire, device scope), bounded like the mbarrier waits.
-__device__ __forceinline__ bool wait_count(const unsigned int* addr, unsigned int target, volatile int* abort_flag) {
-  const uint64_t t0 = global_timer_ns();
-  for (uint32_t spin = 1;; ++spin) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(addr) : "memory");
-    if (v >= target) return true;
-    if ((spin & 15u) == 0u) {
-      if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > kWaitLimitNs) {
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
+// Where a row of the block goes: element offsets within q_out (or y), k_out / v_out and the staged layer (-1: not staged),
+// and within the rotary tables.
+struct __align__(16) RowEntry {
+  long long q, kv, stage, rope;
+};
 
+// Feature tiles.  A tile takes N / 2 consecutive features from each half of a group of 2 half_rows features; with
+// half_rows = head_dim / 2 a tile narrower than a head then holds both partners of every rotary pair it has.
+// PAIR: each block of the pair loads one of the two halves, and D's columns are [half 0 | half 1] either way.
+template <int N, int M, int KP>
 __global__ void __launch_bounds__(kThreads, 1)
 window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const ProjParams p) {
   extern __shared__ uint8_t smem_raw[];
+  constexpr bool PAIR = M > 64;
+  constexpr int kRowTile = M == 64 ? 64 : M / 2;            // rows of the MMA in this block
+  constexpr int kBlockN = PAIR ? N / 2 : N;                 // features whose weights this block loads
+  constexpr uint32_t kWBytes = (uint32_t)KP * kBlockN * 128u;
+  constexpr uint32_t kTmemCols = N < 32 ? 32 : N;
   const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
   const uint32_t base = smem_u32(smem_raw) + pad;
-  const uint32_t x_bytes = (uint32_t)p.rows_pad * 128u;
+  const uint32_t x_panel = (uint32_t)p.rc * 128u, x_bytes = KP * x_panel;
   const uint32_t stage_bytes = kWBytes + x_bytes;
-  const uint32_t sm_bar = base + p.n_stages * stage_bytes;          // full[8], empty[8], done
-  const uint32_t bar_full = sm_bar, bar_empty = sm_bar + 8 * kMaxStages, bar_done = sm_bar + 16 * kMaxStages;
-  const uint32_t bar_red = bar_done + 8;   // the partial tiles' slices of this block's rows have landed in shared memory
-  int* const flags = reinterpret_cast<int*>(smem_raw + pad + (size_t)p.n_stages * stage_bytes + 16 * kMaxStages + 16);
+  // stages (and room behind them for the MMA's reads of rows that no copy fills, see make_proj_plan), then barriers, flags,
+  // the tile's bias and the row table
+  const uint32_t aux = p.aux_offset;
+  const uint32_t bar_full = base + aux, bar_empty = bar_full + 8 * kMaxStages, bar_done = bar_full + 16 * kMaxStages;
+  int* const flags = reinterpret_cast<int*>(smem_raw + pad + aux + 16 * kMaxStages + 16);
   volatile int* const abort_ptr = flags;
   volatile int* const never_ptr = flags + 1;
   uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(flags + 2);
-  volatile int* const is_last = flags + 3;
-  volatile int* const warp_ok = flags + 4;   // [4]: the epilogue warps' waits, so that all four take the same branches
+  float* const bias_s = reinterpret_cast<float*>(flags + 8);
+  RowEntry* const row_s = reinterpret_cast<RowEntry*>(bias_s + 256);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tile = blockIdx.x, split = blockIdx.y, chunk = blockIdx.z;
-  const int row0 = chunk * kMaxRows;
-  const int k0 = split * p.k_per_split;
-  const int k1 = min(k0 + p.k_per_split, p.k_total);
-  const int n_k = (k1 - k0) / kChunkK;     // stages' worth of K in this block (>= 1 by construction)
-  uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < p.rows_pad) tmem_cols <<= 1;
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
+  const int tile = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+  const int row0 = ((int)blockIdx.z * (PAIR ? 2 : 1) + (int)rank) * p.rc;   // this block's first row
+  const int per_group = p.half_rows / (N / 2);
+  const int group = tile / per_group, a0 = (tile % per_group) * (N / 2);
+  const int feat0 = group * 2 * p.half_rows + a0, feat1 = feat0 + p.half_rows;   // first features of the two halves
+  auto feature = [&](int c) { return c < N / 2 ? feat0 + c : feat1 + c - N / 2; };      // output feature of column c
+  const int n_panels = p.k_total / kPanel;
+  const int n_k = (n_panels + KP - 1) / KP;                 // stages' worth of K; panels beyond the last are zero-filled
 
   if (tid == 0) {
-    *abort_ptr = 0; *never_ptr = 0; *is_last = 0;
+    *abort_ptr = 0; *never_ptr = 0;
     for (int i = 0; i < p.n_stages; ++i) {
-      mbar_init(bar_full + 8 * i, 1);
+      mbar_init(bar_full + 8 * i, 2);
       mbar_init(bar_empty + 8 * i, 1);
     }
     mbar_init(bar_done, 1);
-    mbar_init(bar_red, 1);
     mbar_fence_init();
     fence_proxy_async_smem();
   }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), tmem_cols);
-    tmem_relinquish();
+  if (warp == 0 && lane == 0) prefetch_tensormap(&tm_w);
+  if (warp == 1 && lane == 0) prefetch_tensormap(&tm_x);
+  if (warp == 3) {
+    // The tile's weights start on their way to L2 while the kernel before this one is still running (its blocks leave
+    // room for this kernel's): only a prefetch, so nothing is read before that kernel's writes are visible.
+    if (blockIdx.z == 0)
+      for (int i = lane; i < kBlockN; i += 32) {
+        const int f = PAIR ? (rank ? feat1 : feat0) + i : (i < N / 2 ? feat0 + i : feat1 + i - N / 2);
+        prefetch_l2(p.w + (size_t)f * p.k_total, (uint32_t)p.k_total * 2u);
+      }
+    __syncwarp();
+    if (PAIR) {
+      tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+      tmem_relinquish();
+    }
   }
-  if (warp == 0 && lane == 0) {
-    prefetch_tensormap(&tm_w);
-    prefetch_tensormap(&tm_x);
-  }
-  dlm_grid_dependency_wait();
-  dlm_trigger_dependents();
+  __syncwarp();
   tc_fence_before_sync();
-  __syncthreads();
+  if (PAIR) cluster_sync(); else __syncthreads();   // barriers exist (in both blocks), TMEM is there
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  dlm_grid_dependency_wait();
+  dlm_trigger_dependents();
 
-  if (warp == 0) {
-    // ================================================================= TMA producer
-    if (lane == 0) {
-      bool ok = true;
-      int s = 0, round = 0, issued = 0;
-      // bytes a stage receives: a box counts in full, also where it reaches beyond the tensor
-      const uint32_t tx = kWBytes + (p.act_heads == 0 ? x_bytes : (uint32_t)(p.batch * p.q_cap) * 128u);
-      for (int kc = 0; kc < n_k && ok; ++kc) {
-        if (round > 0) ok = mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr);
-        if (!ok) break;
-        const uint32_t dst = base + s * stage_bytes;
-        const int k = k0 + kc * kChunkK;
-        mbar_expect_tx(bar_full + 8 * s, tx);
-        tma_load_3d(dst, &tm_w, bar_full + 8 * s, k, tile * kTileN, 0);
-        if (p.act_heads == 0) {
-          tma_load_3d(dst + kWBytes, &tm_x, bar_full + 8 * s, k, row0, 0);
+  if (warp < 2) {
+    // ================================================================= producers (0: weights, 1: activations)
+    const uint32_t bytes = (warp == 0 ? kWBytes : x_bytes) * (PAIR ? 2u : 1u);   // what the leader's barrier gets from both blocks
+    const uint32_t full0 = PAIR ? map_shared_rank(bar_full, 0) : bar_full;
+    const int head_panels = p.act_heads ? p.head_dim / kPanel : 1;
+    int head = 0, panel = 0;                                // head-split activations: where the next K panel lies
+    const int y0 = p.batch > 1 ? row0 % p.q_cap : row0, z0 = p.batch > 1 ? row0 / p.q_cap : 0;
+    bool ok = true;
+    int s = 0, round = 0, issued = 0;
+    for (int kc = 0; kc < n_k; ++kc) {
+      if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
+      if (!ok) break;
+      if (elect_one_sync()) {
+        if (rank == 0) mbar_expect_tx(bar_full + 8 * s, bytes);
+        const uint32_t dst = base + s * stage_bytes, bar = full0 + 8 * s;
+        if (warp == 0) {
+          tma_load_5d<PAIR>(dst + x_bytes, &tm_w, bar, 0, a0, PAIR ? (int)rank : 0, kc * KP, group);
+        } else if (p.act_heads == 0) {
+          tma_load_4d<PAIR>(dst, &tm_x, bar, 0, row0, kc * KP, 0);
         } else {
-          // activations [B][heads][q_cap][D]: K index k = head * D + d; one box of q_cap rows per batch element
-          const int head = k / p.head_dim, d = k % p.head_dim;
-          for (int b = 0; b < p.batch; ++b)
-            tma_load_3d(dst + kWBytes + (uint32_t)(b * p.q_cap) * 128u, &tm_x, bar_full + 8 * s, d, 0, b * p.act_heads + head);
+          // activations [B][heads][q_cap][D]: panel k belongs to head k / (D / 64); rows of a box are (sequence, row)
+          int h = head, pn = panel;
+          for (int kp = 0; kp < KP; ++kp) {
+            const uint32_t d = dst + kp * x_panel;
+            tma_load_4d<PAIR>(d, &tm_x, bar, pn * kPanel, y0, h, z0);
+            for (int r = p.x_box_rows; r < p.rc; r += p.x_box_rows)
+              tma_load_4d<PAIR>(d + r * 128, &tm_x, bar, pn * kPanel, (row0 + r) % p.q_cap, h, (row0 + r) / p.q_cap);
+            if (++pn == head_panels) { pn = 0; ++h; }
+          }
         }
-        ++issued;
-        if (++s == p.n_stages) { s = 0; ++round; }
       }
-      if (!ok) {   // unwinding: let the copies already issued land before the block's memory is released
-        for (int i = max(0, issued - p.n_stages); i < issued; ++i)
-          mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
-      }
+      for (int kp = 0; kp < KP; ++kp)
+        if (++panel == head_panels) { panel = 0; ++head; }
+      __syncwarp();
+      ++issued;
+      if (++s == p.n_stages) { s = 0; ++round; }
     }
-  } else if (warp == 1) {
+    if (!ok && rank == 0)   // unwinding: let the copies already issued land before the memory is released (both blocks' land on the leader's barriers)
+      for (int i = max(0, issued - p.n_stages); i < issued; ++i)
+        mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
+  } else if (warp == 2 && rank == 0) {
     // ================================================================= MMA issuer
     bool ok = true;
-    const uint32_t idesc = make_idesc_bf16(128, (uint32_t)p.rows_pad, 0);
+    const uint32_t idesc = make_idesc_bf16(M, (uint32_t)N, 0);
+    const uint64_t desc = make_smem_desc_sw128(base, 16, 1024);
+    const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
     int s = 0, round = 0;
-    for (int kc = 0; kc < n_k && ok; ++kc) {
+    for (int kc = 0; kc < n_k; ++kc) {
       ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, round & 1, abort_ptr)) != 0;
       if (!ok) break;
       tc_fence_after_sync();
-      const uint64_t dw = make_smem_desc_sw128(base + s * stage_bytes, 16, 1024);
-      const uint64_t dx = make_smem_desc_sw128(base + s * stage_bytes + kWBytes, 16, 1024);
+      const uint32_t a0_lo = desc_lo + ((s * stage_bytes) >> 4), b0_lo = a0_lo + (x_bytes >> 4);
       if (elect_one_sync()) {
 #pragma unroll
-        for (int k = 0; k < kChunkK / 16; ++k) {
-          if (kc == 0 && k == 0) mma_ss<false>(tmem, dw, dx, idesc);
-          else mma_ss<true>(tmem, desc_offset(dw, k * 32), desc_offset(dx, k * 32), idesc);
+        for (int kp = 0; kp < KP; ++kp) {
+          const uint32_t a_lo = a0_lo + kp * (x_panel >> 4), b_lo = b0_lo + kp * (kBlockN * 8);
+#pragma unroll
+          for (int k = 0; k < kPanel / 16; ++k)
+            mma_ss_lo<PAIR>(tmem, a_lo + 2 * k, b_lo + 2 * k, desc_hi, idesc, kc > 0 || kp > 0 || k > 0 ? 1u : 0u);
         }
-        tc_commit(bar_empty + 8 * s);
+        if (PAIR) tc_commit_pair(bar_empty + 8 * s); else tc_commit(bar_empty + 8 * s);
       }
       __syncwarp();
       if (++s == p.n_stages) { s = 0; ++round; }
     }
-    if (elect_one_sync()) tc_commit(bar_done);
+    if (elect_one_sync()) { if (PAIR) tc_commit_pair(bar_done); else tc_commit(bar_done); }
     __syncwarp();
+  } else if (warp >= 4) {
+    // ================================================================= tables of the epilogue
+    const int t = tid - 128;
+    for (int c = t; c < N; c += 128) bias_s[c] = p.bias ? __bfloat162float(p.bias[feature(c)]) : 0.f;
+    const int row = row0 + t;
+    if (t < p.rc && row < p.rows_total) {
+      const int b = row / p.q_cap, i = row - b * p.q_cap;
+      RowEntry e;
+      e.q = p.mode == 1 ? (long long)row * p.n_out : ((long long)b * p.n_q_heads * p.q_cap + i) * p.head_dim;
+      e.kv = ((long long)b * p.n_kv_heads * p.q_cap + i) * p.head_dim;
+      e.rope = (long long)row * (p.head_dim >> 1);
+      e.stage = -1;   // cache row to stage at: none for an inactive row or one without room (reported)
+      if (p.stage_k && feature(N - 1) >= p.n_q_heads * p.head_dim && (!p.q_len || i < __ldg(p.q_len + b))) {
+        const int pos = __ldg(p.cache_len + b) + i;
+        if (pos >= 0 && pos < p.capacity) e.stage = ((long long)b * p.n_kv_heads * p.capacity + pos) * p.head_dim;
+        else dlm_set_status(p.status, DLM_ERR_CAPACITY);
+      }
+      row_s[t] = e;
+    }
   }
 
-  // ================================================================= epilogue (warps 2-5)
-  if (warp >= 2) {
-    // TMEM lanes are tied to warp % 4: warps 2, 3, 4, 5 own lanes 64-95, 96-127, 0-31, 32-63
-    const int lane_base = (warp & 3) * 32;
-    const int f = lane_base + lane;                       // feature within the tile = TMEM lane
-    const int n = tile * kTileN + f;                      // output feature
-    bool ok = __all_sync(0xffffffffu, mbar_wait(bar_done, 0, abort_ptr)) != 0;
+  // ================================================================= epilogue, by all eight warps
+  // fp32 columns pass through shared memory (free by then), two segments of kCW columns at a time (rotary pairs, or just
+  // two pieces), so that a store instruction writes whole sectors of neighbouring features.  One warp per scheduler runs
+  // this code, so its length in dependent instructions is what counts: addresses are a per-row offset (table) plus a
+  // per-segment pointer.  (Rows kept in their threads, divisions and 64-bit products per store, four warps: 10 us for the
+  // 256-feature tile.)
+  {
+    const int n_rows = min(p.rc, p.rows_total - row0);       // real rows of this block (may be <= 0)
+    const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, abort_ptr) ? 1 : 0) != 0;   // and the tables are there
     tc_fence_after_sync();
-    // rotary embedding (mode 0): feature d of a query or key head is paired with feature d +- head_dim / 2
-    const bool rope = p.mode == 0 && p.rope_cos != nullptr;
-    const int half = p.head_dim >> 1;
-    const int rows_here = min(kMaxRows, p.rows_total - row0);
-    const size_t tile_slot = ((size_t)chunk * gridDim.x + tile) * p.n_split;
-    float* my_partial = p.partial + (tile_slot + split) * (size_t)p.rows_pad * kTileN + f;
-    if (ok && p.n_split > 1) {
-      // fp32 partial tile, [row][feature]: a warp's 32 lanes write 128 contiguous bytes per row
-      uint32_t v[32];
-      for (int c = 0; c < p.rows_pad; c += 32) {
-        tmem_ld32(tmem + ((uint32_t)lane_base << 16) + c, v);
-        tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c + j < rows_here) __stcg(my_partial + (size_t)(c + j) * kTileN, __uint_as_float(v[j]));
-      }
-      __threadfence();
-    }
-    if (lane == 0) warp_ok[warp - 2] = ok ? 1 : 0;
-    named_bar_sync(1, 128);
-    ok = warp_ok[0] && warp_ok[1] && warp_ok[2] && warp_ok[3];
-    // Split K: the n_split blocks of a tile share its final reduction.  Block s takes rows [lo, hi) of the tile; when
-    // all partial tiles are there (arrival counter; the blocks of a launch are all resident: there are no more of
-    // them than SMs) it fetches those rows of every partial tile into the shared memory of the pipeline stages, which
-    // are free by now, with bulk copies, all in flight at once.  (One block folding the other partial tiles with
-    // loads of its own took 6 us of a 16 us call at 32 rows and 37 of 52 us at 256: every batch of loads is a trip of
-    // about 2 us to data other SMs have just written.)  A second counter lets the last block to leave clear both.
-    const int red_lo = p.rows_pad * split / p.n_split, red_hi = p.rows_pad * (split + 1) / p.n_split;
-    const uint32_t slice_bytes = (uint32_t)(red_hi - red_lo) * kTileN * 4u;
-    if (p.n_split > 1) {
-      if (tid == 64) {   // first epilogue thread: every partial store above happened before the barrier
-        int go = 2;
-        unsigned int* const arrive = p.tickets + chunk * gridDim.x + tile;
-        unsigned int* const depart = arrive + kDlmMaxSplitUnits / 2;
-        if (ok) {
-          unsigned int t;
-          asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(arrive) : "memory");
-          if (wait_count(arrive, (unsigned int)p.n_split, abort_ptr)) {
-            fence_proxy_async_all();
-            mbar_expect_tx(bar_red, (uint32_t)p.n_split * slice_bytes);
-            for (int s2 = 0; s2 < p.n_split; ++s2)
-              bulk_load(base + s2 * slice_bytes, p.partial + ((tile_slot + s2) * (size_t)p.rows_pad + red_lo) * kTileN, slice_bytes,
-                        bar_red);
-            if (atomicAdd(depart, 1u) == (unsigned int)p.n_split - 1u) {   // every block of the tile is past its wait
-              *arrive = 0;
-              *depart = 0;
-            }
-            go = 1;
-          }
-        }
-        *is_last = go;
-      }
-      named_bar_sync(1, 128);
-    }
-    // where output feature `feat` of row (b, i) goes: element offset of (b = 0, i = 0) and the two strides
-    // ... and, for a key or value feature of a staging call, where its copy in the cache goes: element offset of
-    // (b = 0, cache row 0); rows are head_dim apart, batch elements n_kv_heads * capacity * head_dim
-    auto place = [&](int feat, __nv_bfloat16*& dst, size_t& row_stride, size_t& b_stride, __nv_bfloat16*& stage) {
-      stage = nullptr;
-      if (p.mode == 0) {
-        const int head = feat / p.head_dim, d = feat % p.head_dim;
-        int heads, h;
-        if (head < p.n_q_heads) { dst = p.q_out; heads = p.n_q_heads; h = head; }
-        else if (head < p.n_q_heads + p.n_kv_heads) { dst = p.k_out; heads = p.n_kv_heads; h = head - p.n_q_heads; stage = p.stage_k; }
-        else { dst = p.v_out; heads = p.n_kv_heads; h = head - p.n_q_heads - p.n_kv_heads; stage = p.stage_v; }
-        dst += (size_t)h * p.q_cap * p.head_dim + d;
-        if (stage) stage += (size_t)h * p.capacity * p.head_dim + d;
-        row_stride = p.head_dim;
-        b_stride = (size_t)heads * p.q_cap * p.head_dim;
-      } else {
-        dst = p.q_out + feat;
-        row_stride = p.n_out;
-        b_stride = (size_t)p.q_cap * p.n_out;
-      }
-    };
-    // cache row that window row i of batch element b is staged at, or -1: inactive row, or no room (reported)
-    auto stage_row = [&](int b, int i) -> int {
-      if (p.q_len && i >= __ldg(p.q_len + b)) return -1;
-      const int pos = __ldg(p.cache_len + b) + i;
-      if (pos < 0 || pos >= p.capacity) {
-        dlm_set_status(p.status, DLM_ERR_CAPACITY);
-        return -1;
-      }
-      return pos;
-    };
-    const size_t stage_b_stride = (size_t)p.n_kv_heads * p.capacity * p.head_dim;
-    if (ok && p.n_split == 1) {
-      // the whole sum is in TMEM: thread = feature, one 2-byte store per row (the output is small beside the weights)
-      const float bias = p.bias ? __bfloat162float(p.bias[n]) : 0.f;
-      __nv_bfloat16* dst;
-      __nv_bfloat16* stage;
-      size_t row_stride, b_stride;
-      place(n, dst, row_stride, b_stride, stage);
-      uint32_t v[32];
-      const bool turn = rope && n / p.head_dim < p.n_q_heads + p.n_kv_heads;   // the same for a feature and its partner
-      const int d = n % p.head_dim;
-      // the partner's values come through shared memory (the pipeline's first stage is free: every MMA has finished);
-      // [feature][33 floats]: 128 x 33 x 4 bytes fit a stage
-      float* const xch = reinterpret_cast<float*>(smem_raw + pad);
-      const int f_partner = d < half ? f + half : f - half;
-      if (!rope && !stage) {
-        // the plain projection: nothing but the bias between the accumulator and the store
-        for (int c = 0; c < p.rows_pad; c += 32) {
-          tmem_ld32(tmem + ((uint32_t)lane_base << 16) + c, v);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int r = row0 + c + j;
-            if (c + j < rows_here) {
-              const int b = r / p.q_cap, i = r % p.q_cap;
-              dst[(size_t)b * b_stride + (size_t)i * row_stride] = __float2bfloat16_rn(__uint_as_float(v[j]) + bias);
-            }
-          }
-        }
-      } else {
-        for (int c = 0; c < p.rows_pad; c += 32) {
-          tmem_ld32(tmem + ((uint32_t)lane_base << 16) + c, v);
-          tmem_ld_wait();
-          if (rope) {   // block-uniform: all four warps meet at the two barriers
-#pragma unroll
-            for (int j = 0; j < 32; ++j) xch[f * 33 + j] = __uint_as_float(v[j]) + bias;
-            named_bar_sync(1, 128);
-          }
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int r = row0 + c + j;
-            if (c + j < rows_here) {
-              const int b = r / p.q_cap, i = r % p.q_cap;
-              float y = __uint_as_float(v[j]) + bias;
-              if (turn) {
-                const size_t a = ((size_t)b * p.q_cap + i) * half + (d < half ? d : d - half);
-                const float cs = p.rope_cos[a], sn = p.rope_sin[a], other = xch[f_partner * 33 + j];
-                y = d < half ? y * cs - other * sn : y * cs + other * sn;
-              }
-              const __nv_bfloat16 yb = __float2bfloat16_rn(y);
-              dst[(size_t)b * b_stride + (size_t)i * row_stride] = yb;
-              if (stage) {
-                const int pos = stage_row(b, i);
-                if (pos >= 0) stage[(size_t)b * stage_b_stride + (size_t)pos * p.head_dim] = yb;
-              }
-            }
-          }
-          if (rope) named_bar_sync(1, 128);   // the next chunk overwrites the exchange area
-        }
-      }
-    } else if (ok && *is_last == 1) {
-      // every block adds its rows of the partial tiles in split order (the sum does not depend on the order of arrival): a
-      // thread takes 4 neighbouring features of every fourth row, 16-byte loads from shared memory, 8-byte stores; a
-      // warp's stores cover 128 features of one row
-      const bool landed = __all_sync(0xffffffffu, mbar_wait(bar_red, 0, abort_ptr)) != 0;
-      // the thread that issued the copies does not go on to the teardown before they have landed
-      if (tid == 64 && !landed) mbar_wait(bar_red, 0, never_ptr);
-      const int t = tid - 64;
-      const int fq = (t & 31) * 4;
-      const int n4 = tile * kTileN + fq;
-      float b4[4] = {0.f, 0.f, 0.f, 0.f};
-      if (p.bias)
-        for (int j = 0; j < 4; ++j) b4[j] = __bfloat162float(p.bias[n4 + j]);
-      __nv_bfloat16* dst;
-      __nv_bfloat16* stage;
-      size_t row_stride, b_stride;
-      place(n4, dst, row_stride, b_stride, stage);
-      const int red_end = landed ? min(red_hi, rows_here) : red_lo;   // rows beyond the call's hold nothing
-      for (int rr0 = red_lo + (t >> 5); rr0 < red_end; rr0 += 16) {
-        float4 accs[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) accs[j] = make_float4(b4[0], b4[1], b4[2], b4[3]);
-        for (int s2 = 0; s2 < p.n_split; ++s2) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (rr0 + 4 * j < red_end) {
-              const float4 x = ld_shared_f4(base + s2 * slice_bytes + (uint32_t)((rr0 + 4 * j - red_lo) * kTileN + fq) * 4u);
-              accs[j].x += x.x; accs[j].y += x.y; accs[j].z += x.z; accs[j].w += x.w;
-            }
-        }
+    if (ok && n_rows > 0) {
+      const int D = p.head_dim, half = D >> 1;
+      const bool rope = p.rope_cos != nullptr;
+      const int n_qk = p.n_q_heads + p.n_kv_heads;
+      constexpr int kCW = N / 2 < 32 ? N / 2 : 32;            // columns of a segment
+      constexpr uint32_t kPitch = 2 * kCW * 4 + 16;           // bytes of a staged row; the 16 spread rows over the banks
+      constexpr int kLanes = kCW / 8, kRowsPerIt = kThreads / kLanes;
+      constexpr int kIts = kRowTile > kRowsPerIt ? kRowTile / kRowsPerIt : 1;
+      const int dist = rope && N > D ? half : N / 2;          // columns between a segment and its partner
+      // TMEM side: warps w and w + 4 read the lanes of quarter w % 4, one segment each.  The row of a lane: M = 64 puts 16
+      // rows in each quarter; M = 128 as a pair puts rows 0-63 twice, lanes 64-127 holding the second half of the columns.
+      const int quarter = warp & 3, seg = warp >> 2;
+      const int my_row = M == 64 ? quarter * 16 + lane : M == 128 ? (quarter & 1) * 32 + lane : quarter * 32 + lane;
+      const bool my_lane = (M != 64 || lane < 16) && my_row < n_rows;
+      const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
+      // store side: where features f .. f + 7 (one head) go
+      struct Dest {
+        __nv_bfloat16 *out, *stage;
+        bool kv;
+      };
+      auto dest = [&](int f) {
+        Dest d;
+        d.stage = nullptr;
+        d.kv = false;
+        if (p.mode == 1) { d.out = p.q_out + f; return d; }
+        const int head = p.head_shift >= 0 ? f >> p.head_shift : f / D, df = f - head * D;
+        if (head < p.n_q_heads) { d.out = p.q_out + (size_t)head * p.q_cap * D + df; return d; }
+        const bool is_k = head < n_qk;
+        const size_t h = is_k ? head - p.n_q_heads : head - n_qk;
+        d.kv = true;
+        d.out = (is_k ? p.k_out : p.v_out) + h * p.q_cap * D + df;
+        if (p.stage_k) d.stage = (is_k ? p.stage_k : p.stage_v) + h * p.capacity * D + df;
+        return d;
+      };
+      auto store8 = [&](const Dest& d, const RowEntry& e, const float* y) {
+        uint32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int rr = rr0 + 4 * j;
-          if (rr >= red_end) break;   // the same for the whole warp
-          float4 acc = accs[j];
-          const int r = row0 + rr;
-          const int b = r / p.q_cap, i = r % p.q_cap;
-          if (rope) {
-            // this lane's 4 features and their partners' (head_dim / 2 features = head_dim / 8 lanes away) turn together;
-            // rr is the same for the whole warp, so every lane is here for the exchange
-            const int dl = p.head_dim >> 3;
-            const float4 o = make_float4(__shfl_xor_sync(0xffffffffu, acc.x, dl), __shfl_xor_sync(0xffffffffu, acc.y, dl),
-                                         __shfl_xor_sync(0xffffffffu, acc.z, dl), __shfl_xor_sync(0xffffffffu, acc.w, dl));
-            const int d = n4 % p.head_dim;
-            if (n4 / p.head_dim < p.n_q_heads + p.n_kv_heads) {
-              const size_t a = ((size_t)b * p.q_cap + i) * half + (d < half ? d : d - half);
-              const float4 cs = __ldg(reinterpret_cast<const float4*>(p.rope_cos + a));
-              const float4 sn = __ldg(reinterpret_cast<const float4*>(p.rope_sin + a));
-              const float sg = d < half ? -1.f : 1.f;
-              acc.x = fmaf(sg * o.x, sn.x, acc.x * cs.x);
-              acc.y = fmaf(sg * o.y, sn.y, acc.y * cs.y);
-              acc.z = fmaf(sg * o.z, sn.z, acc.z * cs.z);
-              acc.w = fmaf(sg * o.w, sn.w, acc.w * cs.w);
+          const __nv_bfloat162 h = __floats2bfloat162_rn(y[2 * j], y[2 * j + 1]);
+          w[j] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(d.out + (d.kv ? e.kv : e.q)) = v;
+        if (d.stage && e.stage >= 0) *reinterpret_cast<uint4*>(d.stage + e.stage) = v;
+      };
+      uint32_t buf = base;
+      for (int g = 0; g < N; g += 2 * dist) {
+        for (int c = g; c < g + dist; c += kCW) {
+          const int cc = c + (tid % kLanes) * 8;             // this thread's 8 columns when it stores, and the 8 at cc + dist
+          const int f0 = feature(cc), f1 = feature(cc + dist);
+          const bool turn = rope && (f0 >> p.head_shift) < n_qk;
+          float4 cs[kIts][2], sn[kIts][2];
+          if (turn) {   // asked for before the accumulator is read
+#pragma unroll
+            for (int it = 0; it < kIts; ++it) {
+              const int r = tid / kLanes + it * kRowsPerIt;
+              if (r < n_rows) {
+                const size_t a = (size_t)row_s[r].rope + (f0 & (D - 1));
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                  cs[it][j] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + a) + j);
+                  sn[it][j] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + a) + j);
+                }
+              }
             }
           }
-          const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
-          uint2 pk;
-          pk.x = *reinterpret_cast<const uint32_t*>(&lo);
-          pk.y = *reinterpret_cast<const uint32_t*>(&hi);
-          *reinterpret_cast<uint2*>(dst + (size_t)b * b_stride + (size_t)i * row_stride) = pk;
-          if (stage) {
-            const int pos = stage_row(b, i);
-            if (pos >= 0) *reinterpret_cast<uint2*>(stage + (size_t)b * stage_b_stride + (size_t)pos * p.head_dim) = pk;
+          int col = c + seg * dist;
+          bool here = true;
+          if (M == 128) {
+            here = col / (N / 2) == quarter >> 1;            // warp-uniform
+            col %= N / 2;
           }
+          if (here) {
+            uint32_t u[kCW];
+            __syncwarp();
+            if (kCW == 32) tmem_ld32(t_row + col, u);
+            else if (kCW == 16) tmem_ld16(t_row + col, u);
+            else tmem_ld8(t_row + col, u);
+            tmem_ld_wait();
+            if (my_lane) {
+              const uint32_t a = buf + my_row * kPitch + seg * kCW * 4;
+#pragma unroll
+              for (int j = 0; j < kCW; j += 4)
+                st_shared_f4(a + j * 4, __uint_as_float(u[j]), __uint_as_float(u[j + 1]), __uint_as_float(u[j + 2]), __uint_as_float(u[j + 3]));
+            }
+          }
+          const Dest d0 = dest(f0), d1 = dest(f1);
+          float b0[8], b1[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) { b0[j] = bias_s[cc + j]; b1[j] = bias_s[cc + dist + j]; }
+          __syncthreads();
+#pragma unroll
+          for (int it = 0; it < kIts; ++it) {
+            const int r = tid / kLanes + it * kRowsPerIt;
+            if (r < n_rows) {
+              const RowEntry e = row_s[r];
+              const uint32_t a = buf + r * kPitch + (tid % kLanes) * 32;
+              float y0[8], y1[8];
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                const float4 lo = ld_shared_f4(a + 16 * j), hi = ld_shared_f4(a + kCW * 4 + 16 * j);
+                y0[4 * j] = lo.x; y0[4 * j + 1] = lo.y; y0[4 * j + 2] = lo.z; y0[4 * j + 3] = lo.w;
+                y1[4 * j] = hi.x; y1[4 * j + 1] = hi.y; y1[4 * j + 2] = hi.z; y1[4 * j + 3] = hi.w;
+              }
+#pragma unroll
+              for (int j = 0; j < 8; ++j) { y0[j] += b0[j]; y1[j] += b1[j]; }
+              if (turn) {
+                const float co[8] = {cs[it][0].x, cs[it][0].y, cs[it][0].z, cs[it][0].w, cs[it][1].x, cs[it][1].y, cs[it][1].z, cs[it][1].w};
+                const float si[8] = {sn[it][0].x, sn[it][0].y, sn[it][0].z, sn[it][0].w, sn[it][1].x, sn[it][1].y, sn[it][1].z, sn[it][1].w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const float lo = y0[j], hi = y1[j];
+                  y0[j] = fmaf(-hi, si[j], lo * co[j]);
+                  y1[j] = fmaf(lo, si[j], hi * co[j]);
+                }
+              }
+              store8(d0, e, y0);
+              store8(d1, e, y1);
+            }
+          }
+          buf = buf == base ? base + kRowTile * kPitch : base;   // the next piece's writes meet no reader of this one
         }
       }
     }
@@ -408,10 +373,11 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   __syncwarp();
   if (tid == 0 && *abort_ptr) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
   tc_fence_before_sync();
-  __syncthreads();
-  if (warp == 1) {
+  // a pair leaves together: the leader's MMAs read the other block's shared memory, both blocks' copies complete on the leader's barriers
+  if (PAIR) cluster_sync(); else __syncthreads();
+  if (warp == 3) {
     tc_fence_after_sync();
-    tmem_dealloc(tmem, tmem_cols);
+    if (PAIR) tmem_dealloc_pair(tmem, kTmemCols); else tmem_dealloc(tmem, kTmemCols);
   }
 }
 
@@ -419,8 +385,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// bf16 tensor viewed as [slabs][rows][inner]; box = 64 elements x box_rows rows x 1 slab, 128-byte swizzle.
-int encode_map3(dlm_ctx* ctx, CUtensorMap* map, const void* base, long long inner, long long rows, long long slabs, int box_rows) {
+// bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle.
+int encode_map(dlm_ctx* ctx, CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+               const cuuint32_t* box) {
   if (!ctx->encode_tiled) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -429,80 +396,131 @@ int encode_map3(dlm_ctx* ctx, CUtensorMap* map, const void* base, long long inne
       return DLM_ERR_CUDA;
     ctx->encode_tiled = fn;
   }
-  const cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)slabs};
-  const cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)rows * inner * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-  const cuuint32_t elem[3] = {1, 1, 1};
+  const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
   const CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
-      map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
+      map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, elem,
       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? DLM_OK : DLM_ERR_CUDA;
 }
 
-struct ProjPlan {
-  int rows_pad, chunks, tiles, n_split, k_per_split, n_stages, smem_bytes;
-  size_t ws_bytes;
+using ProjKernel = void (*)(const CUtensorMap, const CUtensorMap, const ProjParams);
+struct ProjVariant {
+  int n, m, kp;
+  ProjKernel fn;
+};
+// N features, M rows, K panels per stage (stages of 16 - 40 KB)
+const ProjVariant kVariants[] = {
+    {16, 64, 4, window_proj_kernel<16, 64, 4>},     {32, 64, 4, window_proj_kernel<32, 64, 4>},
+    {64, 64, 2, window_proj_kernel<64, 64, 2>},     {128, 64, 2, window_proj_kernel<128, 64, 2>},
+    {64, 128, 2, window_proj_kernel<64, 128, 2>},   {128, 128, 2, window_proj_kernel<128, 128, 2>},
+    {256, 128, 1, window_proj_kernel<256, 128, 1>}, {64, 256, 2, window_proj_kernel<64, 256, 2>},
+    {128, 256, 1, window_proj_kernel<128, 256, 1>}, {256, 256, 1, window_proj_kernel<256, 256, 1>},
 };
 
-// rows: activation rows of the call; whole_rows: every block sees all rows (head-split activations)
-bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, bool whole_rows, ProjPlan& pl) {
-  if (whole_rows && rows > kMaxRows) return false;
-  pl.chunks = (rows + kMaxRows - 1) / kMaxRows;
-  const int rows_chunk = pl.chunks == 1 ? rows : kMaxRows;
-  pl.rows_pad = (rows_chunk + 31) & ~31;
-  pl.tiles = n_out / kTileN;
-  const int k_chunks = k_total / kChunkK;
-  // split K so that about one block per SM streams weights, each with at least four stages' worth of K
-  int split = ctx->num_sms / (pl.tiles * pl.chunks);
-  if (split > k_chunks / 4) split = k_chunks / 4;
-  if (split < 1) split = 1;
-  const int chunks_per_split = (k_chunks + split - 1) / split;
-  pl.n_split = (k_chunks + chunks_per_split - 1) / chunks_per_split;
-  pl.k_per_split = chunks_per_split * kChunkK;
-  const int stage = kWBytes + pl.rows_pad * 128;
-  const int aux = 16 * kMaxStages + 16 + 64;
-  int stages = (ctx->max_smem_optin - 1024 - aux) / stage;
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages > chunks_per_split) stages = chunks_per_split;
-  if (stages < 2) return false;
-  pl.n_stages = stages;
-  // the shared final reduction parks every partial tile's slice of a block's rows in the stages' memory
-  if (pl.n_split > 1 && (long long)stages * stage < (long long)(pl.rows_pad + pl.n_split) * kTileN * 4) {
-    pl.n_split = 1;
-    pl.k_per_split = k_chunks * kChunkK;
+struct ProjPlan {
+  int variant, rc, x_box_rows, chunks, tiles, half_rows, n_stages, aux_offset, smem_bytes;
+};
+
+int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
+
+// rows: activation rows of the call; heads_q_cap > 0: head-split activations (all rows in one chunk) with that many rows
+// per sequence, `batch` sequences.
+bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int head_dim, int batch, int heads_q_cap, ProjPlan& pl) {
+  const int m = rows <= 64 ? 64 : rows <= 128 ? 128 : 256;
+  const bool pair = m > 64;
+  if (heads_q_cap > 0 && rows > kMaxActRows) return false;
+  pl.chunks = pair ? (rows + 255) / 256 : 1;
+  const int blocks_rows = pl.chunks * (pair ? 2 : 1);
+  pl.rc = ((rows + blocks_rows - 1) / blocks_rows + 7) & ~7;
+  pl.x_box_rows = pl.rc;
+  if (heads_q_cap > 0 && batch > 1) {
+    // one copy brings the rows of whole sequences; where the pair's split falls inside one, copies of a common divisor
+    const int nb = (batch + blocks_rows - 1) / blocks_rows;
+    if (nb * heads_q_cap <= (m == 128 ? 64 : 128)) {
+      pl.rc = pl.x_box_rows = nb * heads_q_cap;
+    } else {
+      pl.x_box_rows = gcd(heads_q_cap, m == 128 ? 64 : 128);
+      pl.rc = (pl.rc + pl.x_box_rows - 1) / pl.x_box_rows * pl.x_box_rows;
+    }
   }
-  pl.smem_bytes = 1024 + stages * stage + aux;
-  pl.ws_bytes = pl.n_split > 1 ? (size_t)pl.chunks * pl.tiles * pl.n_split * pl.rows_pad * kTileN * sizeof(float) : 0;
-  return (long long)pl.tiles * pl.chunks <= kDlmMaxSplitUnits / 2;   // two counters per tile
+  // The tile width: estimated cycles of the SM with the most blocks.  Per 16 elements of K a block's MMA takes N / 2
+  // cycles, or what its operands take at 128 bytes per cycle of shared memory, and its operands arrive at about 70 bytes
+  // per cycle and SM (measured); a block costs some fixed time on top.
+  double best = 0;
+  pl.variant = -1;
+  for (int v = 0; v < (int)(sizeof(kVariants) / sizeof(kVariants[0])); ++v) {
+    const ProjVariant& k = kVariants[v];
+    if (k.m != m || n_out % k.n != 0) continue;
+    const long long blocks = (long long)(n_out / k.n) * blocks_rows;
+    const double per_sm = (double)((blocks + ctx->num_sms - 1) / ctx->num_sms);
+    const double mma = m == 256 ? k.n / 2.0 : k.n / 4.0, smem = ((m == 256 ? 4096.0 : 2048.0) + k.n * (pair ? 16.0 : 32.0)) / 128.0;
+    const double intake = (pl.rc + k.n / (pair ? 2 : 1)) * 32.0 / 70.0;
+    double cyc = mma > smem ? mma : smem;
+    if (intake > cyc) cyc = intake;
+    const double t = per_sm * (k_total / 16.0 * cyc + 1000.0 + 12.0 * k.n);
+    if (pl.variant < 0 || t < best) { best = t; pl.variant = v; }
+  }
+  if (pl.variant < 0) return false;
+  const ProjVariant& k = kVariants[pl.variant];
+  pl.tiles = n_out / k.n;
+  // rotary pairs inside a tile: see the kernel
+  pl.half_rows = (head_dim == 64 || head_dim == 128) && k.n < head_dim ? head_dim / 2 : k.n / 2;
+  const int stage = k.kp * 128 * (pl.rc + k.n / (pair ? 2 : 1));
+  const int n_k = (k_total / kPanel + k.kp - 1) / k.kp;
+  // Single blocks stay below half of an SM's shared memory, so that the next kernel's blocks can start beside them and
+  // prefetch their weights; pairs want depth (with 5 stages instead of 3: 20.2 -> 16.4 us at 256 Dream rows).
+  const int fixed = 1024 + 16384 + kAuxBytes;
+  int stages = ((pair ? 220 : 113) * 1024 - fixed) / stage;
+  if (stages < 3) stages = 3;
+  if (stages > kMaxStages) stages = kMaxStages;
+  if (stages > n_k) stages = n_k;
+  pl.n_stages = stages;
+  // Behind the stages: the MMA of the last stage's last activation panel reads the rows up to M, which no copy filled
+  // (their results are never looked at).  The epilogue's two staging buffers lie over the stages.
+  const int row_tile = m == 64 ? 64 : m / 2, cw = k.n / 2 < 32 ? k.n / 2 : 32;
+  const int staging = 2 * row_tile * (2 * cw * 4 + 16);
+  pl.aux_offset = stages * stage + 16384;
+  if (pl.aux_offset < staging) pl.aux_offset = (staging + 127) & ~127;
+  pl.smem_bytes = 1024 + pl.aux_offset + kAuxBytes;
+  return pl.smem_bytes <= ctx->max_smem_optin && pl.chunks <= 65535;
 }
 
-int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, void* workspace,
-                size_t workspace_bytes, cudaStream_t s) {
-  if (pl.ws_bytes > 0 && (!workspace || workspace_bytes < pl.ws_bytes || ((uintptr_t)workspace & 255))) return DLM_ERR_WORKSPACE;
-  if (!ctx->proj_configured) {
-    DLM_CUDA_TRY(cudaFuncSetAttribute(window_proj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin));
-    ctx->proj_configured = true;
+int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, cudaStream_t s) {
+  const ProjVariant& k = kVariants[pl.variant];
+  const int cluster = k.m > 64 ? 2 : 1;
+  if (!(ctx->proj_configured & (1u << pl.variant))) {
+    DLM_CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin));
+    ctx->proj_configured |= 1u << pl.variant;
   }
-  p.partial = static_cast<float*>(workspace);
-  p.tickets = ctx->words->attn_unit_tickets;
-  p.rows_pad = pl.rows_pad;
-  p.n_split = pl.n_split;
-  p.k_per_split = pl.k_per_split;
+  p.rc = pl.rc;
+  p.x_box_rows = pl.x_box_rows;
+  p.half_rows = pl.half_rows;
   p.n_stages = pl.n_stages;
+  p.aux_offset = pl.aux_offset;
+  p.head_shift = p.head_dim == 128 ? 7 : p.head_dim == 64 ? 6 : -1;
   p.status = &ctx->words->status;
-  DLM_CUDA_TRY(dlm_launch(window_proj_kernel, dim3(pl.tiles, pl.n_split, pl.chunks), dim3(kThreads), (size_t)pl.smem_bytes, s, tm_w,
-                          tm_x, p));
+  DLM_CUDA_TRY(dlm_launch_cluster(k.fn, dim3(pl.tiles * cluster, 1, pl.chunks), dim3(kThreads), (size_t)pl.smem_bytes, s,
+                                  cluster, tm_w, tm_x, p));
   return dlm_launch_ok(ctx, 1);
+}
+
+// W seen as [groups][2][half_rows][K / 64][64]; a copy brings n / 2 features of one half (pairs) or of both, kp panels.
+int encode_weights(dlm_ctx* ctx, CUtensorMap* map, const void* w, int n_out, int k_total, const ProjPlan& pl) {
+  const ProjVariant& k = kVariants[pl.variant];
+  const cuuint64_t row = (cuuint64_t)k_total * 2, a = (cuuint64_t)pl.half_rows;
+  const cuuint64_t dims[5] = {(cuuint64_t)kPanel, a, 2, (cuuint64_t)(k_total / kPanel), (cuuint64_t)n_out / (2 * a)};
+  const cuuint64_t strides[4] = {row, a * row, (cuuint64_t)kPanel * 2, 2 * a * row};
+  const cuuint32_t box[5] = {(cuuint32_t)kPanel, (cuuint32_t)k.n / 2, k.m > 64 ? 1u : 2u, (cuuint32_t)k.kp, 1};
+  return encode_map(ctx, map, w, 5, dims, strides, box);
 }
 
 }  // namespace
 
+// The kernels sum all of K in one block (pair) and need no scratch; what is left is a non-zero answer for valid sizes.
 extern "C" size_t dlm_window_proj_workspace_bytes(const dlm_ctx* ctx, int rows, int n_out, int k_total) {
-  if (!ctx || rows <= 0 || n_out <= 0 || k_total <= 0 || n_out % kTileN != 0 || k_total % kChunkK != 0) return 0;
-  ProjPlan pl;
-  if (!make_proj_plan(ctx, rows, n_out, k_total, false, pl)) return 0;
-  return pl.ws_bytes + 256;
+  if (!ctx || rows <= 0 || n_out <= 0 || k_total <= 0 || n_out % 128 != 0 || k_total % kPanel != 0) return 0;
+  return 256;
 }
 
 namespace {
@@ -556,21 +574,27 @@ int qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, co
   if (batch <= 0 || q_cap <= 0 || d_model <= 0 || n_q_heads <= 0 || n_kv_heads <= 0 || head_dim <= 0) return DLM_ERR_SHAPE;
   const long long n_out = (long long)(n_q_heads + 2 * n_kv_heads) * head_dim;
   const long long rows = (long long)batch * q_cap;
-  if (n_out % kTileN != 0 || d_model % kChunkK != 0 || head_dim % 8 != 0 || rows > (1 << 20) || n_out > (1 << 24))
+  if (n_out % 128 != 0 || d_model % kPanel != 0 || head_dim % 8 != 0 || rows > (1 << 20) || n_out > (1 << 24))
     return DLM_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w | (uintptr_t)q_out | (uintptr_t)k_out | (uintptr_t)v_out) & 15) return DLM_ERR_UNSUPPORTED;
   DLM_DEVICE_TRY(ctx);
   ProjPlan pl;
-  if (!make_proj_plan(ctx, (int)rows, (int)n_out, d_model, false, pl)) return DLM_ERR_UNSUPPORTED;
+  if (!make_proj_plan(ctx, (int)rows, (int)n_out, d_model, head_dim, batch, 0, pl)) return DLM_ERR_UNSUPPORTED;
   CUtensorMap tm_w, tm_x;
-  int rc = encode_map3(ctx, &tm_w, w, d_model, n_out, 1, kTileN);
-  if (rc == DLM_OK) rc = encode_map3(ctx, &tm_x, x, d_model, rows, 1, pl.rows_pad);
+  int rc = encode_weights(ctx, &tm_w, w, (int)n_out, d_model, pl);
+  if (rc == DLM_OK) {
+    const cuuint64_t dims[4] = {(cuuint64_t)kPanel, (cuuint64_t)rows, (cuuint64_t)(d_model / kPanel), 1};
+    const cuuint64_t strides[3] = {(cuuint64_t)d_model * 2, (cuuint64_t)kPanel * 2, (cuuint64_t)d_model * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)kPanel, (cuuint32_t)pl.rc, (cuuint32_t)kVariants[pl.variant].kp, 1};
+    rc = encode_map(ctx, &tm_x, x, 4, dims, strides, box);
+  }
   if (rc != DLM_OK) return rc;
   ProjParams p = {};
   p.mode = 0;
   p.q_out = static_cast<__nv_bfloat16*>(q_out);
   p.k_out = static_cast<__nv_bfloat16*>(k_out);
   p.v_out = static_cast<__nv_bfloat16*>(v_out);
+  p.w = static_cast<const __nv_bfloat16*>(w);
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.rope_cos = rope_cos;
   p.rope_sin = rope_sin;
@@ -584,7 +608,7 @@ int qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, co
   }
   p.rows_total = (int)rows; p.q_cap = q_cap; p.n_q_heads = n_q_heads; p.n_kv_heads = n_kv_heads; p.head_dim = head_dim;
   p.n_out = (int)n_out; p.k_total = d_model; p.batch = batch; p.act_heads = 0;
-  return launch_proj(ctx, pl, p, tm_w, tm_x, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
+  return launch_proj(ctx, pl, p, tm_w, tm_x, static_cast<cudaStream_t>(stream));
 }
 }  // namespace
 
@@ -596,23 +620,29 @@ extern "C" int dlm_window_out_project(dlm_ctx* ctx, const void* o, const void* w
   const long long k_total = (long long)n_q_heads * head_dim, rows = (long long)batch * q_cap;
   // a stage holds 64 features of one head for every row of the call: whole heads of 64-element panels, all rows in
   // one block (<= 256), and each batch element's rows starting on a swizzle-atom boundary (8 rows)
-  if (d_model % kTileN != 0 || head_dim % kChunkK != 0 || rows > kMaxRows || (batch > 1 && q_cap % 8 != 0))
+  if (d_model % 128 != 0 || head_dim % kPanel != 0 || rows > kMaxActRows || (batch > 1 && q_cap % 8 != 0))
     return DLM_ERR_UNSUPPORTED;
   if (((uintptr_t)o | (uintptr_t)wo | (uintptr_t)y) & 15) return DLM_ERR_UNSUPPORTED;
   DLM_DEVICE_TRY(ctx);
   ProjPlan pl;
-  if (!make_proj_plan(ctx, (int)rows, d_model, (int)k_total, true, pl)) return DLM_ERR_UNSUPPORTED;
+  if (!make_proj_plan(ctx, (int)rows, d_model, (int)k_total, 0, batch, q_cap, pl)) return DLM_ERR_UNSUPPORTED;
   CUtensorMap tm_w, tm_x;
-  int rc = encode_map3(ctx, &tm_w, wo, k_total, d_model, 1, kTileN);
-  // one box per batch element: q_cap rows; the rows of the panel beyond batch * q_cap stay as they are (their
-  // accumulator columns are never read)
-  if (rc == DLM_OK) rc = encode_map3(ctx, &tm_x, o, head_dim, q_cap, (long long)batch * n_q_heads, q_cap);
+  int rc = encode_weights(ctx, &tm_w, wo, d_model, (int)k_total, pl);
+  if (rc == DLM_OK) {
+    // a box brings one 64-element panel of one head: the rows of whole sequences, or part of one sequence's rows
+    const int box_seqs = batch > 1 && pl.x_box_rows % q_cap == 0 ? pl.x_box_rows / q_cap : 1;
+    const cuuint64_t dims[4] = {(cuuint64_t)head_dim, (cuuint64_t)q_cap, (cuuint64_t)n_q_heads, (cuuint64_t)batch};
+    const cuuint64_t strides[3] = {(cuuint64_t)head_dim * 2, (cuuint64_t)q_cap * head_dim * 2, (cuuint64_t)k_total * q_cap * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)kPanel, (cuuint32_t)(pl.x_box_rows / box_seqs), 1, (cuuint32_t)box_seqs};
+    rc = encode_map(ctx, &tm_x, o, 4, dims, strides, box);
+  }
   if (rc != DLM_OK) return rc;
   ProjParams p = {};
   p.mode = 1;
   p.q_out = static_cast<__nv_bfloat16*>(y);
+  p.w = static_cast<const __nv_bfloat16*>(wo);
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.rows_total = (int)rows; p.q_cap = q_cap; p.n_q_heads = n_q_heads; p.n_kv_heads = 0; p.head_dim = head_dim;
   p.n_out = d_model; p.k_total = (int)k_total; p.batch = batch; p.act_heads = n_q_heads;
-  return launch_proj(ctx, pl, p, tm_w, tm_x, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
+  return launch_proj(ctx, pl, p, tm_w, tm_x, static_cast<cudaStream_t>(stream));
 }

@@ -1,9 +1,10 @@
-"""ctypes binding of libdlm.so: argument marshalling only.
+"""Binding of libdlm.so: argument marshalling only.
 
 Every function has the name and the argument order of its C counterpart in include/dlm.h.
 Tensors are torch CUDA tensors (PyTorch is used for device memory and streams only); each
-call passes raw device pointers and the current CUDA stream.  There is no fallback: if the
-library is missing or a call fails, an exception is raised.
+call passes raw device pointers and the current CUDA stream.  The calls that enqueue kernels come
+from the native module _dlm_calls (csrc/py_calls.cpp); context, size and diagnostic calls go through
+ctypes.  There is no fallback: if the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -150,14 +151,6 @@ def make_kv_cache(k: torch.Tensor, v: torch.Tensor, cache_len: torch.Tensor) -> 
     return c
 
 
-def dlm_kv_cache_commit(ctx, cache, k_new, v_new, src_len, src_idx, dst_pos, dst_mode, n_rows, n_max, advance_len,
-                        layer_begin, layer_end) -> None:
-    _check(lib().dlm_kv_cache_commit(
-        ctx, ctypes.byref(cache), _ptr(k_new, torch.bfloat16), _ptr(v_new, torch.bfloat16), int(src_len),
-        _ptr(src_idx, torch.int32), _ptr(dst_pos, torch.int32), int(dst_mode), _ptr(n_rows, torch.int32), int(n_max),
-        int(bool(advance_len)), int(layer_begin), int(layer_end), _stream()), "dlm_kv_cache_commit")
-
-
 def dlm_attn_workspace_bytes(ctx, cache, n_layers_in_call, n_q_heads, q_cap) -> int:
     return int(lib().dlm_attn_workspace_bytes(ctx, ctypes.byref(cache), int(n_layers_in_call), int(n_q_heads),
                                               int(q_cap)))
@@ -171,51 +164,8 @@ def dlm_selftest_attn_schedule(ctx, cache, n_layers_in_call, n_q_heads, q_cap, c
     return {"grid": g.value, "team": c.value, "whole_units": w.value, "chunk_rows": r.value}
 
 
-def dlm_freecache_attn_step(ctx, cache, layer_begin, layer_end, q, k_new, v_new, n_q_heads, q_cap, q_len,
-                            softmax_scale, cache_len_hint, out, lse, workspace) -> None:
-    _check(lib().dlm_freecache_attn_step(
-        ctx, ctypes.byref(cache), int(layer_begin), int(layer_end), _ptr(q, torch.bfloat16),
-        _ptr(k_new, torch.bfloat16), _ptr(v_new, torch.bfloat16), int(n_q_heads), int(q_cap),
-        _ptr(q_len, torch.int32), float(softmax_scale), int(cache_len_hint), _ptr(out, torch.bfloat16),
-        _ptr(lse, torch.float32), _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
-        "dlm_freecache_attn_step")
-
-
 def dlm_unmask_workspace_bytes(ctx, batch, block_len, vocab) -> int:
     return int(lib().dlm_unmask_workspace_bytes(ctx, int(batch), int(block_len), int(vocab)))
-
-
-def dlm_unmask_select(ctx, logits, batch, block_len, vocab, masked, tokens, k, tok, conf, sel_idx, n_sel,
-                      workspace) -> None:
-    _check(lib().dlm_unmask_select(
-        ctx, _ptr(logits, torch.float32), int(batch), int(block_len), int(vocab), _ptr(masked, torch.uint8),
-        _ptr(tokens, torch.int32), int(k), _ptr(tok, torch.int32), _ptr(conf, torch.float32),
-        _ptr(sel_idx, torch.int32), _ptr(n_sel, torch.int32), _ptr(workspace),
-        workspace.numel() * workspace.element_size(), _stream()), "dlm_unmask_select")
-
-
-def dlm_unmask_select_static(logits, batch, block_len, vocab, masked, tokens, k, tok, conf, sel_idx, n_sel) -> None:
-    """dlm_unmask_select without a context or a workspace (scratch is a fixed array inside the library)."""
-    _check(lib().dlm_unmask_select_static(
-        _ptr(logits, torch.float32), int(batch), int(block_len), int(vocab), _ptr(masked, torch.uint8),
-        _ptr(tokens, torch.int32), int(k), _ptr(tok, torch.int32), _ptr(conf, torch.float32),
-        _ptr(sel_idx, torch.int32), _ptr(n_sel, torch.int32), _stream()), "dlm_unmask_select_static")
-
-
-def dlm_guided_accept(ctx, tok_dlm, tok_ar, batch, block_len, masked, tokens, fallback_source, accept,
-                      acc_idx, n_acc) -> None:
-    _check(lib().dlm_guided_accept(
-        ctx, _ptr(tok_dlm, torch.int32), _ptr(tok_ar, torch.int32), int(batch), int(block_len),
-        _ptr(masked, torch.uint8), _ptr(tokens, torch.int32), int(fallback_source), _ptr(accept, torch.uint8),
-        _ptr(acc_idx, torch.int32), _ptr(n_acc, torch.int32), _stream()), "dlm_guided_accept")
-
-
-def dlm_guided_accept_topk(ctx, tok_dlm, tok_ar_topk, top_k, batch, block_len, masked, tokens, fallback_source, accept,
-                           acc_idx, n_acc) -> None:
-    _check(lib().dlm_guided_accept_topk(
-        ctx, _ptr(tok_dlm, torch.int32), _ptr(tok_ar_topk, torch.int32), int(top_k), int(batch), int(block_len),
-        _ptr(masked, torch.uint8), _ptr(tokens, torch.int32), int(fallback_source), _ptr(accept, torch.uint8),
-        _ptr(acc_idx, torch.int32), _ptr(n_acc, torch.int32), _stream()), "dlm_guided_accept_topk")
 
 
 DLM_SCORE_CONFIDENCE, DLM_SCORE_NEG_ENTROPY, DLM_SCORE_MARGIN, DLM_SCORE_LOG_CONF_PLUS_NOISE = 0, 1, 2, 3
@@ -225,62 +175,8 @@ def dlm_unmask_scored_workspace_bytes(ctx, batch, block_len, vocab) -> int:
     return int(lib().dlm_unmask_scored_workspace_bytes(ctx, int(batch), int(block_len), int(vocab)))
 
 
-def dlm_unmask_select_scored(ctx, logits, batch, block_len, vocab, masked, tokens, k, score_kind, noise, tok, conf, score,
-                             zmax, sel_idx, n_sel, workspace) -> None:
-    _check(lib().dlm_unmask_select_scored(
-        ctx, _ptr(logits, torch.float32), int(batch), int(block_len), int(vocab), _ptr(masked, torch.uint8),
-        _ptr(tokens, torch.int32), int(k), int(score_kind), _ptr(noise, torch.float32), _ptr(tok, torch.int32),
-        _ptr(conf, torch.float32), _ptr(score, torch.float32), _ptr(zmax, torch.float32), _ptr(sel_idx, torch.int32),
-        _ptr(n_sel, torch.int32), _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
-        "dlm_unmask_select_scored")
-
-
-def dlm_guided_accept_threshold(ctx, tok_dlm, zmax_dlm, tok_ar_topk, logit_ar_topk, top_k, tau, batch, block_len, masked,
-                                tokens, fallback_source, accept, acc_idx, n_acc) -> None:
-    _check(lib().dlm_guided_accept_threshold(
-        ctx, _ptr(tok_dlm, torch.int32), _ptr(zmax_dlm, torch.float32), _ptr(tok_ar_topk, torch.int32),
-        _ptr(logit_ar_topk, torch.float32), int(top_k), float(tau), int(batch), int(block_len), _ptr(masked, torch.uint8),
-        _ptr(tokens, torch.int32), int(fallback_source), _ptr(accept, torch.uint8), _ptr(acc_idx, torch.int32),
-        _ptr(n_acc, torch.int32), _stream()), "dlm_guided_accept_threshold")
-
-
 def dlm_window_proj_workspace_bytes(ctx, rows, n_out, k_total) -> int:
     return int(lib().dlm_window_proj_workspace_bytes(ctx, int(rows), int(n_out), int(k_total)))
-
-
-def dlm_window_qkv_project(ctx, x, w, bias, batch, q_cap, d_model, n_q_heads, n_kv_heads, head_dim, q_out, k_out, v_out,
-                           workspace) -> None:
-    _check(lib().dlm_window_qkv_project(
-        ctx, _ptr(x, torch.bfloat16), _ptr(w, torch.bfloat16), _ptr(bias, torch.bfloat16), int(batch), int(q_cap), int(d_model),
-        int(n_q_heads), int(n_kv_heads), int(head_dim), _ptr(q_out, torch.bfloat16), _ptr(k_out, torch.bfloat16),
-        _ptr(v_out, torch.bfloat16), _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
-        "dlm_window_qkv_project")
-
-
-def dlm_window_qkv_project_rope(ctx, x, w, bias, rope_cos, rope_sin, batch, q_cap, d_model, n_q_heads, n_kv_heads, head_dim,
-                                q_out, k_out, v_out, workspace) -> None:
-    _check(lib().dlm_window_qkv_project_rope(
-        ctx, _ptr(x, torch.bfloat16), _ptr(w, torch.bfloat16), _ptr(bias, torch.bfloat16), _ptr(rope_cos, torch.float32),
-        _ptr(rope_sin, torch.float32), int(batch), int(q_cap), int(d_model), int(n_q_heads), int(n_kv_heads), int(head_dim),
-        _ptr(q_out, torch.bfloat16), _ptr(k_out, torch.bfloat16), _ptr(v_out, torch.bfloat16), _ptr(workspace),
-        workspace.numel() * workspace.element_size(), _stream()), "dlm_window_qkv_project_rope")
-
-
-def dlm_window_qkv_project_stage(ctx, x, w, bias, rope_cos, rope_sin, batch, q_cap, d_model, n_q_heads, n_kv_heads, head_dim,
-                                 q_len, q_out, k_out, v_out, cache, layer, workspace) -> None:
-    _check(lib().dlm_window_qkv_project_stage(
-        ctx, _ptr(x, torch.bfloat16), _ptr(w, torch.bfloat16), _ptr(bias, torch.bfloat16), _ptr(rope_cos, torch.float32),
-        _ptr(rope_sin, torch.float32), int(batch), int(q_cap), int(d_model), int(n_q_heads), int(n_kv_heads), int(head_dim),
-        _ptr(q_len, torch.int32), _ptr(q_out, torch.bfloat16), _ptr(k_out, torch.bfloat16), _ptr(v_out, torch.bfloat16),
-        ctypes.byref(cache), int(layer), _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
-        "dlm_window_qkv_project_stage")
-
-
-def dlm_window_out_project(ctx, o, wo, bias, batch, q_cap, d_model, n_q_heads, head_dim, y, workspace) -> None:
-    _check(lib().dlm_window_out_project(
-        ctx, _ptr(o, torch.bfloat16), _ptr(wo, torch.bfloat16), _ptr(bias, torch.bfloat16), int(batch), int(q_cap), int(d_model),
-        int(n_q_heads), int(head_dim), _ptr(y, torch.bfloat16), _ptr(workspace), workspace.numel() * workspace.element_size(),
-        _stream()), "dlm_window_out_project")
 
 
 def dlm_selftest_set_wait_limit(ctx, limit_ns: int) -> None:
@@ -293,3 +189,39 @@ def dlm_selftest_set_attn_team_max(ctx, max_blocks: int, force: bool = False) ->
 
 def dlm_selftest_wait_timeout(ctx, limit_ns: int) -> None:
     _check(lib().dlm_selftest_wait_timeout(ctx, ctypes.c_uint64(int(limit_ns)), _stream()), "dlm_selftest_wait_timeout")
+
+
+# The enqueueing calls.  They are bound to the native functions themselves once _dlm_calls can be loaded; until then (the
+# package is imported by its own build) to stand-ins that load it at the first call or raise.
+_calls = None
+
+
+def _load_calls():
+    global _calls
+    if _calls is None:
+        lib()   # the missing-library message, and the one copy of libdlm.so
+        try:
+            from . import _dlm_calls as m
+        except ImportError as e:
+            raise ImportError(f"{_build.CALLS} cannot be loaded ({e}): run `python -m paper_2505_21467_b200.build` "
+                              "(there is no CPU or PyTorch fallback)") from e
+        m.set_error(DlmError)
+        _calls = m
+    return _calls
+
+
+def _stand_in(name):
+    def call(*args, **kwargs):
+        return getattr(_load_calls(), name)(*args, **kwargs)
+    call.__name__ = call.__qualname__ = name
+    return call
+
+
+try:
+    _load_calls()
+except ImportError:
+    pass
+for _name in ("dlm_kv_cache_commit", "dlm_freecache_attn_step", "dlm_unmask_select", "dlm_unmask_select_static",
+              "dlm_unmask_select_scored", "dlm_guided_accept", "dlm_guided_accept_topk", "dlm_guided_accept_threshold",
+              "dlm_window_qkv_project", "dlm_window_qkv_project_rope", "dlm_window_qkv_project_stage", "dlm_window_out_project"):
+    globals()[_name] = getattr(_calls, _name) if _calls is not None else _stand_in(_name)

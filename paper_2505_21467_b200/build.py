@@ -1,15 +1,19 @@
-"""Builds the C-ABI CUDA library ``libdlm.so`` in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI CUDA library ``libdlm.so`` in-tree with nvcc for sm_100a, and the Python entry points of its calls
+(``_dlm_calls.so``, a CPython module that links it) with g++."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libdlm.so")
+CALLS = os.path.join(HERE, "_dlm_calls.so")
+CALLS_SRC = os.path.join(CSRC, "py_calls.cpp")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -32,6 +36,7 @@ def is_stale() -> bool:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ into libdlm.so (cross-compiles without a GPU)."""
     if not force and not is_stale():
+        build_calls(force=False, verbose=verbose)
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = LIB + f".{os.getpid()}.tmp"
@@ -43,7 +48,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed building libdlm.so")
     check_attention_registers(proc.stdout)
     os.replace(tmp, LIB)
+    build_calls(force=force, verbose=verbose)
     return LIB
+
+
+def build_calls(force: bool = False, verbose: bool = False) -> str:
+    """Compile the Python entry points (needs torch's headers, no GPU)."""
+    deps = [CALLS_SRC, *glob.glob(os.path.join(INCLUDE, "*.h"))]
+    if not force and os.path.exists(CALLS) and all(os.path.getmtime(d) <= os.path.getmtime(CALLS) for d in deps):
+        return CALLS
+    import torch
+    from torch.utils import cpp_extension
+    tmp = CALLS + f".{os.getpid()}.tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", sysconfig.get_paths()["include"]]
+    for d in cpp_extension.include_paths("cuda"):
+        cmd += ["-isystem", d]
+    cmd += ["-o", tmp, CALLS_SRC, "-L", HERE, "-l:libdlm.so", "-Wl,-rpath,$ORIGIN"]
+    for d in cpp_extension.library_paths("cuda"):
+        cmd += ["-L", d]
+    cmd += ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    proc = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if verbose or proc.returncode != 0:
+        sys.stderr.write(proc.stdout)
+    if proc.returncode != 0:
+        raise RuntimeError("g++ failed building _dlm_calls.so")
+    os.replace(tmp, CALLS)
+    return CALLS
 
 
 # The attention kernel moves registers between its warpgroups with setmaxnreg: 8 softmax warps grow to 216 registers a

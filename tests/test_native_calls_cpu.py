@@ -1,0 +1,37 @@
+"""The native entry points check and order their arguments like the Python signatures they stand for (no GPU needed)."""
+import pytest
+import torch
+
+import paper_2505_21467_b200 as dlm
+from paper_2505_21467_b200 import build as _build
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    _build.build()
+
+
+def _args():
+    t = torch.zeros(4, dtype=torch.int32)
+    return dict(ctx=None, tok_dlm=t, tok_ar=t, batch=1, block_len=4, masked=t, tokens=t, fallback_source=0, accept=t, acc_idx=t, n_acc=t)
+
+
+def test_wrong_argument_counts_and_names():
+    a = _args()
+    with pytest.raises(TypeError, match="11 arguments"):
+        dlm.dlm_guided_accept(None, a["tok_dlm"])
+    with pytest.raises(TypeError, match="unexpected or repeated"):
+        dlm.dlm_guided_accept(*list(a.values())[:-1], acc_idx=a["acc_idx"])
+    with pytest.raises(TypeError, match="unexpected or repeated"):
+        dlm.dlm_guided_accept(*list(a.values())[:-1], nonsense=1)
+
+
+def test_tensors_are_checked_before_anything_runs():
+    a = _args()
+    for call in (lambda: dlm.dlm_guided_accept(*a.values()), lambda: dlm.dlm_guided_accept(**a)):
+        with pytest.raises(TypeError, match="contiguous CUDA tensor"):
+            call()
+    with pytest.raises(ValueError):
+        dlm.dlm_guided_accept(None, *([None] * 2), "one", 4, *([None] * 2), 0, *([None] * 3))
+    with pytest.raises(TypeError):      # the cache is not a dlm_kv_cache
+        dlm.dlm_kv_cache_commit(None, None, None, None, 1, None, None, 0, None, 1, 0, 0, 1)

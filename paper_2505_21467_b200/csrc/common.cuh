@@ -14,8 +14,7 @@ constexpr int kDlmMaxSplitUnits = 2048;  // attention units that may be split ac
 struct dlm_device_words {
   int status;
   unsigned int commit_ticket;
-  unsigned int unmask_ticket;
-  unsigned int pad[13];
+  unsigned int pad[14];
   unsigned int unmask_tickets[kDlmUnmaskTickets];     // blocks of a batch element finished so far
   unsigned int attn_unit_tickets[kDlmMaxSplitUnits];  // pieces of a split unit finished so far
 };

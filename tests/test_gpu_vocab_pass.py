@@ -1,0 +1,45 @@
+"""The vocabulary pass at the edges of its chunking: one logit short of and beyond a batch of 4096, rows on and off 16-byte
+boundaries, chunk counts around what the merge keeps in registers, maxima in the first and last logit and repeated across
+batches, warps and chunks.  Against the oracle."""
+import pytest
+
+from helpers import Dev
+from test_gpu_scores_threshold import _compare_scored
+from workloads import make_logits, make_mask
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    return Dev()
+
+
+def _inputs(B, L, V, seed):
+    z = make_logits(B, L, V, (0.5, 6.0), seed)
+    top = float(z.max()) + 1.0
+    z[0, 0, 0] = top                                   # first logit
+    z[0, 1, V - 1] = top                               # last logit
+    z[0, 2, [V // 2, V - 1]] = top                     # twice: the lower index wins
+    z[0, 3, V - 1] = z[0, 3, max(V - 4097, 0)] = top   # twice, a batch apart
+    z[0, 4, : max(V - 2, 1)] = -float("inf")           # nothing finite but the end (V >= 3)
+    return z
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("B,L,V", [(1, 33, 4095), (2, 17, 4096), (1, 9, 8193), (1, 32, 98304), (1, 8, 102401), (3, 40, 12288), (40, 32, 20484)])
+def test_chunk_edges(dev, oracle, B, L, V, kind):
+    masked0 = make_mask(B, L, L - 2, V).numpy()
+    masked0[0, :5] = 1
+    assert _compare_scored(dev, oracle, _inputs(B, L, V, B + L + V), masked0, 0, kind)
+
+
+@pytest.mark.parametrize("L", [31, 32, 33, 64, 1024])
+def test_ranking_of_short_and_long_blocks(dev, oracle, L):
+    """The ranking by one warp (up to 32 positions) and by the block, k beyond and below the number of masked positions."""
+    for k, n_masked in ((1, L), (7, L - 1), (L + 3, L // 2)) if L <= 64 else ((1, L), (L + 3, L // 2)):
+        for seed in range(12):
+            if _compare_scored(dev, oracle, make_logits(2, L, 513, (0.5, 6.0), 10 * L + seed), make_mask(2, L, n_masked, seed).numpy(), k, 0):
+                break
+        else:
+            pytest.skip("near ties in every draw")

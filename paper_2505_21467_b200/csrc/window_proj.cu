@@ -15,12 +15,14 @@
 // form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
 //   rows x K -> features     32 x 3584 -> 4608   12.6 -> 11.2 us (2.9 TB/s of weights)   256 x 3584 -> 4608   25.1 -> 15.5 us
 //                           256 x 4096 -> 12288   167 -> 38.8 us (665 TFLOP/s)          1280 x 3584 -> 4608   237 -> 50 us (845 TFLOP/s)
+// (Prefetching the tile's weights into L2 before the grid dependency wait, tried by rows and by stages, cost more than
+// the head start gave: the stage loads queue behind it.  31 us without, 38 with, at LLaDA's 256 rows.)
 // Both operands are K-major as they lie in memory.  A tensor map with K split into (64-element panel, panel index) lets one
 // copy bring several panels of a stage: a producer's loop costs 200 - 340 cycles per iteration whatever it copies
 // (barrier wait 100, expect 40, each copy 55), which bound the kernel when every 64 elements of K took an iteration.
 //
 // Block = 8 warps: warp 0 weight producer, warp 1 activation producer, warp 2 tcgen05.mma issuer (of the leader block),
-// warp 3 TMEM and the L2 prefetch of the weights, warps 4-7 the epilogue's tables; all eight write the results.
+// warp 3 TMEM, warps 4-7 the epilogue's tables; all eight write the results.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -43,7 +45,6 @@ struct ProjParams {
   __nv_bfloat16* q_out;
   __nv_bfloat16* k_out;
   __nv_bfloat16* v_out;
-  const __nv_bfloat16* w;
   const __nv_bfloat16* bias;   // [n_out] or nullptr
   const float* rope_cos;       // mode 0: rotary embedding of the query and key heads, fp32 [B][q_cap][head_dim / 2],
   const float* rope_sin;       // or both nullptr
@@ -122,14 +123,6 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   if (warp == 0 && lane == 0) prefetch_tensormap(&tm_w);
   if (warp == 1 && lane == 0) prefetch_tensormap(&tm_x);
   if (warp == 3) {
-    // The tile's weights start on their way to L2 while the kernel before this one is still running (its blocks leave
-    // room for this kernel's): only a prefetch, so nothing is read before that kernel's writes are visible.
-    if (blockIdx.z == 0)
-      for (int i = lane; i < kBlockN; i += 32) {
-        const int f = PAIR ? (rank ? feat1 : feat0) + i : (i < N / 2 ? feat0 + i : feat1 + i - N / 2);
-        prefetch_l2(p.w + (size_t)f * p.k_total, (uint32_t)p.k_total * 2u);
-      }
-    __syncwarp();
     if (PAIR) {
       tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
       tmem_relinquish_pair();
@@ -468,19 +461,22 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   pl.half_rows = (head_dim == 64 || head_dim == 128) && k.n < head_dim ? head_dim / 2 : k.n / 2;
   const int stage = k.kp * 128 * (pl.rc + k.n / (pair ? 2 : 1));
   const int n_k = (k_total / kPanel + k.kp - 1) / k.kp;
-  // Single blocks stay below half of an SM's shared memory, so that the next kernel's blocks can start beside them and
-  // prefetch their weights; pairs want depth (with 5 stages instead of 3: 20.2 -> 16.4 us at 256 Dream rows).
-  const int fixed = 1024 + 16384 + kAuxBytes;
-  int stages = ((pair ? 220 : 113) * 1024 - fixed) / stage;
+  // Behind the stages: the MMA reads rows up to M of an activation panel, which no copy filled (their results are never
+  // looked at); for the last panel of the last stage that may reach beyond the weights that follow it.
+  const int row_tile = m == 64 ? 64 : m / 2, cw = k.n / 2 < 32 ? k.n / 2 : 32;
+  const int beyond = (row_tile - pl.rc - k.kp * (k.n / (pair ? 2 : 1))) * 128, slack = beyond > 0 ? beyond : 0;
+  const int fixed = 1024 + slack + kAuxBytes;
+  // One block per SM, with depth (5 stages instead of 3: 20.2 -> 16.4 us at 256 Dream rows).  Two small ones per SM would let
+  // the next kernel's blocks start beside this one's and prefetch their weights, but they also crowd onto the SMs that an
+  // attention kernel before them leaves free: a 28-layer Dream step took 1137 us instead of 995.
+  int stages = (220 * 1024 - fixed) / stage;
   if (stages < 3) stages = 3;
   if (stages > kMaxStages) stages = kMaxStages;
   if (stages > n_k) stages = n_k;
   pl.n_stages = stages;
-  // Behind the stages: the MMA of the last stage's last activation panel reads the rows up to M, which no copy filled
-  // (their results are never looked at).  The epilogue's two staging buffers lie over the stages.
-  const int row_tile = m == 64 ? 64 : m / 2, cw = k.n / 2 < 32 ? k.n / 2 : 32;
+  // the epilogue's two staging buffers lie over the stages
   const int staging = 2 * row_tile * (2 * cw * 4 + 16);
-  pl.aux_offset = stages * stage + 16384;
+  pl.aux_offset = stages * stage + slack;
   if (pl.aux_offset < staging) pl.aux_offset = (staging + 127) & ~127;
   pl.smem_bytes = 1024 + pl.aux_offset + kAuxBytes;
   return pl.smem_bytes <= ctx->max_smem_optin && pl.chunks <= 65535;
@@ -594,7 +590,6 @@ int qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, co
   p.q_out = static_cast<__nv_bfloat16*>(q_out);
   p.k_out = static_cast<__nv_bfloat16*>(k_out);
   p.v_out = static_cast<__nv_bfloat16*>(v_out);
-  p.w = static_cast<const __nv_bfloat16*>(w);
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.rope_cos = rope_cos;
   p.rope_sin = rope_sin;
@@ -640,7 +635,6 @@ extern "C" int dlm_window_out_project(dlm_ctx* ctx, const void* o, const void* w
   ProjParams p = {};
   p.mode = 1;
   p.q_out = static_cast<__nv_bfloat16*>(y);
-  p.w = static_cast<const __nv_bfloat16*>(wo);
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.rows_total = (int)rows; p.q_cap = q_cap; p.n_q_heads = n_q_heads; p.n_kv_heads = 0; p.head_dim = head_dim;
   p.n_out = d_model; p.k_total = (int)k_total; p.batch = batch; p.act_heads = n_q_heads;

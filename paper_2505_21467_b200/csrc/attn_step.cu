@@ -67,6 +67,30 @@ struct Geometry {
   static constexpr uint32_t kColS = 2 * D;                      // S[mt] at 2D + mt * 128 (P aliases it)
 };
 
+// Division by a divisor known on the host: one high multiply, an add and a shift (round-up reciprocal of Granlund and
+// Montgomery, for dividends below 2^31).  The decoding of units and rows stands between a block's start and its first
+// scores; with the compiler's division by run-time divisors, a dozen of them inlined in every role, that code took 1.3 us
+// when it was in the instruction cache and 3.5 - 5.7 us when another kernel had run in between.
+struct FastDiv {
+  uint32_t mul, shift;
+  int d;
+  __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift); }
+  // quotient; `rem` gets the remainder
+  __device__ __forceinline__ int divmod(int n, int& rem) const {
+    const int q = div(n);
+    rem = n - q * d;
+    return q;
+  }
+};
+inline FastDiv make_fast_div(int d) {
+  FastDiv f;
+  f.d = d;
+  f.shift = 0;
+  while ((1ll << f.shift) < d) ++f.shift;
+  f.mul = (uint32_t)((((1ull << 32) * ((1ull << f.shift) - (uint64_t)d)) / (uint64_t)d) + 1);
+  return f;
+}
+
 struct AttnParams {
   const int32_t* cache_len;
   const int32_t* q_len;
@@ -85,19 +109,22 @@ struct AttnParams {
   int team;        // > 1 (with whole_units): blocks [u * team, (u + 1) * team) share unit u, key tiles dealt by rank;
                    // every block then reduces its share of the unit's outputs over all the team's pieces
   int smem_bytes;           // dynamic shared memory of the launch
+  FastDiv by_batch, by_rc, by_kv_heads, by_q_cap, by_team;
   float scale_log2;
   int* status;
   unsigned int* tickets;   // one zero-initialised counter per unit: pieces finished
 };
 
-// Per-block scheduling tables (in the block's dynamic shared memory, sized by batch and grid).
+// Per-block scheduling tables (in the block's dynamic shared memory, sized by batch).
 struct Sched {
   int* prefix;    // [batch + 1]  prefix[b] = tiles of batch elements < b; prefix[batch] = sum
   int* lc;        // [batch]      clamped cache_len
   int* lq;        // [batch]      clamped q_len
-  int* share_lo;  // [grid + 1]   split mode: block c owns items [share_lo[c], share_lo[c + 1])
+  int share, share_rem, n_cta;   // split mode: total items = share * n_cta + share_rem
+  // split mode: block c owns items [lo(c), lo(c + 1)), lo(c) = floor(total * c / n_cta)
+  __device__ __forceinline__ int lo(int c) const { return share * c + (share_rem * c) / n_cta; }
 };
-__host__ __device__ inline int sched_ints(int batch, int grid) { return 3 * (batch + 1) + 2 * (grid + 1); }
+__host__ __device__ inline int sched_ints(int batch) { return 3 * (batch + 1); }
 
 struct Segment {
   int lc_layer, b, kvh, rc;   // unit: layer within the call, batch element, KV head, row chunk
@@ -122,22 +149,19 @@ struct SegmentWalker {
   __device__ SegmentWalker(const AttnParams& p_, const Sched& s_, int cta) : p(p_), s(s_) {
     n_units = p.nl * p.n_kv_heads * p.n_rc * p.batch;
     if (p.whole_units) {
-      unit = p.team > 1 ? cta / p.team : cta;
+      unit = p.team > 1 ? p.by_team.div(cta) : cta;
       end = range_begin = 0;
     } else {
-      range_begin = s.share_lo[cta];
-      end = s.share_lo[cta + 1];
+      range_begin = cta < s.n_cta ? s.lo(cta) : 0;
+      end = cta < s.n_cta ? s.lo(cta + 1) : 0;
       unit = 0;
     }
   }
   __device__ bool next(Segment& g, int n_cta) {
     if (p.whole_units) {
       if (unit >= n_units) return false;
-      const int grp = unit / p.batch;
-      g.b = unit % p.batch;
-      g.rc = grp % p.n_rc;
-      g.lc_layer = (grp / p.n_rc) / p.n_kv_heads;
-      g.kvh = (grp / p.n_rc) % p.n_kv_heads;
+      const int grp = p.by_batch.divmod(unit, g.b);
+      g.lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, g.rc), g.kvh);
       g.Lc = s.lc[g.b];
       g.Lq = s.lq[g.b];
       g.T = s.prefix[g.b + 1] - s.prefix[g.b];
@@ -147,9 +171,9 @@ struct SegmentWalker {
       g.slot = -1;
       g.merger = 0;
       if (p.team > 1) {   // this block's share of the unit's key tiles; the launch has one team per unit
-        const int rank = (int)blockIdx.x % p.team;
-        g.t_begin = g.T * rank / p.team;
-        g.t_end = g.T * (rank + 1) / p.team;
+        const int rank = (int)blockIdx.x - p.by_team.div(blockIdx.x) * p.team;
+        g.t_begin = p.by_team.div(g.T * rank);
+        g.t_end = p.by_team.div(g.T * (rank + 1));
         g.slot = -2;
         unit = n_units;
         return true;
@@ -161,15 +185,18 @@ struct SegmentWalker {
     if (end <= range_begin) return false;
     const int sum = s.prefix[p.batch];
     const int item = end - 1;
-    const int grp = item / sum;
-    const int rem = item - grp * sum;
+    // the divisor is made of lengths, so not known on the host: a float estimate, exact division where it is off
+    int grp = (int)__fdividef((float)item, (float)sum);
+    int rem = item - grp * sum;
+    if (rem < 0 || rem >= sum) {
+      grp = item / sum;
+      rem = item - grp * sum;
+    }
     int b = 0;
     while (s.prefix[b + 1] <= rem) ++b;   // batch is small; units with zero tiles are skipped
     const int unit_start = grp * sum + s.prefix[b];
     g.b = b;
-    g.rc = grp % p.n_rc;
-    g.lc_layer = (grp / p.n_rc) / p.n_kv_heads;
-    g.kvh = (grp / p.n_rc) % p.n_kv_heads;
+    g.lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, g.rc), g.kvh);
     g.Lc = s.lc[b];
     g.Lq = s.lq[b];
     g.T = s.prefix[b + 1] - s.prefix[b];
@@ -201,12 +228,12 @@ struct UnitPieces {
     u0 = ((g.lc_layer * p.n_kv_heads + g.kvh) * p.n_rc + g.rc) * sum + s.prefix[g.b];
     u1 = u0 + g.T;
     c_first = c_last = cta;
-    while (s.share_lo[c_first] > u0) --c_first;
-    while (s.share_lo[c_last + 1] < u1) ++c_last;
+    while (s.lo(c_first) > u0) --c_first;
+    while (s.lo(c_last + 1) < u1) ++c_last;
   }
   // slot of the piece computed by block c (c_first <= c <= c_last): the block's first segment
   // if the piece starts where the block's share starts, else its second one
-  __device__ __forceinline__ int slot_of(int c) const { return s.share_lo[c] >= u0 ? 2 * c : 2 * c + 1; }
+  __device__ __forceinline__ int slot_of(int c) const { return s.lo(c) >= u0 ? 2 * c : 2 * c + 1; }
 };
 
 // Waits until the counter at `addr` reaches `target` (acquire, device scope).  Bounded like the
@@ -232,39 +259,36 @@ __device__ __forceinline__ bool wait_counter(const unsigned int* addr, unsigned 
 // in the workspace as [rank][M tile][head_dim / 4][128 rows] 16-byte vectors (4 columns of a row) and
 // [rank][M tile][128 rows] (m, l) pairs; the unit's n_mt * head_dim / 4 * 128 output vectors are dealt to
 // the ranks in that storage order, rank r reducing vectors [lo, hi) over all pieces.
-// The launch parameters the team schedule's exchange needs, handed to its functions by value.
+// Everything the exchange needs, decoded by the caller and handed over by value.
 struct TeamArgs {
   __nv_bfloat16* out;
   float* lse;
   float* ws_o;
   float* ws_ml;
-  unsigned int* tickets;
-  int team, n_mt, batch, n_rc, n_kv_heads, n_q_heads, group, q_cap, rows, rows_total;
-  __device__ explicit TeamArgs(const AttnParams& p)
-      : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), tickets(p.tickets), team(p.team), n_mt(p.n_mt),
-        batch(p.batch), n_rc(p.n_rc), n_kv_heads(p.n_kv_heads), n_q_heads(p.n_q_heads), group(p.group), q_cap(p.q_cap),
-        rows(p.rows), rows_total(p.rows_total) {}
-};
-
-struct TeamShare {
-  int rank, unit, b, rc, lc_layer, kvh, lo, hi;
-  bool has_keys;
+  unsigned int* arrive;        // the unit's two counters: blocks that have stored their piece ...
+  unsigned int* depart;        // ... and blocks that are past their wait for the first
   size_t piece0;               // index of the team's first piece
+  size_t qrow0;                // output row of the KV head's first query row
+  FastDiv by_q_cap;
+  int team, n_mt, rows, rows_total, rank, r0, Lq, lo, hi;   // r0: the row chunk's first row among the KV head's rows
+  bool has_keys;
   uint32_t ml_bytes, o_bytes;  // bytes fetched from each piece: all its (m, l) rows; this block's share of its vectors
-  __device__ TeamShare(const TeamArgs& p, const int* prefix, int D) {
-    const int C = p.team;
-    rank = (int)blockIdx.x % C;
-    unit = (int)blockIdx.x / C;
-    b = unit % p.batch;
-    const int grp = unit / p.batch;
-    rc = grp % p.n_rc;
-    lc_layer = (grp / p.n_rc) / p.n_kv_heads;
-    kvh = (grp / p.n_rc) % p.n_kv_heads;
-    has_keys = prefix[b + 1] > prefix[b];
+  __device__ __forceinline__ TeamArgs(const AttnParams& p, const Sched& s, int D)
+      : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), by_q_cap(p.by_q_cap), team(p.team), n_mt(p.n_mt), rows(p.rows),
+        rows_total(p.rows_total) {
+    int b, rc, kvh;
+    const int unit = p.by_team.divmod(blockIdx.x, rank);
+    const int grp = p.by_batch.divmod(unit, b), lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
+    has_keys = s.prefix[b + 1] > s.prefix[b];
+    Lq = s.lq[b];
+    r0 = rc * p.chunk_rows;
+    qrow0 = (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group) * p.q_cap;
+    arrive = p.tickets + unit;
+    depart = arrive + kDlmMaxSplitUnits / 2;
     const int n_vec = p.n_mt * (D / 4) * 128;
-    lo = n_vec * rank / C;          // n_vec <= 8192, C <= 16
-    hi = n_vec * (rank + 1) / C;
-    piece0 = (size_t)unit * C * p.n_mt;
+    lo = p.by_team.div(n_vec * rank);          // n_vec <= 8192, team <= 16
+    hi = p.by_team.div(n_vec * (rank + 1));
+    piece0 = (size_t)unit * p.team * p.n_mt;
     ml_bytes = (uint32_t)p.n_mt * 128u * 8u;
     o_bytes = (uint32_t)(hi - lo) * 16u;
   }
@@ -280,53 +304,48 @@ struct TeamShare {
 // longer need (all of the block's MMAs have finished by then: every softmax thread waited for its last one).
 // bar_team = bar_pub + 8 completes when all of it has landed.
 template <int D, bool kNoWait>
-__device__ __noinline__ void team_publish(const TeamArgs p, const int* prefix, uint32_t sm_q, uint32_t bar_pub,
+__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
                                           volatile int* abort_ptr) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   const uint32_t bar_team = bar_pub + 8;
-  const TeamShare ts(p, prefix, D);
-  if (!ts.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
-  unsigned int* const arrive = p.tickets + ts.unit;
-  unsigned int* const depart = p.tickets + kDlmMaxSplitUnits / 2 + ts.unit;
+  if (!p.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
   __threadfence();
-  atomicAdd(arrive, 1u);
-  if (!wait_counter(arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
+  atomicAdd(p.arrive, 1u);
+  if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
   fence_proxy_async_all();
-  mbar_expect_tx(bar_team, (uint32_t)p.team * (ts.ml_bytes + ts.o_bytes));
+  mbar_expect_tx(bar_team, (uint32_t)p.team * (p.ml_bytes + p.o_bytes));
   for (int c = 0; c < p.team; ++c) {
-    bulk_load(sm_q + c * ts.ml_bytes, p.ws_ml + (ts.piece0 + (size_t)c * p.n_mt) * 256, ts.ml_bytes, bar_team);
-    bulk_load(sm_q + p.team * ts.ml_bytes + c * ts.o_bytes,
-              p.ws_o + ((ts.piece0 + (size_t)c * p.n_mt) * (size_t)(D / 4 * 128) + ts.lo) * 4, ts.o_bytes, bar_team);
+    bulk_load(sm_q + c * p.ml_bytes, p.ws_ml + (p.piece0 + (size_t)c * p.n_mt) * 256, p.ml_bytes, bar_team);
+    bulk_load(sm_q + p.team * p.ml_bytes + c * p.o_bytes,
+              p.ws_o + ((p.piece0 + (size_t)c * p.n_mt) * (size_t)(D / 4 * 128) + p.lo) * 4, p.o_bytes, bar_team);
   }
   // every block of the team is past its wait on the arrival counter when the last one gets here: the last
   // one clears both counters for the next launch
-  if (atomicAdd(depart, 1u) == (unsigned int)p.team - 1u) {
-    *arrive = 0;
-    *depart = 0;
+  if (atomicAdd(p.depart, 1u) == (unsigned int)p.team - 1u) {
+    *p.arrive = 0;
+    *p.depart = 0;
   }
   // the copies issued above land in this block's shared memory: this thread does not leave before they have (the
   // softmax threads wait on the same barrier, but may have given up); abort_ptr + 1 is the flag that stays 0
   mbar_wait(bar_team, 0, abort_ptr + 1);
 }
 
-// Softmax threads (all live ones of the block, whole warps): store this thread's row of the block's piece --
+// Softmax threads (all 256 of the block, whole warps).  Live ones store their row of the block's piece --
 // unnormalised O from TMEM at t_o if the block had key tiles, and (m, l), which is (-inf, 0) if it had none
-// (that piece's O is then never read) -- then wait for the publisher's fetch and reduce this block's share of
+// (that piece's O is then never read).  Then all wait for the publisher's fetch and reduce this block's share of
 // the unit's output vectors over the C pieces, in rank order.  Returns false when a wait was given up.
-template <int D, int kChunk, bool kNoWait>
-__device__ __noinline__ bool team_exchange(const TeamArgs p, const int* prefix, uint32_t sm_q, uint32_t bar_pub,
-                                           volatile int* abort_ptr, uint32_t t_o, bool has_tiles, float m_used, float l_run) {
+template <int D, bool kNoWait>
+__device__ __noinline__ bool team_exchange(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
+                                           volatile int* abort_ptr, bool live, uint32_t t_o, bool has_tiles, float m_used, float l_run) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   constexpr int kVecs = D / 4 * 128;          // vectors of one M tile's piece
   const int tid = threadIdx.x, warp = tid >> 5;
   const int mt = warp >> 2, row = tid & 127;
   const int n_live = (p.rows + 31) & ~31;
   const uint32_t bar_team = bar_pub + 8;
-  const TeamShare ts(p, prefix, D);
   const int C = p.team;
-  const int Lq = prefix[p.batch + 1 + p.batch + ts.b];   // the clamped q_len table follows the prefix and cache_len tables
-  {
-    const size_t mine = ts.piece0 + (size_t)ts.rank * p.n_mt + mt;
+  if (live) {
+    const size_t mine = p.piece0 + (size_t)p.rank * p.n_mt + mt;
     if (has_tiles) {
       float4* po = reinterpret_cast<float4*>(p.ws_o) + mine * (size_t)kVecs + row;
       uint32_t v[32];
@@ -341,33 +360,34 @@ __device__ __noinline__ bool team_exchange(const TeamArgs p, const int* prefix, 
       }
     }
     __stcg(reinterpret_cast<float2*>(p.ws_ml) + mine * 128 + row, make_float2(m_used, l_run));
+    // no fence here: the arrival below orders the stores before the publisher's wait (block scope), and the
+    // publisher's fence before it counts the block in carries them to device scope
+    mbar_arrive(bar_pub);
   }
-  // no fence here: the arrival below orders the stores before the publisher's wait (block scope), and the
-  // publisher's fence before it counts the block in carries them to device scope
-  mbar_arrive(bar_pub);
   if (__all_sync(0xffffffffu, mbar_wait_limit(bar_team, 0, abort_ptr, kLimit)) == 0) return false;
-  const uint32_t sm_ml = sm_q, sm_o = sm_q + C * ts.ml_bytes;
-  for (int i = ts.lo + tid; i < ts.hi; i += n_live) {
+  const uint32_t sm_ml = sm_q, sm_o = sm_q + C * p.ml_bytes;
+  for (int i = p.lo + tid; i < p.hi; i += 256) {
     const int mt_i = i / kVecs, rem = i % kVecs, qd = rem / 128, row_i = rem % 128;
     const int r_unit_i = mt_i * 128 + row_i;
-    const int r_kv_i = ts.rc * kChunk + r_unit_i;
+    const int r_kv_i = p.r0 + r_unit_i;
     if (r_unit_i >= n_live || r_kv_i >= p.rows_total) continue;
-    const int hl = r_kv_i / p.q_cap, ir = r_kv_i % p.q_cap;
-    const size_t qrow_i = (((size_t)ts.lc_layer * p.batch + ts.b) * p.n_q_heads + (size_t)ts.kvh * p.group + hl) * p.q_cap + ir;
-    const bool active_i = ir < Lq;
-    const uint32_t a_ml = sm_ml + (uint32_t)r_unit_i * 8u, a_o = sm_o + (uint32_t)(i - ts.lo) * 16u;
+    int ir;
+    p.by_q_cap.divmod(r_kv_i, ir);
+    const size_t qrow_i = p.qrow0 + r_kv_i;                // rows of a KV head's query heads lie one after the other
+    const bool active_i = ir < p.Lq;
+    const uint32_t a_ml = sm_ml + (uint32_t)r_unit_i * 8u, a_o = sm_o + (uint32_t)(i - p.lo) * 16u;
     float m_all = -CUDART_INF_F;
 #pragma unroll 4
     for (int c = 0; c < C; ++c) {
-      const float2 ml = ld_shared_f2(a_ml + c * ts.ml_bytes);
+      const float2 ml = ld_shared_f2(a_ml + c * p.ml_bytes);
       if (ml.y > 0.f) m_all = fmaxf(m_all, ml.x);
     }
     float l_all = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int c = 0; c < C; ++c) {
-      const float2 ml = ld_shared_f2(a_ml + c * ts.ml_bytes);
-      const float4 x = ld_shared_f4(a_o + c * ts.o_bytes);
+      const float2 ml = ld_shared_f2(a_ml + c * p.ml_bytes);
+      const float4 x = ld_shared_f4(a_o + c * p.o_bytes);
       if (ml.y > 0.f) {   // a piece without keys holds no O
         const float w = ex2_approx(ml.x - m_all);
         l_all = fmaf(w, ml.y, l_all);
@@ -585,7 +605,7 @@ template <int D, int kChunk, bool kNoWait>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc,
                        const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ CUtensorMap tm_kn,
-                       const __grid_constant__ CUtensorMap tm_vn, const AttnParams p) {
+                       const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ AttnParams p) {
   using G = Geometry<D>;
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   // Shared memory of the block, all of it dynamic (the scheduling tables are sized by batch and grid):
@@ -606,13 +626,13 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   volatile int* const never_ptr = flags + 1;    // stays 0: for waits that must not be cut short by an abort
   uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(flags + 2);
   volatile int* const merge_ok = flags + 3;
+  volatile int* const any_empty = flags + 4;    // some batch element has no key tile at all
   Sched sched;
   sched.prefix = flags + kFlagBytes / 4;
   sched.lc = sched.prefix + p.batch + 1;
   sched.lq = sched.lc + p.batch;
-  sched.share_lo = sched.lq + p.batch;
   if (smem_pad + (uint32_t)(p.n_mt + KS + VS) * G::kTileBytes + kBarrierBytes + kFlagBytes +
-          4u * (uint32_t)sched_ints(p.batch, gridDim.x) > (uint32_t)p.smem_bytes) {
+          4u * (uint32_t)sched_ints(p.batch) > (uint32_t)p.smem_bytes) {
     // cannot happen with the host's sizing (it leaves room for the largest pad); nothing has been touched yet
     if (threadIdx.x == 0) dlm_set_status(p.status, DLM_ERR_WORKSPACE);
     return;
@@ -636,7 +656,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   // ---- set-up: barriers, TMEM and descriptor prefetch first (they need no data), so that they overlap
   // the cold read of the lengths; then the tile prefix
   if (tid == 0) {
-    *abort_ptr = 0; *never_ptr = 0; *merge_ok = 0;
+    *abort_ptr = 0; *never_ptr = 0; *merge_ok = 0; *any_empty = 0;
     mbar_init(bar_q_full, 1);
     mbar_init(bar_q_empty, (uint32_t)p.n_mt);       // one commit per MMA issuer
     mbar_init(bar_drain, 1);
@@ -684,34 +704,46 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   // tile for this block.
   const bool early_q = p.whole_units != 0;
   if (early_q && warp == 8 && lane == 0) {
-    const int unit = p.team > 1 ? (int)blockIdx.x / p.team : (int)blockIdx.x;
-    const int grp = unit / p.batch, b = unit % p.batch, rc = grp % p.n_rc;
-    const int zq = (((grp / p.n_rc) / p.n_kv_heads) * p.batch + b) * p.n_kv_heads + (grp / p.n_rc) % p.n_kv_heads;
+    int b, rc, kvh;
+    const int grp = p.by_batch.divmod(p.team > 1 ? p.by_team.div(blockIdx.x) : (int)blockIdx.x, b);
+    const int lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
+    const int zq = (lc_layer * p.batch + b) * p.n_kv_heads + kvh;
     mbar_expect_tx(bar_q_full, (uint32_t)(p.n_mt * min(128, p.rows)) * 128u * G::kPanels);
     for (int mt = 0; mt < p.n_mt; ++mt)
       for (int pn = 0; pn < G::kPanels; ++pn)
         tma_load_3d(sm_q + mt * G::kTileBytes + pn * kPanelBytes, &tm_q, bar_q_full, pn * 64, rc * kChunk + mt * 128, zq);
   }
-  for (int b = tid; b < p.batch; b += kThreads) {
-    int Lc = p.cache_len[b];
-    int Lq = p.q_len ? p.q_len[b] : p.q_cap;
-    if (Lc < 0 || Lc > p.capacity || Lq < 0 || Lq > p.q_cap) {
-      dlm_set_status(p.status, DLM_ERR_CAPACITY);
-      Lc = max(0, min(Lc, p.capacity));
-      Lq = max(0, min(Lq, p.q_cap));
-    }
-    sched.lc[b] = Lc;
-    sched.lq[b] = Lq;
-  }
-  __syncthreads();
-  if (tid == 0) {
+  // lengths and tile prefix, by one warp: lane = batch element
+  if (warp == 0) {
     int acc = 0;
-    for (int b = 0; b < p.batch; ++b) {
-      sched.prefix[b] = acc;
-      acc += tiles_of(sched.lc[b], sched.lq[b], p.fresh_box);
+    for (int b0 = 0; b0 < p.batch; b0 += 32) {
+      const int b = b0 + lane;
+      int Lc = 0, Lq = 0, tiles = 0;
+      if (b < p.batch) {
+        Lc = p.cache_len[b];
+        Lq = p.q_len ? p.q_len[b] : p.q_cap;
+        if (Lc < 0 || Lc > p.capacity || Lq < 0 || Lq > p.q_cap) {
+          dlm_set_status(p.status, DLM_ERR_CAPACITY);
+          Lc = max(0, min(Lc, p.capacity));
+          Lq = max(0, min(Lq, p.q_cap));
+        }
+        tiles = tiles_of(Lc, Lq, p.fresh_box);
+        sched.lc[b] = Lc;
+        sched.lq[b] = Lq;
+      }
+      int inc = tiles;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      if (b < p.batch) sched.prefix[b] = acc + inc - tiles;
+      if (__any_sync(0xffffffffu, b < p.batch && tiles == 0) && lane == 0) *any_empty = 1;
+      acc += __shfl_sync(0xffffffffu, inc, 31);
     }
-    sched.prefix[p.batch] = acc;
+    if (lane == 0) sched.prefix[p.batch] = acc;
   }
+  __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -720,10 +752,11 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int total_items = sched.prefix[p.batch] * p.nl * p.n_kv_heads * p.n_rc;
   const int n_cta = p.whole_units ? (int)gridDim.x : min((int)gridDim.x, total_items);
   const bool has_work = p.whole_units || (int)blockIdx.x < n_cta;
+  sched.n_cta = max(n_cta, 1);
+  sched.share = sched.share_rem = 0;
   if (!p.whole_units) {
-    for (int c = tid; c <= n_cta; c += kThreads)
-      sched.share_lo[c] = (int)((long long)total_items * c / max(n_cta, 1));
-    __syncthreads();
+    sched.share = total_items / sched.n_cta;
+    sched.share_rem = total_items - sched.share * sched.n_cta;
   }
 
   // The softmax warps keep a whole score row in registers; the other warpgroup needs few.
@@ -929,7 +962,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // (they arrive on bar_pub and move on), make the stores visible device-wide and count the
       // piece in its unit's counter.
       if (lane == 0 && p.team > 1) {
-        team_publish<D, kNoWait>(TeamArgs(p), sched.prefix, sm_q, bar_pub, abort_ptr);
+        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr);
       } else if (lane == 0 && has_work && !p.whole_units) {
         SegmentWalker walk(p, sched, blockIdx.x);
         Segment g;
@@ -960,10 +993,9 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         return __all_sync(0xffffffffu, mbar_wait_limit(bar, parity, abort_ptr, kLimit)) != 0;
       };
       // this thread's query row in row chunk rc of a KV head: which of its query heads, which active row
+      // (rows of a KV head's query heads lie one after the other)
       auto out_row_of = [&](int lc_layer, int b, int kvh, int rc) {
-        const int r = rc * kChunk + r_unit;
-        const int hl = r < p.rows_total ? r / p.q_cap : 0, ir = r < p.rows_total ? r % p.q_cap : 0;
-        return (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group + hl) * p.q_cap + ir;
+        return (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group) * p.q_cap + rc * kChunk + r_unit;
       };
       auto zero_my_row = [&](size_t qrow, bool real_row) {
         if (real_row) {
@@ -973,14 +1005,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           if (p.lse) p.lse[qrow] = -CUDART_INF_F;
         }
       };
-      if (!p.whole_units) {
+      if (!p.whole_units && *any_empty) {
         // units without any key (inactive batch elements) appear in no share: zero them here
         const int n_units = p.nl * p.n_kv_heads * p.n_rc * p.batch;
         for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-          const int b = unit % p.batch, grp = unit / p.batch, rc = grp % p.n_rc;
+          int b, rc, kvh;
+          const int grp = p.by_batch.divmod(unit, b), lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
           if (sched.prefix[b + 1] == sched.prefix[b])
-            zero_my_row(out_row_of((grp / p.n_rc) / p.n_kv_heads, b, (grp / p.n_rc) % p.n_kv_heads, rc),
-                        rc * kChunk + r_unit < p.rows_total);
+            zero_my_row(out_row_of(lc_layer, b, kvh, rc), rc * kChunk + r_unit < p.rows_total);
         }
       }
       if (has_work) {
@@ -990,15 +1022,11 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         bool ok = true;
         while (ok && walk.next(g, n_cta)) {
           const int n = g.t_end - g.t_begin;
-          const size_t qrow = out_row_of(g.lc_layer, g.b, g.kvh, g.rc);
-          const int r_kv = g.rc * kChunk + r_unit;               // row among all query rows of the KV head
-          const bool real_row = r_kv < p.rows_total;
-          const int i_row = real_row ? r_kv % p.q_cap : 0;
           if (n <= 0) {  // inactive batch element: the unit's rows are zero (team schedule: or no tile for this rank)
             if (g.T == 0) {
-              zero_my_row(qrow, real_row);
+              zero_my_row(out_row_of(g.lc_layer, g.b, g.kvh, g.rc), g.rc * kChunk + r_unit < p.rows_total);
             } else if (g.slot == -2) {   // a piece without key tiles
-              ok = team_exchange<D, kChunk, kNoWait>(TeamArgs(p), sched.prefix, sm_q, bar_pub, abort_ptr, t_o, false, -CUDART_INF_F, 0.f);
+              ok = team_exchange<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
             }
             continue;
           }
@@ -1051,10 +1079,13 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           ok = wait_warp(bar_pv_done + 16 * mt + 8 * ((gt - 1) & 1), ((gt - 1) >> 1) & 1);
           if (!ok) break;
           tc_fence_after_sync();
-          const bool active = real_row && i_row < g.Lq;
+          const size_t qrow = out_row_of(g.lc_layer, g.b, g.kvh, g.rc);
+          const int r_kv = g.rc * kChunk + r_unit;               // row among all query rows of the KV head
+          const bool real_row = r_kv < p.rows_total;
+          const bool active = real_row && r_kv - p.by_q_cap.div(r_kv) * p.q_cap < g.Lq;
           uint32_t v[32];
           if (g.slot == -2) {
-            ok = team_exchange<D, kChunk, kNoWait>(TeamArgs(p), sched.prefix, sm_q, bar_pub, abort_ptr, t_o, true, m_used, l_run);
+            ok = team_exchange<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
           } else if (g.slot < 0) {
             const float inv = active ? 1.f / l_run : 0.f;
 #pragma unroll 1
@@ -1184,6 +1215,10 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
         }
       }
+    } else if (p.team > 1) {
+      // warps without a row of their own help with the reduction
+      const TeamArgs ta(p, sched, D);
+      if (ta.has_keys) team_exchange<D, kNoWait>(ta, sm_q, bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
     }
   }
   // ---- teardown: nothing of this block is in flight any more
@@ -1274,7 +1309,7 @@ struct Plan {
 bool plan_shared_memory(int smem_limit, int head_dim, int batch, Plan& pl) {
   const int tile = head_dim / 64 * kPanelBytes;
   const int stages = head_dim == 128 ? Geometry<128>::kStages : Geometry<64>::kStages;
-  pl.smem_bytes = 1024 + (pl.n_mt + 2 * stages) * tile + kBarrierBytes + kFlagBytes + 4 * sched_ints(batch, pl.grid);
+  pl.smem_bytes = 1024 + (pl.n_mt + 2 * stages) * tile + kBarrierBytes + kFlagBytes + 4 * sched_ints(batch);
   return pl.smem_bytes <= smem_limit;
 }
 
@@ -1434,6 +1469,11 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   p.team = pl.team;
   p.smem_bytes = pl_mut.smem_bytes;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D);
+  p.by_batch = make_fast_div(p.batch);
+  p.by_rc = make_fast_div(p.n_rc);
+  p.by_kv_heads = make_fast_div(p.n_kv_heads);
+  p.by_q_cap = make_fast_div(q_cap);
+  p.by_team = make_fast_div(pl.team);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.status = &ctx->words->status;
   p.tickets = ctx->words->attn_unit_tickets;

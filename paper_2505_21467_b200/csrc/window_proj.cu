@@ -190,14 +190,21 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, round & 1, abort_ptr)) != 0;
       if (!ok) break;
       tc_fence_after_sync();
-      const uint32_t a0_lo = desc_lo + ((s * stage_bytes) >> 4), b0_lo = a0_lo + (x_bytes >> 4);
+      // descriptors of the stage's panels, in warp-uniform code so that they sit in the uniform registers the MMA reads
+      uint32_t a_lo[KP], b_lo[KP];
+      a_lo[0] = desc_lo + ((s * stage_bytes) >> 4);
+      b_lo[0] = a_lo[0] + (x_bytes >> 4);
+#pragma unroll
+      for (int kp = 1; kp < KP; ++kp) {
+        a_lo[kp] = a_lo[kp - 1] + (x_panel >> 4);
+        b_lo[kp] = b_lo[kp - 1] + kBlockN * 8;
+      }
       if (elect_one_sync()) {
 #pragma unroll
         for (int kp = 0; kp < KP; ++kp) {
-          const uint32_t a_lo = a0_lo + kp * (x_panel >> 4), b_lo = b0_lo + kp * (kBlockN * 8);
 #pragma unroll
           for (int k = 0; k < kPanel / 16; ++k)
-            mma_ss_lo<PAIR>(tmem, a_lo + 2 * k, b_lo + 2 * k, desc_hi, idesc, kc > 0 || kp > 0 || k > 0 ? 1u : 0u);
+            mma_ss_lo<PAIR>(tmem, a_lo[kp] + 2 * k, b_lo[kp] + 2 * k, desc_hi, idesc, kc > 0 || kp > 0 || k > 0 ? 1u : 0u);
         }
         if (PAIR) tc_commit_pair(bar_empty + 8 * s); else tc_commit(bar_empty + 8 * s);
       }

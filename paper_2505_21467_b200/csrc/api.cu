@@ -22,14 +22,17 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
   ctx->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
   ctx->launches = 0;
   ctx->encode_tiled = nullptr;
+  ctx->maps = new (std::nothrow) dlm_map_cache();
   ctx->commit_blocks_per_sm[0] = ctx->commit_blocks_per_sm[1] = 0;
   for (int i = 0; i < 8; ++i) ctx->attn_smem_limit[i] = 0;
   ctx->proj_configured = 0;
+  memset(&ctx->attn_plan_key, 0, sizeof ctx->attn_plan_key);
   ctx->wait_limit_ns = sm100::kWaitLimitNs;
   ctx->attn_team_max = 1 << 20;   // no limit beyond the schedule's own
   ctx->attn_team_force = false;
-  if (cudaMalloc(&ctx->words, sizeof(dlm_device_words)) != cudaSuccess ||
+  if (!ctx->maps || cudaMalloc(&ctx->words, sizeof(dlm_device_words)) != cudaSuccess ||
       cudaMemset(ctx->words, 0, sizeof(dlm_device_words)) != cudaSuccess) {
+    delete ctx->maps;
     delete ctx;
     cudaSetDevice(prev);
     return DLM_ERR_CUDA;
@@ -42,6 +45,7 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
 extern "C" int dlm_destroy(dlm_ctx* ctx) {
   if (!ctx) return DLM_ERR_NULL;
   cudaFree(ctx->words);
+  delete ctx->maps;
   delete ctx;
   return DLM_OK;
 }
@@ -60,6 +64,46 @@ extern "C" int dlm_get_status(dlm_ctx* ctx, void* stream) {
     DLM_CUDA_TRY(cudaStreamSynchronize(s));
   }
   return code;
+}
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+const CUtensorMap* dlm_tensor_map(dlm_ctx* ctx, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                                  const cuuint32_t* box) {
+  dlm_map_key k;
+  memset(&k, 0, sizeof k);
+  k.base = base;
+  k.rank = (cuuint32_t)rank;
+  uint64_t h = (uint64_t)(uintptr_t)base >> 4;
+  for (int i = 0; i < rank; ++i) {
+    k.dims[i] = dims[i];
+    k.box[i] = box[i];
+    if (i + 1 < rank) k.strides[i] = strides[i];
+    h = (h ^ dims[i] ^ ((uint64_t)box[i] << 32)) * 0x9e3779b97f4a7c15ull;
+  }
+  const int slot = (int)(h >> 55);   // 9 bits
+  static_assert(kDlmMapSlots == 512, "slots are picked by 9 bits");
+  dlm_map_cache& c = *ctx->maps;
+  if (memcmp(&c.key[slot], &k, sizeof k) == 0) return &c.map[slot];
+  if (!ctx->encode_tiled) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    ctx->encode_tiled = fn;
+  }
+  const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
+  c.key[slot].rank = 0;
+  const CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
+      &c.map[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, elem,
+      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return nullptr;
+  c.key[slot] = k;
+  return &c.map[slot];
 }
 
 extern "C" int64_t dlm_launch_count(const dlm_ctx* ctx) { return ctx ? ctx->launches : 0; }

@@ -31,7 +31,6 @@
 // results (they have lower block indices and computed those pieces first), then folds them into
 // its own O, which is still in TMEM, in block order: the result is deterministic.  When the split
 // would cost more than it saves (the host estimates both) units are dealt whole, round-robin.
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -50,8 +49,6 @@ constexpr int kTmemCols = 512;
 constexpr int kRegsSoftmax = 216;     // registers per thread of the softmax warpgroups after setmaxnreg.inc
 constexpr int kRegsOther = 72;        // ... of the producer / MMA warpgroup after setmaxnreg.dec
 constexpr int kMaxQCap = 4096;         // active rows per call
-constexpr double kTeamMergeTiles = 3.0;   // cost of the team schedule's exchange and reduction per M tile, in key tiles
-                                          // (measured: about 5 us from the last MMA to the output stores, a key tile 1.7 us)
 constexpr int kTeamMax = 16;              // most blocks of a team
 constexpr int kMaxGrid = 256;          // blocks of the persistent grid (one per SM)
 constexpr int kMaxStages = 8;          // barrier slots reserved per ring
@@ -1232,29 +1229,15 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 // bf16 tensor viewed as [slabs][rows][D]; box = 64 elements x box_rows rows x 1 slab, 128-byte swizzle.
 int encode_map(dlm_ctx* ctx, CUtensorMap* map, const void* base, int D, long long rows, long long slabs, int box_rows) {
-  if (!ctx->encode_tiled) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
-        q != cudaDriverEntryPointSuccess)
-      return DLM_ERR_CUDA;
-    ctx->encode_tiled = fn;
-  }
   const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)rows, (cuuint64_t)slabs};
   const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)rows * D * 2};
   const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-  const cuuint32_t elem[3] = {1, 1, 1};
-  const CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
-      map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
-      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? DLM_OK : DLM_ERR_CUDA;
+  const CUtensorMap* m = dlm_tensor_map(ctx, base, 3, dims, strides, box);
+  if (!m) return DLM_ERR_CUDA;
+  *map = *m;
+  return DLM_OK;
 }
 
 // The kernel starts with `numRegs` registers per thread in all 12 warps.  The 8 softmax warps then
@@ -1297,11 +1280,7 @@ int configure_kernel(dlm_ctx* ctx, int which, const void* kern) {
   return DLM_OK;
 }
 
-struct Plan {
-  int n_mt, rows, rows_total, n_rc, grid, whole_units, chunk_rows, team;
-  int smem_bytes;
-  size_t ws_o_bytes, ws_ml_bytes;
-};
+using Plan = dlm_attn_plan;
 
 // Shared memory of a block: Q tiles, the K and V rings, barriers, flags, scheduling tables and up to
 // 1023 bytes of alignment.  (Deeper rings were measured: 2 + 3 and 3 + 3 stages at head_dim 128 were
@@ -1313,70 +1292,92 @@ bool plan_shared_memory(int smem_limit, int head_dim, int batch, Plan& pl) {
   return pl.smem_bytes <= smem_limit;
 }
 
-// Splitting units across blocks balances the load but costs each block a partial store and each
-// unit a wait and a merge that grows with its number of pieces (measured: about 3 key tiles' worth
-// plus 0.7 per further piece); dealing units whole costs idle SMs when the units do not fill a
-// whole number of waves.  The number of shares (= blocks) is chosen to minimise the estimated
-// time in key tiles per block, from the caller's cache length hint; one share per unit or fewer
-// means whole units.
-Plan make_plan(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int cache_len_hint) {
-  Plan pl;
+// Device scratch of a call: room for the partial results of the split and team schedules whenever one of them is possible
+// at all, whichever the hint and the cost estimate then pick.
+struct WorkspaceSize {
+  size_t o_bytes, ml_bytes;
+};
+WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap) {
+  const int rows_total = (n_q_heads / cache->n_kv_heads) * q_cap, sms = ctx->num_sms < kMaxGrid ? ctx->num_sms : kMaxGrid;
+  const long long units = (long long)nl * cache->batch * cache->n_kv_heads * ((rows_total + 255) / 256);
+  const size_t slots = units < 8LL * sms && units <= kDlmMaxSplitUnits ? 2 * (size_t)sms : 0, n_mt = rows_total > 128 ? 2 : 1;
+  return {slots * n_mt * 128 * cache->head_dim * sizeof(float), slots * n_mt * 128 * 2 * sizeof(float)};
+}
+
+// Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer), fitted to measurements of one-layer
+// calls (Dream heads, 1024 - 1152 cached rows; us):    team of 9, 1 tile, one M tile       10.6
+//   256 active rows: team of 5, 2 tiles, two M tiles   18.3     team of 2, 5 tiles, one M tile  19.1     split  23.4
+//   8 sequences:     team of 4, 3 tiles, two M tiles   20.3     team of 2, 5 tiles, one M tile  19.4     split  23.8
+constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer
+constexpr double kTeamCost[2] = {2.3, 4.3};      // the team schedule's exchange and reduction
+constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...
+constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond that
+
+// The best plan with row chunks of `chunk_rows`, and its estimated cost.
+double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
   pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
-  // Row chunks of 256 (two M tiles sharing every K/V tile) read K/V once per KV head.  When a call has
-  // only a handful of such units (one layer of a small batch), chunks of 128 double the units that can
-  // be spread over the SMs and halve every partial result; the second read of K/V comes from L2
-  // (measured on one Dream-shaped layer at batch 1: 15.9 us against 20.9).
-  const long long units256 = (long long)nl * cache->batch * cache->n_kv_heads * ((pl.rows_total + 255) / 256);
-  pl.chunk_rows = (pl.rows_total > 128 && units256 * 8 <= ctx->num_sms) ? 128 : 256;
-  pl.n_rc = (pl.rows_total + pl.chunk_rows - 1) / pl.chunk_rows;
-  pl.rows = pl.rows_total < pl.chunk_rows ? pl.rows_total : pl.chunk_rows;
+  pl.chunk_rows = chunk_rows;
+  pl.n_rc = (pl.rows_total + chunk_rows - 1) / chunk_rows;
+  pl.rows = pl.rows_total < chunk_rows ? pl.rows_total : chunk_rows;
   pl.n_mt = (pl.rows + 127) / 128;
+  const double tile = kTileCost[pl.n_mt - 1];
   const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
   const int sms = ctx->num_sms < kMaxGrid ? ctx->num_sms : kMaxGrid;
   const bool may_split = units < 8LL * sms && units <= kDlmMaxSplitUnits;
-  const int len = (cache_len_hint > 0 && cache_len_hint < cache->capacity) ? cache_len_hint : cache->capacity;
   const long long tiles_unit = (len + 127) / 128 + (q_cap + 127) / 128;
-  const double t_whole = (double)(((units + sms - 1) / sms) * tiles_unit);
-  double best = t_whole;
-  int best_shares = 0;   // 0: whole units
-  if (may_split) {
-    for (long long shares = units + 1; shares <= sms; ++shares) {
-      if (shares > units * tiles_unit) break;   // a share holds at least one item
-      const double pieces = (double)shares / (double)units;
-      const double t = (double)((units * tiles_unit + shares - 1) / shares) + 3.0 + 0.7 * (pieces - 1.0);
-      if (t < best) { best = t; best_shares = (int)shares; }
-    }
-    if (units > sms) {   // more units than SMs: the only split is over all SMs
-      const double t = (double)((units * tiles_unit + sms - 1) / sms) + 3.0 + 0.7;
-      if (t < best) { best = t; best_shares = sms; }
-    }
-  }
-  pl.whole_units = best_shares == 0 ? 1 : 0;
-  pl.grid = pl.whole_units ? (int)(units < sms ? units : sms) : best_shares;
+  // units dealt whole: idle SMs when they do not fill a whole number of waves
+  double best = (double)(((units + sms - 1) / sms) * tiles_unit) * tile;
+  pl.whole_units = 1;
+  pl.team = 1;
+  pl.grid = (int)(units < sms ? units : sms);
+  if (!may_split) return best;
+  // units split across blocks: equal shares, but a partial store per block and a merge per unit
+  auto consider_split = [&](long long shares) {
+    const double pieces = (double)shares / (double)units;
+    const double t = (double)((units * tiles_unit + shares - 1) / shares) * tile + kSplitCost[pl.n_mt - 1] +
+                     (pieces > 1.0 ? kSplitPiece * (pieces - 1.0) : kSplitPiece);
+    if (t < best) { best = t; pl.whole_units = 0; pl.grid = (int)shares; }
+  };
+  for (long long shares = units + 1; shares <= sms && shares <= units * tiles_unit; ++shares) consider_split(shares);
+  if (units > sms) consider_split(sms);   // more units than SMs: the only split is over all SMs
   // Team schedule for calls with few units: C blocks per unit, the unit's key tiles dealt among them, every
   // block reducing a C-th of the outputs over all pieces in parallel (the split schedule's merging block
   // folds the other pieces one after the other).  The smallest C that reaches the fewest tiles per block.
-  pl.team = 1;
-  if (ctx->attn_team_max > 1 && may_split && units * 2 <= sms) {
+  if (ctx->attn_team_max > 1 && units * 2 <= sms) {
     long long C = ctx->attn_team_max < kTeamMax ? ctx->attn_team_max : kTeamMax;
     if (C > sms / units) C = sms / units;
     if (C > tiles_unit) C = tiles_unit;
     if (C > 1) {
       const long long per_block = (tiles_unit + C - 1) / C;
       C = (tiles_unit + per_block - 1) / per_block;
-      const double t = (double)per_block + kTeamMergeTiles * pl.n_mt;   // a piece of two M tiles is twice the bytes
+      const double t = (double)per_block * tile + kTeamCost[pl.n_mt - 1];
       if (C > 1 && (t < best || ctx->attn_team_force)) {
+        best = t;
         pl.team = (int)C;
         pl.whole_units = 1;
         pl.grid = (int)(units * C);
       }
     }
   }
-  // the workspace is sized for the split schedule whenever that schedule is possible at all, so
-  // that its size does not depend on the hint
-  const size_t slots = may_split ? 2 * (size_t)sms : 0;
-  pl.ws_o_bytes = slots * pl.n_mt * 128 * cache->head_dim * sizeof(float);
-  pl.ws_ml_bytes = slots * pl.n_mt * 128 * 2 * sizeof(float);
+  return best;
+}
+
+// Row chunks of 256 (two M tiles sharing every K/V tile) read K/V once per KV head and cost little more per key tile than
+// chunks of 128; those double the units that can be spread over the SMs and halve every partial result, the second read of
+// K/V coming from L2.  Whichever schedule of either has the least estimated cost, from the caller's cache length hint.
+Plan make_plan(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int cache_len_hint) {
+  const int len = (cache_len_hint > 0 && cache_len_hint < cache->capacity) ? cache_len_hint : cache->capacity;
+  Plan pl, narrow;
+  const double cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 256, pl);
+  if (pl.n_mt == 2) {
+    const double narrow_cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 128, narrow);
+    // (a forced team schedule counts as the better one)
+    const bool forced_apart = ctx->attn_team_force && (narrow.team > 1) != (pl.team > 1);
+    if (forced_apart ? narrow.team > 1 : narrow_cost < cost) pl = narrow;
+  }
+  const WorkspaceSize ws = workspace_size(ctx, cache, nl, n_q_heads, q_cap);
+  pl.ws_o_bytes = ws.o_bytes;
+  pl.ws_ml_bytes = ws.ml_bytes;
   return pl;
 }
 
@@ -1387,8 +1388,8 @@ extern "C" size_t dlm_attn_workspace_bytes(const dlm_ctx* ctx, const dlm_kv_cach
   if (!ctx || !cache || n_layers_in_call <= 0 || n_q_heads <= 0 || q_cap <= 0 || cache->n_kv_heads <= 0 ||
       cache->batch <= 0 || n_q_heads % cache->n_kv_heads != 0)
     return 0;
-  const Plan pl = make_plan(ctx, cache, n_layers_in_call, n_q_heads, q_cap, 0);
-  return pl.ws_o_bytes + pl.ws_ml_bytes + 256;
+  const WorkspaceSize ws = workspace_size(ctx, cache, n_layers_in_call, n_q_heads, q_cap);
+  return ws.o_bytes + ws.ml_bytes + 256;
 }
 
 extern "C" int dlm_selftest_attn_schedule(const dlm_ctx* ctx, const dlm_kv_cache* cache, int n_layers_in_call, int n_q_heads,
@@ -1429,15 +1430,20 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   const int nl = layer_end - layer_begin;
   const size_t need = dlm_attn_workspace_bytes(ctx, cache, nl, n_q_heads, q_cap);
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255)) return DLM_ERR_WORKSPACE;
-  const Plan pl = make_plan(ctx, cache, nl, n_q_heads, q_cap, cache_len_hint);
-  {
-    const bool nw = ctx->wait_limit_ns == 0;
-    const int which = kernel_index(D, pl.chunk_rows, nw);
+  const bool nw = ctx->wait_limit_ns == 0;
+  // the plan of the last call serves the calls of a model's other layers too
+  const dlm_attn_plan_key key = {nl, cache->batch, cache->n_kv_heads, cache->capacity, D, n_q_heads, q_cap, cache_len_hint,
+                                 ctx->attn_team_max, ctx->attn_team_force ? 1 : 0, nw ? 1 : 0};
+  if (memcmp(&key, &ctx->attn_plan_key, sizeof key) != 0) {
+    Plan made = make_plan(ctx, cache, nl, n_q_heads, q_cap, cache_len_hint);
+    const int which = kernel_index(D, made.chunk_rows, nw);
     const int rc = configure_kernel(ctx, which, reinterpret_cast<const void*>(kernel_of(which)));
     if (rc != DLM_OK) return rc;
+    if (!plan_shared_memory(ctx->attn_smem_limit[which], D, cache->batch, made)) return DLM_ERR_UNSUPPORTED;
+    ctx->attn_plan = made;
+    ctx->attn_plan_key = key;
   }
-  Plan pl_mut = pl;
-  if (!plan_shared_memory(ctx->attn_smem_limit[kernel_index(D, pl.chunk_rows, ctx->wait_limit_ns == 0)], D, cache->batch, pl_mut)) return DLM_ERR_UNSUPPORTED;
+  const Plan& pl = ctx->attn_plan;
   {  // the split schedule counts (unit, key tile) items in 32 bits
     const long long tiles_per_unit = (cache->capacity + 127) / 128 + (q_cap + 127) / 128 + 1;
     if (!pl.whole_units && (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc * tiles_per_unit >= (1LL << 30))
@@ -1467,7 +1473,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   p.fresh_box = q_cap < 128 ? q_cap : 128;
   p.whole_units = pl.whole_units;
   p.team = pl.team;
-  p.smem_bytes = pl_mut.smem_bytes;
+  p.smem_bytes = pl.smem_bytes;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D);
   p.by_batch = make_fast_div(p.batch);
   p.by_rc = make_fast_div(p.n_rc);
@@ -1490,7 +1496,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   if (rc != DLM_OK) return rc;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DLM_CUDA_TRY(dlm_launch(kernel_of(kernel_index(D, pl.chunk_rows, ctx->wait_limit_ns == 0)), dim3(pl.grid), dim3(kThreads),
+  DLM_CUDA_TRY(dlm_launch(kernel_of(kernel_index(D, pl.chunk_rows, nw)), dim3(pl.grid), dim3(kThreads),
                           (size_t)p.smem_bytes, s, tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
   return dlm_launch_ok(ctx, 1);
 }

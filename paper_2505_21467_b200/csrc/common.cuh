@@ -2,8 +2,10 @@
 // interface is include/dlm.h).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "dlm.h"
 
@@ -19,6 +21,30 @@ struct dlm_device_words {
   unsigned int attn_unit_tickets[kDlmMaxSplitUnits];  // pieces of a split unit finished so far
 };
 
+// TMA descriptors a context has built, by what they describe.  A descriptor is a function of the key alone (an address
+// and sizes; it owns nothing), so a call whose tensors lie where an earlier call's did reuses it: building the five of an
+// attention call costs the host about as much as the launch.  Direct-mapped and fixed in size.
+struct dlm_map_key {
+  const void* base;
+  cuuint64_t dims[5], strides[4];
+  cuuint32_t box[5], rank;
+};
+constexpr int kDlmMapSlots = 512;
+struct dlm_map_cache {
+  dlm_map_key key[kDlmMapSlots];   // rank 0: empty
+  CUtensorMap map[kDlmMapSlots];
+};
+
+// How an attention call's work is dealt out (attn_step.cu), and what that depends on.
+struct dlm_attn_plan {
+  int n_mt, rows, rows_total, n_rc, grid, whole_units, chunk_rows, team;
+  int smem_bytes;
+  size_t ws_o_bytes, ws_ml_bytes;
+};
+struct dlm_attn_plan_key {
+  int nl, batch, n_kv_heads, capacity, head_dim, n_q_heads, q_cap, hint, team_max, team_force, no_wait;
+};
+
 struct dlm_ctx {
   int device;
   int num_sms;
@@ -26,13 +52,21 @@ struct dlm_ctx {
   int64_t launches;
   dlm_device_words* words;  // device
   void* encode_tiled;       // cuTensorMapEncodeTiled entry point (driver API), resolved lazily
+  dlm_map_cache* maps;
   int commit_blocks_per_sm[2];  // resident blocks per SM of the two commit kernels (0 = not asked yet)
   unsigned long long wait_limit_ns;   // limit of the kernels' device-side waits (2 s; a test may shorten it)
   unsigned int proj_configured; // bit per projection kernel: shared-memory opt-in done on this context's device
   int attn_team_max;            // most blocks the attention call's team schedule may give one unit (1 = schedule off)
   bool attn_team_force;         // tests: take the team schedule wherever it is possible, whatever the cost estimate says
+  dlm_attn_plan_key attn_plan_key;   // of the last call's plan (nl = 0: none yet)
+  dlm_attn_plan attn_plan;
   int attn_smem_limit[8];       // dynamic shared memory the two attention kernels may use on this device (0 = not set up yet)
 };
+
+// The descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle;
+// nullptr if the driver refuses it.  Defined in api.cu.
+const CUtensorMap* dlm_tensor_map(dlm_ctx* ctx, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                                  const cuuint32_t* box);
 
 #define DLM_CUDA_TRY(expr)                         \
   do {                                             \

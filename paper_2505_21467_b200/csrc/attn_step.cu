@@ -64,30 +64,9 @@ struct Geometry {
   static constexpr uint32_t kColS = 2 * D;                      // S[mt] at 2D + mt * 128 (P aliases it)
 };
 
-// Division by a divisor known on the host: one high multiply, an add and a shift (round-up reciprocal of Granlund and
-// Montgomery, for dividends below 2^31).  The decoding of units and rows stands between a block's start and its first
-// scores; with the compiler's division by run-time divisors, a dozen of them inlined in every role, that code took 1.3 us
-// when it was in the instruction cache and 3.5 - 5.7 us when another kernel had run in between.
-struct FastDiv {
-  uint32_t mul, shift;
-  int d;
-  __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift); }
-  // quotient; `rem` gets the remainder
-  __device__ __forceinline__ int divmod(int n, int& rem) const {
-    const int q = div(n);
-    rem = n - q * d;
-    return q;
-  }
-};
-inline FastDiv make_fast_div(int d) {
-  FastDiv f;
-  f.d = d;
-  f.shift = 0;
-  while ((1ll << f.shift) < d) ++f.shift;
-  f.mul = (uint32_t)((((1ull << 32) * ((1ull << f.shift) - (uint64_t)d)) / (uint64_t)d) + 1);
-  return f;
-}
-
+// (The decoding of units and rows stands between a block's start and its first scores, in every role: with the compiler's
+// division by run-time divisors it took 1.3 us when it was in the instruction cache and 3.5 - 5.7 us when another
+// kernel had run in between; hence the FastDivs.)
 struct AttnParams {
   const int32_t* cache_len;
   const int32_t* q_len;

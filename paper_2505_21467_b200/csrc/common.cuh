@@ -68,6 +68,28 @@ struct dlm_ctx {
 const CUtensorMap* dlm_tensor_map(dlm_ctx* ctx, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                                   const cuuint32_t* box);
 
+// Division by a divisor known on the host: one high multiply, an add and a shift (round-up reciprocal of Granlund and
+// Montgomery, for dividends below 2^31).
+struct FastDiv {
+  uint32_t mul, shift;
+  int d;
+  __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift); }
+  // quotient; `rem` gets the remainder
+  __device__ __forceinline__ int divmod(int n, int& rem) const {
+    const int q = div(n);
+    rem = n - q * d;
+    return q;
+  }
+};
+static inline FastDiv make_fast_div(int d) {
+  FastDiv f;
+  f.d = d;
+  f.shift = 0;
+  while ((1ll << f.shift) < d) ++f.shift;
+  f.mul = (uint32_t)((((1ull << 32) * ((1ull << f.shift) - (uint64_t)d)) / (uint64_t)d) + 1);
+  return f;
+}
+
 #define DLM_CUDA_TRY(expr)                         \
   do {                                             \
     cudaError_t _e = (expr);                       \

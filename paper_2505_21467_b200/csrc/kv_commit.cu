@@ -7,7 +7,7 @@
 // consecutive (refresh / append).  The item list is cut into equal contiguous ranges, one per
 // block, and the grid is one resident wave, so every SM moves the same number of bytes; a
 // thread keeps kUnroll independent 16-byte loads of K and of V in flight.  Item numbers are
-// decoded with 32-bit arithmetic whenever the call has fewer than 2^31 items (64-bit divisions
+// decoded with 32-bit reciprocals whenever the call has fewer than 2^31 items (64-bit divisions
 // by run-time divisors cost more than the copy).  The last block to finish advances cache_len.
 #include "common.cuh"
 
@@ -28,7 +28,7 @@ struct CommitParams {
   int n_max, src_len, advance_len, layer_begin, n_layers_call, dst_mode;
   int batch, n_kv_heads, capacity;
   int vec_per_row;       // head_dim * 2 / 16
-  int vec_shift;         // log2(vec_per_row) or -1
+  FastDiv by_vec, by_rows, by_heads, by_batch;   // vec_per_row, n_max, n_kv_heads, batch
   long long n_items;     // n_layers_call * batch * heads * n_max * vec_per_row
   long long per_block;   // items per block (a multiple of 32)
   int* status;
@@ -44,75 +44,59 @@ __device__ __forceinline__ int valid_rows(const CommitParams& p, int b, int len0
   return n;
 }
 
+// Where one item comes from and goes to (vector indices), or to = -1: nothing to move.
+struct Move {
+  long long from, to;
+};
+
+// Idx int: item numbers below 2^31, decoded with host-prepared reciprocals.
 template <typename Idx>
-__global__ void __launch_bounds__(kThreads, 4) kv_commit_kernel(const CommitParams p) {
-  dlm_grid_dependency_wait();
-  dlm_trigger_dependents();
-  const Idx begin = (Idx)blockIdx.x * (Idx)p.per_block;
-  const Idx end = (Idx)min((long long)begin + p.per_block, p.n_items);
-  const Idx n_max = (Idx)p.n_max, heads = (Idx)p.n_kv_heads, batch = (Idx)p.batch;
-  for (Idx base = begin + threadIdx.x; base < end; base += kThreads * kUnroll) {
-    uint4 kk[kUnroll], vv[kUnroll];
-    long long to[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      to[u] = -1;
-      const Idx item = base + (Idx)(u * kThreads);
-      if (item >= end) continue;
-      int vec;
-      Idx rest;
-      if (p.vec_shift >= 0) {
-        vec = (int)(item & (Idx)(p.vec_per_row - 1));
-        rest = item >> p.vec_shift;
-      } else {
-        vec = (int)(item % (Idx)p.vec_per_row);
-        rest = item / (Idx)p.vec_per_row;
-      }
-      const int r = (int)(rest % n_max);
-      rest /= n_max;
-      const int h = (int)(rest % heads);
-      rest /= heads;
-      const int b = (int)(rest % batch);
-      const int lc = (int)(rest / batch);  // layer within the call
-      // the index words are read before the row count is checked (their slots always exist), so the
-      // three small loads are in flight together instead of one after the other
-      const int len0 = p.cache_len[b];
-      const long long src = p.src_idx ? p.src_idx[(long long)b * p.n_max + r] : r;
-      const long long dst_given = p.dst_pos ? p.dst_pos[(long long)b * p.n_max + r] : 0;
-      const int n = valid_rows(p, b, len0);
-      if (n < 0) {
-        if (r == 0 && vec == 0 && h == 0 && lc == 0) dlm_set_status(p.status, DLM_ERR_CAPACITY);
-        continue;
-      }
-      if (r >= n) continue;
-      const long long dst = p.dst_pos ? dst_given : (long long)len0 + (p.dst_mode == DLM_DST_WINDOW ? src : r);
-      if (src < 0 || src >= p.src_len || dst < 0 || dst >= p.capacity) {
-        if (vec == 0 && h == 0 && lc == 0) dlm_set_status(p.status, DLM_ERR_INDEX);
-        continue;
-      }
-      const long long from =
-          ((((long long)lc * p.batch + b) * p.n_kv_heads + h) * p.src_len + src) * p.vec_per_row + vec;
-      to[u] = ((((long long)(lc + p.layer_begin) * p.batch + b) * p.n_kv_heads + h) * p.capacity + dst) *
-                  p.vec_per_row + vec;
-      kk[u] = __ldcs(p.k_new + from);
-      vv[u] = __ldcs(p.v_new + from);
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      if (to[u] >= 0) {
-        p.cache_k[to[u]] = kk[u];
-        p.cache_v[to[u]] = vv[u];
-      }
-    }
+__device__ __forceinline__ Move find_move(const CommitParams& p, Idx item) {
+  Move mv = {0, -1};
+  int vec, r, h, b, lc;   // vector of the row, row, head, batch element, layer within the call
+  if (sizeof(Idx) == 4) {
+    lc = p.by_batch.divmod(p.by_heads.divmod(p.by_rows.divmod(p.by_vec.divmod((int)item, vec), r), h), b);
+  } else {
+    long long rest = (long long)item;
+    vec = (int)(rest % p.vec_per_row);
+    rest /= p.vec_per_row;
+    r = (int)(rest % p.n_max);
+    rest /= p.n_max;
+    h = (int)(rest % p.n_kv_heads);
+    rest /= p.n_kv_heads;
+    b = (int)(rest % p.batch);
+    lc = (int)(rest / p.batch);
   }
-  if (!p.advance_len) return;
-  // Serial tail: the last block to arrive bumps cache_len once every row has been written.
+  // the index words are read before the row count is checked (their slots always exist), so the
+  // three small loads are in flight together instead of one after the other
+  const int len0 = p.cache_len[b];
+  const long long src = p.src_idx ? p.src_idx[(long long)b * p.n_max + r] : r;
+  const long long dst_given = p.dst_pos ? p.dst_pos[(long long)b * p.n_max + r] : 0;
+  const int n = valid_rows(p, b, len0);
+  if (n < 0) {
+    if (r == 0 && vec == 0 && h == 0 && lc == 0) dlm_set_status(p.status, DLM_ERR_CAPACITY);
+    return mv;
+  }
+  if (r >= n) return mv;
+  const long long dst = p.dst_pos ? dst_given : (long long)len0 + (p.dst_mode == DLM_DST_WINDOW ? src : r);
+  if (src < 0 || src >= p.src_len || dst < 0 || dst >= p.capacity) {
+    if (vec == 0 && h == 0 && lc == 0) dlm_set_status(p.status, DLM_ERR_INDEX);
+    return mv;
+  }
+  mv.from = ((((long long)lc * p.batch + b) * p.n_kv_heads + h) * p.src_len + src) * p.vec_per_row + vec;
+  mv.to = ((((long long)(lc + p.layer_begin) * p.batch + b) * p.n_kv_heads + h) * p.capacity + dst) * p.vec_per_row + vec;
+  return mv;
+}
+
+// The last block to get here advances cache_len.  That needs every block to have read it, not to have stored its rows: whoever
+// reads the rows is ordered behind the kernel.
+__device__ __forceinline__ void advance_when_last(const CommitParams& p) {
   __shared__ bool is_last;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned int t = atomicAdd(p.ticket, 1u);
-    is_last = (t == gridDim.x - 1);
+    unsigned int t;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(p.ticket) : "memory");
+    is_last = t == gridDim.x - 1;
   }
   __syncthreads();
   if (!is_last) return;
@@ -122,6 +106,59 @@ __global__ void __launch_bounds__(kThreads, 4) kv_commit_kernel(const CommitPara
     if (n > 0) p.cache_len[b] = len0 + n;
   }
   if (threadIdx.x == 0) *p.ticket = 0;
+}
+
+template <typename Idx>
+__global__ void __launch_bounds__(kThreads, 4) kv_commit_kernel(const __grid_constant__ CommitParams p) {
+  dlm_grid_dependency_wait();
+  dlm_trigger_dependents();
+  const Idx begin = (Idx)blockIdx.x * (Idx)p.per_block;
+  const Idx end = (Idx)min((long long)begin + p.per_block, p.n_items);
+  for (Idx base = begin + (Idx)threadIdx.x; base < end; base += (Idx)(kThreads * kUnroll)) {
+    uint4 kk[kUnroll], vv[kUnroll];
+    long long to[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      to[u] = -1;
+      const Idx item = base + (Idx)(u * kThreads);
+      if (item >= end) continue;
+      const Move mv = find_move<Idx>(p, item);
+      to[u] = mv.to;
+      if (mv.to >= 0) {
+        kk[u] = __ldcs(p.k_new + mv.from);
+        vv[u] = __ldcs(p.v_new + mv.from);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      if (to[u] >= 0) {
+        p.cache_k[to[u]] = kk[u];
+        p.cache_v[to[u]] = vv[u];
+      }
+    }
+  }
+  if (p.advance_len) advance_when_last(p);
+}
+
+// Calls too small for a resident wave: one item per thread.  They are a chain of round trips (index words, row, store; with
+// advance_len also ticket and lengths, which go beside the row's): four items a thread put four decodings in front of the
+// first load, and the ticket behind the stores (28 layers x 4 rows: 3.9 us; 8 x 32 rows with advance_len 3.9 us).
+__global__ void __launch_bounds__(kThreads) kv_commit_small_kernel(const __grid_constant__ CommitParams p) {
+  dlm_grid_dependency_wait();
+  dlm_trigger_dependents();
+  const int item = (int)blockIdx.x * kThreads + (int)threadIdx.x;
+  Move mv = {0, -1};
+  if (item < (int)p.n_items) mv = find_move<int>(p, item);
+  uint4 kk = make_uint4(0, 0, 0, 0), vv = kk;
+  if (mv.to >= 0) {
+    kk = __ldcs(p.k_new + mv.from);
+    vv = __ldcs(p.v_new + mv.from);
+  }
+  if (p.advance_len) advance_when_last(p);
+  if (mv.to >= 0) {
+    p.cache_k[mv.to] = kk;
+    p.cache_v[mv.to] = vv;
+  }
 }
 
 }  // namespace
@@ -158,34 +195,39 @@ extern "C" int dlm_kv_cache_commit(dlm_ctx* ctx, const dlm_kv_cache* cache, cons
   p.n_kv_heads = cache->n_kv_heads;
   p.capacity = cache->capacity;
   p.vec_per_row = cache->head_dim * 2 / 16;
-  p.vec_shift = -1;
-  for (int s = 0; s < 16; ++s)
-    if ((1 << s) == p.vec_per_row) p.vec_shift = s;
+  p.by_vec = make_fast_div(p.vec_per_row);
+  p.by_rows = make_fast_div(n_max);
+  p.by_heads = make_fast_div(cache->n_kv_heads);
+  p.by_batch = make_fast_div(cache->batch);
   p.n_items = (long long)p.n_layers_call * p.batch * p.n_kv_heads * n_max * p.vec_per_row;
   p.status = &ctx->words->status;
   p.ticket = &ctx->words->commit_ticket;
 
-  // one resident wave of equal contiguous ranges; small calls get one block per kThreads * kUnroll items
+  // one resident wave of equal contiguous ranges, or one item per thread where that is no more
   const bool narrow = p.n_items < (1LL << 31) - (long long)kThreads * kUnroll;
   int& per_sm = ctx->commit_blocks_per_sm[narrow ? 0 : 1];
   if (per_sm <= 0) {
     int n = 0;
-    const cudaError_t e = narrow ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kv_commit_kernel<unsigned int>, kThreads, 0)
-                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kv_commit_kernel<unsigned long long>, kThreads, 0);
+    const cudaError_t e = narrow ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kv_commit_kernel<int>, kThreads, 0)
+                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kv_commit_kernel<long long>, kThreads, 0);
     if (e != cudaSuccess || n <= 0) return DLM_ERR_CUDA;
     per_sm = n;
   }
+  const long long max_blocks = (long long)ctx->num_sms * per_sm;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (p.n_items <= max_blocks * kThreads) {
+    const unsigned int blocks = (unsigned int)((p.n_items + kThreads - 1) / kThreads);
+    DLM_CUDA_TRY(dlm_launch(kv_commit_small_kernel, dim3(blocks), dim3(kThreads), 0, st, p));
+    return dlm_launch_ok(ctx, 1);
+  }
   const long long per_pass = (long long)kThreads * kUnroll;
   long long blocks = (p.n_items + per_pass - 1) / per_pass;
-  const long long max_blocks = (long long)ctx->num_sms * per_sm;
   if (blocks > max_blocks) blocks = max_blocks;
-  if (blocks < 1) blocks = 1;
   p.per_block = ((p.n_items + blocks - 1) / blocks + 31) & ~31LL;
   blocks = (p.n_items + p.per_block - 1) / p.per_block;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (narrow)
-    DLM_CUDA_TRY(dlm_launch(kv_commit_kernel<unsigned int>, dim3((unsigned)blocks), dim3(kThreads), 0, st, p));
+    DLM_CUDA_TRY(dlm_launch(kv_commit_kernel<int>, dim3((unsigned)blocks), dim3(kThreads), 0, st, p));
   else
-    DLM_CUDA_TRY(dlm_launch(kv_commit_kernel<unsigned long long>, dim3((unsigned)blocks), dim3(kThreads), 0, st, p));
+    DLM_CUDA_TRY(dlm_launch(kv_commit_kernel<long long>, dim3((unsigned)blocks), dim3(kThreads), 0, st, p));
   return dlm_launch_ok(ctx, 1);
 }

@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(kThreads, 4) kv_commit_kernel(const __grid_con
 
 // Calls too small for a resident wave: one item per thread.  They are a chain of round trips (index words, row, store; with
 // advance_len also ticket and lengths, which go beside the row's): four items a thread put four decodings in front of the
-// first load, and the ticket behind the stores (28 layers x 4 rows: 3.9 us; 8 x 32 rows with advance_len 3.9 us).
+// first load, and the ticket behind the stores (28 layers x 4 rows: 3.9 us; 8 x 32 rows with advance_len 3.9 us;
+// now 1.9 and 1.8).
 __global__ void __launch_bounds__(kThreads) kv_commit_small_kernel(const __grid_constant__ CommitParams p) {
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();

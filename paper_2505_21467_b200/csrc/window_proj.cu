@@ -10,13 +10,16 @@
 //                   16 .. 128 features.  Bound by streaming the weights from HBM.
 //   more rows:      chunks of up to 256 rows, each by a pair of blocks (cta_group::2, M = 256): a block holds its half of
 //                   the rows and its half of the tile's features, so it takes in half of what two separate blocks would;
-//                   tiles of 64 .. 256 features.  Bound by the SM's intake from L2 at small tiles, by the tensor pipe at 256.
+//                   tiles of 64 .. 512 features.  Bound by the SM's intake from L2 at small tiles, by the tensor pipe from 256.
+//                   Widths of 192 and beyond 256 exist so that a call's tiles fill the pairs once: 1280 rows of 4608 features
+//                   are 90 tiles of 256, two rounds over 74 pairs (49.3 us), and 60 tiles of 384, one round (37.0 us).
 // Measured (one call per layer over 28 / 32 layers' own weights, back to back, rotary embedding and staging on; before this
 // form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
-//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 11.2 us (2.9 TB/s of weights)   256 x 3584 -> 4608   25.1 -> 15.5 us
-//                           256 x 4096 -> 12288   167 -> 38.8 us (665 TFLOP/s)          1280 x 3584 -> 4608   237 -> 50 us (845 TFLOP/s)
+//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 9.4 us (3.5 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 13.0 us
+//                           256 x 4096 -> 12288   167 -> 29.3 us (880 TFLOP/s)          1280 x 3584 -> 4608   237 -> 37 us (1143 TFLOP/s)
 // (Prefetching the tile's weights into L2 before the grid dependency wait, tried by rows and by stages, cost more than
-// the head start gave: the stage loads queue behind it.  31 us without, 38 with, at LLaDA's 256 rows.)
+// the head start gave: the stage loads queue behind it.  31 us without, 38 with, at LLaDA's 256 rows.  Prefetching
+// 8 - 32 stages ahead as the loads go: 0 - 4 us slower too.)
 // Both operands are K-major as they lie in memory.  A tensor map with K split into (64-element panel, panel index) lets one
 // copy bring several panels of a stage: a producer's loop costs 200 - 340 cycles per iteration whatever it copies
 // (barrier wait 100, expect 40, each copy 55), which bound the kernel when every 64 elements of K took an iteration.
@@ -35,8 +38,9 @@ using namespace sm100;
 constexpr int kThreads = 256;
 constexpr int kPanel = 64;                  // K elements of a 128-byte swizzled panel
 constexpr int kMaxStages = 8;
+constexpr int kMaxN = 512;                  // features of the widest tile (a block's whole TMEM)
 constexpr int kMaxActRows = 256;            // rows of an output projection (one pair sees them all)
-constexpr int kAuxBytes = 16 * kMaxStages + 16 + 32 + 256 * 4 + 128 * 32;   // barriers, flags, bias of the tile, row table
+constexpr int kAuxBytes = 16 * kMaxStages + 16 + 32 + kMaxN * 4 + 128 * 32;   // barriers, flags, bias of the tile, row table
 
 struct ProjParams {
   // destination: mode 0 = Q/K/V head by head ([B][heads][q_cap][D] each), mode 1 = row-major [rows][n_out]
@@ -60,10 +64,13 @@ struct ProjParams {
   int rc;                      // rows per block (a multiple of 8)
   int x_box_rows;              // rows per copy of head-split activations (rc: one copy brings all)
   int half_rows;               // features of a group's half: W is seen as [groups][2][half_rows][K]
+  int w_box_rows;              // tiles of units: features per copy of the weights (32, or 64 where units lie in pairs)
   int n_stages, aux_offset;
   int head_shift;              // log2(head_dim), or -1
   int* status;
 };
+
+__host__ __device__ constexpr bool tile_of_units(int n) { return n == 192 || n > 256; }
 
 // Where a row of the block goes: element offsets within q_out (or y), k_out / v_out and the staged layer (-1: not staged),
 // and within the rotary tables.
@@ -82,7 +89,11 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   constexpr int kRowTile = M == 64 ? 64 : M / 2;            // rows of the MMA in this block
   constexpr int kBlockN = PAIR ? N / 2 : N;                 // features whose weights this block loads
   constexpr uint32_t kWBytes = (uint32_t)KP * kBlockN * 128u;
-  constexpr uint32_t kTmemCols = N < 32 ? 32 : N;
+  constexpr uint32_t kTmemCols = N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : N <= 256 ? 256 : 512;
+  // Tiles of units: a unit is 32 features of a group's first half and the 32 of the second half that they are paired with.
+  // One MMA takes up to 256 columns; a wider tile is two, each [first halves | second halves] of its units.
+  constexpr bool UNITS = tile_of_units(N);
+  constexpr int kN0 = N > 256 ? (N / 64 + 1) / 2 * 64 : N, kN1 = N - kN0;
   const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
   const uint32_t base = smem_u32(smem_raw) + pad;
   const uint32_t x_panel = (uint32_t)p.rc * 128u, x_bytes = KP * x_panel;
@@ -96,16 +107,22 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   volatile int* const never_ptr = flags + 1;
   uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(flags + 2);
   float* const bias_s = reinterpret_cast<float*>(flags + 8);
-  RowEntry* const row_s = reinterpret_cast<RowEntry*>(bias_s + 256);
+  RowEntry* const row_s = reinterpret_cast<RowEntry*>(bias_s + kMaxN);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int tile = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
   const int row0 = ((int)blockIdx.z * (PAIR ? 2 : 1) + (int)rank) * p.rc;   // this block's first row
-  const int per_group = p.half_rows / (N / 2);
+  const int per_group = UNITS ? 1 : p.half_rows / (N / 2);
   const int group = tile / per_group, a0 = (tile % per_group) * (N / 2);
   const int feat0 = group * 2 * p.half_rows + a0, feat1 = feat0 + p.half_rows;   // first features of the two halves
-  auto feature = [&](int c) { return c < N / 2 ? feat0 + c : feat1 + c - N / 2; };      // output feature of column c
+  const int unit_shift = p.half_rows == 64 ? 1 : 0;          // UNITS: log2 of a group's units
+  auto feature = [&](int c) {                                // output feature of column c
+    if (!UNITS) return c < N / 2 ? feat0 + c : feat1 + c - N / 2;
+    const int h = c < kN0 ? kN0 / 2 : kN1 / 2, cc = c < kN0 ? c : c - kN0, second = cc >= h ? 1 : 0;
+    const int r = (c < kN0 ? 0 : kN0 / 2) + cc - second * h, unit = tile * (N / 64) + (r >> 5);
+    return ((2 * (unit >> unit_shift) + second) << (5 + unit_shift)) + ((unit & unit_shift) << 5) + (r & 31);
+  };
   const int n_panels = p.k_total / kPanel;
   const int n_k = (n_panels + KP - 1) / KP;                 // stages' worth of K; panels beyond the last are zero-filled
 
@@ -153,7 +170,12 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       if (elect_one_sync()) {
         if (rank == 0) mbar_expect_tx(bar_full + 8 * s, bytes);
         const uint32_t dst = base + s * stage_bytes, bar = full0 + 8 * s;
-        if (warp == 0) {
+        if (warp == 0 && UNITS) {
+          for (int r = 0; r < kBlockN; r += p.w_box_rows) {   // units beyond the last are zero-filled
+            const int unit = tile * (N / 64) + (r >> 5);
+            tma_load_5d<PAIR>(dst + x_bytes + r * 128, &tm_w, bar, 0, (unit & unit_shift) << 5, (int)rank, kc, unit >> unit_shift);
+          }
+        } else if (warp == 0) {
           tma_load_5d<PAIR>(dst + x_bytes, &tm_w, bar, 0, a0, PAIR ? (int)rank : 0, kc * KP, group);
         } else if (p.act_heads == 0) {
           tma_load_4d<PAIR>(dst, &tm_x, bar, 0, row0, kc * KP, 0);
@@ -181,7 +203,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   } else if (warp == 2 && rank == 0) {
     // ================================================================= MMA issuer
     bool ok = true;
-    const uint32_t idesc = make_idesc_bf16(M, (uint32_t)N, 0);
+    const uint32_t idesc = make_idesc_bf16(M, (uint32_t)kN0, 0), idesc1 = make_idesc_bf16(M, (uint32_t)(kN1 ? kN1 : 64), 0);
     const uint64_t desc = make_smem_desc_sw128(base, 16, 1024);
     const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
     int s = 0, round = 0;
@@ -202,8 +224,11 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
 #pragma unroll
         for (int kp = 0; kp < KP; ++kp) {
 #pragma unroll
-          for (int k = 0; k < kPanel / 16; ++k)
-            mma_ss_lo<PAIR>(tmem, a_lo[kp] + 2 * k, b_lo[kp] + 2 * k, desc_hi, idesc, kc > 0 || kp > 0 || k > 0 ? 1u : 0u);
+          for (int k = 0; k < kPanel / 16; ++k) {
+            const uint32_t add = kc > 0 || kp > 0 || k > 0 ? 1u : 0u;
+            mma_ss_lo<PAIR>(tmem, a_lo[kp] + 2 * k, b_lo[kp] + 2 * k, desc_hi, idesc, add);
+            if (kN1) mma_ss_lo<PAIR>(tmem + kN0, a_lo[kp] + 2 * k, b_lo[kp] + kN0 / 2 * 8 + 2 * k, desc_hi, idesc1, add);
+          }
         }
         if (PAIR) tc_commit_pair(bar_empty + 8 * s); else tc_commit(bar_empty + 8 * s);
       }
@@ -215,7 +240,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   } else if (warp >= 4) {
     // ================================================================= tables of the epilogue
     const int t = tid - 128;
-    for (int c = t; c < N; c += 128) bias_s[c] = p.bias ? __bfloat162float(p.bias[feature(c)]) : 0.f;
+    for (int c = t; c < N; c += 128) bias_s[c] = p.bias && (!UNITS || feature(c) < p.n_out) ? __bfloat162float(p.bias[feature(c)]) : 0.f;
     const int row = row0 + t;
     if (t < p.rc && row < p.rows_total) {
       const int b = row / p.q_cap, i = row - b * p.q_cap;
@@ -251,7 +276,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       constexpr uint32_t kPitch = 2 * kCW * 4 + 16;           // bytes of a staged row; the 16 spread rows over the banks
       constexpr int kLanes = kCW / 8, kRowsPerIt = kThreads / kLanes;
       constexpr int kIts = kRowTile > kRowsPerIt ? kRowTile / kRowsPerIt : 1;
-      const int dist = rope && N > D ? half : N / 2;          // columns between a segment and its partner
+      int dist = UNITS ? kN0 / 2 : rope && N > D ? half : N / 2;   // columns between a segment and its partner
       // TMEM side: warps w and w + 4 read the lanes of quarter w % 4, one segment each.  The row of a lane: M = 64 puts 16
       // rows in each quarter; M = 128 as a pair puts rows 0-63 twice, lanes 64-127 holding the second half of the columns.
       const int quarter = warp & 3, seg = warp >> 2;
@@ -290,9 +315,11 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       };
       uint32_t buf = base;
       for (int g = 0; g < N; g += 2 * dist) {
+        if (UNITS && g > 0) dist = kN1 / 2;                  // the second MMA's columns
         for (int c = g; c < g + dist; c += kCW) {
           const int cc = c + (tid % kLanes) * 8;             // this thread's 8 columns when it stores, and the 8 at cc + dist
           const int f0 = feature(cc), f1 = feature(cc + dist);
+          if (UNITS && f0 >= p.n_out) break;                 // the last tile's units beyond the last feature (uniform: one unit)
           const bool turn = rope && (f0 >> p.head_shift) < n_qk;
           float4 cs[kIts][2], sn[kIts][2];
           if (turn) {   // asked for before the accumulator is read
@@ -391,11 +418,14 @@ const ProjVariant kVariants[] = {
     {64, 64, 2, window_proj_kernel<64, 64, 2>},     {128, 64, 2, window_proj_kernel<128, 64, 2>},
     {64, 128, 2, window_proj_kernel<64, 128, 2>},   {128, 128, 2, window_proj_kernel<128, 128, 2>},
     {256, 128, 1, window_proj_kernel<256, 128, 1>}, {64, 256, 2, window_proj_kernel<64, 256, 2>},
-    {128, 256, 1, window_proj_kernel<128, 256, 1>}, {256, 256, 1, window_proj_kernel<256, 256, 1>},
+    {128, 256, 1, window_proj_kernel<128, 256, 1>}, {192, 256, 1, window_proj_kernel<192, 256, 1>},
+    {256, 256, 1, window_proj_kernel<256, 256, 1>}, {320, 256, 1, window_proj_kernel<320, 256, 1>},
+    {384, 256, 1, window_proj_kernel<384, 256, 1>}, {448, 256, 1, window_proj_kernel<448, 256, 1>},
+    {512, 256, 1, window_proj_kernel<512, 256, 1>},
 };
 
 struct ProjPlan {
-  int variant, rc, x_box_rows, chunks, tiles, half_rows, n_stages, aux_offset, smem_bytes;
+  int variant, rc, x_box_rows, w_box_rows, chunks, tiles, half_rows, n_stages, aux_offset, smem_bytes;
 };
 
 int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
@@ -427,10 +457,10 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   pl.variant = -1;
   for (int v = 0; v < (int)(sizeof(kVariants) / sizeof(kVariants[0])); ++v) {
     const ProjVariant& k = kVariants[v];
-    if (k.m != m || n_out % k.n != 0) continue;
-    const long long blocks = (long long)(n_out / k.n) * blocks_rows;
+    if (k.m != m || (n_out % k.n != 0 && !tile_of_units(k.n))) continue;
+    const long long blocks = (long long)((n_out + k.n - 1) / k.n) * blocks_rows;
     const double per_sm = (double)((blocks + ctx->num_sms - 1) / ctx->num_sms);
-    const double mma = m == 256 ? k.n / 2.0 : k.n / 4.0, smem = ((m == 256 ? 4096.0 : 2048.0) + k.n * (pair ? 16.0 : 32.0)) / 128.0;
+    const double mma = m == 256 ? k.n / 2.0 : k.n / 4.0, smem = ((m == 256 ? 4096.0 : 2048.0) * (k.n > 256 ? 2 : 1) + k.n * (pair ? 16.0 : 32.0)) / 128.0;
     const double intake = (pl.rc + k.n / (pair ? 2 : 1)) * 32.0 / 70.0;
     double cyc = mma > smem ? mma : smem;
     if (intake > cyc) cyc = intake;
@@ -439,9 +469,15 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   }
   if (pl.variant < 0) return false;
   const ProjVariant& k = kVariants[pl.variant];
-  pl.tiles = n_out / k.n;
+  pl.tiles = (n_out + k.n - 1) / k.n;
   // rotary pairs inside a tile: see the kernel
-  pl.half_rows = (head_dim == 64 || head_dim == 128) && k.n < head_dim ? head_dim / 2 : k.n / 2;
+  if (tile_of_units(k.n)) {
+    pl.half_rows = head_dim == 64 ? 32 : 64;
+    pl.w_box_rows = pl.half_rows == 64 && k.n % 128 == 0 ? 64 : 32;
+  } else {
+    pl.half_rows = (head_dim == 64 || head_dim == 128) && k.n < head_dim ? head_dim / 2 : k.n / 2;
+    pl.w_box_rows = k.n / 2;
+  }
   const int stage = k.kp * 128 * (pl.rc + k.n / (pair ? 2 : 1));
   const int n_k = (k_total / kPanel + k.kp - 1) / k.kp;
   // Behind the stages: the MMA reads rows up to M of an activation panel, which no copy filled (their results are never
@@ -475,6 +511,7 @@ int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorM
   p.rc = pl.rc;
   p.x_box_rows = pl.x_box_rows;
   p.half_rows = pl.half_rows;
+  p.w_box_rows = pl.w_box_rows;
   p.n_stages = pl.n_stages;
   p.aux_offset = pl.aux_offset;
   p.head_shift = p.head_dim == 128 ? 7 : p.head_dim == 64 ? 6 : -1;
@@ -484,13 +521,13 @@ int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorM
   return dlm_launch_ok(ctx, 1);
 }
 
-// W seen as [groups][2][half_rows][K / 64][64]; a copy brings n / 2 features of one half (pairs) or of both, kp panels.
+// W seen as [groups][2][half_rows][K / 64][64]; a copy brings w_box_rows features of one half (pairs) or of both, kp panels.
 const CUtensorMap* encode_weights(dlm_ctx* ctx, const void* w, int n_out, int k_total, const ProjPlan& pl) {
   const ProjVariant& k = kVariants[pl.variant];
   const cuuint64_t row = (cuuint64_t)k_total * 2, a = (cuuint64_t)pl.half_rows;
   const cuuint64_t dims[5] = {(cuuint64_t)kPanel, a, 2, (cuuint64_t)(k_total / kPanel), (cuuint64_t)n_out / (2 * a)};
   const cuuint64_t strides[4] = {row, a * row, (cuuint64_t)kPanel * 2, 2 * a * row};
-  const cuuint32_t box[5] = {(cuuint32_t)kPanel, (cuuint32_t)k.n / 2, k.m > 64 ? 1u : 2u, (cuuint32_t)k.kp, 1};
+  const cuuint32_t box[5] = {(cuuint32_t)kPanel, (cuuint32_t)pl.w_box_rows, k.m > 64 ? 1u : 2u, (cuuint32_t)k.kp, 1};
   return dlm_tensor_map(ctx, w, 5, dims, strides, box);
 }
 

@@ -91,6 +91,16 @@ def test_commit_ragged_scatter_append_and_layer_range(dev, oracle, D):
     _run_commit(dev, oracle, ck, cv, [10, 231, 0], kn, vn, advance=True, layer_begin=0, layer_end=3)
 
 
+@pytest.mark.parametrize("rows", [1, 15, 184, 185, 221, 222, 223, 295, 296, 297])
+def test_commit_at_the_edge_of_one_item_per_thread(dev, oracle, rows):
+    # 1024 vectors a row over the layers, sequences and heads; 5, 6 or 8 resident blocks of 256 threads on 148 SMs are 185,
+    # 222 or 296 such rows
+    NL, B, Hkv, D = 4, 2, 8, 128
+    ck, cv = make_cache(NL, B, Hkv, 310, D, 970 + rows)
+    kn, vn = make_kv_rows((NL, B, Hkv, rows, D), 971 + rows), make_kv_rows((NL, B, Hkv, rows, D), 972 + rows)
+    _run_commit(dev, oracle, ck, cv, [3, 13], kn, vn, n_rows=[rows, rows // 2], n_max=rows, advance=True)
+
+
 def test_commit_errors_are_reported_and_suppressed(dev, oracle):
     NL, B, Hkv, Lcap, D, src_len = 2, 2, 2, 40, 64, 8
     ck, cv = make_cache(NL, B, Hkv, Lcap, D, 950)

@@ -6,9 +6,9 @@
 // epilogue thread), N features of one tile its N; a block (pair) sums the whole of K, so there is no workspace, no exchange
 // between blocks and one summation order.  With the row in a thread, a head's features lie along the thread's registers: the
 // rotary embedding pairs two of its own registers and every store is 16 bytes of one row.
-//   up to 64 rows:  one block per tile, M = 128 (rows beyond the call's are never loaded, never read back), tiles of
+//   up to 64 rows:  one block per tile, M = 64 (rows beyond the call's are never loaded, never read back), tiles of
 //                   16 .. 128 features.  Bound by streaming the weights from HBM.
-//   more rows:      chunks of up to 256 rows, each by a pair of blocks (cta_group::2, M = 256): a block holds its half of
+//   more rows:      chunks of up to 256 rows, each by a pair of blocks (cta_group::2, M = 256; M = 128 up to 128 rows): a block holds its half of
 //                   the rows and its half of the tile's features, so it takes in half of what two separate blocks would;
 //                   tiles of 64 .. 512 features.  Bound by the SM's intake from L2 at small tiles, by the tensor pipe from 256.
 //                   Widths of 192 and beyond 256 exist so that a call's tiles fill the pairs once: 1280 rows of 4608 features

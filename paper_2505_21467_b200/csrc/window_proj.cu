@@ -16,7 +16,7 @@
 // Measured (one call per layer over 28 / 32 layers' own weights, back to back, rotary embedding and staging on; before this
 // form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
 //   rows x K -> features     32 x 3584 -> 4608   12.6 -> 9.4 us (3.5 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 13.0 us
-//                           256 x 4096 -> 12288   167 -> 29.3 us (880 TFLOP/s)          1280 x 3584 -> 4608   237 -> 37 us (1143 TFLOP/s)
+//                           256 x 4096 -> 12288   167 -> 29.3 us (880 TFLOP/s)          1280 x 3584 -> 4608   237 -> 35 us (1215 TFLOP/s)
 // (Prefetching the tile's weights into L2 before the grid dependency wait, tried by rows and by stages, cost more than
 // the head start gave: the stage loads queue behind it.  31 us without, 38 with, at LLaDA's 256 rows.  Prefetching
 // 8 - 32 stages ahead as the loads go: 0 - 4 us slower too.)
@@ -72,10 +72,9 @@ struct ProjParams {
 
 __host__ __device__ constexpr bool tile_of_units(int n) { return n == 192 || n > 256; }
 
-// Where a row of the block goes: element offsets within q_out (or y), k_out / v_out and the staged layer (-1: not staged),
-// and within the rotary tables.
+// Where a row of the block goes: element offsets within q_out (or y), k_out / v_out and the staged layer (-1: not staged).
 struct __align__(16) RowEntry {
-  long long q, kv, stage, rope;
+  long long q, kv, stage;
 };
 
 // Feature tiles.  A tile takes N / 2 consecutive features from each half of a group of 2 half_rows features; with
@@ -247,7 +246,6 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       RowEntry e;
       e.q = p.mode == 1 ? (long long)row * p.n_out : ((long long)b * p.n_q_heads * p.q_cap + i) * p.head_dim;
       e.kv = ((long long)b * p.n_kv_heads * p.q_cap + i) * p.head_dim;
-      e.rope = (long long)row * (p.head_dim >> 1);
       e.stage = -1;   // cache row to stage at: none for an inactive row or one without room (reported)
       if (p.stage_k && feature(N - 1) >= p.n_q_heads * p.head_dim && (!p.q_len || i < __ldg(p.q_len + b))) {
         const int pos = __ldg(p.cache_len + b) + i;
@@ -259,30 +257,68 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   }
 
   // ================================================================= epilogue, by all eight warps
-  // fp32 columns pass through shared memory (free by then), two segments of kCW columns at a time (rotary pairs, or just
-  // two pieces), so that a store instruction writes whole sectors of neighbouring features.  One warp per scheduler runs
+  // fp32 columns pass through shared memory (free by then), in pieces of two segments of kCW columns (rotary pairs, or
+  // just two runs), so that a store instruction writes whole sectors of neighbouring features.  One warp per scheduler runs
   // this code, so its length in dependent instructions is what counts: addresses are a per-row offset (table) plus a
-  // per-segment pointer.  (Rows kept in their threads, divisions and 64-bit products per store, four warps: 10 us for the
+  // per-segment pointer, two pieces pass between two barriers, and the rotary factors are in registers before the last
+  // product is done (read piece by piece from L2: 36.4 us instead of 34.8 for 1280 rows of Dream).  (Rows kept in their threads, divisions and 64-bit products per store, four warps: 10 us for the
   // 256-feature tile.)
   {
-    const int n_rows = min(p.rc, p.rows_total - row0);       // real rows of this block (may be <= 0)
+    constexpr int kCW = N / 2 < 32 ? N / 2 : 32;              // columns of a segment
+    constexpr int kPieces = N / (2 * kCW), kPR = kPieces > 1 ? 2 : 1;   // pieces of two segments; pieces per round
+    constexpr uint32_t kPitch = 2 * kCW * 4 + 16;             // bytes of a staged row; the 16 spread rows over the banks
+    constexpr uint32_t kPieceBytes = kRowTile * kPitch;
+    constexpr int kLanes = kCW / 8, kRowsPerIt = kThreads / kLanes;
+    constexpr int kIts = kRowTile > kRowsPerIt ? kRowTile / kRowsPerIt : 1;
+    const int n_rows = min(p.rc, p.rows_total - row0);         // real rows of this block (may be <= 0)
+    const int D = p.head_dim, half = D >> 1;
+    const bool rope = p.rope_cos != nullptr;
+    const int n_qk = p.n_q_heads + p.n_kv_heads;
+    // first column of piece i and the distance from there to its second segment
+    auto column = [&](int i, int& dist) {
+      if (UNITS) {
+        const bool second = i >= kN0 / 64;
+        dist = second ? kN1 / 2 : kN0 / 2;
+        return second ? kN0 + (i - kN0 / 64) * kCW : i * kCW;
+      }
+      dist = rope && N > D ? half : N / 2;
+      if (dist == kCW) return i * 2 * kCW;
+      return dist == N / 2 ? i * kCW : (i >> 1) * 2 * dist + (i & 1) * kCW;   // half a head: 32 or 64 columns
+    };
+    // cos / sin of this thread's rows and columns: every other piece has the same (a head's half is one or two segments), so
+    // they are read once, while the products are still running
+    float4 cs[kPR][kIts][2], sn[kPR][kIts][2];
+    if (rope) {
+#pragma unroll
+      for (int pr = 0; pr < kPR; ++pr) {
+        int dist;
+        const int f = feature(column(pr, dist) + (tid % kLanes) * 8);
+        if ((f >> p.head_shift) < n_qk) {
+#pragma unroll
+          for (int it = 0; it < kIts; ++it) {
+            const int r = tid / kLanes + it * kRowsPerIt;
+            if (r < n_rows) {
+              const size_t a = (size_t)(row0 + r) * half + (f & (D - 1));
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                cs[pr][it][q] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + a) + q);
+                sn[pr][it][q] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + a) + q);
+              }
+            }
+          }
+        }
+      }
+    }
     const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, abort_ptr) ? 1 : 0) != 0;   // and the tables are there
     tc_fence_after_sync();
     if (ok && n_rows > 0) {
-      const int D = p.head_dim, half = D >> 1;
-      const bool rope = p.rope_cos != nullptr;
-      const int n_qk = p.n_q_heads + p.n_kv_heads;
-      constexpr int kCW = N / 2 < 32 ? N / 2 : 32;            // columns of a segment
-      constexpr uint32_t kPitch = 2 * kCW * 4 + 16;           // bytes of a staged row; the 16 spread rows over the banks
-      constexpr int kLanes = kCW / 8, kRowsPerIt = kThreads / kLanes;
-      constexpr int kIts = kRowTile > kRowsPerIt ? kRowTile / kRowsPerIt : 1;
-      int dist = UNITS ? kN0 / 2 : rope && N > D ? half : N / 2;   // columns between a segment and its partner
       // TMEM side: warps w and w + 4 read the lanes of quarter w % 4, one segment each.  The row of a lane: M = 64 puts 16
       // rows in each quarter; M = 128 as a pair puts rows 0-63 twice, lanes 64-127 holding the second half of the columns.
       const int quarter = warp & 3, seg = warp >> 2;
       const int my_row = M == 64 ? quarter * 16 + lane : M == 128 ? (quarter & 1) * 32 + lane : quarter * 32 + lane;
       const bool my_lane = (M != 64 || lane < 16) && my_row < n_rows;
       const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t bias_a = smem_u32(bias_s);
       // store side: where features f .. f + 7 (one head) go
       struct Dest {
         __nv_bfloat16 *out, *stage;
@@ -314,29 +350,14 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
         if (d.stage && e.stage >= 0) *reinterpret_cast<uint4*>(d.stage + e.stage) = v;
       };
       uint32_t buf = base;
-      for (int g = 0; g < N; g += 2 * dist) {
-        if (UNITS && g > 0) dist = kN1 / 2;                  // the second MMA's columns
-        for (int c = g; c < g + dist; c += kCW) {
-          const int cc = c + (tid % kLanes) * 8;             // this thread's 8 columns when it stores, and the 8 at cc + dist
-          const int f0 = feature(cc), f1 = feature(cc + dist);
-          if (UNITS && f0 >= p.n_out) break;                 // the last tile's units beyond the last feature (uniform: one unit)
-          const bool turn = rope && (f0 >> p.head_shift) < n_qk;
-          float4 cs[kIts][2], sn[kIts][2];
-          if (turn) {   // asked for before the accumulator is read
+#pragma unroll 1
+      for (int i0 = 0; i0 < kPieces; i0 += kPR) {
 #pragma unroll
-            for (int it = 0; it < kIts; ++it) {
-              const int r = tid / kLanes + it * kRowsPerIt;
-              if (r < n_rows) {
-                const size_t a = (size_t)row_s[r].rope + (f0 & (D - 1));
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                  cs[it][j] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + a) + j);
-                  sn[it][j] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + a) + j);
-                }
-              }
-            }
-          }
-          int col = c + seg * dist;
+        for (int pr = 0; pr < kPR; ++pr) {
+          if (kPieces % kPR != 0 && i0 + pr >= kPieces) break;
+          int dist;
+          int col = column(i0 + pr, dist);
+          col += seg * dist;
           bool here = true;
           if (M == 128) {
             here = col / (N / 2) == quarter >> 1;            // warp-uniform
@@ -350,23 +371,36 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
             else tmem_ld8(t_row + col, u);
             tmem_ld_wait();
             if (my_lane) {
-              const uint32_t a = buf + my_row * kPitch + seg * kCW * 4;
+              const uint32_t a = buf + pr * kPieceBytes + my_row * kPitch + seg * kCW * 4;
 #pragma unroll
               for (int j = 0; j < kCW; j += 4)
                 st_shared_f4(a + j * 4, __uint_as_float(u[j]), __uint_as_float(u[j + 1]), __uint_as_float(u[j + 2]), __uint_as_float(u[j + 3]));
             }
           }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int pr = 0; pr < kPR; ++pr) {
+          if (kPieces % kPR != 0 && i0 + pr >= kPieces) break;
+          int dist;
+          const int cc = column(i0 + pr, dist) + (tid % kLanes) * 8;   // this thread's 8 columns, and the 8 at cc + dist
+          const int f0 = feature(cc), f1 = feature(cc + dist);
+          if (UNITS && f0 >= p.n_out) break;                 // the last tile's units beyond the last feature (uniform: one unit)
+          const bool turn = rope && (f0 >> p.head_shift) < n_qk;
           const Dest d0 = dest(f0), d1 = dest(f1);
           float b0[8], b1[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) { b0[j] = bias_s[cc + j]; b1[j] = bias_s[cc + dist + j]; }
-          __syncthreads();
+          for (int j = 0; j < 8; j += 4) {
+            const float4 x = ld_shared_f4(bias_a + (cc + j) * 4), y = ld_shared_f4(bias_a + (cc + dist + j) * 4);
+            b0[j] = x.x; b0[j + 1] = x.y; b0[j + 2] = x.z; b0[j + 3] = x.w;
+            b1[j] = y.x; b1[j + 1] = y.y; b1[j + 2] = y.z; b1[j + 3] = y.w;
+          }
 #pragma unroll
           for (int it = 0; it < kIts; ++it) {
             const int r = tid / kLanes + it * kRowsPerIt;
             if (r < n_rows) {
               const RowEntry e = row_s[r];
-              const uint32_t a = buf + r * kPitch + (tid % kLanes) * 32;
+              const uint32_t a = buf + pr * kPieceBytes + r * kPitch + (tid % kLanes) * 32;
               float y0[8], y1[8];
 #pragma unroll
               for (int j = 0; j < 2; ++j) {
@@ -377,8 +411,9 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
 #pragma unroll
               for (int j = 0; j < 8; ++j) { y0[j] += b0[j]; y1[j] += b1[j]; }
               if (turn) {
-                const float co[8] = {cs[it][0].x, cs[it][0].y, cs[it][0].z, cs[it][0].w, cs[it][1].x, cs[it][1].y, cs[it][1].z, cs[it][1].w};
-                const float si[8] = {sn[it][0].x, sn[it][0].y, sn[it][0].z, sn[it][0].w, sn[it][1].x, sn[it][1].y, sn[it][1].z, sn[it][1].w};
+                const float4 (&c4)[2] = cs[pr][it], (&s4)[2] = sn[pr][it];
+                const float co[8] = {c4[0].x, c4[0].y, c4[0].z, c4[0].w, c4[1].x, c4[1].y, c4[1].z, c4[1].w};
+                const float si[8] = {s4[0].x, s4[0].y, s4[0].z, s4[0].w, s4[1].x, s4[1].y, s4[1].z, s4[1].w};
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                   const float lo = y0[j], hi = y1[j];
@@ -390,8 +425,8 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
               store8(d1, e, y1);
             }
           }
-          buf = buf == base ? base + kRowTile * kPitch : base;   // the next piece's writes meet no reader of this one
         }
+        buf = buf == base ? base + kPR * kPieceBytes : base;   // the next round's writes meet no reader of this one
       }
     }
   }
@@ -493,8 +528,8 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   if (stages > kMaxStages) stages = kMaxStages;
   if (stages > n_k) stages = n_k;
   pl.n_stages = stages;
-  // the epilogue's two staging buffers lie over the stages
-  const int staging = 2 * row_tile * (2 * cw * 4 + 16);
+  // the epilogue's two staging buffers, of one or two pieces each, lie over the stages
+  const int staging = (k.n > 2 * cw ? 4 : 2) * row_tile * (2 * cw * 4 + 16);
   pl.aux_offset = stages * stage + slack;
   if (pl.aux_offset < staging) pl.aux_offset = (staging + 127) & ~127;
   pl.smem_bytes = 1024 + pl.aux_offset + kAuxBytes;

@@ -1,6 +1,7 @@
 """The vocabulary pass at the edges of its chunking: one logit short of and beyond a batch of 4096, rows on and off 16-byte
 boundaries, chunk counts around what the merge keeps in registers, maxima in the first and last logit and repeated across
 batches, warps and chunks.  Against the oracle."""
+import numpy as np
 import pytest
 
 from helpers import Dev
@@ -43,3 +44,14 @@ def test_ranking_of_short_and_long_blocks(dev, oracle, L):
                 break
         else:
             pytest.skip("near ties in every draw")
+
+
+@pytest.mark.parametrize("L", [1, 32, 33, 100])
+def test_tickets_of_few_masked_rows(dev, oracle, L):
+    """Which blocks take a ticket: elements with no masked row, the first only, the last only, all but the first; twice, since
+    the last block resets the count."""
+    masked0 = np.zeros((4, L), np.uint8)
+    masked0[1, 0] = masked0[2, L - 1] = masked0[3, 1:] = 1
+    for _ in range(2):
+        for k in (0, 1, 3):
+            assert any(_compare_scored(dev, oracle, make_logits(4, L, 9001, (0.5, 6.0), 50 * L + seed), masked0, k, 0) for seed in range(12))

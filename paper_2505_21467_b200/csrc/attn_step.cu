@@ -1291,6 +1291,11 @@ constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two 
 constexpr double kTeamCost[2] = {2.3, 4.3};      // the team schedule's exchange and reduction
 constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...
 constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond that
+// With more units than SMs a block has whole units to compute while its first piece travels, and merges one unit at most.
+// 40 layer-batched calls, split against whole: with two M tiles the split was 4 - 9 us slower where it saves one key tile a
+// block, equal at two and 1 - 2 us faster at three (4 us at four: 5 layers x 2 x 419 rows 88.8 -> 84.5); with one M tile
+// 2 - 4 us slower at one and two, equal at three, 1 - 2 us faster at four.
+constexpr double kSplitManyCost[2] = {3.2, 2.7};
 
 // The best plan with row chunks of `chunk_rows`, and its estimated cost.
 double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
@@ -1311,14 +1316,15 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
   pl.grid = (int)(units < sms ? units : sms);
   if (!may_split) return best;
   // units split across blocks: equal shares, but a partial store per block and a merge per unit
-  auto consider_split = [&](long long shares) {
-    const double pieces = (double)shares / (double)units;
+  for (long long shares = units + 1; shares <= sms && shares <= units * tiles_unit; ++shares) {
     const double t = (double)((units * tiles_unit + shares - 1) / shares) * tile + kSplitCost[pl.n_mt - 1] +
-                     (pieces > 1.0 ? kSplitPiece * (pieces - 1.0) : kSplitPiece);
+                     kSplitPiece * ((double)shares / (double)units - 1.0);
     if (t < best) { best = t; pl.whole_units = 0; pl.grid = (int)shares; }
-  };
-  for (long long shares = units + 1; shares <= sms && shares <= units * tiles_unit; ++shares) consider_split(shares);
-  if (units > sms) consider_split(sms);   // more units than SMs: the only split is over all SMs
+  }
+  if (units > sms) {   // more units than SMs: the only split is over all SMs
+    const double t = (double)((units * tiles_unit + sms - 1) / sms) * tile + kSplitManyCost[pl.n_mt - 1];
+    if (t < best) { best = t; pl.whole_units = 0; pl.grid = sms; }
+  }
   // Team schedule for calls with few units: C blocks per unit, the unit's key tiles dealt among them, every
   // block reducing a C-th of the outputs over all pieces in parallel (the split schedule's merging block
   // folds the other pieces one after the other).  The smallest C that reaches the fewest tiles per block.

@@ -25,7 +25,8 @@
 // (barrier wait 100, expect 40, each copy 55), which bound the kernel when every 64 elements of K took an iteration.
 //
 // Block = 8 warps: warp 0 weight producer, warp 1 activation producer, warp 2 tcgen05.mma issuer (of the leader block),
-// warp 3 TMEM, warps 4-7 the epilogue's tables; all eight write the results.
+// warp 3 TMEM and, for activations in many pieces, half of their copies, warps 4-7 the epilogue's tables; all eight write
+// the results.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -63,6 +64,7 @@ struct ProjParams {
   int act_heads;               // activations are [B][act_heads][q_cap][D] (0: plain [rows][K])
   int rc;                      // rows per block (a multiple of 8)
   int x_box_rows;              // rows per copy of head-split activations (rc: one copy brings all)
+  int pieces;                  // copies that bring a panel of a block's activation rows
   int half_rows;               // features of a group's half: W is seen as [groups][2][half_rows][K]
   int w_box_rows;              // tiles of units: features per copy of the weights (32, or 64 where units lie in pairs)
   int n_stages, aux_offset;
@@ -154,7 +156,33 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();
 
-  if (warp < 2) {
+  if (p.pieces > 1 && (warp == 1 || warp == 3)) {
+    // ================================================================= activations in pieces of sequences
+    // Head-split activations [B][heads][q_cap][D] whose rows of a block end inside a sequence.  A lane of warps 1 and 3 has its
+    // copy of every stage, its coordinates but the panel's known beforehand (all by one lane, with the divisions in the loop
+    // below: 125 cycles a copy).
+    const uint32_t full0 = PAIR ? map_shared_rank(bar_full, 0) : bar_full;
+    const int head_panels = p.head_dim / kPanel, item = (lane << 1) + (warp >> 1);
+    const int my_kp = item / p.pieces, my_row = (item - my_kp * p.pieces) * p.x_box_rows;
+    const int z = (row0 + my_row) / p.q_cap, y = row0 + my_row - z * p.q_cap;
+    int head = my_kp / head_panels, panel = my_kp - head * head_panels, s = 0, round = 0, issued = 0;
+    bool ok = true;
+    for (int kc = 0; kc < n_k; ++kc) {
+      if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
+      if (!ok) break;
+      if (warp == 1 && rank == 0 && lane == 0) mbar_expect_tx(bar_full + 8 * s, x_bytes * 2u);   // pieces: always a pair
+      __syncwarp();
+      if (my_kp < KP)
+        tma_load_4d<PAIR>(base + s * stage_bytes + my_kp * x_panel + my_row * 128, &tm_x, full0 + 8 * s, panel * kPanel, y, head, z);
+      for (panel += KP; panel >= head_panels; panel -= head_panels) ++head;
+      __syncwarp();
+      ++issued;
+      if (++s == p.n_stages) { s = 0; ++round; }
+    }
+    if (!ok && rank == 0)   // as below
+      for (int i = max(0, issued - p.n_stages); i < issued; ++i)
+        mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
+  } else if (warp < 2) {
     // ================================================================= producers (0: weights, 1: activations)
     const uint32_t bytes = (warp == 0 ? kWBytes : x_bytes) * (PAIR ? 2u : 1u);   // what the leader's barrier gets from both blocks
     const uint32_t full0 = PAIR ? map_shared_rank(bar_full, 0) : bar_full;
@@ -182,10 +210,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
           // activations [B][heads][q_cap][D]: panel k belongs to head k / (D / 64); rows of a box are (sequence, row)
           int h = head, pn = panel;
           for (int kp = 0; kp < KP; ++kp) {
-            const uint32_t d = dst + kp * x_panel;
-            tma_load_4d<PAIR>(d, &tm_x, bar, pn * kPanel, y0, h, z0);
-            for (int r = p.x_box_rows; r < p.rc; r += p.x_box_rows)
-              tma_load_4d<PAIR>(d + r * 128, &tm_x, bar, pn * kPanel, (row0 + r) % p.q_cap, h, (row0 + r) / p.q_cap);
+            tma_load_4d<PAIR>(dst + kp * x_panel, &tm_x, bar, pn * kPanel, y0, h, z0);
             if (++pn == head_panels) { pn = 0; ++h; }
           }
         }
@@ -463,12 +488,13 @@ struct ProjPlan {
   int variant, rc, x_box_rows, w_box_rows, chunks, tiles, half_rows, n_stages, aux_offset, smem_bytes;
 };
 
-int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
-
 // rows: activation rows of the call; heads_q_cap > 0: head-split activations (all rows in one chunk) with that many rows
 // per sequence, `batch` sequences.
 bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int head_dim, int batch, int heads_q_cap, ProjPlan& pl) {
-  const int m = rows <= 64 ? 64 : rows <= 128 ? 128 : 256;
+  // (head-split activations whose half of the sequences is more than the 64 rows of a pair's block take the wide pairs: one
+  // copy per panel instead of pieces of a sequence)
+  const bool wide = heads_q_cap > 0 && batch > 1 && (batch + 1) / 2 * heads_q_cap > 64;
+  const int m = rows <= 64 ? 64 : rows <= 128 && !wide ? 128 : 256;
   const bool pair = m > 64;
   if (heads_q_cap > 0 && rows > kMaxActRows) return false;
   pl.chunks = pair ? (rows + 255) / 256 : 1;
@@ -476,13 +502,19 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   pl.rc = ((rows + blocks_rows - 1) / blocks_rows + 7) & ~7;
   pl.x_box_rows = pl.rc;
   if (heads_q_cap > 0 && batch > 1) {
-    // one copy brings the rows of whole sequences; where the pair's split falls inside one, copies of a common divisor
+    // one copy brings the rows of whole sequences; where the pair's split falls inside one, copies of the largest divisor of a
+    // sequence (in eights) that leaves no block more than its rows.  With the common divisor of sequence and block, 14 copies of 8 rows a
+    // panel at 3 x 72 rows, an output projection of Dream took 65.5 us; with the 5 of 24, dealt over lanes, 13.9.
     const int nb = (batch + blocks_rows - 1) / blocks_rows;
     if (nb * heads_q_cap <= (m == 128 ? 64 : 128)) {
       pl.rc = pl.x_box_rows = nb * heads_q_cap;
     } else {
-      pl.x_box_rows = gcd(heads_q_cap, m == 128 ? 64 : 128);
-      pl.rc = (pl.rc + pl.x_box_rows - 1) / pl.x_box_rows * pl.x_box_rows;
+      const int half = (rows + 1) / 2, limit = m == 128 ? 64 : 128;
+      for (int d = heads_q_cap; d >= 8; d -= 8) {   // d = 8 always fits
+        pl.x_box_rows = d;
+        pl.rc = (half + d - 1) / d * d;
+        if (heads_q_cap % d == 0 && pl.rc <= limit) break;
+      }
     }
   }
   // The tile width: estimated cycles of the SM with the most blocks.  Per 16 elements of K a block's MMA takes N / 2
@@ -545,6 +577,7 @@ int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorM
   }
   p.rc = pl.rc;
   p.x_box_rows = pl.x_box_rows;
+  p.pieces = p.act_heads ? pl.rc / pl.x_box_rows : 1;
   p.half_rows = pl.half_rows;
   p.w_box_rows = pl.w_box_rows;
   p.n_stages = pl.n_stages;

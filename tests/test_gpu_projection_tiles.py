@@ -72,6 +72,10 @@ def test_qkv_projection_tiles(dev, oracle, B, q_cap, dm, Hq, Hkv, D):
     (1, 200, 256, 3, 64),
     (3, 80, 128, 5, 64),          # 240 rows: as above, with 128 rows a block
     (9, 24, 256, 2, 128),
+    (3, 72, 128, 3, 64),          # 216 rows in pieces of 24
+    (5, 48, 384, 2, 128),         # the same, five sequences
+    (5, 24, 128, 3, 128),         # 120 rows whose half of the sequences exceeds the narrow pair's rows
+    (3, 56, 256, 1, 192),         # heads of three panels
 ])
 def test_out_projection_tiles(dev, oracle, B, q_cap, dm, Hq, D):
     seed = 17 * B + q_cap

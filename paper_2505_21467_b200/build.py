@@ -3,6 +3,7 @@
 from __future__ import annotations
 
 import glob
+import hashlib
 import os
 import subprocess
 import sys
@@ -52,15 +53,40 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def calls_abi() -> str:
+    """Whose C++ and C objects _dlm_calls.so reads: this torch's and this Python's."""
+    import torch
+    return f"torch {torch.__version__} {torch.version.git_version} {sys.implementation.cache_tag}"
+
+
+def calls_fingerprint() -> str:
+    """What _dlm_calls.so is built from and for.  The module carries it (DLM_CALLS_BUILT_FOR), so that one built for another
+    torch or another Python counts as stale however new its file is."""
+    h = hashlib.sha256()
+    for d in [CALLS_SRC, *sorted(glob.glob(os.path.join(INCLUDE, "*.h")))]:
+        with open(d, "rb") as f:
+            h.update(f.read())
+    return f"dlm_calls for {calls_abi()}, sources {h.hexdigest()}"
+
+
+def calls_built_for(what: str) -> bool:
+    """Whether the _dlm_calls.so in place carries `what` (read from the file: a module for another torch is not loaded)."""
+    try:
+        with open(CALLS, "rb") as f:
+            return what.encode() in f.read()
+    except OSError:
+        return False
+
+
 def build_calls(force: bool = False, verbose: bool = False) -> str:
     """Compile the Python entry points (needs torch's headers, no GPU)."""
-    deps = [CALLS_SRC, *glob.glob(os.path.join(INCLUDE, "*.h"))]
-    if not force and os.path.exists(CALLS) and all(os.path.getmtime(d) <= os.path.getmtime(CALLS) for d in deps):
+    if not force and calls_built_for(calls_fingerprint()):
         return CALLS
     import torch
     from torch.utils import cpp_extension
     tmp = CALLS + f".{os.getpid()}.tmp"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DDLM_CALLS_BUILT_FOR="{calls_fingerprint()}"',
            "-I", INCLUDE, "-I", sysconfig.get_paths()["include"]]
     for d in cpp_extension.include_paths("cuda"):
         cmd += ["-isystem", d]

@@ -382,8 +382,14 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_dlm_calls", nullptr, -1, g_meth
 
 }  // namespace
 
+#ifndef DLM_CALLS_BUILT_FOR   // the torch, the Python and the sources of this build (build.py)
+#define DLM_CALLS_BUILT_FOR "unknown"
+#endif
+
 PyMODINIT_FUNC PyInit__dlm_calls() {
   fill_methods(std::make_integer_sequence<int, kNumEntries>());
   g_methods[kNumEntries] = {"set_error", set_error, METH_O, nullptr};
-  return PyModule_Create(&g_module);
+  PyObject* m = PyModule_Create(&g_module);
+  if (m && PyModule_AddStringConstant(m, "built_for", DLM_CALLS_BUILT_FOR) != 0) Py_CLEAR(m);
+  return m;
 }

@@ -35,3 +35,24 @@ def test_tensors_are_checked_before_anything_runs():
         dlm.dlm_guided_accept(None, *([None] * 2), "one", 4, *([None] * 2), 0, *([None] * 3))
     with pytest.raises(TypeError):      # the cache is not a dlm_kv_cache
         dlm.dlm_kv_cache_commit(None, None, None, None, 1, None, None, 0, None, 1, 0, 0, 1)
+
+
+def test_a_module_for_another_torch_is_stale_and_not_loaded(monkeypatch):
+    """The module reads torch's C++ objects: one built for another torch (or Python) is rebuilt however new its file is, and is
+    refused before it is loaded."""
+    from paper_2505_21467_b200 import _binding
+    assert _build.calls_built_for(_build.calls_fingerprint()) and _binding._load_calls().built_for == _build.calls_fingerprint()
+    built = []
+    monkeypatch.setattr(_build.subprocess, "run", lambda cmd, **kw: built.append(cmd) or _Failed())
+    assert _build.build_calls() == _build.CALLS and not built      # fresh: nothing to do
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    with pytest.raises(RuntimeError, match="_dlm_calls"):           # stale: the compiler is called (and fails here)
+        _build.build_calls()
+    assert len(built) == 1
+    monkeypatch.setattr(_binding, "_calls", None)
+    with pytest.raises(ImportError, match="not built for torch 9.9.9"):
+        _binding._load_calls()
+
+
+class _Failed:
+    returncode, stdout = 1, ""

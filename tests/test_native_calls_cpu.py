@@ -50,7 +50,17 @@ def test_a_module_for_another_torch_is_stale_and_not_loaded(monkeypatch):
         _build.build_calls()
     assert len(built) == 1
     monkeypatch.setattr(_binding, "_calls", None)
-    with pytest.raises(ImportError, match="not built for torch 9.9.9"):
+    with pytest.raises(ImportError, match="not built .* for torch 9.9.9"):
+        _binding._load_calls()
+
+
+def test_a_module_of_other_sources_is_not_loaded(monkeypatch):
+    """Nor is one whose functions may be other ones than the package calls: importing the package has to stay possible, or it
+    could not be built again."""
+    from paper_2505_21467_b200 import _binding
+    monkeypatch.setattr(_build, "CALLS_SRC", __file__)
+    monkeypatch.setattr(_binding, "_calls", None)
+    with pytest.raises(ImportError, match="present sources"):
         _binding._load_calls()
 
 

@@ -209,6 +209,7 @@ def _load_calls():
             raise ImportError(f"{_build.CALLS} cannot be loaded ({e}): run `python -m paper_2505_21467_b200.build` "
                               "(there is no CPU or PyTorch fallback)") from e
         m.set_error(DlmError)
+        m.set_types(ctypes.c_void_p, dlm_kv_cache)
         _calls = m
     return _calls
 

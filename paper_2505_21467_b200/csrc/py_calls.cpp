@@ -14,6 +14,9 @@
 namespace {
 
 PyObject* g_error = nullptr;   // DlmError(code, where), set by the package
+// The classes whose memory is read as a pointer and as a dlm_kv_cache (ctypes.c_void_p and the package's structure), set by
+// the package.  Nothing else will do: the bytes of another object would be taken for device addresses.
+PyTypeObject *g_handle_type = nullptr, *g_cache_type = nullptr;
 
 struct Args;
 typedef int (*CallFn)(Args&);
@@ -35,14 +38,24 @@ struct Args {
   void* handle(int i) {
     PyObject* o = v[i];
     if (o == Py_None) return nullptr;
-    if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
-    return *static_cast<void**>(buffer(i, sizeof(void*)));
+    if (PyLong_Check(o)) {
+      void* const p = PyLong_AsVoidPtr(o);
+      if (!p && PyErr_Occurred()) failed = true;
+      return p;
+    }
+    return *static_cast<void**>(buffer(i, g_handle_type, sizeof(void*)));
   }
-  // address of the memory behind a ctypes object of at least `bytes` bytes (the argument stays alive during the call)
-  void* buffer(int i, Py_ssize_t bytes) {
+  // address of the memory behind a ctypes object of class `type` and at least `bytes` bytes (the argument stays alive during the call)
+  void* buffer(int i, PyTypeObject* type, Py_ssize_t bytes) {
     static void* zero[16] = {};
+    if (failed) return zero;
+    if (!type || !PyObject_TypeCheck(v[i], type)) {
+      PyErr_Format(PyExc_TypeError, "expected %s, got %s", type ? type->tp_name : "a ctypes object", Py_TYPE(v[i])->tp_name);
+      failed = true;
+      return zero;
+    }
     Py_buffer b;
-    if (failed || PyObject_GetBuffer(v[i], &b, PyBUF_SIMPLE) != 0) { failed = true; return zero; }
+    if (PyObject_GetBuffer(v[i], &b, PyBUF_SIMPLE) != 0) { failed = true; return zero; }
     void* p = b.buf;
     const bool ok = b.len >= bytes;
     PyBuffer_Release(&b);
@@ -53,7 +66,7 @@ struct Args {
     }
     return p;
   }
-  const dlm_kv_cache* cache(int i) { return static_cast<const dlm_kv_cache*>(buffer(i, sizeof(dlm_kv_cache))); }
+  const dlm_kv_cache* cache(int i) { return static_cast<const dlm_kv_cache*>(buffer(i, g_cache_type, sizeof(dlm_kv_cache))); }
   int integer(int i) {
     if (failed) return 0;
     if (PyLong_Check(v[i])) return (int)PyLong_AsUnsignedLongMask(v[i]);
@@ -371,7 +384,17 @@ PyObject* set_error(PyObject*, PyObject* cls) {
   Py_RETURN_NONE;
 }
 
-PyMethodDef g_methods[kNumEntries + 2];
+PyObject* set_types(PyObject*, PyObject* args) {
+  PyObject *handle, *cache;
+  if (!PyArg_ParseTuple(args, "O!O!", &PyType_Type, &handle, &PyType_Type, &cache)) return nullptr;
+  Py_INCREF(handle);
+  Py_INCREF(cache);
+  Py_XSETREF(g_handle_type, reinterpret_cast<PyTypeObject*>(handle));
+  Py_XSETREF(g_cache_type, reinterpret_cast<PyTypeObject*>(cache));
+  Py_RETURN_NONE;
+}
+
+PyMethodDef g_methods[kNumEntries + 3];
 
 template <int... I>
 void fill_methods(std::integer_sequence<int, I...>) {
@@ -389,6 +412,7 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_dlm_calls", nullptr, -1, g_meth
 PyMODINIT_FUNC PyInit__dlm_calls() {
   fill_methods(std::make_integer_sequence<int, kNumEntries>());
   g_methods[kNumEntries] = {"set_error", set_error, METH_O, nullptr};
+  g_methods[kNumEntries + 1] = {"set_types", set_types, METH_VARARGS, nullptr};
   PyObject* m = PyModule_Create(&g_module);
   if (m && PyModule_AddStringConstant(m, "built_for", DLM_CALLS_BUILT_FOR) != 0) Py_CLEAR(m);
   return m;

@@ -1,4 +1,7 @@
 """The native entry points check and order their arguments like the Python signatures they stand for (no GPU needed)."""
+import ctypes
+
+import numpy as np
 import pytest
 import torch
 
@@ -35,6 +38,19 @@ def test_tensors_are_checked_before_anything_runs():
         dlm.dlm_guided_accept(None, *([None] * 2), "one", 4, *([None] * 2), 0, *([None] * 3))
     with pytest.raises(TypeError):      # the cache is not a dlm_kv_cache
         dlm.dlm_kv_cache_commit(None, None, None, None, 1, None, None, 0, None, 1, 0, 0, 1)
+
+
+def test_bytes_of_other_objects_are_not_taken_for_addresses():
+    """A context or a cache is what the package makes, not any object with a buffer of that size."""
+    other = [b"\0" * 64, bytearray(64), np.zeros(64, np.uint8), (ctypes.c_char * 64)(), ctypes.c_int64(0)]
+    for wrong in other:
+        with pytest.raises(TypeError, match="expected"):
+            dlm.dlm_guided_accept(wrong, None, None, 1, 4, None, None, 0, None, None, None)
+    for wrong in other + [ctypes.c_void_p(), 0]:
+        with pytest.raises(TypeError, match="expected"):
+            dlm.dlm_kv_cache_commit(None, wrong, None, None, 1, None, None, 0, None, 1, 0, 0, 1)
+    with pytest.raises(OverflowError):
+        dlm.dlm_guided_accept(1 << 70, None, None, 1, 4, None, None, 0, None, None, None)
 
 
 def test_a_module_for_another_torch_is_stale_and_not_loaded(monkeypatch):

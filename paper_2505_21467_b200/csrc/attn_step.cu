@@ -797,14 +797,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
           ++seg;
         }
-        if (!ok) {
-          // unwinding: let the copies already issued land before the block's memory is released
-          for (uint32_t i = (kt > (uint32_t)KS ? kt - KS : 0); i < kt; ++i)
-            mbar_wait(bar_k_full + 8 * (i % KS), (i / KS) & 1, never_ptr);
-          for (uint32_t i = (vt > (uint32_t)VS ? vt - VS : 0); i < vt; ++i)
-            mbar_wait(bar_v_full + 8 * (i % VS), (i / VS) & 1, never_ptr);
-          if (q_issued > 0) mbar_wait(bar_q_full, (q_issued - 1) & 1, never_ptr);
-        }
+        // No copy lands after the block has released its shared memory: wait for those whose consumer may not have, also when
+        // this lane itself never had to give up (its last copies were issued before another role did, or a unit without key
+        // tiles has its Q on the way).  They have landed long since unless the block is unwinding.
+        for (uint32_t i = (kt > (uint32_t)KS ? kt - KS : 0); i < kt; ++i)
+          mbar_wait(bar_k_full + 8 * (i % KS), (i / KS) & 1, never_ptr);
+        for (uint32_t i = (vt > (uint32_t)VS ? vt - VS : 0); i < vt; ++i)
+          mbar_wait(bar_v_full + 8 * (i % VS), (i / VS) & 1, never_ptr);
+        if (q_issued > 0) mbar_wait(bar_q_full, (q_issued - 1) & 1, never_ptr);
       }
     } else if (warp == 9 || warp == 10) {
       // ============================================ MMA issuers: warp 9 for M tile 0, warp 10 for M tile 1

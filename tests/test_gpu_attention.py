@@ -252,6 +252,33 @@ def test_the_attention_kernel_gives_up_cleanly_when_its_waits_may_not_wait(dev, 
     assert e.value.code == dlm.DLM_ERR_SHAPE
 
 
+@pytest.mark.parametrize("D,cache_len,q_len", [
+    (128, [100, 90], None),         # two key tiles: the producer has issued everything before it would have to wait
+    (128, [100, 0], [16, 0]),       # a unit without key tiles, whose Q is copied all the same
+    (64, [330, 200], [16, 9]),      # the deeper rings of heads of 64: up to four key tiles
+])
+def test_giving_up_lets_copies_land_that_nobody_waits_for(dev, oracle, D, cache_len, q_len):
+    """A launch that gives up although its producer never had to wait ends only when its copies have landed: the blocks of the
+    next launch, right behind it on the same SMs, take over that shared memory.  Units dealt whole (no counters to clear)."""
+    ck, cv = make_cache(2, 2, 4, 400, D, 1)
+    q, kn, vn = make_attn_inputs(2, 2, 28, 4, 16, D, 2)
+    cl, ql = _i32(cache_len), None if q_len is None else _i32(q_len)
+    args = [t.cuda() for t in (ck, cv)] + [cl] + [t.cuda() for t in (q, kn, vn)] + [ql]
+    assert _schedule(dev, 2, 2, 28, 4, D, 400, 16, 2, 1)["whole_units"] == 1 == _schedule(dev, 2, 2, 28, 4, D, 400, 16, 2, 1)["team"]
+    ref = oracle_attn_layers(oracle, ck, cv, cl, q, kn, vn, ql)
+    gpu_attn_step(dev, *args, hint=1)
+    for _ in range(4):
+        dlm.dlm_selftest_set_wait_limit(dev.ctx, 0)
+        try:
+            gpu_attn_step(dev, *args, hint=1)
+        finally:
+            dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
+        out, lse = gpu_attn_step(dev, *args, hint=1)
+        assert dev.status() == dlm.DLM_ERR_TIMEOUT
+        for lc in ref:
+            assert_attn_close(out, lse, ref[lc], lc)
+
+
 def _schedule(dev, NL, B, Hq, Hkv, D, Lcap, q_cap, nl, hint=0):
     ck = torch.empty(NL, B, Hkv, Lcap, D, dtype=torch.bfloat16, device="cuda")
     cache = dlm.make_kv_cache(ck, ck, _i32([0] * B))

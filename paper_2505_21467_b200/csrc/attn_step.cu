@@ -278,9 +278,10 @@ struct TeamArgs {
 // (bar_pub), count the block in the unit's arrival counter; when the whole team has arrived, fetch this
 // block's share of every piece, and every piece's (m, l) rows, into the shared memory the Q, K and V buffers no
 // longer need (all of the block's MMAs have finished by then: every softmax thread waited for its last one).
-// bar_team = bar_pub + 8 completes when all of it has landed.
+// bar_team = bar_pub + 8 completes when all of it has landed.  A block without a key tile of its own has run no MMA, and
+// its Q may still be on its way to that shared memory: bar_q is waited for too.
 template <int D, bool kNoWait>
-__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
+__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_q, uint32_t bar_pub,
                                           volatile int* abort_ptr) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   const uint32_t bar_team = bar_pub + 8;
@@ -288,6 +289,7 @@ __device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint3
   __threadfence();
   atomicAdd(p.arrive, 1u);
   if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
+  if (!mbar_wait_limit(bar_q, 0, abort_ptr, kLimit)) return;
   fence_proxy_async_all();
   mbar_expect_tx(bar_team, (uint32_t)p.team * (p.ml_bytes + p.o_bytes));
   for (int c = 0; c < p.team; ++c) {
@@ -938,7 +940,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // (they arrive on bar_pub and move on), make the stores visible device-wide and count the
       // piece in its unit's counter.
       if (lane == 0 && p.team > 1) {
-        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr);
+        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_q_full, bar_pub, abort_ptr);
       } else if (lane == 0 && has_work && !p.whole_units) {
         SegmentWalker walk(p, sched, blockIdx.x);
         Segment g;

@@ -336,6 +336,21 @@ def test_team_schedule_repeated_launches_leave_the_counters_clean(dev, oracle):
     _case(dev, oracle, 2, 2, 28, 4, 128, 1400, 32, [1368, 900], [32, 17], seed=77)
 
 
+def test_team_members_without_key_tiles(dev, oracle):
+    """Sequences much shorter than the hint: most blocks of a team have no key tile and are done before the Q they were sent
+    has landed in the shared memory that the others' pieces go to.  Many launches back to back, every one the same."""
+    B, Lcap, q_cap = 2, 2200, 32
+    assert _schedule(dev, 1, B, 28, 4, 128, Lcap, q_cap, 1)["team"] > 2
+    out, lse, _ = _case(dev, oracle, 1, B, 28, 4, 128, Lcap, q_cap, [0, 60], [1, 32], seed=811)
+    ck, cv = make_cache(1, B, 4, Lcap, 128, 811, device="cpu")
+    q, kn, vn = make_attn_inputs(1, B, 28, 4, q_cap, 128, 812, device="cpu")
+    args = [t.cuda() for t in (ck, cv)] + [_i32([0, 60])] + [t.cuda() for t in (q, kn, vn)] + [_i32([1, 32])]
+    again = [gpu_attn_step(dev, *args) for _ in range(64)]
+    assert dev.status() == 0
+    for o, l in again:
+        assert torch.equal(o, out) and torch.equal(l, lse)
+
+
 def test_team_schedule_gives_up_cleanly_when_its_waits_may_not_wait(dev, oracle):
     """The give-up path under the team schedule: with the wait limit at 0 every wait, the one for the team's other
     blocks included, gives up at once.  The kernel ends normally with DLM_ERR_TIMEOUT, reading the status clears

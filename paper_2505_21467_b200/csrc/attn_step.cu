@@ -53,6 +53,7 @@ constexpr int kTeamMax = 16;              // most blocks of a team
 constexpr int kMaxGrid = 256;          // blocks of the persistent grid (one per SM)
 constexpr int kMaxStages = 8;          // barrier slots reserved per ring
 constexpr int kBarrierBytes = 512;     // mbarriers of a block
+constexpr int kBarPub = 32 + 4 * 8 * kMaxStages + 3 * 32;   // distance of the publisher's barrier from the first, which is Q's
 constexpr int kFlagBytes = 64;         // abort / never flags, TMEM slot, merge flag
 
 template <int D>
@@ -279,9 +280,9 @@ struct TeamArgs {
 // block's share of every piece, and every piece's (m, l) rows, into the shared memory the Q, K and V buffers no
 // longer need (all of the block's MMAs have finished by then: every softmax thread waited for its last one).
 // bar_team = bar_pub + 8 completes when all of it has landed.  A block without a key tile of its own has run no MMA, and
-// its Q may still be on its way to that shared memory: bar_q is waited for too.
+// its Q may still be on its way to that shared memory: the barrier of Q, bar_pub - kBarPub, is waited for too.
 template <int D, bool kNoWait>
-__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_q, uint32_t bar_pub,
+__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
                                           volatile int* abort_ptr) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   const uint32_t bar_team = bar_pub + 8;
@@ -289,7 +290,7 @@ __device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint3
   __threadfence();
   atomicAdd(p.arrive, 1u);
   if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
-  if (!mbar_wait_limit(bar_q, 0, abort_ptr, kLimit)) return;
+  if (!mbar_wait_limit(bar_pub - kBarPub, 0, abort_ptr, kLimit)) return;
   fence_proxy_async_all();
   mbar_expect_tx(bar_team, (uint32_t)p.team * (p.ml_bytes + p.o_bytes));
   for (int c = 0; c < p.team; ++c) {
@@ -624,7 +625,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t bar_pv_done = bar_p_ready + 32;                 // [M tile][half-step parity] P V product finished.  Two P V
                                                                  // products can be in flight, so consecutive half-steps use different
                                                                  // barriers: a parity wait cannot tell phases two apart
-  const uint32_t bar_pub = bar_pv_done + 32;                     // partial result of a segment stored by every softmax thread
+  const uint32_t bar_pub = sm_bar + kBarPub;                     // partial result of a segment stored by every softmax thread
   const uint32_t bar_team = bar_pub + 8;                         // team schedule: the team's pieces of this block's share have landed
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -940,7 +941,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // (they arrive on bar_pub and move on), make the stores visible device-wide and count the
       // piece in its unit's counter.
       if (lane == 0 && p.team > 1) {
-        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_q_full, bar_pub, abort_ptr);
+        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr);
       } else if (lane == 0 && has_work && !p.whole_units) {
         SegmentWalker walk(p, sched, blockIdx.x);
         Segment g;

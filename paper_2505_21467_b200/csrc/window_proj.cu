@@ -156,6 +156,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();
 
+  int issued = 0;   // stages this producer warp has issued
   if (p.pieces > 1 && (warp == 1 || warp == 3)) {
     // ================================================================= activations in pieces of sequences
     // Head-split activations [B][heads][q_cap][D] whose rows of a block end inside a sequence.  A lane of warps 1 and 3 has its
@@ -165,7 +166,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     const int head_panels = p.head_dim / kPanel, item = (lane << 1) + (warp >> 1);
     const int my_kp = item / p.pieces, my_row = (item - my_kp * p.pieces) * p.x_box_rows;
     const int z = (row0 + my_row) / p.q_cap, y = row0 + my_row - z * p.q_cap;
-    int head = my_kp / head_panels, panel = my_kp - head * head_panels, s = 0, round = 0, issued = 0;
+    int head = my_kp / head_panels, panel = my_kp - head * head_panels, s = 0, round = 0;
     bool ok = true;
     for (int kc = 0; kc < n_k; ++kc) {
       if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
@@ -179,9 +180,6 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       ++issued;
       if (++s == p.n_stages) { s = 0; ++round; }
     }
-    if (!ok && rank == 0)   // as below
-      for (int i = max(0, issued - p.n_stages); i < issued; ++i)
-        mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
   } else if (warp < 2) {
     // ================================================================= producers (0: weights, 1: activations)
     const uint32_t bytes = (warp == 0 ? kWBytes : x_bytes) * (PAIR ? 2u : 1u);   // what the leader's barrier gets from both blocks
@@ -190,7 +188,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     int head = 0, panel = 0;                                // head-split activations: where the next K panel lies
     const int y0 = p.batch > 1 ? row0 % p.q_cap : row0, z0 = p.batch > 1 ? row0 / p.q_cap : 0;
     bool ok = true;
-    int s = 0, round = 0, issued = 0;
+    int s = 0, round = 0;
     for (int kc = 0; kc < n_k; ++kc) {
       if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
       if (!ok) break;
@@ -221,9 +219,6 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       ++issued;
       if (++s == p.n_stages) { s = 0; ++round; }
     }
-    if (!ok && rank == 0)   // unwinding: let the copies already issued land before the memory is released (both blocks' land on the leader's barriers)
-      for (int i = max(0, issued - p.n_stages); i < issued; ++i)
-        mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
   } else if (warp == 2 && rank == 0) {
     // ================================================================= MMA issuer
     bool ok = true;
@@ -334,9 +329,18 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
         }
       }
     }
-    const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, abort_ptr) ? 1 : 0) != 0;   // and the tables are there
+    // The last MMA is waited for whether or not a role of this block has given up: it reads the stages and writes TMEM.  (The
+    // tables are there too.)
+    const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, never_ptr) ? 1 : 0) != 0;
     tc_fence_after_sync();
-    if (ok && n_rows > 0) {
+    // Unwinding: the copies already issued land before anything else is put in their place or the memory is released, also those
+    // of a producer that never had to wait (the issuer may have given up behind it).  Both blocks' copies complete on the
+    // leader's barriers.  Otherwise the issuer has waited for every one of them.
+    const bool gave_up = *abort_ptr != 0;
+    if (gave_up && rank == 0)
+      for (int i = max(0, issued - p.n_stages); i < issued; ++i)
+        mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
+    if (ok && !gave_up && n_rows > 0) {
       // TMEM side: warps w and w + 4 read the lanes of quarter w % 4, one segment each.  The row of a lane: M = 64 puts 16
       // rows in each quarter; M = 128 as a pair puts rows 0-63 twice, lanes 64-127 holding the second half of the columns.
       const int quarter = warp & 3, seg = warp >> 2;
@@ -457,7 +461,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
   }
   // ---- teardown
   __syncwarp();
-  if (tid == 0 && *abort_ptr) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
+  if (tid == 0 && (*abort_ptr || *never_ptr)) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
   tc_fence_before_sync();
   // a pair leaves together: the leader's MMAs read the other block's shared memory, both blocks' copies complete on the leader's barriers
   if (PAIR) cluster_sync(); else __syncthreads();

@@ -18,7 +18,7 @@
  *   - Pointers documented "device" are caller-owned device pointers on the context's GPU and
  *     must stay valid until the enqueued work has finished.  The library never allocates,
  *     frees or retains tensor memory; the only device memory it owns is about 12 KB of
- *     status and ticket words inside the context.
+ *     status and ticket words per context, and dlm_unmask_select_static's array.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  All calls
  *     only enqueue work; none synchronises except dlm_get_status.
  *   - Data-dependent errors (an index out of range, an append beyond capacity, a bounded
@@ -59,8 +59,9 @@ typedef struct dlm_ctx dlm_ctx;
 /* Creates a context bound to CUDA device `device` (must be compute capability 10.x).
  * Every later call that takes the context must be made with that device current on the
  * calling thread (else DLM_ERR_DEVICE, nothing launched).
- * The context owns only its status / ticket words.  Not thread-safe: use one context per
- * host thread or serialise calls.  Kernels enqueued through one context on different
+ * The context owns its status / ticket words and, on the host, what its calls keep for the next ones: TMA descriptors
+ * (functions of an address and sizes) and the last attention call's plan (a function of sizes).  Not thread-safe: use
+ * one context per host thread or serialise calls.  Kernels enqueued through one context on different
  * streams must not overlap in time (they share the context's ticket words). */
 int dlm_create(dlm_ctx** out, int device);
 int dlm_destroy(dlm_ctx* ctx);

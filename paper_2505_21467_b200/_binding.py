@@ -46,53 +46,24 @@ def lib() -> ctypes.CDLL:
         raise ImportError(f"{path} is missing: run `python -m paper_2505_21467_b200.build` "
                           "(there is no CPU or PyTorch fallback)")
     L = ctypes.CDLL(path)
-    vp, i32, f32, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_size_t
-    L.dlm_create.argtypes = [ctypes.POINTER(vp), i32]
-    L.dlm_destroy.argtypes = [vp]
-    L.dlm_get_status.argtypes = [vp, vp]
-    L.dlm_strerror.argtypes = [i32]
-    L.dlm_strerror.restype = ctypes.c_char_p
-    L.dlm_selftest_wait_timeout.argtypes = [vp, ctypes.c_uint64, vp]
-    L.dlm_selftest_wait_timeout.restype = i32
-    L.dlm_selftest_set_wait_limit.argtypes = [vp, ctypes.c_uint64]
-    L.dlm_selftest_set_wait_limit.restype = i32
-    L.dlm_selftest_set_attn_team_max.argtypes = [vp, ctypes.c_int, ctypes.c_int]
-    L.dlm_selftest_set_attn_team_max.restype = i32
-    L.dlm_launch_count.argtypes = [vp]
-    L.dlm_launch_count.restype = ctypes.c_int64
-    L.dlm_kv_cache_commit.argtypes = [vp, ctypes.POINTER(dlm_kv_cache), vp, vp, i32, vp, vp, i32, vp, i32, i32,
-                                      i32, i32, vp]
-    L.dlm_attn_workspace_bytes.argtypes = [vp, ctypes.POINTER(dlm_kv_cache), i32, i32, i32]
-    L.dlm_attn_workspace_bytes.restype = sz
-    ip = ctypes.POINTER(ctypes.c_int)
-    L.dlm_selftest_attn_schedule.argtypes = [vp, ctypes.POINTER(dlm_kv_cache), i32, i32, i32, i32, ip, ip, ip, ip]
-    L.dlm_selftest_attn_schedule.restype = i32
-    L.dlm_freecache_attn_step.argtypes = [vp, ctypes.POINTER(dlm_kv_cache), i32, i32, vp, vp, vp, i32, i32,
-                                          vp, f32, i32, vp, vp, vp, sz, vp]
-    L.dlm_unmask_workspace_bytes.argtypes = [vp, i32, i32, i32]
-    L.dlm_unmask_workspace_bytes.restype = sz
-    L.dlm_unmask_select.argtypes = [vp, vp, i32, i32, i32, vp, vp, i32, vp, vp, vp, vp, vp, sz, vp]
-    L.dlm_unmask_select_static.argtypes = [vp, i32, i32, i32, vp, vp, i32, vp, vp, vp, vp, vp]
-    L.dlm_guided_accept.argtypes = [vp, vp, vp, i32, i32, vp, vp, i32, vp, vp, vp, vp]
-    L.dlm_guided_accept_topk.argtypes = [vp, vp, vp, i32, i32, i32, vp, vp, i32, vp, vp, vp, vp]
-    L.dlm_unmask_scored_workspace_bytes.argtypes = [vp, i32, i32, i32]
-    L.dlm_unmask_scored_workspace_bytes.restype = sz
-    L.dlm_unmask_select_scored.argtypes = [vp, vp, i32, i32, i32, vp, vp, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
-    L.dlm_guided_accept_threshold.argtypes = [vp, vp, vp, vp, vp, i32, f32, i32, i32, vp, vp, i32, vp, vp, vp, vp]
-    L.dlm_window_proj_workspace_bytes.argtypes = [vp, i32, i32, i32]
-    L.dlm_window_proj_workspace_bytes.restype = sz
-    L.dlm_window_qkv_project.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, i32, vp, vp, vp, vp, sz, vp]
-    L.dlm_window_qkv_project_rope.argtypes = [vp, vp, vp, vp, vp, vp, i32, i32, i32, i32, i32, i32, vp, vp, vp, vp, sz, vp]
-    L.dlm_window_qkv_project_stage.argtypes = [vp, vp, vp, vp, vp, vp, i32, i32, i32, i32, i32, i32, vp, vp, vp, vp,
-                                               ctypes.POINTER(dlm_kv_cache), i32, vp, sz, vp]
-    L.dlm_window_qkv_project_stage.restype = i32
-    L.dlm_window_out_project.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp, sz, vp]
-    for name in ("dlm_unmask_select_scored", "dlm_guided_accept_threshold", "dlm_window_qkv_project", "dlm_window_qkv_project_rope",
-                 "dlm_window_out_project"):
-        getattr(L, name).restype = i32
-    for name in ("dlm_create", "dlm_destroy", "dlm_get_status", "dlm_kv_cache_commit",
-                 "dlm_freecache_attn_step", "dlm_unmask_select", "dlm_unmask_select_static", "dlm_guided_accept", "dlm_guided_accept_topk"):
-        getattr(L, name).restype = i32
+    vp, i32, sz, u64, ip = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint64, ctypes.POINTER(ctypes.c_int)
+    cache = ctypes.POINTER(dlm_kv_cache)
+    for name, restype, argtypes in (
+            ("dlm_create", i32, [ctypes.POINTER(vp), i32]),
+            ("dlm_destroy", i32, [vp]),
+            ("dlm_get_status", i32, [vp, vp]),
+            ("dlm_strerror", ctypes.c_char_p, [i32]),
+            ("dlm_launch_count", ctypes.c_int64, [vp]),
+            ("dlm_attn_workspace_bytes", sz, [vp, cache, i32, i32, i32]),
+            ("dlm_unmask_workspace_bytes", sz, [vp, i32, i32, i32]),
+            ("dlm_unmask_scored_workspace_bytes", sz, [vp, i32, i32, i32]),
+            ("dlm_window_proj_workspace_bytes", sz, [vp, i32, i32, i32]),
+            ("dlm_selftest_wait_timeout", i32, [vp, u64, vp]),
+            ("dlm_selftest_set_wait_limit", i32, [vp, u64]),
+            ("dlm_selftest_set_attn_team_max", i32, [vp, i32, i32]),
+            ("dlm_selftest_attn_schedule", i32, [vp, cache, i32, i32, i32, i32, ip, ip, ip, ip])):
+        f = getattr(L, name)
+        f.restype, f.argtypes = restype, argtypes
     _lib = L
     return L
 

@@ -630,7 +630,8 @@ extern "C" int dlm_window_qkv_project_rope(dlm_ctx* ctx, const void* x, const vo
                                            int n_kv_heads, int head_dim, void* q_out, void* k_out, void* v_out, void* workspace,
                                            size_t workspace_bytes, void* stream) {
   if (!rope_cos || !rope_sin) return DLM_ERR_NULL;
-  // a feature and its partner must lie in one 128-feature tile, and 4 neighbouring features in one half of a head
+  // a tile's halves are a head's halves, or units of 32 features of either (make_proj_plan knows 64 and 128), and the factors
+  // are read as 16-byte vectors
   if (head_dim != 64 && head_dim != 128) return DLM_ERR_UNSUPPORTED;
   if (((uintptr_t)rope_cos | (uintptr_t)rope_sin) & 15) return DLM_ERR_UNSUPPORTED;
   return qkv_project(ctx, x, w, bias, rope_cos, rope_sin, batch, q_cap, d_model, n_q_heads, n_kv_heads, head_dim, q_out, k_out,

@@ -82,3 +82,14 @@ def test_a_module_of_other_sources_is_not_loaded(monkeypatch):
 
 class _Failed:
     returncode, stdout = 1, ""
+
+
+def test_ctypes_declares_the_calls_that_go_through_it_and_no_others():
+    """One declaration per function: the enqueueing calls have theirs in the native module."""
+    import re
+    from paper_2505_21467_b200 import _binding
+    source = open(_binding.__file__).read()
+    used = set(re.findall(r"lib\(\)\.(dlm_\w+)", source))
+    declared = set(re.findall(r'\("(dlm_\w+)", \S+, \[', source)) | set(re.findall(r"\bL\.(dlm_\w+)\.", source))
+    assert declared == used
+    assert all(getattr(_binding.lib(), name).argtypes is None for name in dir(_binding._load_calls()) if name.startswith("dlm_"))

@@ -289,8 +289,8 @@ __device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint3
   if (!p.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
   __threadfence();
   atomicAdd(p.arrive, 1u);
-  if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
   if (!mbar_wait_limit(bar_pub - kBarPub, 0, abort_ptr, kLimit)) return;
+  if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
   fence_proxy_async_all();
   mbar_expect_tx(bar_team, (uint32_t)p.team * (p.ml_bytes + p.o_bytes));
   for (int c = 0; c < p.team; ++c) {

@@ -330,17 +330,17 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       }
     }
     // The last MMA is waited for whether or not a role of this block has given up: it reads the stages and writes TMEM.  (The
-    // tables are there too.)
-    const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, never_ptr) ? 1 : 0) != 0;
+    // tables are there too.)  Who raised the abort flag sees it here.
+    const bool clean = *abort_ptr == 0;
+    const bool ok = __syncthreads_and(mbar_wait(bar_done, 0, never_ptr) && clean) != 0;
     tc_fence_after_sync();
-    // Unwinding: the copies already issued land before anything else is put in their place or the memory is released, also those
-    // of a producer that never had to wait (the issuer may have given up behind it).  Both blocks' copies complete on the
-    // leader's barriers.  Otherwise the issuer has waited for every one of them.
-    const bool gave_up = *abort_ptr != 0;
-    if (gave_up && rank == 0)
+    // Unwinding: the copies already issued land before the memory is released, also those of a producer that never had to wait
+    // (the issuer may have given up behind it).  Both blocks' copies complete on the leader's barriers.  Otherwise the
+    // issuer has waited for every one of them.
+    if (!ok && rank == 0)
       for (int i = max(0, issued - p.n_stages); i < issued; ++i)
         mbar_wait(bar_full + 8 * (i % p.n_stages), (i / p.n_stages) & 1, never_ptr);
-    if (ok && !gave_up && n_rows > 0) {
+    if (ok && n_rows > 0) {
       // TMEM side: warps w and w + 4 read the lanes of quarter w % 4, one segment each.  The row of a lane: M = 64 puts 16
       // rows in each quarter; M = 128 as a pair puts rows 0-63 twice, lanes 64-127 holding the second half of the columns.
       const int quarter = warp & 3, seg = warp >> 2;

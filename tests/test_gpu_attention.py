@@ -35,6 +35,25 @@ def _case(dev, oracle, NL, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len=None, se
     return out, lse, errs
 
 
+def _schedule(dev, NL, B, Hq, Hkv, D, Lcap, q_cap, nl, hint=0):
+    ck = torch.empty(NL, B, Hkv, Lcap, D, dtype=torch.bfloat16, device="cuda")
+    cache = dlm.make_kv_cache(ck, ck, _i32([0] * B))
+    return dlm.dlm_selftest_attn_schedule(dev.ctx, cache, nl, Hq, q_cap, hint)
+
+
+def _each_schedule(dev, names, NL, B, Hq, Hkv, D, Lcap, q_cap):
+    """For every schedule of `names`, makes a call of this shape take it and yields the length hint to pass."""
+    try:
+        for name in names:
+            hint = 1 if name == "whole" else 0
+            dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20 if name == "team" else 1)
+            sch = _schedule(dev, NL, B, Hq, Hkv, D, Lcap, q_cap, NL, hint)
+            assert name == ("team" if sch["team"] > 1 else "whole" if sch["whole_units"] else "split"), sch
+            yield hint
+    finally:
+        dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)
+
+
 def test_tiny_config_full(dev, oracle):
     cfg = get_config(0)
     _case(dev, oracle, cfg.n_layers, cfg.batch, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.capacity,
@@ -57,21 +76,22 @@ def test_shapes_and_ragged_lengths(dev, oracle, Hq, Hkv, D, Lcap, q_cap, cache_l
             assert torch.all(out[:, b, :, n:] == 0)
 
 
-@pytest.mark.parametrize("hint", [1, 0])
-def test_both_schedules_whole_units_and_split(dev, oracle, hint):
-    """The length hint only picks the schedule: a tiny hint deals the units whole, the default (capacity)
-    splits these 16 long units across the SMs; both must match the oracle."""
-    _case(dev, oracle, 2, 2, 28, 4, 128, 1400, 32, [1368, 900], [32, 17], seed=77, hint=hint)
+@pytest.mark.parametrize("name", ["whole", "split", "team"])
+def test_each_schedule(dev, oracle, name):
+    """How the units are dealt is the host's choice: whole, split across the SMs, or to teams; all three match the oracle."""
+    for hint in _each_schedule(dev, [name], 2, 2, 28, 4, 128, 1400, 32):
+        _case(dev, oracle, 2, 2, 28, 4, 128, 1400, 32, [1368, 900], [32, 17], seed=77, hint=hint)
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,Lcap,q_cap,cache_len,q_len", [
     (28, 4, 128, 600, 256, [300], None),                # the paper's window: 256 active rows, Dream heads (7 chunks of 256 rows)
     (4, 4, 128, 520, 512, [0, 0], [512, 333]),          # initial full pass: empty cache, 512 active rows, ragged
     (4, 2, 64, 400, 300, [77, 100], [300, 130]),        # rows per KV head not a multiple of 256, head_dim 64
+    (16, 4, 64, 1100, 256, [1001, 844, 3], [256, 200, 256]),   # units of two M tiles when split
 ])
 def test_large_windows_in_row_chunks(dev, oracle, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len):
     B = len(cache_len)
-    for hint in (1, 0):   # both schedules
+    for hint in _each_schedule(dev, ["whole", "split", "team"], 1, B, Hq, Hkv, D, Lcap, q_cap):
         out, lse, _ = _case(dev, oracle, 1, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len, seed=Hq * 1000 + q_cap, hint=hint)
         if q_len is not None:
             for b, n in enumerate(q_len):
@@ -82,14 +102,14 @@ def test_large_windows_in_row_chunks(dev, oracle, Hq, Hkv, D, Lcap, q_cap, cache
 def test_scores_that_keep_outgrowing_the_running_maximum(dev, oracle, scale):
     """Keys grow along the cache and the softmax scale is large, so later tiles bring scores far above the
     maximum in use (by tens of powers of two): the deferred rescaling of O has to fire, repeatedly, and the result
-    must still match.  Both schedules."""
+    must still match.  Every schedule."""
     NL, B, Hq, Hkv, D, Lc, q_cap = 1, 2, 14, 2, 128, 1500, 32
     ck, cv = make_cache(NL, B, Hkv, Lc + 40, D, 91)
     q, kn, vn = make_attn_inputs(NL, B, Hq, Hkv, q_cap, D, 92)
     grow = (1.0 + 4.0 * torch.arange(Lc + 40, dtype=torch.float32) / Lc).view(1, 1, 1, -1, 1)
     ck = (ck.float() * grow).to(torch.bfloat16)
     cl = _i32([Lc, Lc - 333])
-    for hint in (1, 0):
+    for hint in _each_schedule(dev, ["whole", "split", "team"], NL, B, Hq, Hkv, D, Lc + 40, q_cap):
         out, lse = gpu_attn_step(dev, ck.cuda(), cv.cuda(), cl, q.cuda(), kn.cuda(), vn.cuda(), None, scale, hint=hint)
         assert dev.status() == 0
         ref = oracle_attn_layers(oracle, ck, cv, cl, q, kn, vn, None, scale)
@@ -111,30 +131,34 @@ def test_layer_range_and_explicit_scale(dev, oracle):
     _case(dev, oracle, 5, 1, 4, 2, 128, 300, 32, [290], seed=9, layer_begin=2, nl=2, scale=0.05)
 
 
-def test_poisoned_invisible_rows_do_not_leak(dev, oracle):
+@pytest.mark.parametrize("name,Lcap", [("whole", 520), ("team", 520), ("split", 1400)])
+def test_poisoned_invisible_rows_do_not_leak(dev, oracle, name, Lcap):
     """Rows at or beyond cache_len / q_len may hold NaN: the result must not change (bit for bit)."""
-    NL, B, Hq, Hkv, D, Lcap, q_cap = 1, 2, 14, 2, 128, 520, 32
-    ck, cv = make_cache(NL, B, Hkv, Lcap, D, 31, device="cuda")
-    q, kn, vn = make_attn_inputs(NL, B, Hq, Hkv, q_cap, D, 32, device="cuda")
+    NL, B, Hq, Hkv, D, q_cap = 1, 2, 14, 2, 128, 32
     cl, ql = _i32([300, 5]), _i32([32, 9])
-    base, base_lse = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, ql)
-    nan = float("nan")
-    ck[:, 0, :, 300:] = nan; cv[:, 0, :, 300:] = nan
-    ck[:, 1, :, 5:] = nan; cv[:, 1, :, 5:] = nan
-    kn[:, 1, :, 9:] = nan; vn[:, 1, :, 9:] = nan; q[:, 1, :, 9:] = nan
-    out, lse = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, ql)
-    assert dev.status() == 0
-    assert torch.equal(out, base) and torch.equal(lse, base_lse)
-    assert torch.isfinite(out.float()).all()
+    for hint in _each_schedule(dev, [name], NL, B, Hq, Hkv, D, Lcap, q_cap):
+        ck, cv = make_cache(NL, B, Hkv, Lcap, D, 31, device="cuda")
+        q, kn, vn = make_attn_inputs(NL, B, Hq, Hkv, q_cap, D, 32, device="cuda")
+        base, base_lse = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, ql, hint=hint)
+        nan = float("nan")
+        ck[:, 0, :, 300:] = nan; cv[:, 0, :, 300:] = nan
+        ck[:, 1, :, 5:] = nan; cv[:, 1, :, 5:] = nan
+        kn[:, 1, :, 9:] = nan; vn[:, 1, :, 9:] = nan; q[:, 1, :, 9:] = nan
+        out, lse = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, ql, hint=hint)
+        assert dev.status() == 0
+        assert torch.equal(out, base) and torch.equal(lse, base_lse)
+        assert torch.isfinite(out.float()).all()
 
 
-def test_deterministic(dev):
+@pytest.mark.parametrize("name", ["whole", "split", "team"])
+def test_deterministic(dev, name):
     ck, cv = make_cache(2, 1, 4, 1100, 128, 41, device="cuda")
     q, kn, vn = make_attn_inputs(2, 1, 28, 4, 32, 128, 42, device="cuda")
     cl = _i32([1056])
-    a, al = gpu_attn_step(dev, ck, cv, cl, q, kn, vn)
-    b, bl = gpu_attn_step(dev, ck, cv, cl, q, kn, vn)
-    assert torch.equal(a, b) and torch.equal(al, bl)
+    for hint in _each_schedule(dev, [name], 2, 1, 28, 4, 128, 1100, 32):
+        a, al = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, hint=hint)
+        b, bl = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, hint=hint)
+        assert torch.equal(a, b) and torch.equal(al, bl)
 
 
 def test_argument_errors(dev):
@@ -199,6 +223,8 @@ def test_guided_shape_more_units_than_sms_split_schedule(dev, oracle):
     cfg = get_config(4)
     cache_len = [1024, 1031, 1056, 1100, 1247, 1279, 1088, 1150]
     q_len = [32, 25, 32, 20, 1, 1, 32, 2]
+    sch = _schedule(dev, 10, cfg.batch, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.capacity, cfg.block_len, 10)
+    assert sch["whole_units"] == 0 and sch["team"] == 1
     _case(dev, oracle, 10, cfg.batch, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.capacity, cfg.block_len,
           cache_len, q_len, seed=seed_for(4, 7), layers=[0, 9], device="cuda")
 
@@ -229,24 +255,25 @@ def test_a_wait_that_runs_out_reports_timeout_and_leaves_the_context_usable(dev,
     assert e.value.code == dlm.DLM_ERR_SHAPE
 
 
-@pytest.mark.parametrize("hint", [1, 0])
-def test_the_attention_kernel_gives_up_cleanly_when_its_waits_may_not_wait(dev, oracle, hint):
-    """The kernel's own unwinding, in both schedules: with the wait limit set to 0 the first wait whose data is still
+@pytest.mark.parametrize("name", ["whole", "split"])
+def test_the_attention_kernel_gives_up_cleanly_when_its_waits_may_not_wait(dev, oracle, name):
+    """The kernel's own unwinding, units whole and split: with the wait limit set to 0 the first wait whose data is still
     on its way gives up; the producer lets its copies land, the MMA issuers drain, every role reaches the teardown,
     TMEM is released and the kernel ends normally with DLM_ERR_TIMEOUT.  With the limit restored the next call on the
     same context is correct again (nothing of the aborted launch is left behind, ticket words included)."""
-    args = dict(NL=2, B=2, Hq=28, Hkv=4, D=128, Lcap=700, q_cap=32, cache_len=[517, 640], seed=4242, hint=hint)
-    dlm.dlm_selftest_set_wait_limit(dev.ctx, 0)
-    try:
-        ck, cv = make_cache(2, 2, 4, 700, 128, 1, device="cuda")
-        q, kn, vn = make_attn_inputs(2, 2, 28, 4, 32, 128, 2, device="cuda")
-        gpu_attn_step(dev, ck, cv, _i32([517, 640]), q, kn, vn, hint=hint)
-        torch.cuda.synchronize()
-        assert dev.status() == dlm.DLM_ERR_TIMEOUT
-    finally:
-        dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
-    assert dev.status() == 0
-    _case(dev, oracle, **args)
+    for hint in _each_schedule(dev, [name], 2, 2, 28, 4, 128, 700, 32):
+        args = dict(NL=2, B=2, Hq=28, Hkv=4, D=128, Lcap=700, q_cap=32, cache_len=[517, 640], seed=4242, hint=hint)
+        dlm.dlm_selftest_set_wait_limit(dev.ctx, 0)
+        try:
+            ck, cv = make_cache(2, 2, 4, 700, 128, 1, device="cuda")
+            q, kn, vn = make_attn_inputs(2, 2, 28, 4, 32, 128, 2, device="cuda")
+            gpu_attn_step(dev, ck, cv, _i32([517, 640]), q, kn, vn, hint=hint)
+            torch.cuda.synchronize()
+            assert dev.status() == dlm.DLM_ERR_TIMEOUT
+        finally:
+            dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
+        assert dev.status() == 0
+        _case(dev, oracle, **args)
     with pytest.raises(dlm.DlmError) as e:
         dlm.dlm_selftest_set_wait_limit(dev.ctx, 3_000_000_000)
     assert e.value.code == dlm.DLM_ERR_SHAPE
@@ -277,12 +304,6 @@ def test_giving_up_lets_copies_land_that_nobody_waits_for(dev, oracle, D, cache_
         assert dev.status() == dlm.DLM_ERR_TIMEOUT
         for lc in ref:
             assert_attn_close(out, lse, ref[lc], lc)
-
-
-def _schedule(dev, NL, B, Hq, Hkv, D, Lcap, q_cap, nl, hint=0):
-    ck = torch.empty(NL, B, Hkv, Lcap, D, dtype=torch.bfloat16, device="cuda")
-    cache = dlm.make_kv_cache(ck, ck, _i32([0] * B))
-    return dlm.dlm_selftest_attn_schedule(dev.ctx, cache, nl, Hq, q_cap, hint)
 
 
 @pytest.mark.parametrize("NL,B,Hq,Hkv,D,Lcap,q_cap,cache_len,q_len", [
@@ -323,7 +344,7 @@ def test_team_schedule_against_the_oracle_at_every_team_size(dev, oracle, NL, B,
 
 
 def test_team_schedule_repeated_launches_leave_the_counters_clean(dev, oracle):
-    """The team's arrival and departure counters are cleared by the last warp to leave: many launches in a row on
+    """The team's arrival and departure counters are cleared by the last block to leave: many launches in a row on
     the same units (also of different team sizes) stay correct, and so does a split-schedule call afterwards."""
     shape = dict(NL=1, B=1, Hq=28, Hkv=4, D=128, Lcap=2200, q_cap=32)
     try:
@@ -333,7 +354,8 @@ def test_team_schedule_repeated_launches_leave_the_counters_clean(dev, oracle):
             _case(dev, oracle, cache_len=[1500 + 100 * i], seed=300 + i, **shape)
     finally:
         dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)
-    _case(dev, oracle, 2, 2, 28, 4, 128, 1400, 32, [1368, 900], [32, 17], seed=77)
+    for hint in _each_schedule(dev, ["split"], 2, 2, 28, 4, 128, 1400, 32):
+        _case(dev, oracle, 2, 2, 28, 4, 128, 1400, 32, [1368, 900], [32, 17], seed=77, hint=hint)
 
 
 def test_team_members_without_key_tiles(dev, oracle):

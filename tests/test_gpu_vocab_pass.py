@@ -28,7 +28,7 @@ def _inputs(B, L, V, seed):
 
 
 @pytest.mark.parametrize("kind", [0, 1, 2])
-@pytest.mark.parametrize("B,L,V", [(1, 33, 4095), (2, 17, 4096), (1, 9, 8193), (1, 32, 98304), (1, 8, 102401), (3, 40, 12288), (40, 32, 20484)])
+@pytest.mark.parametrize("B,L,V", [(1, 33, 4095), (2, 17, 4096), (1, 9, 8193), (1, 32, 98304), (1, 8, 98304), (1, 8, 98305), (1, 8, 102401), (3, 40, 12288), (40, 32, 20484)])
 def test_chunk_edges(dev, oracle, B, L, V, kind):
     masked0 = make_mask(B, L, L - 2, V).numpy()
     masked0[0, :5] = 1

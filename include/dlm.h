@@ -60,7 +60,7 @@ typedef struct dlm_ctx dlm_ctx;
  * Every later call that takes the context must be made with that device current on the
  * calling thread (else DLM_ERR_DEVICE, nothing launched).
  * The context owns its status / ticket words and, on the host, what its calls keep for the next ones: TMA descriptors
- * (functions of an address and sizes) and the last attention call's plan (a function of sizes).  Not thread-safe: use
+ * and the last attention call's plan, both functions of sizes alone.  Not thread-safe: use
  * one context per host thread or serialise calls.  Kernels enqueued through one context on different
  * streams must not overlap in time (they share the context's ticket words). */
 int dlm_create(dlm_ctx** out, int device);

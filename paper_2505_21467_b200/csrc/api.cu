@@ -21,7 +21,7 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
   ctx->num_sms = prop.multiProcessorCount;
   ctx->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
   ctx->launches = 0;
-  ctx->encode_tiled = nullptr;
+  ctx->encode_tiled = ctx->replace_address = nullptr;
   ctx->maps = new (std::nothrow) dlm_map_cache();
   ctx->commit_blocks_per_sm[0] = ctx->commit_blocks_per_sm[1] = 0;
   for (int i = 0; i < 8; ++i) ctx->attn_smem_limit[i] = 0;
@@ -70,40 +70,44 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-const CUtensorMap* dlm_tensor_map(dlm_ctx* ctx, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
-                                  const cuuint32_t* box) {
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+
+static void* driver_entry(const char* name) {
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  return cudaGetDriverEntryPoint(name, &fn, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr;
+}
+
+bool dlm_tensor_map(dlm_ctx* ctx, CUtensorMap* out, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                    const cuuint32_t* box) {
+  if (!ctx->encode_tiled) ctx->encode_tiled = driver_entry("cuTensorMapEncodeTiled");
+  if (!ctx->replace_address) ctx->replace_address = driver_entry("cuTensorMapReplaceAddress");
+  if (!ctx->encode_tiled || !ctx->replace_address) return false;
   dlm_map_key k;
   memset(&k, 0, sizeof k);
-  k.base = base;
   k.rank = (cuuint32_t)rank;
-  uint64_t h = (uint64_t)(uintptr_t)base >> 4;
+  uint64_t h = (uint64_t)rank;
   for (int i = 0; i < rank; ++i) {
     k.dims[i] = dims[i];
     k.box[i] = box[i];
     if (i + 1 < rank) k.strides[i] = strides[i];
     h = (h ^ dims[i] ^ ((uint64_t)box[i] << 32)) * 0x9e3779b97f4a7c15ull;
   }
-  const int slot = (int)(h >> 55);   // 9 bits
-  static_assert(kDlmMapSlots == 512, "slots are picked by 9 bits");
+  const int slot = (int)(h >> 57);   // 7 bits
+  static_assert(kDlmMapSlots == 128, "slots are picked by 7 bits");
   dlm_map_cache& c = *ctx->maps;
-  if (memcmp(&c.key[slot], &k, sizeof k) == 0) return &c.map[slot];
-  if (!ctx->encode_tiled) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
-        q != cudaDriverEntryPointSuccess)
-      return nullptr;
-    ctx->encode_tiled = fn;
+  if (memcmp(&c.key[slot], &k, sizeof k) != 0) {
+    const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
+    c.key[slot].rank = 0;
+    if (reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
+            &c.map[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return false;
+    c.key[slot] = k;
   }
-  const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
-  c.key[slot].rank = 0;
-  const CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
-      &c.map[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, elem,
-      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return nullptr;
-  c.key[slot] = k;
-  return &c.map[slot];
+  *out = c.map[slot];
+  return reinterpret_cast<ReplaceAddressFn>(ctx->replace_address)(out, const_cast<void*>(base)) == CUDA_SUCCESS;
 }
 
 extern "C" int64_t dlm_launch_count(const dlm_ctx* ctx) { return ctx ? ctx->launches : 0; }

@@ -1216,10 +1216,7 @@ int encode_map(dlm_ctx* ctx, CUtensorMap* map, const void* base, int D, long lon
   const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)rows, (cuuint64_t)slabs};
   const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)rows * D * 2};
   const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-  const CUtensorMap* m = dlm_tensor_map(ctx, base, 3, dims, strides, box);
-  if (!m) return DLM_ERR_CUDA;
-  *map = *m;
-  return DLM_OK;
+  return dlm_tensor_map(ctx, map, base, 3, dims, strides, box) ? DLM_OK : DLM_ERR_CUDA;
 }
 
 // The kernel starts with `numRegs` registers per thread in all 12 warps.  The 8 softmax warps then

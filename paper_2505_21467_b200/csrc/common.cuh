@@ -21,15 +21,14 @@ struct dlm_device_words {
   unsigned int attn_unit_tickets[kDlmMaxSplitUnits];  // pieces of a split unit finished so far
 };
 
-// TMA descriptors a context has built, by what they describe.  A descriptor is a function of the key alone (an address
-// and sizes; it owns nothing), so a call whose tensors lie where an earlier call's did reuses it: building the five of an
-// attention call costs the host about as much as the launch.  Direct-mapped and fixed in size.
+// TMA descriptors a context has built, by the sizes they describe and not by the tensor: a call copies the one of its sizes
+// and writes its own address into the copy (9 ns; building one takes 57 ns, and an attention call has five), on new
+// tensors as on old ones.  Direct-mapped and fixed in size.
 struct dlm_map_key {
-  const void* base;
   cuuint64_t dims[5], strides[4];
   cuuint32_t box[5], rank;
 };
-constexpr int kDlmMapSlots = 512;
+constexpr int kDlmMapSlots = 128;
 struct dlm_map_cache {
   dlm_map_key key[kDlmMapSlots];   // rank 0: empty
   CUtensorMap map[kDlmMapSlots];
@@ -51,7 +50,8 @@ struct dlm_ctx {
   int max_smem_optin;       // largest dynamic shared memory a block may opt in to, bytes
   int64_t launches;
   dlm_device_words* words;  // device
-  void* encode_tiled;       // cuTensorMapEncodeTiled entry point (driver API), resolved lazily
+  void* encode_tiled;       // cuTensorMapEncodeTiled and cuTensorMapReplaceAddress (driver API), resolved lazily
+  void* replace_address;
   dlm_map_cache* maps;
   int commit_blocks_per_sm[2];  // resident blocks per SM of the two commit kernels (0 = not asked yet)
   unsigned long long wait_limit_ns;   // limit of the kernels' device-side waits (2 s; a test may shorten it)
@@ -63,10 +63,10 @@ struct dlm_ctx {
   int attn_smem_limit[8];       // dynamic shared memory the two attention kernels may use on this device (0 = not set up yet)
 };
 
-// The descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle;
-// nullptr if the driver refuses it.  Defined in api.cu.
-const CUtensorMap* dlm_tensor_map(dlm_ctx* ctx, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
-                                  const cuuint32_t* box);
+// Writes the descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle,
+// to `out`; false if the driver refuses it.  Defined in api.cu.
+bool dlm_tensor_map(dlm_ctx* ctx, CUtensorMap* out, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                    const cuuint32_t* box);
 
 // Division by a divisor known on the host: one high multiply, an add and a shift (round-up reciprocal of Granlund and
 // Montgomery, for dividends below 2^31).

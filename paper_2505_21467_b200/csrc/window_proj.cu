@@ -594,13 +594,13 @@ int launch_proj(dlm_ctx* ctx, const ProjPlan& pl, ProjParams& p, const CUtensorM
 }
 
 // W seen as [groups][2][half_rows][K / 64][64]; a copy brings w_box_rows features of one half (pairs) or of both, kp panels.
-const CUtensorMap* encode_weights(dlm_ctx* ctx, const void* w, int n_out, int k_total, const ProjPlan& pl) {
+bool encode_weights(dlm_ctx* ctx, CUtensorMap* map, const void* w, int n_out, int k_total, const ProjPlan& pl) {
   const ProjVariant& k = kVariants[pl.variant];
   const cuuint64_t row = (cuuint64_t)k_total * 2, a = (cuuint64_t)pl.half_rows;
   const cuuint64_t dims[5] = {(cuuint64_t)kPanel, a, 2, (cuuint64_t)(k_total / kPanel), (cuuint64_t)n_out / (2 * a)};
   const cuuint64_t strides[4] = {row, a * row, (cuuint64_t)kPanel * 2, 2 * a * row};
   const cuuint32_t box[5] = {(cuuint32_t)kPanel, (cuuint32_t)pl.w_box_rows, k.m > 64 ? 1u : 2u, (cuuint32_t)k.kp, 1};
-  return dlm_tensor_map(ctx, w, 5, dims, strides, box);
+  return dlm_tensor_map(ctx, map, w, 5, dims, strides, box);
 }
 
 }  // namespace
@@ -669,16 +669,14 @@ int qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, co
   DLM_DEVICE_TRY(ctx);
   ProjPlan pl;
   if (!make_proj_plan(ctx, (int)rows, (int)n_out, d_model, head_dim, batch, 0, pl)) return DLM_ERR_UNSUPPORTED;
-  const CUtensorMap *tm_w = encode_weights(ctx, w, (int)n_out, d_model, pl), *tm_x = nullptr;
-  if (!tm_w) return DLM_ERR_CUDA;
-  const CUtensorMap w_map = *tm_w;   // the next descriptor may take its slot
+  CUtensorMap tm_w, tm_x;
+  if (!encode_weights(ctx, &tm_w, w, (int)n_out, d_model, pl)) return DLM_ERR_CUDA;
   {
     const cuuint64_t dims[4] = {(cuuint64_t)kPanel, (cuuint64_t)rows, (cuuint64_t)(d_model / kPanel), 1};
     const cuuint64_t strides[3] = {(cuuint64_t)d_model * 2, (cuuint64_t)kPanel * 2, (cuuint64_t)d_model * 2};
     const cuuint32_t box[4] = {(cuuint32_t)kPanel, (cuuint32_t)pl.rc, (cuuint32_t)kVariants[pl.variant].kp, 1};
-    tm_x = dlm_tensor_map(ctx, x, 4, dims, strides, box);
+    if (!dlm_tensor_map(ctx, &tm_x, x, 4, dims, strides, box)) return DLM_ERR_CUDA;
   }
-  if (!tm_x) return DLM_ERR_CUDA;
   ProjParams p = {};
   p.mode = 0;
   p.q_out = static_cast<__nv_bfloat16*>(q_out);
@@ -697,7 +695,7 @@ int qkv_project(dlm_ctx* ctx, const void* x, const void* w, const void* bias, co
   }
   p.rows_total = (int)rows; p.q_cap = q_cap; p.n_q_heads = n_q_heads; p.n_kv_heads = n_kv_heads; p.head_dim = head_dim;
   p.n_out = (int)n_out; p.k_total = d_model; p.batch = batch; p.act_heads = 0;
-  return launch_proj(ctx, pl, p, w_map, *tm_x, static_cast<cudaStream_t>(stream));
+  return launch_proj(ctx, pl, p, tm_w, tm_x, static_cast<cudaStream_t>(stream));
 }
 }  // namespace
 
@@ -715,23 +713,21 @@ extern "C" int dlm_window_out_project(dlm_ctx* ctx, const void* o, const void* w
   DLM_DEVICE_TRY(ctx);
   ProjPlan pl;
   if (!make_proj_plan(ctx, (int)rows, d_model, (int)k_total, 0, batch, q_cap, pl)) return DLM_ERR_UNSUPPORTED;
-  const CUtensorMap *tm_w = encode_weights(ctx, wo, d_model, (int)k_total, pl), *tm_x = nullptr;
-  if (!tm_w) return DLM_ERR_CUDA;
-  const CUtensorMap w_map = *tm_w;   // the next descriptor may take its slot
+  CUtensorMap tm_w, tm_x;
+  if (!encode_weights(ctx, &tm_w, wo, d_model, (int)k_total, pl)) return DLM_ERR_CUDA;
   {
     // a box brings one 64-element panel of one head: the rows of whole sequences, or part of one sequence's rows
     const int box_seqs = batch > 1 && pl.x_box_rows % q_cap == 0 ? pl.x_box_rows / q_cap : 1;
     const cuuint64_t dims[4] = {(cuuint64_t)head_dim, (cuuint64_t)q_cap, (cuuint64_t)n_q_heads, (cuuint64_t)batch};
     const cuuint64_t strides[3] = {(cuuint64_t)head_dim * 2, (cuuint64_t)q_cap * head_dim * 2, (cuuint64_t)k_total * q_cap * 2};
     const cuuint32_t box[4] = {(cuuint32_t)kPanel, (cuuint32_t)(pl.x_box_rows / box_seqs), 1, (cuuint32_t)box_seqs};
-    tm_x = dlm_tensor_map(ctx, o, 4, dims, strides, box);
+    if (!dlm_tensor_map(ctx, &tm_x, o, 4, dims, strides, box)) return DLM_ERR_CUDA;
   }
-  if (!tm_x) return DLM_ERR_CUDA;
   ProjParams p = {};
   p.mode = 1;
   p.q_out = static_cast<__nv_bfloat16*>(y);
   p.bias = static_cast<const __nv_bfloat16*>(bias);
   p.rows_total = (int)rows; p.q_cap = q_cap; p.n_q_heads = n_q_heads; p.n_kv_heads = 0; p.head_dim = head_dim;
   p.n_out = d_model; p.k_total = (int)k_total; p.batch = batch; p.act_heads = n_q_heads;
-  return launch_proj(ctx, pl, p, w_map, *tm_x, static_cast<cudaStream_t>(stream));
+  return launch_proj(ctx, pl, p, tm_w, tm_x, static_cast<cudaStream_t>(stream));
 }

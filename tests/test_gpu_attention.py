@@ -161,6 +161,26 @@ def test_deterministic(dev, name):
         assert torch.equal(a, b) and torch.equal(al, bl)
 
 
+def test_the_same_sizes_on_other_tensors(dev):
+    """What a context keeps of a call (descriptors, plan) depends on sizes alone: calls of two shapes in turn, each time on
+    other copies of the same tensors, one of them at an odd multiple of 16 bytes, give the same bits."""
+    def shifted(t, n):      # a copy that starts n * 16 bytes into a buffer of its own
+        buf = torch.empty(t.numel() + 8 * n, dtype=t.dtype, device="cuda")
+        return buf[8 * n:].view_as(t).copy_(t)
+
+    shapes = [(2, 1, 28, 4, 32, 128, 300, [280]), (1, 3, 4, 2, 40, 64, 500, [400, 0, 77])]
+    first = {}
+    for turn in range(3):
+        for i, (NL, B, Hq, Hkv, q_cap, D, Lcap, lens) in enumerate(shapes):
+            ck, cv = make_cache(NL, B, Hkv, Lcap, D, 60 + i, device="cuda")
+            t = [ck, cv, *make_attn_inputs(NL, B, Hq, Hkv, q_cap, D, 70 + i, device="cuda")]
+            ck, cv, q, kn, vn = [shifted(x, 2 * turn + 1) for x in t]
+            out, lse = gpu_attn_step(dev, ck, cv, _i32(lens), q, kn, vn)
+            assert dev.status() == 0
+            a, b = first.setdefault(i, (out, lse))
+            assert torch.equal(a, out) and torch.equal(b, lse)
+
+
 def test_argument_errors(dev):
     ck, cv = make_cache(1, 1, 2, 64, 128, 1, device="cuda")
     cl = _i32([10])

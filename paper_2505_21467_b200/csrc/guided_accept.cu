@@ -3,14 +3,16 @@
 // Integer-only and tiny (one block of positions per batch element), so it is bound by launch
 // latency.  One warp per batch element walks the block 32 positions at a time; ballots give
 // the masked set, the first disagreement and the ascending output order without any sort.
+// (No pointer is declared __restrict__: the inputs would then be read through the read-only path, which asks that they do not
+// change while the kernel runs, and it starts while the vocabulary pass is still writing them; see dlm_grid_dependency_wait.)
 #include "common.cuh"
 
 namespace {
 
 __global__ void __launch_bounds__(32)
-guided_accept_kernel(const int32_t* __restrict__ tok_dlm, const int32_t* __restrict__ tok_ar, int top_k, int block_len,
-                     uint8_t* __restrict__ masked, int32_t* __restrict__ tokens, int fallback_source,
-                     uint8_t* __restrict__ accept, int32_t* __restrict__ acc_idx, int32_t* __restrict__ n_acc) {
+guided_accept_kernel(const int32_t* tok_dlm, const int32_t* tok_ar, int top_k, int block_len,
+                     uint8_t* masked, int32_t* tokens, int fallback_source,
+                     uint8_t* accept, int32_t* acc_idx, int32_t* n_acc) {
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();
   const int b = blockIdx.x;
@@ -68,11 +70,11 @@ guided_accept_kernel(const int32_t* __restrict__ tok_dlm, const int32_t* __restr
 // above (fallback included) united with every masked position whose largest DLM logit exceeds tau times the largest
 // of the guider's top_k logits for it.  Same walk as above; the accepted set need not be a prefix any more.
 __global__ void __launch_bounds__(32)
-guided_accept_threshold_kernel(const int32_t* __restrict__ tok_dlm, const float* __restrict__ zmax_dlm,
-                               const int32_t* __restrict__ tok_ar, const float* __restrict__ logit_ar, int top_k, float tau,
-                               int block_len, uint8_t* __restrict__ masked, int32_t* __restrict__ tokens,
-                               int fallback_source, uint8_t* __restrict__ accept, int32_t* __restrict__ acc_idx,
-                               int32_t* __restrict__ n_acc) {
+guided_accept_threshold_kernel(const int32_t* tok_dlm, const float* zmax_dlm,
+                               const int32_t* tok_ar, const float* logit_ar, int top_k, float tau,
+                               int block_len, uint8_t* masked, int32_t* tokens,
+                               int fallback_source, uint8_t* accept, int32_t* acc_idx,
+                               int32_t* n_acc) {
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();
   const int b = blockIdx.x;

@@ -197,3 +197,36 @@ def test_threshold_guided_config_shape_with_the_scored_pass(dev, oracle):
     ar_logit = (o[3][..., None] * rng.uniform(1.2, 3.0, (B, L, K))).astype(np.float32)
     n = _compare_threshold(dev, oracle, d, o[3], ar_tok, ar_logit, 0.5, masked0, 0)
     assert n.min() >= 1
+
+
+@pytest.mark.parametrize("B,L,V", [(1, 32, 3000), (8, 70, 9001)])
+def test_accepting_right_behind_the_pass_that_proposes(dev, B, L, V):
+    """The accept kernel starts while the vocabulary pass still writes the proposals and largest logits it reads: calls in a
+    row, without a wait between them, give what they give one by one."""
+    rounds, K = 12, 2
+    logits = [make_logits(B, L, V, (1.0, 6.0), 700 + r, device="cuda") for r in range(rounds)]
+    best = [z.argmax(-1).int() for z in logits]
+    rng = torch.Generator().manual_seed(9)
+    ar = [torch.stack([torch.where((torch.rand(B, L, generator=rng) < 0.8).cuda(), t, (t + 1) % V), (t + 2) % V], -1).contiguous() for t in best]
+    lg = [(10 + 30 * torch.rand(B, L, K, generator=rng)).cuda() for _ in range(rounds)]
+    tok, conf, score, zmax = (torch.empty(B, L, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32, torch.float32))
+    ws = dev.workspace(dlm.dlm_unmask_scored_workspace_bytes(dev.ctx, B, L, V))
+
+    def run(wait):
+        masked = torch.ones(rounds, 2, B, L, dtype=torch.uint8, device="cuda")
+        tokens, idx = (torch.full((rounds, 2, B, L), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+        n, accept = torch.empty(rounds, 2, B, dtype=torch.int32, device="cuda"), torch.empty(rounds, 2, B, L, dtype=torch.uint8, device="cuda")
+        for r in range(rounds):
+            for i in range(2):
+                dlm.dlm_unmask_select_scored(dev.ctx, logits[r], B, L, V, masked[r, i], tokens[r, i], 0, 0, None, tok, conf, score, zmax, None, None, ws)
+                if wait:
+                    torch.cuda.synchronize()
+                if i == 0:
+                    dlm.dlm_guided_accept_topk(dev.ctx, tok, ar[r], K, B, L, masked[r, i], tokens[r, i], 0, accept[r, i], idx[r, i], n[r, i])
+                else:
+                    dlm.dlm_guided_accept_threshold(dev.ctx, tok, zmax, ar[r], lg[r], K, 0.5, B, L, masked[r, i], tokens[r, i], 0,
+                                                    accept[r, i], idx[r, i], n[r, i])
+        assert dev.status() == 0
+        return masked, tokens, idx, n, accept
+    for a, b in zip(run(False), run(True)):
+        assert torch.equal(a, b)

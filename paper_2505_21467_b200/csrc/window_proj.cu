@@ -267,8 +267,8 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       e.q = p.mode == 1 ? (long long)row * p.n_out : ((long long)b * p.n_q_heads * p.q_cap + i) * p.head_dim;
       e.kv = ((long long)b * p.n_kv_heads * p.q_cap + i) * p.head_dim;
       e.stage = -1;   // cache row to stage at: none for an inactive row or one without room (reported)
-      if (p.stage_k && feature(N - 1) >= p.n_q_heads * p.head_dim && (!p.q_len || i < __ldg(p.q_len + b))) {
-        const int pos = __ldg(p.cache_len + b) + i;
+      if (p.stage_k && feature(N - 1) >= p.n_q_heads * p.head_dim && (!p.q_len || i < p.q_len[b])) {
+        const int pos = p.cache_len[b] + i;   // (not through the read-only path: the commit before may still be advancing it when this kernel starts)
         if (pos >= 0 && pos < p.capacity) e.stage = ((long long)b * p.n_kv_heads * p.capacity + pos) * p.head_dim;
         else dlm_set_status(p.status, DLM_ERR_CAPACITY);
       }
@@ -321,8 +321,8 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
               const size_t a = (size_t)(row0 + r) * half + (f & (D - 1));
 #pragma unroll
               for (int q = 0; q < 2; ++q) {
-                cs[pr][it][q] = __ldg(reinterpret_cast<const float4*>(p.rope_cos + a) + q);
-                sn[pr][it][q] = __ldg(reinterpret_cast<const float4*>(p.rope_sin + a) + q);
+                cs[pr][it][q] = reinterpret_cast<const float4*>(p.rope_cos + a)[q];
+                sn[pr][it][q] = reinterpret_cast<const float4*>(p.rope_sin + a)[q];
               }
             }
           }

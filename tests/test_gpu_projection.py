@@ -267,3 +267,24 @@ def test_two_steps_without_a_commit_call(dev, oracle):
             o_ck[b, :, o_len[b]:o_len[b] + q_cap] = rk[b]
             o_cv[b, :, o_len[b]:o_len[b] + q_cap] = rv[b]
         o_len += q_cap
+
+
+def test_staging_right_behind_a_commit_that_advances(dev):
+    """Every round a commit lengthens the cache by a row and the projection behind it stages behind that row: the kernel starts
+    while the commit still runs, and must not see the old length."""
+    rounds, B, q_cap, dm, Hq, Hkv, D, L0 = 24, 3, 4, 128, 2, 1, 128, 5
+    x, w = make_kv_rows((B, q_cap, dm), 1, "cuda"), make_kv_rows(((Hq + 2 * Hkv) * D, dm), 2, "cuda")
+    ck, cv = make_kv_rows((rounds, B, Hkv, 40, D), 3, "cuda"), make_kv_rows((rounds, B, Hkv, 40, D), 4, "cuda")
+    cl = torch.full((B,), L0, dtype=torch.int32, device="cuda")
+    cache = dlm.make_kv_cache(ck, cv, cl)
+    row_k, row_v = make_kv_rows((1, B, Hkv, 1, D), 5, "cuda"), make_kv_rows((1, B, Hkv, 1, D), 6, "cuda")
+    q, k = torch.empty(B, Hq, q_cap, D, dtype=torch.bfloat16, device="cuda"), torch.empty(B, Hkv, q_cap, D, dtype=torch.bfloat16, device="cuda")
+    v, ws = torch.empty_like(k), dev.workspace(256)
+    for r in range(rounds):
+        dlm.dlm_kv_cache_commit(dev.ctx, cache, row_k, row_v, 1, None, None, dlm.DLM_DST_APPEND, None, 1, 1, r, r + 1)
+        dlm.dlm_window_qkv_project_stage(dev.ctx, x, w, None, None, None, B, q_cap, dm, Hq, Hkv, D, None, q, k, v, cache, r, ws)
+    assert dev.status() == 0 and bool((cl == L0 + rounds).all())
+    for r in range(rounds):
+        n = L0 + r
+        assert torch.equal(ck[r, :, :, n:n + 1], row_k[0]) and torch.equal(cv[r, :, :, n:n + 1], row_v[0])
+        assert torch.equal(ck[r, :, :, n + 1:n + 1 + q_cap], k) and torch.equal(cv[r, :, :, n + 1:n + 1 + q_cap], v)

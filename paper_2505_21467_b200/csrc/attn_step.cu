@@ -1287,6 +1287,9 @@ WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int 
 // calls (Dream heads, 1024 - 1152 cached rows; us):    team of 9, 1 tile, one M tile       10.6
 //   256 active rows: team of 5, 2 tiles, two M tiles   18.3     team of 2, 5 tiles, one M tile  19.1     split  23.4
 //   8 sequences:     team of 4, 3 tiles, two M tiles   20.3     team of 2, 5 tiles, one M tile  19.4     split  23.8
+// Heads of 64, which were not in the fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule,
+// the choice is the fastest or within 2 % of it.  The same calls with heads of 128: within 2 % but one (64 units of 9 tiles,
+// one M tile: team of 2 19.6 us, split over 128 blocks 18.2).
 constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer
 constexpr double kTeamCost[2] = {2.3, 4.3};      // the team schedule's exchange and reduction
 constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...

@@ -12,11 +12,13 @@
 //                   the rows and its half of the tile's features, so it takes in half of what two separate blocks would;
 //                   tiles of 64 .. 512 features.  Bound by the SM's intake from L2 at small tiles, by the tensor pipe from 256.
 //                   Widths of 192 and beyond 256 exist so that a call's tiles fill the pairs once: 1280 rows of 4608 features
-//                   are 90 tiles of 256, two rounds over 74 pairs (49.3 us), and 60 tiles of 384, one round (37.0 us).
+//                   are 90 tiles of 256, two rounds over 74 pairs (52.1 us), and 60 tiles of 384, one round (36.2 us).
 // Measured (one call per layer over 28 / 32 layers' own weights, back to back, rotary embedding and staging on; before this
 // form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
-//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 9.4 us (3.5 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 13.0 us
-//                           256 x 4096 -> 12288   167 -> 29.3 us (880 TFLOP/s)          1280 x 3584 -> 4608   237 -> 35 us (1215 TFLOP/s)
+//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 9.4 us (3.5 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 12.9 us
+//                           256 x 4096 -> 12288   167 -> 28.6 us (900 TFLOP/s)          1280 x 3584 -> 4608   237 -> 36.1 us (1170 TFLOP/s)
+// at SM clocks of 1927 - 1965 MHz (bursts of 12 ms); one call after the other for longer, the power cap brings 1280 rows to 1670
+// MHz and 41 us, 256 x 4096 -> 12288 to 1600 MHz and 32 us.
 // (Prefetching the tile's weights into L2 before the grid dependency wait, tried by rows and by stages, cost more than
 // the head start gave: the stage loads queue behind it.  31 us without, 38 with, at LLaDA's 256 rows.  Prefetching
 // 8 - 32 stages ahead as the loads go: 0 - 4 us slower too.)
@@ -521,9 +523,14 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
       }
     }
   }
-  // The tile width: estimated cycles of the SM with the most blocks.  Per 16 elements of K a block's MMA takes N / 2
-  // cycles, or what its operands take at 128 bytes per cycle of shared memory, and its operands arrive at about 70 bytes
-  // per cycle and SM (measured); a block costs some fixed time on top.
+  // The tile width: the one with the least estimate for the SM with the most blocks.  Per 16 elements of K a block's MMA takes
+  // N / 2 cycles, or what its operands take at 128 bytes per cycle of shared memory, or what they take to arrive at 70 bytes
+  // per cycle and SM; a block costs some fixed time on top.  It ranks widths and is not a time: HBM, latencies, the producers'
+  // loop and the power cap are not in it, and calls take 1.3 to 3.6 times as long (32 x 3584 -> 4608: 4.0 us against 9.4
+  // measured, 256 x 3584 -> 4608 9.2 against 12.9, 1280 x 3584 -> 4608 24.7 against 36.1, 256 x 4096 -> 12288 15.0 against 28.6,
+  // and 28.5 with the weights in L2: it is not HBM that is missing there).  Of 125 calls with every width timed (both
+  // projections of five models' widths, 1 - 3000 rows) it picks the fastest or one within 2 % in 123; the two are 800 rows of
+  // 12288 features (384: 96.5 us, 256: 93.0) and 2000 (192: 210, 512: 189), both under the power cap.
   double best = 0;
   pl.variant = -1;
   for (int v = 0; v < (int)(sizeof(kVariants) / sizeof(kVariants[0])); ++v) {

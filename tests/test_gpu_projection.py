@@ -42,13 +42,13 @@ def _qkv_case(dev, oracle, B, q_cap, dm, Hq, Hkv, D, with_bias, seed):
 
 
 @pytest.mark.parametrize("B,q_cap,dm,Hq,Hkv,D,with_bias", [
-    (1, 32, 3584, 28, 4, 128, True),      # Dream-7B widths, one block of 32 rows: K split over the SMs
+    (1, 32, 3584, 28, 4, 128, True),      # Dream-7B widths, one block of 32 rows
     (8, 32, 3584, 28, 4, 128, True),      # the guided config's batch: 256 rows
     (1, 256, 3584, 28, 4, 128, False),    # the paper's window of 256 rows
     (4, 64, 4096, 32, 32, 128, False),    # LLaDA-8B widths (no bias), batch 4 x block 64
     (1, 20, 512, 4, 2, 128, True),        # ragged rows (20 of 32)
     (3, 100, 256, 2, 1, 128, True),       # 300 rows: two row chunks, the second ragged
-    (2, 7, 128, 4, 2, 64, False),         # head_dim 64 (two heads per feature tile), K too short to split
+    (2, 7, 128, 4, 2, 64, False),         # head_dim 64, tiles narrower than a head, K of one stage
 ])
 def test_qkv_projection(dev, oracle, B, q_cap, dm, Hq, Hkv, D, with_bias):
     _qkv_case(dev, oracle, B, q_cap, dm, Hq, Hkv, D, with_bias, seed=B * 1000 + q_cap)
@@ -114,15 +114,14 @@ def _rope_tables(B, q_cap, D, seed, positions=None):
 
 
 @pytest.mark.parametrize("B,q_cap,dm,Hq,Hkv,D,with_bias", [
-    (1, 32, 3584, 28, 4, 128, True),      # Dream-7B widths: K split, the partner feature is 16 lanes away in the final reduction
+    (1, 32, 3584, 28, 4, 128, True),      # Dream-7B widths: tiles of 32 features, 16 of each half of a head
     (8, 32, 3584, 28, 4, 128, False),     # 256 rows
     (4, 64, 4096, 32, 32, 128, False),    # LLaDA-8B widths
     (1, 20, 512, 4, 2, 128, True),        # ragged rows
     (3, 100, 256, 2, 1, 128, True),       # two row chunks
-    (2, 7, 128, 4, 2, 64, False),         # head_dim 64, K too short to split: the partner comes through shared memory
-    (2, 40, 1024, 6, 3, 64, True),        # head_dim 64 with the K split: two heads per tile, partner 8 lanes away; a tile
-                                          # straddles the last key head and the first value head
-    (1, 9, 128, 1, 1, 128, True),         # K too short to split, head_dim 128: the partner sits in another warp
+    (2, 7, 128, 4, 2, 64, False),         # head_dim 64, 14 rows
+    (2, 40, 1024, 6, 3, 64, True),        # head_dim 64, 80 rows: pairs of blocks, tiles of one head
+    (1, 9, 128, 1, 1, 128, True),         # the fewest heads, K of one stage
 ])
 def test_qkv_projection_with_rotary_embedding(dev, oracle, B, q_cap, dm, Hq, Hkv, D, with_bias):
     seed = 7 * B + q_cap
@@ -163,9 +162,9 @@ def test_rotary_projection_argument_errors(dev):
 
 
 @pytest.mark.parametrize("B,q_cap,dm,Hq,Hkv,D,Lcap,cache_len,q_len,rope", [
-    (1, 32, 3584, 28, 4, 128, 1100, [1024], None, True),          # Dream-7B widths: K split, 8-byte stores into the cache
+    (1, 32, 3584, 28, 4, 128, 1100, [1024], None, True),          # Dream-7B widths
     (4, 64, 1024, 8, 8, 128, 300, [200, 0, 236, 17], [64, 5, 64, 0], False),   # ragged active rows, one slot range ending at capacity
-    (2, 7, 128, 4, 2, 64, 40, [3, 30], [7, 6], True),             # unsplit K: element-wise stores
+    (2, 7, 128, 4, 2, 64, 40, [3, 30], [7, 6], True),             # head_dim 64, 14 rows, one of them inactive
 ])
 def test_projection_stages_the_window_rows_in_the_cache(dev, oracle, B, q_cap, dm, Hq, Hkv, D, Lcap, cache_len, q_len, rope):
     """K/V of the window written by the projection's epilogue to cache rows cache_len[b] + i of one layer: those rows

@@ -30,7 +30,9 @@ def dev():
     (1, 100, 192, 40, 4, 128),    # 128-feature pair tiles of 64 rows
     (1, 100, 128, 128, 16, 64),   # 256-feature pair tiles of 64 rows: four heads of 64
     (1, 250, 192, 88, 4, 64),     # 128-feature pair tiles of 128 rows: two heads of 64
-    (1, 250, 64, 72, 4, 128),     # 256-feature pair tiles of 128 rows: two heads of 128
+    (1, 250, 64, 72, 4, 128),     # 192-feature pair tiles of 128 rows, units of heads of 128
+    (1, 130, 64, 104, 4, 128),    # 256-feature pair tiles of 128 rows: two heads of 128
+    (1, 300, 64, 104, 4, 64),     # the same, four heads of 64, two chunks of rows
     (1, 33, 128, 14, 1, 24),      # a head size without rotary embedding
     (1, 160, 64, 192, 10, 64),    # 192-feature tiles, units of 32 two to a group, the last tile ragged
     (1, 160, 128, 84, 8, 128),    # the same with heads of 128

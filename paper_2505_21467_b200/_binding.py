@@ -171,7 +171,7 @@ def _load_calls():
     global _calls
     if _calls is None:
         lib()   # the missing-library message, and the one copy of libdlm.so
-        if os.path.exists(_build.CALLS) and not _build.calls_built_for(_build.calls_fingerprint()):
+        if os.path.exists(_build.CALLS) and not _build.calls_loadable():
             raise ImportError(f"{_build.CALLS} was not built from its present sources for {_build.calls_abi()}, whose objects it "
                               "would read: run `python -m paper_2505_21467_b200.build`")
         try:

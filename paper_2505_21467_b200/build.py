@@ -78,6 +78,13 @@ def calls_built_for(what: str) -> bool:
         return False
 
 
+def calls_loadable() -> bool:
+    """Whether the _dlm_calls.so in place may be loaded: built for this torch and Python and, where the sources are at hand (a
+    copy of the built package may come without them), from them."""
+    at_hand = os.path.exists(CALLS_SRC) and os.path.exists(os.path.join(INCLUDE, "dlm.h"))
+    return calls_built_for(calls_fingerprint() if at_hand else f"dlm_calls for {calls_abi()}, ")
+
+
 def build_calls(force: bool = False, verbose: bool = False) -> str:
     """Compile the Python entry points (needs torch's headers, no GPU)."""
     if not force and calls_built_for(calls_fingerprint()):

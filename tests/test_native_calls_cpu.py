@@ -78,6 +78,12 @@ def test_a_module_of_other_sources_is_not_loaded(monkeypatch):
     monkeypatch.setattr(_binding, "_calls", None)
     with pytest.raises(ImportError, match="present sources"):
         _binding._load_calls()
+    monkeypatch.setattr(_build, "CALLS_SRC", __file__ + ".not_there")     # a copy of the built package without its sources
+    assert _binding._load_calls().built_for
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    monkeypatch.setattr(_binding, "_calls", None)
+    with pytest.raises(ImportError, match="torch 9.9.9"):
+        _binding._load_calls()
 
 
 class _Failed:

@@ -15,7 +15,7 @@
 //                   are 90 tiles of 256, two rounds over 74 pairs (52.1 us), and 60 tiles of 384, one round (36.2 us).
 // Measured (one call per layer over 28 / 32 layers' own weights, back to back, rotary embedding and staging on; before this
 // form: one 128-feature block per tile with K split over blocks and partial tiles through the workspace):
-//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 9.4 us (3.5 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 12.9 us
+//   rows x K -> features     32 x 3584 -> 4608   12.6 -> 8.5 us (3.9 TB/s of weights)    256 x 3584 -> 4608   25.1 -> 12.4 us
 //                           256 x 4096 -> 12288   167 -> 28.6 us (900 TFLOP/s)          1280 x 3584 -> 4608   237 -> 36.1 us (1170 TFLOP/s)
 // at SM clocks of 1927 - 1965 MHz (bursts of 12 ms); one call after the other for longer, the power cap brings 1280 rows to 1670
 // MHz and 41 us, 256 x 4096 -> 12288 to 1600 MHz and 32 us.
@@ -171,7 +171,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     int head = my_kp / head_panels, panel = my_kp - head * head_panels, s = 0, round = 0;
     bool ok = true;
     for (int kc = 0; kc < n_k; ++kc) {
-      if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
+      if (round > 0) ok = mbar_wait_warp(bar_empty + 8 * s, (round - 1) & 1, abort_ptr);
       if (!ok) break;
       if (warp == 1 && rank == 0 && lane == 0) mbar_expect_tx(bar_full + 8 * s, x_bytes * 2u);   // pieces: always a pair
       __syncwarp();
@@ -192,7 +192,7 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     bool ok = true;
     int s = 0, round = 0;
     for (int kc = 0; kc < n_k; ++kc) {
-      if (round > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty + 8 * s, (round - 1) & 1, abort_ptr)) != 0;
+      if (round > 0) ok = mbar_wait_warp(bar_empty + 8 * s, (round - 1) & 1, abort_ptr);
       if (!ok) break;
       if (elect_one_sync()) {
         if (rank == 0) mbar_expect_tx(bar_full + 8 * s, bytes);
@@ -223,40 +223,50 @@ window_proj_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
     }
   } else if (warp == 2 && rank == 0) {
     // ================================================================= MMA issuer
-    bool ok = true;
     const uint32_t idesc = make_idesc_bf16(M, (uint32_t)kN0, 0), idesc1 = make_idesc_bf16(M, (uint32_t)(kN1 ? kN1 : 64), 0);
     const uint64_t desc = make_smem_desc_sw128(base, 16, 1024);
     const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
-    int s = 0, round = 0;
-    for (int kc = 0; kc < n_k; ++kc) {
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, round & 1, abort_ptr)) != 0;
-      if (!ok) break;
-      tc_fence_after_sync();
-      // descriptors of the stage's panels, in warp-uniform code so that they sit in the uniform registers the MMA reads
-      uint32_t a_lo[KP], b_lo[KP];
-      a_lo[0] = desc_lo + ((s * stage_bytes) >> 4);
-      b_lo[0] = a_lo[0] + (x_bytes >> 4);
+    // One lane runs the whole loop, waits included, so that the MMAs of a stage follow one another at the tensor pipe's rate: with
+    // the warp taking part in every wait and one lane elected per stage, a stage of 16 MMAs of 64 x 32 x 16 took 710 cycles, 320
+    // more than the pipe needs (32 x 3584 -> 4608: 9.3 us, now 8.5; 32 x 3584 -> 3584: 8.5, now 7.5; with the weights in L2 8.1, now
+    // 6.8).  Whether the next stage is there too is asked before this one's MMAs are issued, which hides the answer's latency.
+    auto issue = [&](uint32_t off, bool first) {
+      const uint32_t a_lo = desc_lo + (off >> 4), b_lo = a_lo + (x_bytes >> 4);
 #pragma unroll
-      for (int kp = 1; kp < KP; ++kp) {
-        a_lo[kp] = a_lo[kp - 1] + (x_panel >> 4);
-        b_lo[kp] = b_lo[kp - 1] + kBlockN * 8;
-      }
-      if (elect_one_sync()) {
+      for (int kp = 0; kp < KP; ++kp) {
 #pragma unroll
-        for (int kp = 0; kp < KP; ++kp) {
-#pragma unroll
-          for (int k = 0; k < kPanel / 16; ++k) {
-            const uint32_t add = kc > 0 || kp > 0 || k > 0 ? 1u : 0u;
-            mma_ss_lo<PAIR>(tmem, a_lo[kp] + 2 * k, b_lo[kp] + 2 * k, desc_hi, idesc, add);
-            if (kN1) mma_ss_lo<PAIR>(tmem + kN0, a_lo[kp] + 2 * k, b_lo[kp] + kN0 / 2 * 8 + 2 * k, desc_hi, idesc1, add);
-          }
+        for (int k = 0; k < kPanel / 16; ++k) {
+          const uint32_t add = !first || kp > 0 || k > 0 ? 1u : 0u, ka = a_lo + kp * (x_panel >> 4) + 2 * k, kb = b_lo + kp * (kBlockN * 8) + 2 * k;
+          mma_ss_lo<PAIR>(tmem, ka, kb, desc_hi, idesc, add);
+          if (kN1) mma_ss_lo<PAIR>(tmem + kN0, ka, kb + kN0 / 2 * 8, desc_hi, idesc1, add);
         }
-        if (PAIR) tc_commit_pair(bar_empty + 8 * s); else tc_commit(bar_empty + 8 * s);
       }
-      __syncwarp();
-      if (++s == p.n_stages) { s = 0; ++round; }
+    };
+    if (n_k <= 2) {   // K in one or two stages, each with a buffer of its own: nothing to overlap, and this way it takes 0.1 us less
+      bool ok = true;
+      for (int kc = 0; ok && kc < n_k; ++kc) {
+        ok = mbar_wait_warp(bar_full + 8 * kc, 0, abort_ptr);
+        tc_fence_after_sync();
+        if (ok && elect_one_sync()) issue(kc * stage_bytes, kc == 0);
+        __syncwarp();
+      }
+      if (elect_one_sync()) { if (PAIR) tc_commit_pair(bar_done); else tc_commit(bar_done); }
+    } else if (elect_one_sync()) {
+      int s = 0, round = 0;
+      uint32_t off = 0;
+      bool here = false;   // the stage's data has been seen to be there
+      for (int kc = 0; kc < n_k; ++kc) {
+        if (!here && !mbar_wait(bar_full + 8 * s, round & 1, abort_ptr)) break;
+        tc_fence_after_sync();
+        const uint32_t cur = off, bar = bar_empty + 8 * s;
+        off += stage_bytes;
+        if (++s == p.n_stages) { s = 0; off = 0; ++round; }
+        here = kc + 1 < n_k && mbar_test_wait(bar_full + 8 * s, round & 1);
+        issue(cur, kc == 0);
+        if (PAIR) tc_commit_pair(bar); else tc_commit(bar);
+      }
+      if (PAIR) tc_commit_pair(bar_done); else tc_commit(bar_done);
     }
-    if (elect_one_sync()) { if (PAIR) tc_commit_pair(bar_done); else tc_commit(bar_done); }
     __syncwarp();
   } else if (warp >= 4) {
     // ================================================================= tables of the epilogue

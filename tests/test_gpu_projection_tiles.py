@@ -88,3 +88,10 @@ def test_out_projection_tiles(dev, oracle, B, q_cap, dm, Hq, D):
     dlm.dlm_window_out_project(dev.ctx, o, wo, None, B, q_cap, dm, Hq, D, y, ws)
     assert dev.status() == 0
     _close(y, oracle.out_project(widen(o), widen(wo), None), "y")
+
+
+# K of one stage, of two (a stage holds 256 elements of K, or 128 with more than 64 rows), of one more, and of more than the ring holds
+@pytest.mark.parametrize("dm", [128, 256, 512, 576, 2304])
+@pytest.mark.parametrize("q_cap", [17, 100, 200])
+def test_qkv_projection_stages_of_k(dev, oracle, q_cap, dm):
+    _qkv_case(dev, oracle, 1, q_cap, dm, 4, 1, 128, True, q_cap + dm)

@@ -14,7 +14,7 @@
 //   warps 0-3   softmax of M tile 0 (thread = query row = TMEM lane)
 //   warps 4-7   softmax of M tile 1
 //   warp  8     TMA producer (one lane): Q once per segment, K and V tiles through two rings
-//   warp  9/10  tcgen05.mma issuer of M tile 0 / 1 (one elected lane each): S = Q K^T into one of two
+//   warp  9/10  tcgen05.mma issuer of M tile 0 / 1 (one lane each): S = Q K^T into one of two
 //               64-column score buffers in TMEM, two half-steps ahead of the softmax; then
 //               O += P V with P read from TMEM (it overwrites S in place as packed bf16)
 //   warp  11    publisher (one lane): makes a finished partial result visible device-wide and
@@ -812,16 +812,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     } else if (warp == 9 || warp == 10) {
       // ============================================ MMA issuers: warp 9 for M tile 0, warp 10 for M tile 1
       // One warp per M tile, so that the scalar work around one tile's MMAs (barrier waits and
-      // commits) runs while the tensor pipe executes the other tile's.  The whole warp runs the
-      // loop and one elected lane issues: in warp-uniform code the descriptors live in uniform
-      // registers, which is what tcgen05.mma reads; issued from a divergent single-lane branch
-      // every MMA paid for moving its operands there.  The K, V and Q buffers are
-      // released when every issuer has committed (their "empty" barriers count n_mt arrivals).
+      // commits) runs while the tensor pipe executes the other tile's.  One elected lane runs the whole
+      // loop, waits included: with the warp taking part in every wait and a lane elected per product, waits on
+      // complete barriers and the elections stood between P's arrival and the products it releases (an LLaDA layer, one M tile
+      // per block: 31.5 us, now 29.5; two M tiles, where the softmax warps bound the loop, 0 - 2 %).  The K, V and Q
+      // buffers are released when every issuer has committed (their "empty" barriers count n_mt arrivals).
       const int mt = warp - 9;
-      if (has_work && mt < p.n_mt) {
-        auto wait_warp = [&](uint32_t bar, uint32_t parity) {
-          return __all_sync(0xffffffffu, mbar_wait_limit(bar, parity, abort_ptr, kLimit)) != 0;
-        };
+      if (has_work && mt < p.n_mt && elect_one_sync()) {
+        auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_limit(bar, parity, abort_ptr, kLimit); };
         SegmentWalker walk(p, sched, blockIdx.x);
         Segment g;
         uint32_t kt = 0, vt = 0, gt = 0, seg = 0;
@@ -838,34 +836,23 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const uint32_t idesc = make_idesc_bf16(128, (uint32_t)n16, 0);
           const uint64_t dk = desc_offset(desc_k0, ks * G::kTileBytes + k0 * 128);
           const uint32_t d = t_s + buf * kHalfKeys;
-          if (elect_one_sync()) {
-            mma_ss<false>(d, desc_q, dk, idesc);
 #pragma unroll
-            for (int k = 1; k < D / 16; ++k) {
-              const uint32_t off = (k >> 2) * kPanelBytes + (k & 3) * 32;
-              mma_ss<true>(d, desc_offset(desc_q, off), desc_offset(dk, off), idesc);
-            }
+          for (int k = 0; k < D / 16; ++k) {
+            const uint32_t off = ((k >> 2) * kPanelBytes + (k & 3) * 32) >> 4;
+            mma_ss_lo<false>(d, (uint32_t)desc_q + off, (uint32_t)dk + off, (uint32_t)(desc_q >> 32), idesc, k > 0 ? 1u : 0u);
           }
-          __syncwarp();
         };
         // O (+)= P V for the same keys, P in score buffer `buf`, V tile in stage `vs`
         auto issue_pv = [&](uint32_t vs, int k0, int n16, uint32_t buf, bool first) {
           const uint64_t dv = desc_offset(desc_v0, vs * G::kTileBytes + k0 * 128);
           const uint32_t a = t_s + buf * kHalfKeys;
-          if (elect_one_sync()) {
-            if (first) mma_ts<false>(t_o, a, dv, idesc_pv); else mma_ts<true>(t_o, a, dv, idesc_pv);
-            if (n16 == kHalfKeys) {
+          if (first) mma_ts<false>(t_o, a, dv, idesc_pv); else mma_ts<true>(t_o, a, dv, idesc_pv);
+          if (n16 == kHalfKeys) {
 #pragma unroll
-              for (int st = 1; st < kHalfKeys / 16; ++st) mma_ts<true>(t_o, a + st * 8, desc_offset(dv, st * 2048), idesc_pv);
-            } else {
-              for (int st = 1; st < n16 / 16; ++st) mma_ts<true>(t_o, a + st * 8, desc_offset(dv, st * 2048), idesc_pv);
-            }
+            for (int st = 1; st < kHalfKeys / 16; ++st) mma_ts<true>(t_o, a + st * 8, desc_offset(dv, st * 2048), idesc_pv);
+          } else {
+            for (int st = 1; st < n16 / 16; ++st) mma_ts<true>(t_o, a + st * 8, desc_offset(dv, st * 2048), idesc_pv);
           }
-          __syncwarp();
-        };
-        auto commit = [&](uint32_t bar) {
-          if (elect_one_sync()) tc_commit(bar);
-          __syncwarp();
         };
         uint32_t js = 0;   // half-steps whose scores have been issued (global count: buffer = js & 1)
         bool q_ahead = early_q;   // the Q of the block's first unit was copied before the lengths were known
@@ -874,15 +861,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           q_ahead = false;
           if (g.t_end <= g.t_begin) {
             if (q_here) {   // no key tile for this block after all: take that Q and release it
-              ok = wait_warp(bar_q_full, seg & 1);
+              ok = wait(bar_q_full, seg & 1);
               if (!ok) break;
-              if (lane == 0) mbar_arrive(bar_q_empty);
-              __syncwarp();
+              mbar_arrive(bar_q_empty);
               ++seg;
             }
             continue;
           }
-          ok = wait_warp(bar_q_full, seg & 1);
+          ok = wait(bar_q_full, seg & 1);
           if (!ok) break;
           HalfIter si(g, p.fresh_box), pi(g, p.fresh_box);
           // scores of the next half-step of the segment that has none yet, into buffer js & 1
@@ -891,17 +877,17 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             if (!si.get(hs)) return true;
             const uint32_t ks = kt % KS;
             if (hs.first_of_tile) {
-              if (!wait_warp(bar_k_full + 8 * ks, (kt / KS) & 1)) return false;
+              if (!wait(bar_k_full + 8 * ks, (kt / KS) & 1)) return false;
               tc_fence_after_sync();
             }
             issue_s(ks, hs.k0, (hs.nkeys + 15) & ~15, js & 1);
-            commit(bar_s_ready + 16 * mt + 8 * (js & 1));
+            tc_commit(bar_s_ready + 16 * mt + 8 * (js & 1));
             ++js;
             si.advance(hs);
             if (hs.last_of_tile) {
-              commit(bar_k_empty + 8 * ks);
+              tc_commit(bar_k_empty + 8 * ks);
               ++kt;
-              if (si.t >= g.t_end) commit(bar_q_empty);   // Q is not read again in this segment
+              if (si.t >= g.t_end) tc_commit(bar_q_empty);   // Q is not read again in this segment
             }
             return true;
           };
@@ -911,17 +897,17 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           while (ok && pi.get(hs)) {
             const uint32_t vs = vt % VS;
             if (hs.first_of_tile) {
-              ok = wait_warp(bar_v_full + 8 * vs, (vt / VS) & 1);
+              ok = wait(bar_v_full + 8 * vs, (vt / VS) & 1);
               if (!ok) break;
             }
-            ok = wait_warp(bar_p_ready + 16 * mt + 8 * (gt & 1), (gt >> 1) & 1);
+            ok = wait(bar_p_ready + 16 * mt + 8 * (gt & 1), (gt >> 1) & 1);
             if (!ok) break;
             tc_fence_after_sync();
             issue_pv(vs, hs.k0, (hs.nkeys + 15) & ~15, gt & 1, first);
-            commit(bar_pv_done + 16 * mt + 8 * (gt & 1));
+            tc_commit(bar_pv_done + 16 * mt + 8 * (gt & 1));
             first = false;
             if (hs.last_of_tile) {
-              commit(bar_v_empty + 8 * vs);
+              tc_commit(bar_v_empty + 8 * vs);
               ++vt;
             }
             ++gt;
@@ -930,9 +916,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
           ++seg;
         }
-        // every MMA issued by this warp has finished before TMEM is released
-        if (elect_one_sync()) tc_commit(bar_drain + 8 * mt);
-        __syncwarp();
+        // every MMA issued by this lane has finished before TMEM is released
+        tc_commit(bar_drain + 8 * mt);
         mbar_wait(bar_drain + 8 * mt, 0, never_ptr);
       }
     } else {
@@ -968,9 +953,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const int n_live_mt = min(128, n_live - 128 * mt);   // live softmax threads of this M tile
       // the warp leaves a wait together, so the .sync.aligned TMEM instructions that follow
       // always see a converged warp, also when a wait is given up
-      auto wait_warp = [&](uint32_t bar, uint32_t parity) {
-        return __all_sync(0xffffffffu, mbar_wait_limit(bar, parity, abort_ptr, kLimit)) != 0;
-      };
+      auto wait_warp = [&](uint32_t bar, uint32_t parity) { return mbar_wait_warp(bar, parity, abort_ptr, kLimit); };
       // this thread's query row in row chunk rc of a KV head: which of its query heads, which active row
       // (rows of a KV head's query heads lie one after the other)
       auto out_row_of = [&](int lc_layer, int b, int kvh, int rc) {

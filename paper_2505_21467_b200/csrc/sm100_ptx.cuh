@@ -266,7 +266,7 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"(both) : "memory");
 }
-// The same MMA with the descriptors given by their low words and one high word they share (operands of the same layout).
+// D[tmem] (+)= A[smem] * B[smem], kind::f16, with the descriptors given by their low words and one high word they share (operands of the same layout).
 // The issuing thread's scalar work sets the rate of small MMAs: with 64-bit descriptor arithmetic an MMA of 64 x 32 x 16
 // took 45 cycles to issue, this way 26, which is what its operands take to read.
 template <bool PAIR>
@@ -281,19 +281,9 @@ __device__ __forceinline__ void mma_ss_lo(uint32_t d_tmem, uint32_t a_lo, uint32
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; kind::f16 (bf16 inputs, fp32 accumulate).  ACC is a compile-time
+// D[tmem] (+)= A[tmem] * B[smem]; kind::f16 (bf16 inputs, fp32 accumulate).  ACC is a compile-time
 // flag: the issuing thread runs alone, so every scalar instruction it spends per MMA is exposed
 // latency; descriptors are prepared once and only offset by constants (desc_offset).
-template <bool ACC>
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-  if (ACC)
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, 1, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc) : "memory");
-  else
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, 0, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc) : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem].
 template <bool ACC>
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
   if (ACC)

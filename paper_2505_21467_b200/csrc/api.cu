@@ -24,7 +24,7 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
   ctx->encode_tiled = ctx->replace_address = nullptr;
   ctx->maps = new (std::nothrow) dlm_map_cache();
   ctx->commit_blocks_per_sm[0] = ctx->commit_blocks_per_sm[1] = 0;
-  for (int i = 0; i < 8; ++i) ctx->attn_smem_limit[i] = 0;
+  for (int& limit : ctx->attn_smem_limit) limit = 0;
   ctx->proj_configured = 0;
   memset(&ctx->attn_plan_key, 0, sizeof ctx->attn_plan_key);
   ctx->wait_limit_ns = sm100::kWaitLimitNs;

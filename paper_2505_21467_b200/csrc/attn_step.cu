@@ -107,7 +107,7 @@ struct Segment {
   int lc_layer, b, kvh, rc;   // unit: layer within the call, batch element, KV head, row chunk
   int Lc, Lq, n_ct, T;    // lengths, cache tiles, total tiles of the unit
   int t_begin, t_end;     // tile range of this segment
-  int slot;               // partial slot; -1 when the segment is the whole unit; -2 for a piece of the team schedule
+  int slot;               // partial slot; -1 when the segment is the whole unit
   int merger;             // partial segment holding the unit's last tile: this block merges the unit
 };
 
@@ -116,17 +116,49 @@ __device__ __forceinline__ int tiles_of(int Lc, int Lq, int fresh_box) {
   return (Lc + kTileKeys - 1) / kTileKeys + (Lq + fresh_box - 1) / fresh_box;
 }
 
+// Launches in which a block has one unit at most (kSingle: whole units on as many SMs, and teams): which one does not depend on
+// the lengths, so it is decoded while the kernel before is still running; of the lengths a block needs those of its unit's
+// batch element only, and every role reads them for itself: no tables and no barrier behind the wait for the kernel before.
+// They are kernels of their own because what stands in front of the first copies is code that is not in the instruction
+// cache (another kernel has run in between): with all schedules in one kernel and the tables, a one-layer call of Dream issued
+// its first K copy 5360 cycles after that wait, now 2260.  Us a call, before -> now: one sequence 10.6 -> 9.3, window of 256
+// rows 18.2 -> 16.8, 8 sequences 19.2 -> 17.2, an LLaDA layer (whole units) 29.5 -> 28.0, 28 layers in one call 26.7 -> 25.3.
+__device__ __forceinline__ void decode_single(const AttnParams& p, Segment& g) {
+  const int unit = p.team > 1 ? p.by_team.div(blockIdx.x) : (int)blockIdx.x;
+  const int grp = p.by_batch.divmod(unit, g.b);
+  g.lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, g.rc), g.kvh);
+}
+__device__ __forceinline__ void set_single_lengths(const AttnParams& p, Segment& g, int Lc, int Lq) {
+  g.Lc = Lc;
+  g.Lq = Lq;
+  g.n_ct = (Lc + kTileKeys - 1) / kTileKeys;
+  g.T = tiles_of(Lc, Lq, p.fresh_box);
+  g.t_begin = 0;
+  g.t_end = g.T;
+  if (p.team > 1) {   // this block's share of the unit's key tiles; the launch has one team per unit
+    const int rank = (int)blockIdx.x - p.by_team.div(blockIdx.x) * p.team;
+    g.t_begin = p.by_team.div(g.T * rank);
+    g.t_end = p.by_team.div(g.T * (rank + 1));
+  }
+}
+
 // Walks the segments of block `cta`.  Identical in every role, so the roles agree on the
 // sequence without communicating.  Item counts fit 32 bits (the host refuses larger launches).
+template <bool kSingle>
 struct SegmentWalker {
   const AttnParams& p;
   const Sched& s;
   int end, range_begin;   // split mode: items [range_begin, end) are still to do
   int unit, n_units;
-  __device__ SegmentWalker(const AttnParams& p_, const Sched& s_, int cta) : p(p_), s(s_) {
+  __device__ __forceinline__ SegmentWalker(const AttnParams& p_, const Sched& s_, int cta) : p(p_), s(s_) {
+    if (kSingle) {
+      unit = end = range_begin = 0;
+      n_units = 1;
+      return;
+    }
     n_units = p.nl * p.n_kv_heads * p.n_rc * p.batch;
     if (p.whole_units) {
-      unit = p.team > 1 ? p.by_team.div(cta) : cta;
+      unit = cta;
       end = range_begin = 0;
     } else {
       range_begin = cta < s.n_cta ? s.lo(cta) : 0;
@@ -134,7 +166,12 @@ struct SegmentWalker {
       unit = 0;
     }
   }
-  __device__ bool next(Segment& g, int n_cta) {
+  __device__ __forceinline__ bool next(Segment& g, int n_cta) {
+    if (kSingle) {   // g holds the block's unit already
+      const bool more = unit < n_units;
+      unit = n_units;
+      return more;
+    }
     if (p.whole_units) {
       if (unit >= n_units) return false;
       const int grp = p.by_batch.divmod(unit, g.b);
@@ -147,14 +184,6 @@ struct SegmentWalker {
       g.t_end = g.T;
       g.slot = -1;
       g.merger = 0;
-      if (p.team > 1) {   // this block's share of the unit's key tiles; the launch has one team per unit
-        const int rank = (int)blockIdx.x - p.by_team.div(blockIdx.x) * p.team;
-        g.t_begin = p.by_team.div(g.T * rank);
-        g.t_end = p.by_team.div(g.T * (rank + 1));
-        g.slot = -2;
-        unit = n_units;
-        return true;
-      }
       unit += n_cta;
       return true;
     }
@@ -247,19 +276,16 @@ struct TeamArgs {
   size_t piece0;               // index of the team's first piece
   size_t qrow0;                // output row of the KV head's first query row
   FastDiv by_q_cap;
-  int team, n_mt, rows, rows_total, rank, r0, Lq, lo, hi;   // r0: the row chunk's first row among the KV head's rows
+  int team, n_mt, rows, rows_total, rank, Lq;
   bool has_keys;
+  int r0, lo, hi;              // r0: the row chunk's first row among the KV head's rows
   uint32_t ml_bytes, o_bytes;  // bytes fetched from each piece: all its (m, l) rows; this block's share of its vectors
-  __device__ __forceinline__ TeamArgs(const AttnParams& p, const Sched& s, int D)
+  __device__ __forceinline__ TeamArgs(const AttnParams& p, const Segment& g, int D)
       : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), by_q_cap(p.by_q_cap), team(p.team), n_mt(p.n_mt), rows(p.rows),
-        rows_total(p.rows_total) {
-    int b, rc, kvh;
+        rows_total(p.rows_total), Lq(g.Lq), has_keys(g.T > 0) {
     const int unit = p.by_team.divmod(blockIdx.x, rank);
-    const int grp = p.by_batch.divmod(unit, b), lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
-    has_keys = s.prefix[b + 1] > s.prefix[b];
-    Lq = s.lq[b];
-    r0 = rc * p.chunk_rows;
-    qrow0 = (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group) * p.q_cap;
+    r0 = g.rc * p.chunk_rows;
+    qrow0 = (((size_t)g.lc_layer * p.batch + g.b) * p.n_q_heads + (size_t)g.kvh * p.group) * p.q_cap;
     arrive = p.tickets + unit;
     depart = arrive + kDlmMaxSplitUnits / 2;
     const int n_vec = p.n_mt * (D / 4) * 128;
@@ -580,7 +606,7 @@ __device__ __noinline__ bool softmax_half_ragged(uint32_t t_s, uint32_t t_o, int
 // its barrier once and gives up if the data is not there yet (waits that let issued copies and MMAs finish keep the
 // 2 s limit).  The limit is a compile-time constant because the waits sit on the critical path of the MMA issuers
 // (a run-time limit cost 2 % at the Dream shape).
-template <int D, int kChunk, bool kNoWait>
+template <int D, int kChunk, bool kSingle, bool kNoWait>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc,
                        const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ CUtensorMap tm_kn,
@@ -632,8 +658,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   // softmax threads that own a real query row, rounded up to whole warps (they are tid 0 .. n_live-1)
   const int n_live = (p.rows + 31) & ~31;
 
-  // ---- set-up: barriers, TMEM and descriptor prefetch first (they need no data), so that they overlap
-  // the cold read of the lengths; then the tile prefix
+  // ---- set-up: barriers, TMEM, descriptor prefetch and which unit is this block's first (they need no data), so that they
+  // overlap the kernel before; then the lengths
   if (tid == 0) {
     *abort_ptr = 0; *never_ptr = 0; *merge_ok = 0; *any_empty = 0;
     mbar_init(bar_q_full, 1);
@@ -673,27 +699,49 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     prefetch_tensormap(&tm_kn);
     prefetch_tensormap(&tm_vn);
   }
-  // everything above needed no data; from here on the inputs of the call are read
-  __syncthreads();   // the barriers exist for the producer's first copy below
-  dlm_grid_dependency_wait();
-  dlm_trigger_dependents();
-  // Whole units and teams: which unit a block starts with does not depend on the lengths, so the copy of its Q
-  // rows starts now, while the lengths are read and the tile prefix is built (about 1 us, and Q no longer queues
-  // in front of the first K tile).  The roles below consume this Q also when the unit turns out to have no key
-  // tile for this block.
-  const bool early_q = p.whole_units != 0;
-  if (early_q && warp == 8 && lane == 0) {
-    int b, rc, kvh;
-    const int grp = p.by_batch.divmod(p.team > 1 ? p.by_team.div(blockIdx.x) : (int)blockIdx.x, b);
-    const int lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
-    const int zq = (lc_layer * p.batch + b) * p.n_kv_heads + kvh;
-    mbar_expect_tx(bar_q_full, (uint32_t)(p.n_mt * min(128, p.rows)) * 128u * G::kPanels);
+  Segment one;
+  if (kSingle) decode_single(p, one);
+  __syncwarp();
+  tc_fence_before_sync();
+  __syncthreads();   // the barriers exist and TMEM is there
+  tc_fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  // Everything above needed no data.  Whole units and teams: which unit a block starts with does not depend on the lengths, so
+  // the copy of its Q rows starts before they are read (about 1 us, and Q does not queue in front of the first K tile).  The
+  // roles below consume this Q also when the unit turns out to have no key tile for this block.
+  const bool early_q = kSingle || p.whole_units != 0;
+  auto expect_q = [&]() { mbar_expect_tx(bar_q_full, (uint32_t)(p.n_mt * min(128, p.rows)) * 128u * G::kPanels); };   // a box counts in full
+  auto copy_q = [&](int zq, int rc) {
     for (int mt = 0; mt < p.n_mt; ++mt)
       for (int pn = 0; pn < G::kPanels; ++pn)
         tma_load_3d(sm_q + mt * G::kTileBytes + pn * kPanelBytes, &tm_q, bar_q_full, pn * 64, rc * kChunk + mt * 128, zq);
+  };
+  // From here on the inputs of the call are read: all threads wait for the kernel before.  In a block of a single unit each role
+  // does so where it starts, so that the code up to there has been fetched by then, and reads its unit's lengths for itself.
+  auto wait_for_inputs = [&]() {
+    dlm_grid_dependency_wait();
+    dlm_trigger_dependents();
+  };
+  auto read_lengths = [&]() {
+    int Lc = p.cache_len[one.b], Lq = p.q_len ? p.q_len[one.b] : p.q_cap;
+    if (Lc < 0 || Lc > p.capacity || Lq < 0 || Lq > p.q_cap) {
+      if (tid == 0) dlm_set_status(p.status, DLM_ERR_CAPACITY);
+      Lc = max(0, min(Lc, p.capacity));
+      Lq = max(0, min(Lq, p.q_cap));
+    }
+    set_single_lengths(p, one, Lc, Lq);
+  };
+  if (!kSingle) {
+    wait_for_inputs();
+    if (early_q && warp == 8 && lane == 0) {
+      int b, rc, kvh;
+      const int lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(p.by_batch.divmod(blockIdx.x, b), rc), kvh);
+      expect_q();
+      copy_q((lc_layer * p.batch + b) * p.n_kv_heads + kvh, rc);
+    }
   }
   // lengths and tile prefix, by one warp: lane = batch element
-  if (warp == 0) {
+  if (!kSingle && warp == 0) {
     int acc = 0;
     for (int b0 = 0; b0 < p.batch; b0 += 32) {
       const int b = b0 + lane;
@@ -722,21 +770,19 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
     if (lane == 0) sched.prefix[p.batch] = acc;
   }
-  __syncwarp();
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  if (!kSingle) __syncthreads();
   // number of shares the item list is cut into (every share holds at least one item)
-  const int total_items = sched.prefix[p.batch] * p.nl * p.n_kv_heads * p.n_rc;
-  const int n_cta = p.whole_units ? (int)gridDim.x : min((int)gridDim.x, total_items);
-  const bool has_work = p.whole_units || (int)blockIdx.x < n_cta;
-  sched.n_cta = max(n_cta, 1);
+  int n_cta = (int)gridDim.x;
+  sched.n_cta = n_cta;
   sched.share = sched.share_rem = 0;
-  if (!p.whole_units) {
+  if (!kSingle && !p.whole_units) {
+    const int total_items = sched.prefix[p.batch] * p.nl * p.n_kv_heads * p.n_rc;
+    n_cta = min(n_cta, total_items);
+    sched.n_cta = max(n_cta, 1);
     sched.share = total_items / sched.n_cta;
     sched.share_rem = total_items - sched.share * sched.n_cta;
   }
+  const bool has_work = kSingle || p.whole_units || (int)blockIdx.x < n_cta;
 
   // The softmax warps keep a whole score row in registers; the other warpgroup needs few.
   // setmaxnreg.inc waits, without a bound, until the registers it asks for are free: the host
@@ -746,9 +792,16 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     setmaxnreg_dec<kRegsOther>();
     if (warp == 8) {
       // ================================================================= TMA producer
+      if (kSingle) {
+        const int zq = (one.lc_layer * p.batch + one.b) * p.n_kv_heads + one.kvh;
+        if (lane == 0) expect_q();
+        wait_for_inputs();
+        if (lane == 0) copy_q(zq, one.rc);
+        read_lengths();
+      }
       if (lane == 0 && has_work) {
-        SegmentWalker walk(p, sched, blockIdx.x);
-        Segment g;
+        SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
+        Segment g = one;
         uint32_t kt = 0, vt = 0, seg = 0, q_issued = early_q ? 1 : 0;
         bool ok = true;
         bool q_ahead = early_q;   // the Q of the block's first unit is already on its way
@@ -764,12 +817,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           if (!q_here) {
             if (seg > 0) ok = mbar_wait_limit(bar_q_empty, (seg - 1) & 1, abort_ptr, kLimit);
             if (!ok) break;
-            const int q_box = min(128, p.rows);
-            mbar_expect_tx(bar_q_full, (uint32_t)(p.n_mt * q_box) * 128u * G::kPanels);  // a box counts in full
-            for (int mt = 0; mt < p.n_mt; ++mt)
-              for (int pn = 0; pn < G::kPanels; ++pn)
-                tma_load_3d(sm_q + mt * G::kTileBytes + pn * kPanelBytes, &tm_q, bar_q_full, pn * 64,
-                            g.rc * kChunk + mt * 128, zq);
+            expect_q();
+            copy_q(zq, g.rc);
             ++q_issued;
           }
           for (int t = g.t_begin; t < g.t_end && ok; ++t) {
@@ -818,10 +867,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // per block: 31.5 us, now 29.5; two M tiles, where the softmax warps bound the loop, 0 - 2 %).  The K, V and Q
       // buffers are released when every issuer has committed (their "empty" barriers count n_mt arrivals).
       const int mt = warp - 9;
+      if (kSingle) {
+        wait_for_inputs();
+        read_lengths();
+      }
       if (has_work && mt < p.n_mt && elect_one_sync()) {
         auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_limit(bar, parity, abort_ptr, kLimit); };
-        SegmentWalker walk(p, sched, blockIdx.x);
-        Segment g;
+        SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
+        Segment g = one;
         uint32_t kt = 0, vt = 0, gt = 0, seg = 0;
         bool ok = true;
         const uint32_t idesc_pv = make_idesc_bf16(128, D, 1);
@@ -925,11 +978,15 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // A piece that some other block will merge: once every softmax thread has stored its row
       // (they arrive on bar_pub and move on), make the stores visible device-wide and count the
       // piece in its unit's counter.
-      if (lane == 0 && p.team > 1) {
-        team_publish<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr);
-      } else if (lane == 0 && has_work && !p.whole_units) {
-        SegmentWalker walk(p, sched, blockIdx.x);
-        Segment g;
+      if (kSingle) {
+        wait_for_inputs();
+        read_lengths();
+      }
+      if (kSingle && lane == 0 && p.team > 1) {
+        team_publish<D, kNoWait>(TeamArgs(p, one, D), sm_q, bar_pub, abort_ptr);
+      } else if (!kSingle && lane == 0 && has_work && !p.whole_units) {
+        SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
+        Segment g = one;
         uint32_t pub = 0;
         while (walk.next(g, n_cta)) {
           if (g.slot < 0 || g.merger || g.t_end <= g.t_begin) continue;
@@ -942,6 +999,10 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   } else {
     setmaxnreg_inc<kRegsSoftmax>();
+    if (kSingle) {
+      wait_for_inputs();
+      read_lengths();
+    }
     if (tid < n_live) {
       // ================================================= softmax warps (those that own real rows)
       const int mt = warp >> 2;
@@ -967,7 +1028,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           if (p.lse) p.lse[qrow] = -CUDART_INF_F;
         }
       };
-      if (!p.whole_units && *any_empty) {
+      if (!kSingle && !p.whole_units && *any_empty) {
         // units without any key (inactive batch elements) appear in no share: zero them here
         const int n_units = p.nl * p.n_kv_heads * p.n_rc * p.batch;
         for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
@@ -978,8 +1039,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         }
       }
       if (has_work) {
-        SegmentWalker walk(p, sched, blockIdx.x);
-        Segment g;
+        SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
+        Segment g = one;
         uint32_t gt = 0, vt = 0;   // half-steps and key tiles done so far
         bool ok = true;
         while (ok && walk.next(g, n_cta)) {
@@ -987,15 +1048,16 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           if (n <= 0) {  // inactive batch element: the unit's rows are zero (team schedule: or no tile for this rank)
             if (g.T == 0) {
               zero_my_row(out_row_of(g.lc_layer, g.b, g.kvh, g.rc), g.rc * kChunk + r_unit < p.rows_total);
-            } else if (g.slot == -2) {   // a piece without key tiles
-              ok = team_exchange<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
+            } else if (kSingle && p.team > 1) {   // a piece without key tiles
+              ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), sm_q, bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
             }
             continue;
           }
           float m_used = -CUDART_INF_F, l_run = 0.f;
           bool first = true;
+          const int n_whole = g.Lc / kTileKeys;   // tiles of 128 visible cache rows
           for (int t = g.t_begin; t < g.t_end && ok; ++t, ++vt) {
-            const int valid = tile_valid(g, t, p.fresh_box);
+            const int valid = t < n_whole ? kTileKeys : tile_valid(g, t, p.fresh_box);
             const int n16 = (valid + 15) & ~15;
             if (valid < n16) {
               // V rows in [valid, n16) would be multiplied by P = 0: clear them so that stale
@@ -1046,9 +1108,9 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const bool real_row = r_kv < p.rows_total;
           const bool active = real_row && r_kv - p.by_q_cap.div(r_kv) * p.q_cap < g.Lq;
           uint32_t v[32];
-          if (g.slot == -2) {
-            ok = team_exchange<D, kNoWait>(TeamArgs(p, sched, D), sm_q, bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
-          } else if (g.slot < 0) {
+          if (kSingle && p.team > 1) {
+            ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), sm_q, bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
+          } else if (kSingle || g.slot < 0) {
             const float inv = active ? 1.f / l_run : 0.f;
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
@@ -1177,9 +1239,9 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
         }
       }
-    } else if (p.team > 1) {
+    } else if (kSingle && p.team > 1) {
       // warps without a row of their own help with the reduction
-      const TeamArgs ta(p, sched, D);
+      const TeamArgs ta(p, one, D);
       if (ta.has_keys) team_exchange<D, kNoWait>(ta, sm_q, bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
     }
   }
@@ -1209,24 +1271,27 @@ bool register_budget_ok(const cudaFuncAttributes& a) {
   return a.numRegs >= kRegsOther && 8 * (kRegsSoftmax - a.numRegs) <= 4 * (a.numRegs - kRegsOther);
 }
 
-// The eight instantiations: head_dim 128 / 64, row chunks of 256 / 128, normal / no-wait (test) waits.
+// The sixteen instantiations: head_dim 128 / 64, row chunks of 256 / 128, normal / no-wait (test) waits, blocks of any number of
+// segments / of one.
 using AttnKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                             const AttnParams);
-inline int kernel_index(int head_dim, int chunk_rows, bool no_wait) {
-  return (head_dim == 128 ? 0 : 1) + (chunk_rows == 256 ? 0 : 2) + (no_wait ? 4 : 0);
+inline int kernel_index(int head_dim, const dlm_attn_plan& pl, bool no_wait) {
+  return (head_dim == 128 ? 0 : 1) + (pl.chunk_rows == 256 ? 0 : 2) + (no_wait ? 4 : 0) + (pl.single ? 8 : 0);
 }
+template <bool kSingle>
 AttnKernel kernel_of(int which) {
-  switch (which) {
-    case 0: return attn_step_sm100_kernel<128, 256, false>;
-    case 1: return attn_step_sm100_kernel<64, 256, false>;
-    case 2: return attn_step_sm100_kernel<128, 128, false>;
-    case 3: return attn_step_sm100_kernel<64, 128, false>;
-    case 4: return attn_step_sm100_kernel<128, 256, true>;
-    case 5: return attn_step_sm100_kernel<64, 256, true>;
-    case 6: return attn_step_sm100_kernel<128, 128, true>;
-    default: return attn_step_sm100_kernel<64, 128, true>;
+  switch (which & 7) {
+    case 0: return attn_step_sm100_kernel<128, 256, kSingle, false>;
+    case 1: return attn_step_sm100_kernel<64, 256, kSingle, false>;
+    case 2: return attn_step_sm100_kernel<128, 128, kSingle, false>;
+    case 3: return attn_step_sm100_kernel<64, 128, kSingle, false>;
+    case 4: return attn_step_sm100_kernel<128, 256, kSingle, true>;
+    case 5: return attn_step_sm100_kernel<64, 256, kSingle, true>;
+    case 6: return attn_step_sm100_kernel<128, 128, kSingle, true>;
+    default: return attn_step_sm100_kernel<64, 128, kSingle, true>;
   }
 }
+AttnKernel kernel_of(int which) { return which & 8 ? kernel_of<true>(which) : kernel_of<false>(which); }
 
 // First use of an attention kernel on a context's device: checks the register budget and opts in to
 // all the dynamic shared memory the device allows a block (less the kernel's static part).
@@ -1346,6 +1411,7 @@ Plan make_plan(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_he
     const bool forced_apart = ctx->attn_team_force && (narrow.team > 1) != (pl.team > 1);
     if (forced_apart ? narrow.team > 1 : narrow_cost < cost) pl = narrow;
   }
+  pl.single = pl.whole_units && (pl.team > 1 || (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc <= pl.grid);
   const WorkspaceSize ws = workspace_size(ctx, cache, nl, n_q_heads, q_cap);
   pl.ws_o_bytes = ws.o_bytes;
   pl.ws_ml_bytes = ws.ml_bytes;
@@ -1407,7 +1473,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
                                  ctx->attn_team_max, ctx->attn_team_force ? 1 : 0, nw ? 1 : 0};
   if (memcmp(&key, &ctx->attn_plan_key, sizeof key) != 0) {
     Plan made = make_plan(ctx, cache, nl, n_q_heads, q_cap, cache_len_hint);
-    const int which = kernel_index(D, made.chunk_rows, nw);
+    const int which = kernel_index(D, made, nw);
     const int rc = configure_kernel(ctx, which, reinterpret_cast<const void*>(kernel_of(which)));
     if (rc != DLM_OK) return rc;
     if (!plan_shared_memory(ctx->attn_smem_limit[which], D, cache->batch, made)) return DLM_ERR_UNSUPPORTED;
@@ -1467,7 +1533,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   if (rc != DLM_OK) return rc;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DLM_CUDA_TRY(dlm_launch(kernel_of(kernel_index(D, pl.chunk_rows, nw)), dim3(pl.grid), dim3(kThreads),
+  DLM_CUDA_TRY(dlm_launch(kernel_of(kernel_index(D, pl, nw)), dim3(pl.grid), dim3(kThreads),
                           (size_t)p.smem_bytes, s, tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
   return dlm_launch_ok(ctx, 1);
 }

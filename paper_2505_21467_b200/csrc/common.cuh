@@ -37,6 +37,7 @@ struct dlm_map_cache {
 // How an attention call's work is dealt out (attn_step.cu), and what that depends on.
 struct dlm_attn_plan {
   int n_mt, rows, rows_total, n_rc, grid, whole_units, chunk_rows, team;
+  int single;      // whole units or teams, and no block has more than one unit (or piece of one)
   int smem_bytes;
   size_t ws_o_bytes, ws_ml_bytes;
 };
@@ -60,7 +61,7 @@ struct dlm_ctx {
   bool attn_team_force;         // tests: take the team schedule wherever it is possible, whatever the cost estimate says
   dlm_attn_plan_key attn_plan_key;   // of the last call's plan (nl = 0: none yet)
   dlm_attn_plan attn_plan;
-  int attn_smem_limit[8];       // dynamic shared memory the two attention kernels may use on this device (0 = not set up yet)
+  int attn_smem_limit[16];      // dynamic shared memory the attention kernels may use on this device (0 = not set up yet)
 };
 
 // Writes the descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle,

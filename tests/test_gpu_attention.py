@@ -410,3 +410,15 @@ def test_team_schedule_gives_up_cleanly_when_its_waits_may_not_wait(dev, oracle)
         dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
     assert dev.status() == 0
     _case(dev, oracle, cache_len=[2048], seed=99, **shape)
+
+
+# as many units as SMs (a block of a single unit each) and a few more (some blocks have two), one M tile and two; with inactive elements
+@pytest.mark.parametrize("B,Hkv,group,D,q_cap", [(37, 4, 2, 64, 40), (50, 3, 2, 128, 40), (37, 4, 7, 128, 20), (50, 3, 5, 64, 30)])
+def test_whole_units_as_many_as_sms_and_more(dev, oracle, B, Hkv, group, D, q_cap):
+    rng = np.random.default_rng(B + D)
+    cl, ql = rng.integers(0, 201, B), rng.integers(0, q_cap + 1, B)
+    ql[[0, B // 2]] = 0
+    for hint in _each_schedule(dev, ["whole"], 1, B, Hkv * group, Hkv, D, 200, q_cap):
+        out, lse, _ = _case(dev, oracle, 1, B, Hkv * group, Hkv, D, 200, q_cap, cl, ql, seed=B, hint=hint)
+    for b in np.flatnonzero(ql == 0):
+        assert not out[0, b].any() and bool((lse[0, b] == -float("inf")).all())

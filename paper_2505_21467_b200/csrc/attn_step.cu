@@ -53,7 +53,6 @@ constexpr int kTeamMax = 16;              // most blocks of a team
 constexpr int kMaxGrid = 256;          // blocks of the persistent grid (one per SM)
 constexpr int kMaxStages = 8;          // barrier slots reserved per ring
 constexpr int kBarrierBytes = 512;     // mbarriers of a block
-constexpr int kBarPub = 32 + 4 * 8 * kMaxStages + 3 * 32;   // distance of the publisher's barrier from the first, which is Q's
 constexpr int kFlagBytes = 64;         // abort / never flags, TMEM slot, merge flag
 
 template <int D>
@@ -79,7 +78,7 @@ struct AttnParams {
   int rows_total;  // group * q_cap: query rows per (layer, batch element, KV head)
   int n_rc;        // row chunks: rows_total cut into units of up to 256 rows (each re-reads the K/V tiles)
   int rows;        // query rows per unit = min(chunk_rows, rows_total)
-  int chunk_rows;  // 256 (two M tiles share every K/V tile) or 128 (one M tile per unit)
+  int chunk_rows;  // 256 (two M tiles share every K/V tile), 128 (one M tile per unit) or 64 (half an M tile; teams)
   int n_mt;        // M tiles per unit (1 or 2)
   int fresh_box;   // rows per TMA box of the fresh K/V tensors = min(128, q_cap)
   int whole_units; // 1: deal whole units round-robin, no partials
@@ -262,9 +261,9 @@ __device__ __forceinline__ bool wait_counter(const unsigned int* addr, unsigned 
 }
 
 // Team schedule: what a block of a team works on after its share of the key tiles.  The team's pieces lie
-// in the workspace as [rank][M tile][head_dim / 4][128 rows] 16-byte vectors (4 columns of a row) and
-// [rank][M tile][128 rows] (m, l) pairs; the unit's n_mt * head_dim / 4 * 128 output vectors are dealt to
-// the ranks in that storage order, rank r reducing vectors [lo, hi) over all pieces.
+// in the workspace as [rank][M tile][head_dim / 4][R rows] 16-byte vectors (4 columns of a row) and
+// [rank][M tile][R rows] (m, l) pairs, R the unit's rows in an M tile rounded up to 32, 64 or 128; the unit's n_mt * head_dim / 4 * R
+// output vectors are dealt to the ranks in that storage order, rank r reducing vectors [lo, hi) over all pieces.
 // Everything the exchange needs, decoded by the caller and handed over by value.
 struct TeamArgs {
   __nv_bfloat16* out;
@@ -279,7 +278,7 @@ struct TeamArgs {
   int team, n_mt, rows, rows_total, rank, Lq;
   bool has_keys;
   int r0, lo, hi;              // r0: the row chunk's first row among the KV head's rows
-  uint32_t ml_bytes, o_bytes;  // bytes fetched from each piece: all its (m, l) rows; this block's share of its vectors
+  int r_shift;                 // log2 R
   __device__ __forceinline__ TeamArgs(const AttnParams& p, const Segment& g, int D)
       : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), by_q_cap(p.by_q_cap), team(p.team), n_mt(p.n_mt), rows(p.rows),
         rows_total(p.rows_total), Lq(g.Lq), has_keys(g.T > 0) {
@@ -288,12 +287,11 @@ struct TeamArgs {
     qrow0 = (((size_t)g.lc_layer * p.batch + g.b) * p.n_q_heads + (size_t)g.kvh * p.group) * p.q_cap;
     arrive = p.tickets + unit;
     depart = arrive + kDlmMaxSplitUnits / 2;
-    const int n_vec = p.n_mt * (D / 4) * 128;
+    r_shift = p.rows > 64 ? 7 : p.rows > 32 ? 6 : 5;
+    const int n_vec = (p.n_mt * (D / 4)) << r_shift;
     lo = p.by_team.div(n_vec * rank);          // n_vec <= 8192, team <= 16
     hi = p.by_team.div(n_vec * (rank + 1));
     piece0 = (size_t)unit * p.team * p.n_mt;
-    ml_bytes = (uint32_t)p.n_mt * 128u * 8u;
-    o_bytes = (uint32_t)(hi - lo) * 16u;
   }
 };
 
@@ -302,57 +300,107 @@ struct TeamArgs {
 // layer-batched calls, which never run them).
 //
 // Publisher warp, one thread: once every softmax thread of this block has stored its row of the block's piece
-// (bar_pub), count the block in the unit's arrival counter; when the whole team has arrived, fetch this
-// block's share of every piece, and every piece's (m, l) rows, into the shared memory the Q, K and V buffers no
-// longer need (all of the block's MMAs have finished by then: every softmax thread waited for its last one).
-// bar_team = bar_pub + 8 completes when all of it has landed.  A block without a key tile of its own has run no MMA, and
-// its Q may still be on its way to that shared memory: the barrier of Q, bar_pub - kBarPub, is waited for too.
-template <int D, bool kNoWait>
-__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
-                                          volatile int* abort_ptr) {
+// (bar_pub), count the block in the unit's arrival counter; when the whole team has arrived, let the softmax threads go on
+// (bar_team = bar_pub + 8).
+template <bool kNoWait>
+__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t bar_pub, volatile int* abort_ptr) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
-  const uint32_t bar_team = bar_pub + 8;
   if (!p.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
   __threadfence();
   atomicAdd(p.arrive, 1u);
-  if (!mbar_wait_limit(bar_pub - kBarPub, 0, abort_ptr, kLimit)) return;
   if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
-  fence_proxy_async_all();
-  mbar_expect_tx(bar_team, (uint32_t)p.team * (p.ml_bytes + p.o_bytes));
-  for (int c = 0; c < p.team; ++c) {
-    bulk_load(sm_q + c * p.ml_bytes, p.ws_ml + (p.piece0 + (size_t)c * p.n_mt) * 256, p.ml_bytes, bar_team);
-    bulk_load(sm_q + p.team * p.ml_bytes + c * p.o_bytes,
-              p.ws_o + ((p.piece0 + (size_t)c * p.n_mt) * (size_t)(D / 4 * 128) + p.lo) * 4, p.o_bytes, bar_team);
-  }
+  mbar_arrive(bar_pub + 8);
   // every block of the team is past its wait on the arrival counter when the last one gets here: the last
   // one clears both counters for the next launch
   if (atomicAdd(p.depart, 1u) == (unsigned int)p.team - 1u) {
     *p.arrive = 0;
     *p.depart = 0;
   }
-  // the copies issued above land in this block's shared memory: this thread does not leave before they have (the
-  // softmax threads wait on the same barrier, but may have given up); abort_ptr + 1 is the flag that stays 0
-  mbar_wait(bar_team, 0, abort_ptr + 1);
 }
 
 // Softmax threads (all 256 of the block, whole warps).  Live ones store their row of the block's piece --
 // unnormalised O from TMEM at t_o if the block had key tiles, and (m, l), which is (-inf, 0) if it had none
-// (that piece's O is then never read).  Then all wait for the publisher's fetch and reduce this block's share of
-// the unit's output vectors over the C pieces, in rank order.  Returns false when a wait was given up.
+// (that piece's O is then never read).  Then all wait for the team and reduce this block's share of
+// the unit's output vectors over the C pieces, in rank order.  A thread's vectors lie in one row of an M tile, whose weights it takes
+// once, and what it needs of up to kMax pieces it asks L2 for at once: one round trip for the weights and the first vectors, one
+// for each further pair or single vector.  (Bulk copies of the shares into shared memory, 2 C of them issued by one lane, took 2400 -
+// 2900 cycles until they had landed, and the reduction from there 1400 - 6000.)  Returns false when a wait was given up.
+template <int D, bool kNoWait, int kMax>
+__device__ __forceinline__ void team_reduce(const TeamArgs& p) {
+  constexpr int kVec = 16 / kMax;             // vectors in flight
+  const int kVecs = (D / 4) << p.r_shift, R = 1 << p.r_shift;   // vectors of one M tile's piece
+  const int tid = threadIdx.x, C = p.team;
+  const int row = (p.lo + tid) & (R - 1);     // 256 is a multiple of R
+  const float4* const o = reinterpret_cast<const float4*>(p.ws_o) + ((p.piece0 * (D / 4)) << p.r_shift);
+  const size_t piece = (size_t)kVecs * p.n_mt;
+  int mt = -1;
+  bool real = false, active = false;
+  float w[kMax], m_all = 0.f, l_all = 0.f, inv = 0.f;
+  size_t qrow = 0;
+  for (int i = p.lo + tid; i < p.hi; i += 256 * kVec) {
+    float4 x[kVec][kMax];
+#pragma unroll
+    for (int u = 0; u < kVec; ++u)
+#pragma unroll
+      for (int c = 0; c < kMax; ++c)
+        if (c < C && i + 256 * u < p.hi) x[u][c] = __ldcg(o + c * piece + i + 256 * u);
+#pragma unroll
+    for (int u = 0; u < kVec; ++u) {
+      const int iu = i + 256 * u, mt_i = iu >= kVecs ? 1 : 0, qd = (iu - mt_i * kVecs) >> p.r_shift;
+      if (iu >= p.hi) break;
+      if (mt_i != mt) {
+        mt = mt_i;
+        const int r_unit = mt * 128 + row, r_kv = p.r0 + r_unit;
+        real = r_unit < ((p.rows + 31) & ~31) && r_kv < p.rows_total;
+        qrow = p.qrow0 + r_kv;                // rows of a KV head's query heads lie one after the other
+        int ir;
+        p.by_q_cap.divmod(r_kv, ir);
+        active = ir < p.Lq;
+        const float2* const a_ml = reinterpret_cast<const float2*>(p.ws_ml) + ((p.piece0 + mt) << p.r_shift) + row;
+        float2 ml[kMax];
+#pragma unroll
+        for (int c = 0; c < kMax; ++c) ml[c] = c < C && real ? __ldcg(a_ml + (((size_t)c * p.n_mt) << p.r_shift)) : make_float2(-CUDART_INF_F, 0.f);
+        m_all = -CUDART_INF_F;
+#pragma unroll
+        for (int c = 0; c < kMax; ++c)
+          if (ml[c].y > 0.f) m_all = fmaxf(m_all, ml[c].x);
+        l_all = 0.f;
+#pragma unroll
+        for (int c = 0; c < kMax; ++c) {
+          w[c] = ml[c].y > 0.f ? ex2_approx(ml[c].x - m_all) : 0.f;
+          l_all = fmaf(w[c], ml[c].y, l_all);
+        }
+        inv = active ? 1.f / l_all : 0.f;
+      }
+      if (!real) continue;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < kMax; ++c) {
+        if (c < C && w[c] != 0.f) {           // a piece without keys holds no O
+          acc.x = fmaf(w[c], x[u][c].x, acc.x);
+          acc.y = fmaf(w[c], x[u][c].y, acc.y);
+          acc.z = fmaf(w[c], x[u][c].z, acc.z);
+          acc.w = fmaf(w[c], x[u][c].w, acc.w);
+        }
+      }
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(active ? acc.x * inv : 0.f, active ? acc.y * inv : 0.f);
+      const __nv_bfloat162 h1 = __floats2bfloat162_rn(active ? acc.z * inv : 0.f, active ? acc.w * inv : 0.f);
+      *reinterpret_cast<uint2*>(p.out + qrow * D + qd * 4) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+      if (qd == 0 && p.lse) p.lse[qrow] = active ? (m_all + lg2_approx(l_all)) * 0.6931471805599453f : -CUDART_INF_F;
+    }
+  }
+}
+
 template <int D, bool kNoWait>
-__device__ __noinline__ bool team_exchange(const TeamArgs p, uint32_t sm_q, uint32_t bar_pub,
-                                           volatile int* abort_ptr, bool live, uint32_t t_o, bool has_tiles, float m_used, float l_run) {
+__device__ __noinline__ bool team_exchange(const TeamArgs p, uint32_t bar_pub, volatile int* abort_ptr, bool live, uint32_t t_o,
+                                           bool has_tiles, float m_used, float l_run) {
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
-  constexpr int kVecs = D / 4 * 128;          // vectors of one M tile's piece
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int mt = warp >> 2, row = tid & 127;
-  const int n_live = (p.rows + 31) & ~31;
-  const uint32_t bar_team = bar_pub + 8;
-  const int C = p.team;
+  const int tid = threadIdx.x, mt = tid >> 7, row = tid & 127;
   if (live) {
     const size_t mine = p.piece0 + (size_t)p.rank * p.n_mt + mt;
     if (has_tiles) {
-      float4* po = reinterpret_cast<float4*>(p.ws_o) + mine * (size_t)kVecs + row;
+      float4* po = reinterpret_cast<float4*>(p.ws_o) + ((mine * (D / 4)) << p.r_shift) + row;
       uint32_t v[32];
 #pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
@@ -360,55 +408,17 @@ __device__ __noinline__ bool team_exchange(const TeamArgs p, uint32_t sm_q, uint
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          __stcg(po + (c * 8 + j) * 128, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                     __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
+          __stcg(po + ((c * 8 + j) << p.r_shift), make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                              __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
       }
     }
-    __stcg(reinterpret_cast<float2*>(p.ws_ml) + mine * 128 + row, make_float2(m_used, l_run));
+    __stcg(reinterpret_cast<float2*>(p.ws_ml) + (mine << p.r_shift) + row, make_float2(m_used, l_run));
     // no fence here: the arrival below orders the stores before the publisher's wait (block scope), and the
     // publisher's fence before it counts the block in carries them to device scope
     mbar_arrive(bar_pub);
   }
-  if (__all_sync(0xffffffffu, mbar_wait_limit(bar_team, 0, abort_ptr, kLimit)) == 0) return false;
-  const uint32_t sm_ml = sm_q, sm_o = sm_q + C * p.ml_bytes;
-  for (int i = p.lo + tid; i < p.hi; i += 256) {
-    const int mt_i = i / kVecs, rem = i % kVecs, qd = rem / 128, row_i = rem % 128;
-    const int r_unit_i = mt_i * 128 + row_i;
-    const int r_kv_i = p.r0 + r_unit_i;
-    if (r_unit_i >= n_live || r_kv_i >= p.rows_total) continue;
-    int ir;
-    p.by_q_cap.divmod(r_kv_i, ir);
-    const size_t qrow_i = p.qrow0 + r_kv_i;                // rows of a KV head's query heads lie one after the other
-    const bool active_i = ir < p.Lq;
-    const uint32_t a_ml = sm_ml + (uint32_t)r_unit_i * 8u, a_o = sm_o + (uint32_t)(i - p.lo) * 16u;
-    float m_all = -CUDART_INF_F;
-#pragma unroll 4
-    for (int c = 0; c < C; ++c) {
-      const float2 ml = ld_shared_f2(a_ml + c * p.ml_bytes);
-      if (ml.y > 0.f) m_all = fmaxf(m_all, ml.x);
-    }
-    float l_all = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int c = 0; c < C; ++c) {
-      const float2 ml = ld_shared_f2(a_ml + c * p.ml_bytes);
-      const float4 x = ld_shared_f4(a_o + c * p.o_bytes);
-      if (ml.y > 0.f) {   // a piece without keys holds no O
-        const float w = ex2_approx(ml.x - m_all);
-        l_all = fmaf(w, ml.y, l_all);
-        acc.x = fmaf(w, x.x, acc.x);
-        acc.y = fmaf(w, x.y, acc.y);
-        acc.z = fmaf(w, x.z, acc.z);
-        acc.w = fmaf(w, x.w, acc.w);
-      }
-    }
-    const float inv = active_i ? 1.f / l_all : 0.f;
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(active_i ? acc.x * inv : 0.f, active_i ? acc.y * inv : 0.f);
-    const __nv_bfloat162 h1 = __floats2bfloat162_rn(active_i ? acc.z * inv : 0.f, active_i ? acc.w * inv : 0.f);
-    *reinterpret_cast<uint2*>(p.out + qrow_i * D + qd * 4) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-    if (qd == 0 && p.lse) p.lse[qrow_i] = active_i ? (m_all + lg2_approx(l_all)) * 0.6931471805599453f : -CUDART_INF_F;
-  }
+  if (!mbar_wait_warp(bar_pub + 8, 0, abort_ptr, kLimit)) return false;
+  if (p.team <= 8) team_reduce<D, kNoWait, 8>(p); else team_reduce<D, kNoWait, 16>(p);
   __syncwarp();
   return true;
 }
@@ -651,8 +661,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t bar_pv_done = bar_p_ready + 32;                 // [M tile][half-step parity] P V product finished.  Two P V
                                                                  // products can be in flight, so consecutive half-steps use different
                                                                  // barriers: a parity wait cannot tell phases two apart
-  const uint32_t bar_pub = sm_bar + kBarPub;                     // partial result of a segment stored by every softmax thread
-  const uint32_t bar_team = bar_pub + 8;                         // team schedule: the team's pieces of this block's share have landed
+  const uint32_t bar_pub = bar_pv_done + 32;                   // partial result of a segment stored by every softmax thread
+  const uint32_t bar_team = bar_pub + 8;                         // team schedule: the whole team's pieces are there
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // softmax threads that own a real query row, rounded up to whole warps (they are tid 0 .. n_live-1)
@@ -983,7 +993,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         read_lengths();
       }
       if (kSingle && lane == 0 && p.team > 1) {
-        team_publish<D, kNoWait>(TeamArgs(p, one, D), sm_q, bar_pub, abort_ptr);
+        team_publish<kNoWait>(TeamArgs(p, one, D), bar_pub, abort_ptr);
       } else if (!kSingle && lane == 0 && has_work && !p.whole_units) {
         SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
         Segment g = one;
@@ -1049,7 +1059,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             if (g.T == 0) {
               zero_my_row(out_row_of(g.lc_layer, g.b, g.kvh, g.rc), g.rc * kChunk + r_unit < p.rows_total);
             } else if (kSingle && p.team > 1) {   // a piece without key tiles
-              ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), sm_q, bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
+              ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
             }
             continue;
           }
@@ -1109,7 +1119,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const bool active = real_row && r_kv - p.by_q_cap.div(r_kv) * p.q_cap < g.Lq;
           uint32_t v[32];
           if (kSingle && p.team > 1) {
-            ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), sm_q, bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
+            ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
           } else if (kSingle || g.slot < 0) {
             const float inv = active ? 1.f / l_run : 0.f;
 #pragma unroll 1
@@ -1242,7 +1252,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     } else if (kSingle && p.team > 1) {
       // warps without a row of their own help with the reduction
       const TeamArgs ta(p, one, D);
-      if (ta.has_keys) team_exchange<D, kNoWait>(ta, sm_q, bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
+      if (ta.has_keys) team_exchange<D, kNoWait>(ta, bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
     }
   }
   // ---- teardown: nothing of this block is in flight any more
@@ -1271,11 +1281,12 @@ bool register_budget_ok(const cudaFuncAttributes& a) {
   return a.numRegs >= kRegsOther && 8 * (kRegsSoftmax - a.numRegs) <= 4 * (a.numRegs - kRegsOther);
 }
 
-// The sixteen instantiations: head_dim 128 / 64, row chunks of 256 / 128, normal / no-wait (test) waits, blocks of any number of
-// segments / of one.
+// The instantiations: head_dim 128 / 64, row chunks of 256 / 128, normal / no-wait (test) waits, blocks of any number of
+// segments / of one; and chunks of 64 for teams.
 using AttnKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                             const AttnParams);
 inline int kernel_index(int head_dim, const dlm_attn_plan& pl, bool no_wait) {
+  if (pl.chunk_rows == 64) return 16 + (head_dim == 128 ? 0 : 1) + (no_wait ? 2 : 0);
   return (head_dim == 128 ? 0 : 1) + (pl.chunk_rows == 256 ? 0 : 2) + (no_wait ? 4 : 0) + (pl.single ? 8 : 0);
 }
 template <bool kSingle>
@@ -1291,7 +1302,15 @@ AttnKernel kernel_of(int which) {
     default: return attn_step_sm100_kernel<64, 128, kSingle, true>;
   }
 }
-AttnKernel kernel_of(int which) { return which & 8 ? kernel_of<true>(which) : kernel_of<false>(which); }
+AttnKernel kernel_of(int which) {
+  switch (which) {
+    case 16: return attn_step_sm100_kernel<128, 64, true, false>;
+    case 17: return attn_step_sm100_kernel<64, 64, true, false>;
+    case 18: return attn_step_sm100_kernel<128, 64, true, true>;
+    case 19: return attn_step_sm100_kernel<64, 64, true, true>;
+    default: return which & 8 ? kernel_of<true>(which) : kernel_of<false>(which);
+  }
+}
 
 // First use of an attention kernel on a context's device: checks the register budget and opts in to
 // all the dynamic shared memory the device allows a block (less the kernel's static part).
@@ -1332,14 +1351,16 @@ WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int 
 }
 
 // Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer), fitted to measurements of one-layer
-// calls (Dream heads, 1024 - 1152 cached rows; us):    team of 9, 1 tile, one M tile       10.6
-//   256 active rows: team of 5, 2 tiles, two M tiles   18.3     team of 2, 5 tiles, one M tile  19.1     split  23.4
-//   8 sequences:     team of 4, 3 tiles, two M tiles   20.3     team of 2, 5 tiles, one M tile  19.4     split  23.8
-// Heads of 64, which were not in the fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule,
-// the choice is the fastest or within 2 % of it.  The same calls with heads of 128: within 2 % but one (64 units of 9 tiles,
-// one M tile: team of 2 19.6 us, split over 128 blocks 18.2).
+// calls (Dream heads, 1024 - 1152 cached rows; us):    team of 9, 1 tile, 128 rows         9.4     of 64 rows              9.0
+//   256 active rows: team of 5, 2 tiles, two M tiles   16.4    team of 2, 5 tiles, one M tile  18.3     split  23.4
+//   8 sequences:     team of 4, 3 tiles, two M tiles   18.4    team of 2, 5 tiles, one M tile  16.9     split  23.8
+// and of 15 more (300 - 4096 cached rows, 16 - 256 active, 1 - 8 sequences, four models' heads) under four sets of team costs: this set has the
+// fastest or one within 1 % everywhere; with the exchange dearer (1.8, 2.3, 4.3) 2 sequences of 32 heads at 3000 rows were dealt
+// whole, 29.1 us instead of 24.9, with 128 rows as cheap as 64 one sequence took 9.4 instead of 9.0 (300 rows: 8.9, 7.9).
+// Heads of 64, which were not in the fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule with
+// the costs before these, the choice was the fastest or within 2 % of it.
 constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer
-constexpr double kTeamCost[2] = {2.3, 4.3};      // the team schedule's exchange and reduction
+constexpr double kTeamCost[3] = {1.4, 1.8, 3.6};      // the team schedule's exchange and reduction, for 64 / 128 / 256 rows
 constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...
 constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond that
 // With more units than SMs a block has whole units to compute while its first piece travels, and merges one unit at most.
@@ -1386,7 +1407,7 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
     if (C > 1) {
       const long long per_block = (tiles_unit + C - 1) / C;
       C = (tiles_unit + per_block - 1) / per_block;
-      const double t = (double)per_block * tile + kTeamCost[pl.n_mt - 1];
+      const double t = (double)per_block * tile + kTeamCost[pl.rows <= 64 ? 0 : pl.n_mt];
       if (C > 1 && (t < best || ctx->attn_team_force)) {
         best = t;
         pl.team = (int)C;
@@ -1400,16 +1421,21 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
 
 // Row chunks of 256 (two M tiles sharing every K/V tile) read K/V once per KV head and cost little more per key tile than
 // chunks of 128; those double the units that can be spread over the SMs and halve every partial result, the second read of
-// K/V coming from L2.  Whichever schedule of either has the least estimated cost, from the caller's cache length hint.
+// K/V coming from L2.  Chunks of 64, half an M tile, halve the partial results once more: for teams only, whose exchange is
+// half of a short call.  Whichever schedule of any has the least estimated cost, from the caller's cache length hint.
 Plan make_plan(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int cache_len_hint) {
   const int len = (cache_len_hint > 0 && cache_len_hint < cache->capacity) ? cache_len_hint : cache->capacity;
   Plan pl, narrow;
-  const double cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 256, pl);
+  double cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 256, pl);
   if (pl.n_mt == 2) {
     const double narrow_cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 128, narrow);
     // (a forced team schedule counts as the better one)
     const bool forced_apart = ctx->attn_team_force && (narrow.team > 1) != (pl.team > 1);
-    if (forced_apart ? narrow.team > 1 : narrow_cost < cost) pl = narrow;
+    if (forced_apart ? narrow.team > 1 : narrow_cost < cost) { pl = narrow; cost = narrow_cost; }
+  }
+  if (pl.rows > 64) {
+    const double slim_cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 64, narrow);
+    if (narrow.team > 1 && slim_cost < cost && !ctx->attn_team_force) pl = narrow;
   }
   pl.single = pl.whole_units && (pl.team > 1 || (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc <= pl.grid);
   const WorkspaceSize ws = workspace_size(ctx, cache, nl, n_q_heads, q_cap);

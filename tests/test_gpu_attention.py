@@ -422,3 +422,17 @@ def test_whole_units_as_many_as_sms_and_more(dev, oracle, B, Hkv, group, D, q_ca
         out, lse, _ = _case(dev, oracle, 1, B, Hkv * group, Hkv, D, 200, q_cap, cl, ql, seed=B, hint=hint)
     for b in np.flatnonzero(ql == 0):
         assert not out[0, b].any() and bool((lse[0, b] == -float("inf")).all())
+
+
+# teams on row chunks of 64: a ragged last chunk, inactive rows and an inactive element, blocks without a key tile, both head sizes
+@pytest.mark.parametrize("B,Hq,Hkv,D,Lcap,q_cap,cache_len,q_len", [
+    (1, 28, 4, 128, 1100, 32, [1024], None),
+    (1, 28, 4, 128, 1100, 32, [500], [9]),
+    (2, 9, 3, 64, 700, 24, [700, 3], [24, 0]),
+    (1, 5, 1, 128, 1990, 13, [1500], None),
+])
+def test_teams_of_half_m_tiles(dev, oracle, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len):
+    sch = _schedule(dev, 2, B, Hq, Hkv, D, Lcap, q_cap, 1, max(cache_len))
+    assert sch["team"] > 1 and sch["chunk_rows"] == 64, sch
+    for _ in range(2):   # and leave the counters clean
+        _case(dev, oracle, 2, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len, seed=Hq, layer_begin=1, hint=max(cache_len))

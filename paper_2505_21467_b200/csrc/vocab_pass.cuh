@@ -14,7 +14,7 @@
 // and identical rows give identical bits.
 //
 // A chunk's statistics (Entry) go to the workspace; the last block of a batch element to finish (a release-acquire ticket)
-// merges that element's entries, eight lanes per row, and ranks the positions.
+// merges that element's entries, eight or four lanes per row, and ranks the positions.
 #pragma once
 
 #include <math_constants.h>
@@ -291,7 +291,7 @@ __device__ __forceinline__ void reduce_chunk(const float* __restrict__ z, int be
 
 // ---- selection for batch element b by the whole block
 struct SelectScratch {
-  float key[kMaxBlockLen];     // ranking score; meaningless where `on` is 0
+  float key[kMaxBlockLen];     // ranking score; NaN where `on` is 0
   int32_t tok[kMaxBlockLen];
   uint8_t on[kMaxBlockLen];
   uint32_t sel[kMaxBlockLen / 32];
@@ -306,39 +306,35 @@ __device__ __forceinline__ float score_of(const Args& a, int score_kind, size_t 
   return a.noise[pos] - __logf(s);
 }
 
-template <int KIND>
-__device__ void select_batch(const Args& a, int score_kind, int b, SelectScratch& sc) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int L = a.block_len, k = a.k;
-  const size_t p0 = (size_t)b * L;
-  if (tid < kMaxBlockLen / 32) sc.sel[tid] = 0;
-  if (tid == 0) sc.n_on = 0;
-  // (1) eight lanes per row merge the row's entries (lanes over chunks, fixed shuffle tree), so that a warp does four rows at
-  // once and the block 32: one round trip to L2 and one pass through this code for a block of 32 positions.  The entries are
-  // asked for beside the mask byte (a row that is not masked has stale ones, which are then ignored).
-  const int sub = lane & 7;
-  for (int i0 = warp * 4; i0 < L; i0 += kWarps * 4) {
-    const int i = i0 + (lane >> 3);
+// (1) of the selection: LANES lanes per row merge the row's entries (lanes over chunks, fixed shuffle tree), 32 / LANES rows a warp,
+// KEEP entries a lane in registers (further ones are read twice).  The entries are asked for beside the mask byte (a row that
+// is not masked has stale ones, which are then ignored).
+template <int KIND, int LANES, int KEEP>
+__device__ __forceinline__ void merge_rows(const Args& a, int score_kind, size_t p0, SelectScratch& sc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & (LANES - 1), L = a.block_len;
+  constexpr int kRows = 32 / LANES;
+#pragma unroll 1
+  for (int i0 = warp * kRows; i0 < L; i0 += kWarps * kRows) {
+    const int i = i0 + lane / LANES;
     const size_t p = p0 + min(i, L - 1);
     const bool on = i < L && __ldcg(a.masked + p) != 0;
     const float4* e = reinterpret_cast<const float4*>(a.entries + p * a.n_chunks);
-    constexpr int kKeep = 3;   // entries a lane keeps in registers (rows of up to 24 chunks); further ones are read twice
-    float4 v[kKeep];
+    float4 v[KEEP];
 #pragma unroll
-    for (int h = 0; h < kKeep; ++h) {
-      const int c = sub + 8 * h;
+    for (int h = 0; h < KEEP; ++h) {
+      const int c = sub + LANES * h;
       v[h] = c < a.n_chunks ? __ldcg(e + c) : make_float4(-CUDART_INF_F, __int_as_float(0x7fffffff), 0.f, KIND == kMargin ? -CUDART_INF_F : 0.f);
     }
     float m = v[0].x, m2 = v[0].w;
     int idx = __float_as_int(v[0].y);
 #pragma unroll
-    for (int h = 1; h < kKeep; ++h) merge_max<KIND>(m, idx, m2, v[h].x, __float_as_int(v[h].y), v[h].w);
-    for (int c = sub + 8 * kKeep; c < a.n_chunks; c += 8) {
+    for (int h = 1; h < KEEP; ++h) merge_max<KIND>(m, idx, m2, v[h].x, __float_as_int(v[h].y), v[h].w);
+    for (int c = sub + LANES * KEEP; c < a.n_chunks; c += LANES) {
       const float4 w = __ldcg(e + c);
       merge_max<KIND>(m, idx, m2, w.x, __float_as_int(w.y), w.w);
     }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
+    for (int o = LANES / 2; o > 0; o >>= 1) {
       const float om = __shfl_xor_sync(0xffffffffu, m, o);
       const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
       const float o2 = KIND == kMargin ? __shfl_xor_sync(0xffffffffu, m2, o) : 0.f;
@@ -352,10 +348,10 @@ __device__ void select_batch(const Args& a, int score_kind, int b, SelectScratch
       if (KIND == kEntropy) x += tw;
     };
 #pragma unroll
-    for (int h = 0; h < kKeep; ++h) take(v[h]);
-    for (int c = sub + 8 * kKeep; c < a.n_chunks; c += 8) take(__ldcg(e + c));
+    for (int h = 0; h < KEEP; ++h) take(v[h]);
+    for (int c = sub + LANES * KEEP; c < a.n_chunks; c += LANES) take(__ldcg(e + c));
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
+    for (int o = LANES / 2; o > 0; o >>= 1) {
       s += __shfl_xor_sync(0xffffffffu, s, o);
       if (KIND == kEntropy) x += __shfl_xor_sync(0xffffffffu, x, o);
     }
@@ -365,46 +361,45 @@ __device__ void select_batch(const Args& a, int score_kind, int b, SelectScratch
       a.tok[p] = on ? idx : -1;
       a.conf[p] = on ? 1.0f / s : -1.f;
       if (a.score) { a.score[p] = score; a.zmax[p] = on ? m : 0.f; }
-      sc.key[i] = score;
+      sc.key[i] = on ? score : CUDART_NAN_F;
       sc.tok[i] = idx;
       sc.on[i] = on;
     }
   }
+}
+
+template <int KIND, bool WIDE>
+__device__ __forceinline__ void select_batch(const Args& a, int score_kind, int b, SelectScratch& sc) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int L = a.block_len, k = a.k;
+  const size_t p0 = (size_t)b * L;
+  if (tid < kMaxBlockLen / 32) sc.sel[tid] = 0;
+  if (tid == 0) sc.n_on = 0;
+  // Up to 32 positions are one pass of eight lanes a row, one round trip to L2; more (WIDE) take four lanes a row, 64 rows a pass
+  // (4 x 64 positions of 6 chunks, a block's life with two passes of eight lanes: 346 us, now 313).  Which one is the kernel's, not a
+  // branch: this code runs once, and what it holds beside what it needs costs fetches and the streaming loop registers.
+  if (!WIDE) merge_rows<KIND, 8, 3>(a, score_kind, p0, sc); else merge_rows<KIND, 4, 5>(a, score_kind, p0, sc);
   if (k <= 0) return;
   __syncthreads();
-  // (2) rank among the masked positions: (score desc, position asc)
-  if (L <= 32) {   // one warp, a position per lane
-    if (warp != 0) return;
-    const bool on = lane < L && sc.on[lane];
-    const unsigned all = __ballot_sync(0xffffffffu, on);
-    const float mine = on ? sc.key[lane] : 0.f;
+  // (2) rank among the masked positions: (score desc, position asc).  Eight lanes a position, each comparing it with every eighth
+  // one (a position that is not masked has a NaN, which outranks nothing).  (One warp with 32 unrolled shuffles for up to 32
+  // positions, one thread a position for more: 2900 and 5000 - 10000 cycles behind the merge, most of it code seen for the
+  // first time and a serial chain; now 1500.)
+#pragma unroll 1
+  for (int i0 = warp * 4; i0 < L; i0 += kWarps * 4) {
+    const int i = i0 + (lane >> 3), first = lane & 7;
+    const float mine = sc.key[min(i, L - 1)];
     int rank = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float sj = __shfl_sync(0xffffffffu, mine, j);
-      rank += ((all >> j) & 1u) && (sj > mine || (sj == mine && j < lane)) ? 1 : 0;
-    }
-    const unsigned chosen = __ballot_sync(0xffffffffu, on && rank < k);
-    const int order = __popc(chosen & ((1u << lane) - 1u)), count = min(k, __popc(all));
-    if (((chosen >> lane) & 1u) && order < k) {   // more than k only with NaN scores
-      a.sel_idx[(size_t)b * k + order] = lane;
-      a.tokens[p0 + lane] = sc.tok[lane];
-      a.masked[p0 + lane] = 0;
-    }
-    for (int j = count + lane; j < k; j += 32) a.sel_idx[(size_t)b * k + j] = -1;
-    if (lane == 0) a.n_sel[b] = count;
-    return;
-  }
-  for (int i = tid; i < L; i += kThreads) {
-    if (!sc.on[i]) continue;
-    atomicAdd(&sc.n_on, 1);
-    const float mine = sc.key[i];
-    int rank = 0;
-    for (int j = 0; j < L; ++j) {
+    for (int j = first; j < L; j += 8) {
       const float sj = sc.key[j];
-      rank += sc.on[j] && (sj > mine || (sj == mine && j < i)) ? 1 : 0;
+      rank += sj > mine || (sj == mine && j < i) ? 1 : 0;
     }
-    if (rank < k) atomicOr(&sc.sel[i >> 5], 1u << (i & 31));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (first == 0 && i < L && sc.on[i]) {
+      atomicAdd(&sc.n_on, 1);
+      if (rank < k) atomicOr(&sc.sel[i >> 5], 1u << (i & 31));
+    }
   }
   __syncthreads();
   for (int i = tid; i < L; i += kThreads) {
@@ -422,7 +417,7 @@ __device__ void select_batch(const Args& a, int score_kind, int b, SelectScratch
 }
 
 // ---- kernels
-template <int KIND, bool VEC>
+template <int KIND, bool VEC, bool WIDE>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm) vocab_pass_kernel(const __grid_constant__ Args a, int score_kind) {
   __shared__ SelectScratch scratch;
   __shared__ bool is_last;
@@ -462,16 +457,16 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) vocab_pass_kernel(cons
     if (is_last) a.tickets[b] = 0;   // ready for the next launch
   }
   __syncthreads();
-  if (is_last) select_batch<KIND>(a, score_kind, b, scratch);
+  if (is_last) select_batch<KIND, WIDE>(a, score_kind, b, scratch);
 }
 
 // The selection as a kernel of its own, one block per batch element (no tickets).
-template <int KIND>
+template <int KIND, bool WIDE>
 __global__ void __launch_bounds__(kThreads) vocab_select_kernel(const __grid_constant__ Args a, int score_kind) {
   __shared__ SelectScratch scratch;
   dlm_grid_dependency_wait();
   dlm_trigger_dependents();
-  select_batch<KIND>(a, score_kind, blockIdx.x, scratch);
+  select_batch<KIND, WIDE>(a, score_kind, blockIdx.x, scratch);
 }
 
 // Chunks of 1 .. 8 batches: about two resident waves of blocks, so that the last ones to run find the memory busy, but no
@@ -491,17 +486,22 @@ inline void plan_chunks(Args& a, int num_sms) {
   a.by_block_len = make_fast_div(a.block_len);
 }
 
-template <int KIND>
-inline int launch_kind(Args& a, int score_kind, int batch, int num_sms, cudaStream_t s) {
+template <int KIND, bool WIDE>
+inline int launch_sized(Args& a, int score_kind, int batch, int num_sms, cudaStream_t s) {
   plan_chunks(a, num_sms);
   const bool vec = a.vocab % 4 == 0 && ((uintptr_t)a.logits & 15) == 0;
   const dim3 grid(a.n_chunks, a.rows);
-  const cudaError_t e = vec ? dlm_launch(vocab_pass_kernel<KIND, true>, grid, dim3(kThreads), 0, s, a, score_kind)
-                            : dlm_launch(vocab_pass_kernel<KIND, false>, grid, dim3(kThreads), 0, s, a, score_kind);
+  const cudaError_t e = vec ? dlm_launch(vocab_pass_kernel<KIND, true, WIDE>, grid, dim3(kThreads), 0, s, a, score_kind)
+                            : dlm_launch(vocab_pass_kernel<KIND, false, WIDE>, grid, dim3(kThreads), 0, s, a, score_kind);
   if (e != cudaSuccess) return -1;
   if (a.tickets != nullptr) return 1;
-  if (dlm_launch(vocab_select_kernel<KIND>, dim3(batch), dim3(kThreads), 0, s, a, score_kind) != cudaSuccess) return -1;
+  if (dlm_launch(vocab_select_kernel<KIND, WIDE>, dim3(batch), dim3(kThreads), 0, s, a, score_kind) != cudaSuccess) return -1;
   return 2;
+}
+
+template <int KIND>
+inline int launch_kind(Args& a, int score_kind, int batch, int num_sms, cudaStream_t s) {
+  return a.block_len > 32 ? launch_sized<KIND, true>(a, score_kind, batch, num_sms, s) : launch_sized<KIND, false>(a, score_kind, batch, num_sms, s);
 }
 
 }  // namespace vocab

@@ -55,3 +55,13 @@ def test_tickets_of_few_masked_rows(dev, oracle, L):
     for _ in range(2):
         for k in (0, 1, 3):
             assert any(_compare_scored(dev, oracle, make_logits(4, L, 9001, (0.5, 6.0), 50 * L + seed), masked0, k, 0) for seed in range(12))
+
+
+# more than 32 positions are merged by four lanes a row, which hold 20 chunks: exactly that many, one more, and more than a pass of 64 rows
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("L,V", [(40, 163840), (40, 163841), (65, 98304), (130, 9000)])
+def test_merge_of_long_blocks(dev, oracle, L, V, kind):
+    masked0 = make_mask(1, L, L - 3, V).numpy()
+    masked0[0, :5] = 1
+    assert any(_compare_scored(dev, oracle, _inputs(1, L, V, L + V + seed), masked0, k, kind) for k in (0, 3) for seed in range(6))
+    assert _compare_scored(dev, oracle, _inputs(1, L, V, L + V), masked0, 0, kind)

@@ -18,7 +18,8 @@
 //               64-column score buffers in TMEM, two half-steps ahead of the softmax; then
 //               O += P V with P read from TMEM (it overwrites S in place as packed bf16)
 //   warp  11    publisher (one lane): makes a finished partial result visible device-wide and
-//               bumps its unit's counter, so the softmax warps need not wait for that
+//               bumps its unit's counter, so the softmax warps need not wait for that; teams: tells
+//               them when the whole team has
 // Online softmax in fp32 with base-2 exponentials; a half-step's scores sit in registers; O stays
 // in TMEM and is rescaled only when a row's scores have outgrown the maximum in use by a lot.
 //

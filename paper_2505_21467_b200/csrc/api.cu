@@ -25,6 +25,7 @@ extern "C" int dlm_create(dlm_ctx** out, int device) {
   ctx->maps = new (std::nothrow) dlm_map_cache();
   ctx->commit_blocks_per_sm[0] = ctx->commit_blocks_per_sm[1] = 0;
   for (int& limit : ctx->attn_smem_limit) limit = 0;
+  for (int& n : ctx->attn_clusters) n = 0;
   ctx->proj_configured = 0;
   memset(&ctx->attn_plan_key, 0, sizeof ctx->attn_plan_key);
   ctx->wait_limit_ns = sm100::kWaitLimitNs;

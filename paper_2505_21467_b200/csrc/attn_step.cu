@@ -6,7 +6,7 @@
 // query heads of a KV head, q_cap rows each, are cut into chunks of 256 rows = two 128-row M
 // tiles that share every K/V tile (at the block sizes of the configs, g * q_cap <= 256: one chunk,
 // K/V read from HBM once per KV head; larger windows re-read them per chunk, normally from L2;
-// calls with very few units use chunks of 128 rows, one M tile, to have more units to spread).
+// calls with few units use chunks of 128 rows or fewer, one M tile, to have more units to spread).
 // Keys are loaded in tiles of 128 rows, first the visible cache rows, then the fresh rows, and
 // processed in half-steps of 64.
 //
@@ -18,8 +18,7 @@
 //               64-column score buffers in TMEM, two half-steps ahead of the softmax; then
 //               O += P V with P read from TMEM (it overwrites S in place as packed bf16)
 //   warp  11    publisher (one lane): makes a finished partial result visible device-wide and
-//               bumps its unit's counter, so the softmax warps need not wait for that; teams: tells
-//               them when the whole team has
+//               bumps its unit's counter, so the softmax warps need not wait for that
 // Online softmax in fp32 with base-2 exponentials; a half-step's scores sit in registers; O stays
 // in TMEM and is rescaled only when a row's scores have outgrown the maximum in use by a lot.
 //
@@ -32,6 +31,10 @@
 // results (they have lower block indices and computed those pieces first), then folds them into
 // its own O, which is still in TMEM, in block order: the result is deterministic.  When the split
 // would cost more than it saves (the host estimates both) units are dealt whole, round-robin.
+// Calls with few units give each unit a team: a thread-block cluster that deals the unit's key tiles among its blocks and
+// exchanges the partial results through the blocks' shared memory (team_share and below).  A team's block with one M tile
+// has a chain of warps to spare, so it splits the keys: warps 0-3 and issuer 9 take the first 64 keys of every tile, warps 4-7
+// and issuer 10 the others, each half with an O, maximum and sum of its own.
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -55,6 +58,7 @@ constexpr int kMaxGrid = 256;          // blocks of the persistent grid (one per
 constexpr int kMaxStages = 8;          // barrier slots reserved per ring
 constexpr int kBarrierBytes = 512;     // mbarriers of a block
 constexpr int kFlagBytes = 64;         // abort / never flags, TMEM slot, merge flag
+constexpr int kFoldBytes = 2 * 128 * 8;   // (running max, running sum) of every row of the two key halves
 
 template <int D>
 struct Geometry {
@@ -86,7 +90,7 @@ struct AttnParams {
   int team;        // > 1 (with whole_units): blocks [u * team, (u + 1) * team) share unit u, key tiles dealt by rank;
                    // every block then reduces its share of the unit's outputs over all the team's pieces
   int smem_bytes;           // dynamic shared memory of the launch
-  FastDiv by_batch, by_rc, by_kv_heads, by_q_cap, by_team;
+  FastDiv by_batch, by_rc, by_kv_heads, by_q_cap, by_team, by_live;
   float scale_log2;
   int* status;
   unsigned int* tickets;   // one zero-initialised counter per unit: pieces finished
@@ -261,167 +265,143 @@ __device__ __forceinline__ bool wait_counter(const unsigned int* addr, unsigned 
   }
 }
 
-// Team schedule: what a block of a team works on after its share of the key tiles.  The team's pieces lie
-// in the workspace as [rank][M tile][head_dim / 4][R rows] 16-byte vectors (4 columns of a row) and
-// [rank][M tile][R rows] (m, l) pairs, R the unit's rows in an M tile rounded up to 32, 64 or 128; the unit's n_mt * head_dim / 4 * R
-// output vectors are dealt to the ranks in that storage order, rank r reducing vectors [lo, hi) over all pieces.
-// Everything the exchange needs, decoded by the caller and handed over by value.
-struct TeamArgs {
-  __nv_bfloat16* out;
-  float* lse;
-  float* ws_o;
-  float* ws_ml;
-  unsigned int* arrive;        // the unit's two counters: blocks that have stored their piece ...
-  unsigned int* depart;        // ... and blocks that are past their wait for the first
-  size_t piece0;               // index of the team's first piece
-  size_t qrow0;                // output row of the KV head's first query row
-  FastDiv by_q_cap;
-  int team, n_mt, rows, rows_total, rank, Lq;
-  bool has_keys;
-  int r0, lo, hi;              // r0: the row chunk's first row among the KV head's rows
-  int r_shift;                 // log2 R
-  __device__ __forceinline__ TeamArgs(const AttnParams& p, const Segment& g, int D)
-      : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), by_q_cap(p.by_q_cap), team(p.team), n_mt(p.n_mt), rows(p.rows),
-        rows_total(p.rows_total), Lq(g.Lq), has_keys(g.T > 0) {
-    const int unit = p.by_team.divmod(blockIdx.x, rank);
-    r0 = g.rc * p.chunk_rows;
-    qrow0 = (((size_t)g.lc_layer * p.batch + g.b) * p.n_q_heads + (size_t)g.kvh * p.group) * p.q_cap;
-    arrive = p.tickets + unit;
-    depart = arrive + kDlmMaxSplitUnits / 2;
-    r_shift = p.rows > 64 ? 7 : p.rows > 32 ? 6 : 5;
-    const int n_vec = (p.n_mt * (D / 4)) << r_shift;
-    lo = p.by_team.div(n_vec * rank);          // n_vec <= 8192, team <= 16
-    hi = p.by_team.div(n_vec * (rank + 1));
-    piece0 = (size_t)unit * p.team * p.n_mt;
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// 32 columns of a row's O at `t`; with the keys split, the weighted sum of both halves' (at t and t2, which
+// lie D columns apart).  (A half without keys holds no O: then t2 is the other half's again and the weights are halves of its.)
+template <bool kKeys>
+__device__ __forceinline__ void read_o(uint32_t t, uint32_t t2, const float (&w)[2], uint32_t (&v)[32]) {
+  tmem_ld32(t, v);
+  if (!kKeys) {
+    tmem_ld_wait();
+    return;
   }
+  uint32_t u[32];
+  tmem_ld32(t2, u);
+  tmem_ld_wait();
+  const uint64_t w0 = pack2(w[0], w[0]), w1 = pack2(w[1], w[1]);
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    const uint64_t a = pack2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), b = pack2(__uint_as_float(u[j]), __uint_as_float(u[j + 1]));
+    float x, y;
+    unpack2(fma2(w1, b, mul2(w0, a)), x, y);
+    v[j] = __float_as_uint(x);
+    v[j + 1] = __float_as_uint(y);
+  }
+}
+
+// Team schedule: what the blocks of a team, which are a thread-block cluster, do after their shares of the key tiles.  A block's
+// piece -- unnormalised O, and (m, l), for every row -- is laid out in its own shared memory, over the rings, which are read no
+// more: [warp of 32 rows][head_dim / 4][32] 16-byte vectors, R the unit's rows in whole warps.  Each block finishes some of the unit's output
+// columns, in units of 8, over all the team's pieces: bulk copies bring it those columns of the others' pieces and their (m, l),
+// counted in on a barrier of its own.
+//   What bounds it is neither bytes nor the shared memory network but the number of instructions, run once and partly fetched for
+// the first time: so it is short and in loops, what can be made ready before the last product is, and the reduction is spread over
+// all eight softmax warps.  Cycles from the last product to the end of the block, 64 rows in teams of 4 in a step: straight from
+// registers into the others' shared memory, 1500 unrolled instructions, 7900 (2450 to send, 1400 for the weights of 4 pieces, 1400 to
+// reduce, 200 of waiting; in loops 6000: such stores move 16 - 18 bytes a cycle); bulk copies by one lane of the publisher 6100; by every
+// warp as soon as its rows are laid out 5500.  Through L2 with counters, as before, a block of a team of 9 took 9800.
+//   One-layer calls, before (through L2, keys not split) -> now, us: 256 active rows of Dream 16.4 -> 12.9, 8 sequences 16.9 -> 13.2, 4 13.2 -> 11.2,
+// one 8.95 -> 8.55 (64 blocks instead of 144), 300 cached rows 7.7 -> 7.15, the tiny configuration 6.85 -> 6.65, 2 x 8 heads of 100 rows 10.6 ->
+// 9.5, 4 sequences of 8 KV heads at 2000 rows 14.7 -> 13.4.  The split of the keys alone, with the exchange through L2: 8 sequences 16.9 ->
+// 15.9, 4 13.2 -> 12.7, 64 rows and fewer equal (it is not used for whole units: an LLaDA layer, 64 rows a unit, is bound by HBM and took
+// 0.2 us more).
+__host__ __device__ inline int team_share(int head_dim, int team) { return (head_dim / 8 + team - 1) / team; }   // largest share, units
+__host__ __device__ inline int team_bytes(int head_dim, int team, int rows) {
+  return (team - 1) * team_share(head_dim, team) * rows * 32 + team * rows * 8;
+}
+struct TeamShape {
+  FastDiv by_team;
+  int team, rank, R, share;
+  uint32_t sm_piece;     // the block's own piece
+  uint32_t sm_x;         // the others': [team - 1][R / 32][share][2][32] vectors
+  uint32_t sm_ml;        // [team][R] (m, l), the block's own last
+  __device__ __forceinline__ int lo(int D, int r) const { return by_team.div(D / 8 * r); }   // first unit of rank r
 };
 
-// The two halves of the team schedule's exchange are functions of their own, not inlined: they run once per
-// launch, and inlined they changed the register allocation of the kernel's main loops (measured: 2 - 3 % on the
-// layer-batched calls, which never run them).
-//
-// Publisher warp, one thread: once every softmax thread of this block has stored its row of the block's piece
-// (bar_pub), count the block in the unit's arrival counter; when the whole team has arrived, let the softmax threads go on
-// (bar_team = bar_pub + 8).
-template <bool kNoWait>
-__device__ __noinline__ void team_publish(const TeamArgs p, uint32_t bar_pub, volatile int* abort_ptr) {
-  constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
-  if (!p.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
-  __threadfence();
-  atomicAdd(p.arrive, 1u);
-  if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
-  mbar_arrive(bar_pub + 8);
-  // every block of the team is past its wait on the arrival counter when the last one gets here: the last
-  // one clears both counters for the next launch
-  if (atomicAdd(p.depart, 1u) == (unsigned int)p.team - 1u) {
-    *p.arrive = 0;
-    *p.depart = 0;
-  }
+// What the others will send: O those that have tiles (dealt so that no block has two before each has one), (m, l) all.
+template <int D>
+__device__ __forceinline__ void team_expect(const TeamShape& p, uint32_t bar_team, int T, bool has_tiles) {
+  const int mine = p.lo(D, p.rank + 1) - p.lo(D, p.rank), with_tiles = min(T, p.team) - (has_tiles ? 1 : 0);
+  mbar_expect_tx(bar_team, (uint32_t)(p.R * (with_tiles * mine * 32 + (p.team - 1) * 8)));
 }
 
-// Softmax threads (all 256 of the block, whole warps).  Live ones store their row of the block's piece --
-// unnormalised O from TMEM at t_o if the block had key tiles, and (m, l), which is (-inf, 0) if it had none
-// (that piece's O is then never read).  Then all wait for the team and reduce this block's share of
-// the unit's output vectors over the C pieces, in rank order.  A thread's vectors lie in one row of an M tile, whose weights it takes
-// once, and what it needs of up to kMax pieces it asks L2 for at once: one round trip for the weights and the first vectors, one
-// for each further pair or single vector.  (Bulk copies of the shares into shared memory, 2 C of them issued by one lane, took 2400 -
-// 2900 cycles until they had landed, and the reduction from there 1400 - 6000.)  Returns false when a wait was given up.
-template <int D, bool kNoWait, int kMax>
-__device__ __forceinline__ void team_reduce(const TeamArgs& p) {
-  constexpr int kVec = 16 / kMax;             // vectors in flight
-  const int kVecs = (D / 4) << p.r_shift, R = 1 << p.r_shift;   // vectors of one M tile's piece
-  const int tid = threadIdx.x, C = p.team;
-  const int row = (p.lo + tid) & (R - 1);     // 256 is a multiple of R
-  const float4* const o = reinterpret_cast<const float4*>(p.ws_o) + ((p.piece0 * (D / 4)) << p.r_shift);
-  const size_t piece = (size_t)kVecs * p.n_mt;
-  int mt = -1;
-  bool real = false, active = false;
-  float w[kMax], m_all = 0.f, l_all = 0.f, inv = 0.f;
-  size_t qrow = 0;
-  for (int i = p.lo + tid; i < p.hi; i += 256 * kVec) {
-    float4 x[kVec][kMax];
-#pragma unroll
-    for (int u = 0; u < kVec; ++u)
-#pragma unroll
-      for (int c = 0; c < kMax; ++c)
-        if (c < C && i + 256 * u < p.hi) x[u][c] = __ldcg(o + c * piece + i + 256 * u);
-#pragma unroll
-    for (int u = 0; u < kVec; ++u) {
-      const int iu = i + 256 * u, mt_i = iu >= kVecs ? 1 : 0, qd = (iu - mt_i * kVecs) >> p.r_shift;
-      if (iu >= p.hi) break;
-      if (mt_i != mt) {
-        mt = mt_i;
-        const int r_unit = mt * 128 + row, r_kv = p.r0 + r_unit;
-        real = r_unit < ((p.rows + 31) & ~31) && r_kv < p.rows_total;
-        qrow = p.qrow0 + r_kv;                // rows of a KV head's query heads lie one after the other
-        int ir;
-        p.by_q_cap.divmod(r_kv, ir);
-        active = ir < p.Lq;
-        const float2* const a_ml = reinterpret_cast<const float2*>(p.ws_ml) + ((p.piece0 + mt) << p.r_shift) + row;
-        float2 ml[kMax];
-#pragma unroll
-        for (int c = 0; c < kMax; ++c) ml[c] = c < C && real ? __ldcg(a_ml + (((size_t)c * p.n_mt) << p.r_shift)) : make_float2(-CUDART_INF_F, 0.f);
-        m_all = -CUDART_INF_F;
-#pragma unroll
-        for (int c = 0; c < kMax; ++c)
-          if (ml[c].y > 0.f) m_all = fmaxf(m_all, ml[c].x);
-        l_all = 0.f;
-#pragma unroll
-        for (int c = 0; c < kMax; ++c) {
-          w[c] = ml[c].y > 0.f ? ex2_approx(ml[c].x - m_all) : 0.f;
-          l_all = fmaf(w[c], ml[c].y, l_all);
-        }
-        inv = active ? 1.f / l_all : 0.f;
-      }
-      if (!real) continue;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int c = 0; c < kMax; ++c) {
-        if (c < C && w[c] != 0.f) {           // a piece without keys holds no O
-          acc.x = fmaf(w[c], x[u][c].x, acc.x);
-          acc.y = fmaf(w[c], x[u][c].y, acc.y);
-          acc.z = fmaf(w[c], x[u][c].z, acc.z);
-          acc.w = fmaf(w[c], x[u][c].w, acc.w);
-        }
-      }
-      const __nv_bfloat162 h0 = __floats2bfloat162_rn(active ? acc.x * inv : 0.f, active ? acc.y * inv : 0.f);
-      const __nv_bfloat162 h1 = __floats2bfloat162_rn(active ? acc.z * inv : 0.f, active ? acc.w * inv : 0.f);
-      *reinterpret_cast<uint2*>(p.out + qrow * D + qd * 4) =
-          make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-      if (qd == 0 && p.lse) p.lse[qrow] = active ? (m_all + lg2_approx(l_all)) * 0.6931471805599453f : -CUDART_INF_F;
-    }
+// What lane d of a warp sends block d of the warp's 32 rows (number `w` of the unit): the units that block finishes of [u0, u1), and,
+// for every n_parts-th block from `part` on, the rows' (m, l).  Made ready while the block's first keys are on their way.
+struct TeamParcel {
+  uint32_t src, dst, bytes, ml_dst, bar;   // bytes, ml_dst: 0 for none
+};
+template <int D>
+__device__ __forceinline__ TeamParcel team_parcel(const TeamShape& p, uint32_t bar_team, int w, int u0, int u1, int part, int n_parts) {
+  const int d = threadIdx.x & 31;
+  TeamParcel c = {0, 0, 0, 0, 0};
+  if (d < p.team && d != p.rank) {
+    const int lo_d = p.lo(D, d), lo = max(lo_d, u0), n = min(p.lo(D, d + 1), u1) - lo, slot = p.rank < d ? p.rank : p.rank - 1;
+    c.src = p.sm_piece + (w * (D / 8) + lo) * 1024;
+    c.dst = map_shared_rank(p.sm_x, d) + ((slot * (p.R >> 5) + w) * p.share + lo - lo_d) * 1024;
+    c.bytes = n > 0 ? n * 1024 : 0;
+    c.ml_dst = d % n_parts == part ? map_shared_rank(p.sm_ml, d) + (slot * p.R + w * 32) * 8 : 0;
+    c.bar = map_shared_rank(bar_team, d);
   }
+  return c;
 }
 
-template <int D, bool kNoWait>
-__device__ __noinline__ bool team_exchange(const TeamArgs p, uint32_t bar_pub, volatile int* abort_ptr, bool live, uint32_t t_o,
-                                           bool has_tiles, float m_used, float l_run) {
-  constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
-  const int tid = threadIdx.x, mt = tid >> 7, row = tid & 127;
-  if (live) {
-    const size_t mine = p.piece0 + (size_t)p.rank * p.n_mt + mt;
-    if (has_tiles) {
-      float4* po = reinterpret_cast<float4*>(p.ws_o) + ((mine * (D / 4)) << p.r_shift) + row;
-      uint32_t v[32];
+// Softmax threads, all 256: row `row` of the unit and every n_groups-th unit of the block's columns from the group's on, two units
+// and two pieces at a time (a unit or piece beyond the last is the last again, not stored or without weight).
+template <int D>
+__device__ __forceinline__ void team_reduce(const TeamShape& p, int row, int group, int n_groups, bool real, bool active, __nv_bfloat16* out, float* lse) {
+  const int lo = p.lo(D, p.rank), n = p.lo(D, p.rank + 1) - lo, last = p.team - 1;
+  const uint32_t at = (uint32_t)((row & 31) * 16), ml = p.sm_ml + row * 8, ml_step = p.R * 8, x_step = p.share * p.R * 32;
+  const uint32_t x0 = p.sm_x + (uint32_t)((row >> 5) * p.share) * 1024 + at, own = p.sm_piece + (uint32_t)((row >> 5) * (D / 8) + lo) * 1024 + at;
+  float m_all = -CUDART_INF_F;
+#pragma unroll 4
+  for (int s = 0; s <= last; ++s) m_all = fmaxf(m_all, ld_shared_f2(ml + s * ml_step).x);
 #pragma unroll 1
-      for (int c = 0; c < D / 32; ++c) {
-        tmem_ld32(t_o + c * 32, v);
-        tmem_ld_wait();
+  for (int u = group; u < n; u += 2 * n_groups) {
+    const int u1 = min(u + n_groups, n - 1);
+    float acc[2][8] = {}, l_all = 0.f;
+#pragma unroll 1
+    for (int s = 0; s <= last; s += 2) {
+      float2 a[2];
+      float4 x[2][2], y[2][2];
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          __stcg(po + ((c * 8 + j) << p.r_shift), make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                              __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
+      for (int j = 0; j < 2; ++j) {
+        const int sj = min(s + j, last);
+        const uint32_t from = sj == last ? own : x0 + sj * x_step;
+        a[j] = ld_shared_f2(ml + sj * ml_step);
+        if (s + j > last) a[j].y = 0.f;
+        x[j][0] = ld_shared_f4(from + u * 1024);
+        y[j][0] = ld_shared_f4(from + u * 1024 + 512);
+        x[j][1] = ld_shared_f4(from + u1 * 1024);
+        y[j][1] = ld_shared_f4(from + u1 * 1024 + 512);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (!__any_sync(0xffffffffu, a[j].y != 0.f)) continue;   // a piece without key tiles holds no O
+        const float w = ex2_approx(a[j].x - m_all);
+        l_all = fmaf(w, a[j].y, l_all);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          acc[i][0] = fmaf(w, x[j][i].x, acc[i][0]); acc[i][1] = fmaf(w, x[j][i].y, acc[i][1]);
+          acc[i][2] = fmaf(w, x[j][i].z, acc[i][2]); acc[i][3] = fmaf(w, x[j][i].w, acc[i][3]);
+          acc[i][4] = fmaf(w, y[j][i].x, acc[i][4]); acc[i][5] = fmaf(w, y[j][i].y, acc[i][5]);
+          acc[i][6] = fmaf(w, y[j][i].z, acc[i][6]); acc[i][7] = fmaf(w, y[j][i].w, acc[i][7]);
+        }
       }
     }
-    __stcg(reinterpret_cast<float2*>(p.ws_ml) + (mine << p.r_shift) + row, make_float2(m_used, l_run));
-    // no fence here: the arrival below orders the stores before the publisher's wait (block scope), and the
-    // publisher's fence before it counts the block in carries them to device scope
-    mbar_arrive(bar_pub);
+    const float inv = 1.f / l_all;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      uint32_t h[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) h[j] = active ? pack_bf16(acc[i][2 * j] * inv, acc[i][2 * j + 1] * inv) : 0u;
+      if (real) *reinterpret_cast<uint4*>(out + (lo + (i ? u1 : u)) * 8) = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+    if (lo + u == 0 && real && lse) *lse = active ? (m_all + lg2_approx(l_all)) * 0.6931471805599453f : -CUDART_INF_F;
   }
-  if (!mbar_wait_warp(bar_pub + 8, 0, abort_ptr, kLimit)) return false;
-  if (p.team <= 8) team_reduce<D, kNoWait, 8>(p); else team_reduce<D, kNoWait, 16>(p);
-  __syncwarp();
-  return true;
 }
 
 // A key tile is processed in half-steps of up to 64 keys.  Each M tile has two 64-column score
@@ -435,21 +415,26 @@ struct HalfStep {
   int nkeys;      // valid keys (1..64)
   bool first_of_tile, last_of_tile;
 };
+// In kernels that split the keys (kKeys) chain h has half-step h of every tile that reaches it.
+template <bool kKeys>
 struct HalfIter {
   const Segment& g;
   int fresh_box, t, h;
-  __device__ HalfIter(const Segment& g_, int fresh_box_) : g(g_), fresh_box(fresh_box_), t(g_.t_begin), h(0) {}
+  __device__ HalfIter(const Segment& g_, int fresh_box_, int chain) : g(g_), fresh_box(fresh_box_), t(g_.t_begin), h(kKeys ? chain : 0) {}
+  // kKeys: the chain has nothing in tile t
+  __device__ __forceinline__ bool skips() const { return kKeys && h != 0 && t < g.t_end && tile_valid(g, t, fresh_box) <= kHalfKeys; }
   __device__ __forceinline__ bool get(HalfStep& s) const {
     if (t >= g.t_end) return false;
     const int valid = tile_valid(g, t, fresh_box);
     s.t = t;
     s.k0 = h * kHalfKeys;
     s.nkeys = min(kHalfKeys, valid - s.k0);
-    s.first_of_tile = (h == 0);
-    s.last_of_tile = (h == 1) || valid <= kHalfKeys;
+    s.first_of_tile = kKeys || (h == 0);
+    s.last_of_tile = kKeys || (h == 1) || valid <= kHalfKeys;
     return true;
   }
   __device__ __forceinline__ void advance(const HalfStep& s) {
+    if (kKeys) { ++t; return; }
     if (s.last_of_tile) { ++t; h = 0; } else { h = 1; }
   }
 };
@@ -506,11 +491,6 @@ __device__ __forceinline__ float row_max64(const uint32_t (&s)[64]) {
     for (int c = 0; c < 8; ++c) mx[c] = fmaxf(mx[c], __uint_as_float(s[j + c]));
   }
   return fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // P = 2^(s * scale - m) for 32 scores, packed to bf16 pairs and written to 16 TMEM columns at t_p;
@@ -613,17 +593,25 @@ __device__ __noinline__ bool softmax_half_ragged(uint32_t t_s, uint32_t t_o, int
   return true;
 }
 
+enum BlockWork { kManySegments, kOneUnit, kPartOfTeam };   // what a block of a launch has
+
 // kNoWait = true is the instantiation a test selects to run the give-up path: every wait on work still to come tests
 // its barrier once and gives up if the data is not there yet (waits that let issued copies and MMAs finish keep the
 // 2 s limit).  The limit is a compile-time constant because the waits sit on the critical path of the MMA issuers
 // (a run-time limit cost 2 % at the Dream shape).
-template <int D, int kChunk, bool kSingle, bool kNoWait>
+template <int D, int kChunk, BlockWork kWork, bool kNoWait>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kc,
                        const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ CUtensorMap tm_kn,
                        const __grid_constant__ CUtensorMap tm_vn, const __grid_constant__ AttnParams p) {
   using G = Geometry<D>;
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
+  // One M tile per block: the two chains of warps that otherwise have an M tile each share it and split the keys, chain h taking
+  // keys 64 h .. 64 h + 63 of every tile into an O, maximum and sum of its own, folded at the end.
+  constexpr bool kSingle = kWork != kManySegments, kTeam = kWork == kPartOfTeam, kKeys = kTeam && kChunk <= 128;
+  const int n_chains = kKeys ? 2 : p.n_mt;
+  // softmax threads that own a real query row, rounded up to whole warps (tid 0 .. n_live-1; keys split: of either half)
+  const int n_live = (p.rows + 31) & ~31;
   // Shared memory of the block, all of it dynamic (the scheduling tables are sized by batch and grid):
   // [Q: n_mt tiles][K ring][V ring][barriers][flags][scheduling tables], from the first 1024-byte
   // boundary (the swizzled tiles need that alignment).
@@ -644,12 +632,15 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   volatile int* const merge_ok = flags + 3;
   volatile int* const any_empty = flags + 4;    // some batch element has no key tile at all
   Sched sched;
+  float2* const fold = reinterpret_cast<float2*>(flags + kFlagBytes / 4);   // [key half][row]
+  const uint32_t sm_x = smem_u32(fold) + kFoldBytes;                        // kSingle: what the team's other blocks send (team_bytes)
   sched.prefix = flags + kFlagBytes / 4;
   sched.lc = sched.prefix + p.batch + 1;
   sched.lq = sched.lc + p.batch;
   if (smem_pad + (uint32_t)(p.n_mt + KS + VS) * G::kTileBytes + kBarrierBytes + kFlagBytes +
-          4u * (uint32_t)sched_ints(p.batch) > (uint32_t)p.smem_bytes) {
-    // cannot happen with the host's sizing (it leaves room for the largest pad); nothing has been touched yet
+          (kTeam ? (uint32_t)(kFoldBytes + team_bytes(D, p.team, n_live)) : kSingle ? 0u : 4u * (uint32_t)sched_ints(p.batch)) > (uint32_t)p.smem_bytes ||
+      (kTeam && cluster_nctarank() != (uint32_t)p.team)) {
+    // cannot happen with the host's sizing (it leaves room for the largest pad) and launch; nothing has been touched yet
     if (threadIdx.x == 0) dlm_set_status(p.status, DLM_ERR_WORKSPACE);
     return;
   }
@@ -663,32 +654,32 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                                                                  // products can be in flight, so consecutive half-steps use different
                                                                  // barriers: a parity wait cannot tell phases two apart
   const uint32_t bar_pub = bar_pv_done + 32;                   // partial result of a segment stored by every softmax thread
-  const uint32_t bar_team = bar_pub + 8;                         // team schedule: the whole team's pieces are there
+  const uint32_t bar_team = bar_pub + 8;                         // team schedule: the other blocks' pieces are there
+  const uint32_t bar_fold = bar_team + 8;                        // keys split: both halves' O, maxima and sums are there
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // softmax threads that own a real query row, rounded up to whole warps (they are tid 0 .. n_live-1)
-  const int n_live = (p.rows + 31) & ~31;
 
   // ---- set-up: barriers, TMEM, descriptor prefetch and which unit is this block's first (they need no data), so that they
   // overlap the kernel before; then the lengths
   if (tid == 0) {
     *abort_ptr = 0; *never_ptr = 0; *merge_ok = 0; *any_empty = 0;
     mbar_init(bar_q_full, 1);
-    mbar_init(bar_q_empty, (uint32_t)p.n_mt);       // one commit per MMA issuer
+    mbar_init(bar_q_empty, (uint32_t)n_chains);     // one commit per MMA issuer
     mbar_init(bar_drain, 1);
     mbar_init(bar_drain + 8, 1);
-    mbar_init(bar_pub, (uint32_t)n_live);
+    mbar_init(bar_pub, (uint32_t)(kSingle ? n_live / 32 * (kKeys ? 2 : 1) : n_live));   // teams: one arrival per warp
     mbar_init(bar_team, 1);
+    mbar_init(bar_fold, (uint32_t)n_live / 16);     // one arrival per live warp of either half
     for (int i = 0; i < KS; ++i) {
       mbar_init(bar_k_full + 8 * i, 1);
-      mbar_init(bar_k_empty + 8 * i, (uint32_t)p.n_mt);
+      mbar_init(bar_k_empty + 8 * i, (uint32_t)n_chains);
     }
     for (int i = 0; i < VS; ++i) {
       mbar_init(bar_v_full + 8 * i, 1);
-      mbar_init(bar_v_empty + 8 * i, (uint32_t)p.n_mt);
+      mbar_init(bar_v_empty + 8 * i, (uint32_t)n_chains);
     }
     for (int i = 0; i < 2; ++i) {
-      const uint32_t live_i = (uint32_t)max(32, min(128, n_live - 128 * i)) / 32;   // one arrival per live warp
+      const uint32_t live_i = (uint32_t)(kKeys ? n_live : max(32, min(128, n_live - 128 * i))) / 32;   // one arrival per live warp
       for (int u = 0; u < 2; ++u) {
         mbar_init(bar_s_ready + 16 * i + 8 * u, 1);
         mbar_init(bar_p_ready + 16 * i + 8 * u, live_i);
@@ -714,7 +705,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (kSingle) decode_single(p, one);
   __syncwarp();
   tc_fence_before_sync();
-  __syncthreads();   // the barriers exist and TMEM is there
+  // the barriers exist and TMEM is there; in a team, so do the other blocks' barriers
+  if (kTeam) cluster_sync(); else __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   // Everything above needed no data.  Whole units and teams: which unit a block starts with does not depend on the lengths, so
@@ -725,7 +717,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   auto copy_q = [&](int zq, int rc) {
     for (int mt = 0; mt < p.n_mt; ++mt)
       for (int pn = 0; pn < G::kPanels; ++pn)
-        tma_load_3d(sm_q + mt * G::kTileBytes + pn * kPanelBytes, &tm_q, bar_q_full, pn * 64, rc * kChunk + mt * 128, zq);
+        tma_load_3d(sm_q + mt * G::kTileBytes + pn * kPanelBytes, &tm_q, bar_q_full, pn * 64, rc * (kKeys ? p.chunk_rows : kChunk) + mt * 128, zq);
   };
   // From here on the inputs of the call are read: all threads wait for the kernel before.  In a block of a single unit each role
   // does so where it starts, so that the code up to there has been fetched by then, and reads its unit's lengths for itself.
@@ -741,6 +733,18 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       Lq = max(0, min(Lq, p.q_cap));
     }
     set_single_lengths(p, one, Lc, Lq);
+  };
+  auto team_shape = [&]() {
+    TeamShape a;
+    a.by_team = p.by_team;
+    a.team = p.team;
+    p.by_team.divmod(blockIdx.x, a.rank);
+    a.R = n_live;
+    a.share = team_share(D, p.team);
+    a.sm_piece = sm_k;
+    a.sm_x = sm_x;
+    a.sm_ml = sm_x + (uint32_t)((p.team - 1) * a.share * n_live * 32);
+    return a;
   };
   if (!kSingle) {
     wait_for_inputs();
@@ -870,19 +874,19 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         if (q_issued > 0) mbar_wait(bar_q_full, (q_issued - 1) & 1, never_ptr);
       }
     } else if (warp == 9 || warp == 10) {
-      // ============================================ MMA issuers: warp 9 for M tile 0, warp 10 for M tile 1
+      // ============================================ MMA issuers: warp 9 for M tile (or key half) 0, warp 10 for 1
       // One warp per M tile, so that the scalar work around one tile's MMAs (barrier waits and
       // commits) runs while the tensor pipe executes the other tile's.  One elected lane runs the whole
       // loop, waits included: with the warp taking part in every wait and a lane elected per product, waits on
       // complete barriers and the elections stood between P's arrival and the products it releases (an LLaDA layer, one M tile
       // per block: 31.5 us, now 29.5; two M tiles, where the softmax warps bound the loop, 0 - 2 %).  The K, V and Q
-      // buffers are released when every issuer has committed (their "empty" barriers count n_mt arrivals).
+      // buffers are released when every issuer has committed (their "empty" barriers count as many arrivals).
       const int mt = warp - 9;
       if (kSingle) {
         wait_for_inputs();
         read_lengths();
       }
-      if (has_work && mt < p.n_mt && elect_one_sync()) {
+      if (has_work && mt < n_chains && elect_one_sync()) {
         auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_limit(bar, parity, abort_ptr, kLimit); };
         SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
         Segment g = one;
@@ -890,7 +894,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         bool ok = true;
         const uint32_t idesc_pv = make_idesc_bf16(128, D, 1);
         // descriptors of the first K-step of each operand buffer; the loops only add constants
-        const uint64_t desc_q = make_smem_desc_sw128(sm_q + mt * G::kTileBytes, 16, 1024);
+        const uint64_t desc_q = make_smem_desc_sw128(sm_q + (kKeys ? 0 : mt) * G::kTileBytes, 16, 1024);
         const uint64_t desc_k0 = make_smem_desc_sw128(sm_k, 16, 1024);
         const uint64_t desc_v0 = make_smem_desc_sw128(sm_v, kPanelBytes, 1024);
         const uint32_t t_o = tmem + G::kColO + mt * D;
@@ -934,10 +938,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
           ok = wait(bar_q_full, seg & 1);
           if (!ok) break;
-          HalfIter si(g, p.fresh_box), pi(g, p.fresh_box);
+          HalfIter<kKeys> si(g, p.fresh_box, mt), pi(g, p.fresh_box, mt);
           // scores of the next half-step of the segment that has none yet, into buffer js & 1
           auto issue_next_s = [&]() -> bool {
             HalfStep hs;
+            for (; si.skips(); ++si.t, ++kt) {   // (behind the copy, so that the arrival counts for this use of the buffer)
+              if (!wait(bar_k_full + 8 * (kt % KS), (kt / KS) & 1)) return false;
+              mbar_arrive(bar_k_empty + 8 * (kt % KS));
+            }
             if (!si.get(hs)) return true;
             const uint32_t ks = kt % KS;
             if (hs.first_of_tile) {
@@ -958,7 +966,14 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           ok = issue_next_s() && issue_next_s();   // both score buffers filled ahead
           bool first = true;
           HalfStep hs;
-          while (ok && pi.get(hs)) {
+          auto skip_v = [&]() -> bool {
+            for (; pi.skips(); ++pi.t, ++vt) {
+              if (!wait(bar_v_full + 8 * (vt % VS), (vt / VS) & 1)) return false;
+              mbar_arrive(bar_v_empty + 8 * (vt % VS));
+            }
+            return true;
+          };
+          while (ok && (ok = skip_v()) && pi.get(hs)) {
             const uint32_t vs = vt % VS;
             if (hs.first_of_tile) {
               ok = wait(bar_v_full + 8 * vs, (vt / VS) & 1);
@@ -993,8 +1008,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         wait_for_inputs();
         read_lengths();
       }
-      if (kSingle && lane == 0 && p.team > 1) {
-        team_publish<kNoWait>(TeamArgs(p, one, D), bar_pub, abort_ptr);
+      if (kTeam && lane == 0 && one.T > 0) {
+        team_expect<D>(team_shape(), bar_team, one.T, one.t_end > one.t_begin);
       } else if (!kSingle && lane == 0 && has_work && !p.whole_units) {
         SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
         Segment g = one;
@@ -1014,22 +1029,65 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       wait_for_inputs();
       read_lengths();
     }
-    if (tid < n_live) {
+    // teams: what this thread reduces, made ready while the first keys are on their way
+    TeamShape sh;
+    int red_row = 0, red_group = 0, red_groups = 0;
+    bool red_real = false, red_active = false;
+    __nv_bfloat16* red_out = nullptr;
+    float* red_lse = nullptr;
+    if (kTeam) {
+      sh = team_shape();
+      red_group = p.by_live.divmod(tid, red_row);
+      red_groups = p.by_live.div(256);
+      const int r_kv = one.rc * (kKeys ? p.chunk_rows : kChunk) + red_row;
+      red_real = red_row < p.rows && r_kv < p.rows_total;
+      red_active = red_real && r_kv - p.by_q_cap.div(r_kv) * p.q_cap < one.Lq;
+      const size_t qrow = (((size_t)one.lc_layer * p.batch + one.b) * p.n_q_heads + (size_t)one.kvh * p.group) * p.q_cap + r_kv;
+      red_out = p.out + qrow * D;
+      if (p.lse) red_lse = p.lse + qrow;
+    }
+    if ((kKeys ? tid & 127 : tid) < n_live) {
       // ================================================= softmax warps (those that own real rows)
       const int mt = warp >> 2;
       const int row = (warp & 3) * 32 + lane;                 // row of the M tile = TMEM lane
       const uint32_t t_lane = (uint32_t)((warp & 3) * 32) << 16;
       const uint32_t t_s = tmem + t_lane + G::kColS + mt * 128;
       const uint32_t t_o = tmem + t_lane + G::kColO + mt * D;
-      const int r_unit = mt * 128 + row;                      // row within the unit (== tid)
-      const int n_live_mt = min(128, n_live - 128 * mt);   // live softmax threads of this M tile
+      const int r_unit = kKeys ? row : mt * 128 + row;        // row within the unit
+      const int n_live_mt = kKeys ? n_live : min(128, n_live - 128 * mt);   // live softmax threads of this M tile
       // the warp leaves a wait together, so the .sync.aligned TMEM instructions that follow
       // always see a converged warp, also when a wait is given up
       auto wait_warp = [&](uint32_t bar, uint32_t parity) { return mbar_wait_warp(bar, parity, abort_ptr, kLimit); };
+      const int chunk_rows = kKeys ? p.chunk_rows : kChunk;
       // this thread's query row in row chunk rc of a KV head: which of its query heads, which active row
       // (rows of a KV head's query heads lie one after the other)
       auto out_row_of = [&](int lc_layer, int b, int kvh, int rc) {
-        return (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group) * p.q_cap + rc * kChunk + r_unit;
+        return (((size_t)lc_layer * p.batch + b) * p.n_q_heads + (size_t)kvh * p.group) * p.q_cap + rc * chunk_rows + r_unit;
+      };
+      constexpr int kCols = kKeys ? D / 2 : D;               // of O that this thread folds and stores
+      const int c0 = kKeys ? mt * kCols : 0;
+      TeamParcel parcel;
+      if (kTeam) parcel = team_parcel<D>(sh, bar_team, r_unit >> 5, c0 / 8, (c0 + kCols) / 8, kKeys ? mt : 0, kKeys ? 2 : 1);
+      // teams: the row's (m, l) and O to the block's piece; O complete in TMEM at t (and t2), or the block has no key tile
+      auto lay_out_piece = [&](bool has_tiles, uint32_t t, uint32_t t2, const float (&w)[2], float m, float l) {
+        st_shared_f2(sh.sm_ml + ((p.team - 1) * n_live + r_unit) * 8, m, l);
+        if (has_tiles) {
+          uint32_t to = sh.sm_piece + ((r_unit >> 5) * (D / 4) + c0 / 4) * 512 + lane * 16;
+#pragma unroll 1
+          for (int c = c0; c < c0 + kCols; c += 32) {
+            uint32_t v[32];
+            read_o<kKeys>(t + c, t2 + c, w, v);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4, to += 512)
+              st_shared_f4(to, __uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
+          }
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_pub);   // for the block's own other warps
+        if (parcel.ml_dst) bulk_copy_to_cluster(parcel.ml_dst, sh.sm_ml + ((p.team - 1) * n_live + (r_unit & ~31)) * 8, 256, parcel.bar);
+        if (has_tiles && parcel.bytes) bulk_copy_to_cluster(parcel.dst, parcel.src, parcel.bytes, parcel.bar);
+        __syncwarp();
       };
       auto zero_my_row = [&](size_t qrow, bool real_row) {
         if (real_row) {
@@ -1046,7 +1104,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           int b, rc, kvh;
           const int grp = p.by_batch.divmod(unit, b), lc_layer = p.by_kv_heads.divmod(p.by_rc.divmod(grp, rc), kvh);
           if (sched.prefix[b + 1] == sched.prefix[b])
-            zero_my_row(out_row_of(lc_layer, b, kvh, rc), rc * kChunk + r_unit < p.rows_total);
+            zero_my_row(out_row_of(lc_layer, b, kvh, rc), rc * chunk_rows + r_unit < p.rows_total);
         }
       }
       if (has_work) {
@@ -1058,9 +1116,10 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const int n = g.t_end - g.t_begin;
           if (n <= 0) {  // inactive batch element: the unit's rows are zero (team schedule: or no tile for this rank)
             if (g.T == 0) {
-              zero_my_row(out_row_of(g.lc_layer, g.b, g.kvh, g.rc), g.rc * kChunk + r_unit < p.rows_total);
-            } else if (kSingle && p.team > 1) {   // a piece without key tiles
-              ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
+              zero_my_row(out_row_of(g.lc_layer, g.b, g.kvh, g.rc), g.rc * chunk_rows + r_unit < p.rows_total);
+            } else if (kTeam) {   // a piece without key tiles
+              const float none[2] = {0.f, 0.f};
+              lay_out_piece(false, 0, 0, none, -CUDART_INF_F, 0.f);
             }
             continue;
           }
@@ -1070,11 +1129,12 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           for (int t = g.t_begin; t < g.t_end && ok; ++t, ++vt) {
             const int valid = t < n_whole ? kTileKeys : tile_valid(g, t, p.fresh_box);
             const int n16 = (valid + 15) & ~15;
-            if (valid < n16) {
+            const int k_begin = kKeys ? mt * kHalfKeys : 0, k_end = kKeys ? min(valid, k_begin + kHalfKeys) : valid;
+            if (valid < n16 && k_begin < valid && k_end == valid) {
               // V rows in [valid, n16) would be multiplied by P = 0: clear them so that stale
               // NaN / Inf bit patterns cannot reach O.  Each M tile's warps do it before they
               // announce the P of the tile's first half-step, so it precedes that tile's P V
-              // products (the two M tiles write the same zeros).
+              // products (the two M tiles write the same zeros; with the keys split, the half that has them).
               const uint32_t vs = vt % VS;
               ok = wait_warp(bar_v_full + 8 * vs, (vt / VS) & 1);
               if (!ok) break;
@@ -1087,7 +1147,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               fence_proxy_async_smem();
             }
             // the tile's half-steps (the same enumeration as HalfIter, which the MMA warps use)
-            for (int k0 = 0; k0 < valid && ok; k0 += kHalfKeys, ++gt) {
+            for (int k0 = k_begin; k0 < k_end && ok; k0 += kHalfKeys, ++gt) {
               const int nkeys = min(kHalfKeys, valid - k0);
               const uint32_t buf = gt & 1;
               ok = wait_warp(bar_s_ready + 16 * mt + 8 * buf, (gt >> 1) & 1);
@@ -1111,22 +1171,44 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
           if (!ok) break;
           // ---- epilogue of the segment: O is complete once the last P V product has finished
-          ok = wait_warp(bar_pv_done + 16 * mt + 8 * ((gt - 1) & 1), ((gt - 1) >> 1) & 1);
+          if (!kKeys || gt > 0) ok = wait_warp(bar_pv_done + 16 * mt + 8 * ((gt - 1) & 1), ((gt - 1) >> 1) & 1);
           if (!ok) break;
           tc_fence_after_sync();
+          float w[2] = {1.f, 0.f};                               // of the key halves' O, at t_first and t_second
+          uint32_t t_first = t_o, t_second = t_o;
+          if (kKeys) {
+            // both halves' threads of a row learn of each other's maximum and sum ((-inf, 0) without keys); then each has
+            // half of the columns
+            fold[tid] = make_float2(m_used, l_run);
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_fold);
+            ok = wait_warp(bar_fold, 0);
+            if (!ok) break;
+            tc_fence_after_sync();
+            const float2 a = fold[row], b = fold[128 + row];
+            m_used = fmaxf(a.x, b.x);
+            w[0] = ex2_approx(a.x - m_used);
+            w[1] = ex2_approx(b.x - m_used);     // 0 without keys
+            l_run = fmaf(w[0], a.y, w[1] * b.y);
+            t_first = t_second = t_o - mt * D;
+            if (__any_sync(0xffffffffu, b.y != 0.f)) t_second += D;
+            else w[0] = w[1] = 0.5f * w[0];
+          }
           const size_t qrow = out_row_of(g.lc_layer, g.b, g.kvh, g.rc);
-          const int r_kv = g.rc * kChunk + r_unit;               // row among all query rows of the KV head
+          const int r_kv = g.rc * chunk_rows + r_unit;           // row among all query rows of the KV head
           const bool real_row = r_kv < p.rows_total;
           const bool active = real_row && r_kv - p.by_q_cap.div(r_kv) * p.q_cap < g.Lq;
           uint32_t v[32];
-          if (kSingle && p.team > 1) {
-            ok = team_exchange<D, kNoWait>(TeamArgs(p, g, D), bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
+          if (kTeam) {
+            lay_out_piece(true, t_first, t_second, w, m_used, l_run);
           } else if (kSingle || g.slot < 0) {
             const float inv = active ? 1.f / l_run : 0.f;
+            constexpr int kChunks = kKeys ? D / 64 : D / 32;
+            const int c0 = kKeys ? mt * kChunks : 0;
 #pragma unroll 1
-            for (int c = 0; c < D / 32; ++c) {
-              tmem_ld32(t_o + c * 32, v);
-              tmem_ld_wait();
+            for (int c = c0; c < c0 + kChunks; ++c) {
+              read_o<kKeys>(t_first + c * 32, t_second + c * 32, w, v);
               if (real_row) {
                 uint4* o = reinterpret_cast<uint4*>(p.out + qrow * D + c * 32);
 #pragma unroll
@@ -1143,7 +1225,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 }
               }
             }
-            if (real_row && p.lse)
+            if (real_row && p.lse && (!kKeys || mt == 0))
               p.lse[qrow] = active ? (m_used + lg2_approx(l_run)) * 0.6931471805599453f : -CUDART_INF_F;
           } else {
             // ---- a piece of a split unit.  Partial O is stored as 16-byte vectors of 4 columns,
@@ -1250,21 +1332,28 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           }
         }
       }
-    } else if (kSingle && p.team > 1) {
-      // warps without a row of their own help with the reduction
-      const TeamArgs ta(p, one, D);
-      if (ta.has_keys) team_exchange<D, kNoWait>(ta, bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
+    }
+    if (kTeam && one.T > 0) {
+      // teams: the columns that this block finishes, by all softmax threads
+      if (mbar_wait_warp(bar_pub, 0, abort_ptr, kLimit) && mbar_wait_warp(bar_team, 0, abort_ptr, kLimit)) {
+        if (red_group < red_groups) team_reduce<D>(sh, red_row, red_group, red_groups, red_real, red_active, red_out, red_lse);
+      }
     }
   }
-  // ---- teardown: nothing of this block is in flight any more
+  // ---- teardown: nothing of this block is in flight any more.  A team's blocks leave together: none before the others have
+  // stopped sending to its shared memory (every block gets here, also one that gave up, which then waits for what may be on its way).
+  if (kTeam && tid == 0 && *abort_ptr && one.T > 0) mbar_wait(bar_team, 0, never_ptr);
   __syncwarp();
+  if (kTeam) cluster_arrive();
   if (tid == 0 && *abort_ptr) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 9) {
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
+    __syncwarp();
   }
+  if (kTeam) cluster_wait();
 }
 
 // bf16 tensor viewed as [slabs][rows][D]; box = 64 elements x box_rows rows x 1 slab, 128-byte swizzle.
@@ -1282,36 +1371,32 @@ bool register_budget_ok(const cudaFuncAttributes& a) {
   return a.numRegs >= kRegsOther && 8 * (kRegsSoftmax - a.numRegs) <= 4 * (a.numRegs - kRegsOther);
 }
 
-// The instantiations: head_dim 128 / 64, row chunks of 256 / 128, normal / no-wait (test) waits, blocks of any number of
-// segments / of one; and chunks of 64 for teams.
+// The instantiations: head_dim 128 / 64; blocks of any number of segments, of one unit, parts of a team; units of up to 256 rows (two M
+// tiles) / 128 (one; in teams with the keys split); normal / no-wait (test) waits.
 using AttnKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                             const AttnParams);
 inline int kernel_index(int head_dim, const dlm_attn_plan& pl, bool no_wait) {
-  if (pl.chunk_rows == 64) return 16 + (head_dim == 128 ? 0 : 1) + (no_wait ? 2 : 0);
-  return (head_dim == 128 ? 0 : 1) + (pl.chunk_rows == 256 ? 0 : 2) + (no_wait ? 4 : 0) + (pl.single ? 8 : 0);
+  const bool narrow = pl.single ? pl.n_mt == 1 : pl.chunk_rows == 128;
+  return (head_dim == 128 ? 0 : 1) + (narrow ? 2 : 0) + (pl.team > 1 ? 8 : pl.single ? 4 : 0) + (no_wait ? 12 : 0);
 }
-template <bool kSingle>
-AttnKernel kernel_of(int which) {
-  switch (which & 7) {
-    case 0: return attn_step_sm100_kernel<128, 256, kSingle, false>;
-    case 1: return attn_step_sm100_kernel<64, 256, kSingle, false>;
-    case 2: return attn_step_sm100_kernel<128, 128, kSingle, false>;
-    case 3: return attn_step_sm100_kernel<64, 128, kSingle, false>;
-    case 4: return attn_step_sm100_kernel<128, 256, kSingle, true>;
-    case 5: return attn_step_sm100_kernel<64, 256, kSingle, true>;
-    case 6: return attn_step_sm100_kernel<128, 128, kSingle, true>;
-    default: return attn_step_sm100_kernel<64, 128, kSingle, true>;
-  }
-}
-AttnKernel kernel_of(int which) {
+template <bool kNoWait>
+AttnKernel kernel_of_waits(int which) {
   switch (which) {
-    case 16: return attn_step_sm100_kernel<128, 64, true, false>;
-    case 17: return attn_step_sm100_kernel<64, 64, true, false>;
-    case 18: return attn_step_sm100_kernel<128, 64, true, true>;
-    case 19: return attn_step_sm100_kernel<64, 64, true, true>;
-    default: return which & 8 ? kernel_of<true>(which) : kernel_of<false>(which);
+    case 0: return attn_step_sm100_kernel<128, 256, kManySegments, kNoWait>;
+    case 1: return attn_step_sm100_kernel<64, 256, kManySegments, kNoWait>;
+    case 2: return attn_step_sm100_kernel<128, 128, kManySegments, kNoWait>;
+    case 3: return attn_step_sm100_kernel<64, 128, kManySegments, kNoWait>;
+    case 4: return attn_step_sm100_kernel<128, 256, kOneUnit, kNoWait>;
+    case 5: return attn_step_sm100_kernel<64, 256, kOneUnit, kNoWait>;
+    case 6: return attn_step_sm100_kernel<128, 128, kOneUnit, kNoWait>;
+    case 7: return attn_step_sm100_kernel<64, 128, kOneUnit, kNoWait>;
+    case 9: return attn_step_sm100_kernel<64, 256, kPartOfTeam, kNoWait>;
+    case 10: return attn_step_sm100_kernel<128, 128, kPartOfTeam, kNoWait>;
+    case 11: return attn_step_sm100_kernel<64, 128, kPartOfTeam, kNoWait>;
+    default: return nullptr;   // teams on two M tiles of heads of 128: their pieces have no room in shared memory
   }
 }
+AttnKernel kernel_of(int which) { return which >= 12 ? kernel_of_waits<true>(which - 12) : kernel_of_waits<false>(which); }
 
 // First use of an attention kernel on a context's device: checks the register budget and opts in to
 // all the dynamic shared memory the device allows a block (less the kernel's static part).
@@ -1323,6 +1408,7 @@ int configure_kernel(dlm_ctx* ctx, int which, const void* kern) {
   const int limit = ctx->max_smem_optin - (int)a.sharedSizeBytes;
   if (limit <= 0) return DLM_ERR_UNSUPPORTED;
   DLM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  if (which % 12 >= 8) DLM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   ctx->attn_smem_limit[which] = limit;
   return DLM_OK;
 }
@@ -1335,7 +1421,8 @@ using Plan = dlm_attn_plan;
 bool plan_shared_memory(int smem_limit, int head_dim, int batch, Plan& pl) {
   const int tile = head_dim / 64 * kPanelBytes;
   const int stages = head_dim == 128 ? Geometry<128>::kStages : Geometry<64>::kStages;
-  pl.smem_bytes = 1024 + (pl.n_mt + 2 * stages) * tile + kBarrierBytes + kFlagBytes + 4 * sched_ints(batch);
+  pl.smem_bytes = 1024 + (pl.n_mt + 2 * stages) * tile + kBarrierBytes + kFlagBytes +
+                  (pl.team > 1 ? kFoldBytes + team_bytes(head_dim, pl.team, (pl.rows + 31) & ~31) : pl.single ? 0 : 4 * sched_ints(batch));
   return pl.smem_bytes <= smem_limit;
 }
 
@@ -1352,16 +1439,10 @@ WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int 
 }
 
 // Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer), fitted to measurements of one-layer
-// calls (Dream heads, 1024 - 1152 cached rows; us):    team of 9, 1 tile, 128 rows         9.4     of 64 rows              9.0
-//   256 active rows: team of 5, 2 tiles, two M tiles   16.4    team of 2, 5 tiles, one M tile  18.3     split  23.4
-//   8 sequences:     team of 4, 3 tiles, two M tiles   18.4    team of 2, 5 tiles, one M tile  16.9     split  23.8
-// and of 15 more (300 - 4096 cached rows, 16 - 256 active, 1 - 8 sequences, four models' heads) under four sets of team costs: this set has the
-// fastest or one within 1 % everywhere; with the exchange dearer (1.8, 2.3, 4.3) 2 sequences of 32 heads at 3000 rows were dealt
-// whole, 29.1 us instead of 24.9, with 128 rows as cheap as 64 one sequence took 9.4 instead of 9.0 (300 rows: 8.9, 7.9).
-// Heads of 64, which were not in the fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule with
-// the costs before these, the choice was the fastest or within 2 % of it.
+// calls: units split across all SMs take 23.4 us with 256 active rows of Dream at 1024 cached ones, 23.8 with 8 sequences of 32.
+// Heads of 64, which were not in that fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule, the choice
+// was the fastest or within 2 % of it.
 constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer
-constexpr double kTeamCost[3] = {1.4, 1.8, 3.6};      // the team schedule's exchange and reduction, for 64 / 128 / 256 rows
 constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...
 constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond that
 // With more units than SMs a block has whole units to compute while its first piece travels, and merges one unit at most.
@@ -1370,6 +1451,32 @@ constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond
 // 2 - 4 us slower at one and two, equal at three, 1 - 2 us faster at four.
 constexpr double kSplitManyCost[2] = {3.2, 2.7};
 
+// The team schedule's call in us, fitted to 190 one-layer calls (28 shapes of six models' heads, 1 - 256 active and 0 - 4096 cached rows, 1 -
+// 8 sequences, every team size that fits, rows in chunks of 64, 96 and 128; rms error 6 %).  t: the key tiles of the block with the most;
+// r: rows of a piece / 128; d: head_dim / 128; full: the teams' part of the clusters that the device runs at a time; g: blocks per SM;
+// even: all blocks finish equally many columns.  Of the teams timed it takes the fastest or one within 5 % for every shape but one (11 %).
+// In the unit above a call of whole units takes (us - kWholeCall) / kTileUs.
+constexpr double kWholeCall = 3.2, kTileUs = 2.2;
+double team_us(double t, double r, double d, int team, double full, double g, bool even) {
+  return 4.9 + t * (0.55 + 0.45 * d) + 1.6 * r + 0.2 * team * full + 0.5 * t * d * g * g + (even ? 0.0 : 0.25);
+}
+
+// A unit's key tiles: the cache's, then the fresh rows'.
+struct UnitTiles {
+  long long len, q_cap, box, n_cache, n;
+  UnitTiles(long long len_, long long q_cap_) : len(len_), q_cap(q_cap_), box(q_cap_ < 128 ? q_cap_ : 128), n_cache((len_ + 127) / 128),
+                                                n(n_cache + (q_cap_ + 127) / 128) {}
+  // what tiles [from, to) cost: a ragged one 0.3 and 0.7 of its share
+  double cost(long long from, long long to) const {
+    double sum = 0;
+    for (long long i = from; i < to; ++i) {
+      const long long left = i < n_cache ? len - i * 128 : q_cap - (i - n_cache) * box, most = i < n_cache ? 128 : box;
+      sum += 0.3 + 0.7 / 128 * (double)(left < most ? left : most);
+    }
+    return sum;
+  }
+};
+
 // The best plan with row chunks of `chunk_rows`, and its estimated cost.
 double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
   pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
@@ -1377,11 +1484,11 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
   pl.n_rc = (pl.rows_total + chunk_rows - 1) / chunk_rows;
   pl.rows = pl.rows_total < chunk_rows ? pl.rows_total : chunk_rows;
   pl.n_mt = (pl.rows + 127) / 128;
-  const double tile = kTileCost[pl.n_mt - 1];
   const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
   const int sms = ctx->num_sms < kMaxGrid ? ctx->num_sms : kMaxGrid;
   const bool may_split = units < 8LL * sms && units <= kDlmMaxSplitUnits;
-  const long long tiles_unit = (len + 127) / 128 + (q_cap + 127) / 128;
+  const long long tiles_unit = UnitTiles(len, q_cap).n;
+  const double tile = kTileCost[pl.n_mt - 1];
   // units dealt whole: idle SMs when they do not fill a whole number of waves
   double best = (double)(((units + sms - 1) / sms) * tiles_unit) * tile;
   pl.whole_units = 1;
@@ -1398,23 +1505,61 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
     const double t = (double)((units * tiles_unit + sms - 1) / sms) * tile + kSplitManyCost[pl.n_mt - 1];
     if (t < best) { best = t; pl.whole_units = 0; pl.grid = sms; }
   }
-  // Team schedule for calls with few units: C blocks per unit, the unit's key tiles dealt among them, every
-  // block reducing a C-th of the outputs over all pieces in parallel (the split schedule's merging block
-  // folds the other pieces one after the other).  The smallest C that reaches the fewest tiles per block.
-  if (ctx->attn_team_max > 1 && units * 2 <= sms) {
-    long long C = ctx->attn_team_max < kTeamMax ? ctx->attn_team_max : kTeamMax;
-    if (C > sms / units) C = sms / units;
-    if (C > tiles_unit) C = tiles_unit;
-    if (C > 1) {
-      const long long per_block = (tiles_unit + C - 1) / C;
-      C = (tiles_unit + per_block - 1) / per_block;
-      const double t = (double)per_block * tile + kTeamCost[pl.rows <= 64 ? 0 : pl.n_mt];
-      if (C > 1 && (t < best || ctx->attn_team_force)) {
-        best = t;
-        pl.team = (int)C;
-        pl.whole_units = 1;
-        pl.grid = (int)(units * C);
-      }
+  return best;
+}
+
+// How many clusters of `team` blocks, one block per SM, the device runs at a time (0: none).  It depends on which SMs a die has: 74 of 2,
+// 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 - 9, 7 of 16 on one card.
+int team_clusters(dlm_ctx* ctx, int team) {
+  int& known = ctx->attn_clusters[team];
+  if (known == 0) {
+    constexpr int kTeamKernel = 10;   // head_dim 128, one M tile (kernel_index)
+    const AttnKernel kern = kernel_of(kTeamKernel);
+    known = -1;
+    if (configure_kernel(ctx, kTeamKernel, reinterpret_cast<const void*>(kern)) == DLM_OK) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(team);
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = ctx->attn_smem_limit[kTeamKernel];
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = team;
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) known = n;
+      else cudaGetLastError();
+    }
+  }
+  return known > 0 ? known : 0;
+}
+
+// The best plan with teams on row chunks of `chunk_rows`, and its estimated cost (negative: there is none).
+double plan_teams(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
+  pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
+  pl.chunk_rows = chunk_rows;
+  pl.n_rc = (pl.rows_total + chunk_rows - 1) / chunk_rows;
+  pl.rows = pl.rows_total < chunk_rows ? pl.rows_total : chunk_rows;
+  pl.n_mt = (pl.rows + 127) / 128;
+  pl.whole_units = pl.single = 1;
+  const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
+  const UnitTiles tiles(len, q_cap);
+  Plan at = pl;
+  double best = -1;
+  for (int team = 2; team <= kTeamMax && team <= ctx->attn_team_max && team <= tiles.n && units * team <= ctx->num_sms; ++team) {
+    at.team = team;
+    const int clusters = team_clusters(ctx, team);
+    if (!plan_shared_memory(ctx->max_smem_optin, cache->head_dim, cache->batch, at) || units > clusters) continue;
+    double most = 0;
+    for (int r = 0; r < team; ++r) most = fmax(most, tiles.cost(tiles.n * r / team, tiles.n * (r + 1) / team));
+    const double us = team_us(most * pl.n_mt, ((pl.rows + 31) & ~31) / 128.0, cache->head_dim / 128.0, team, (double)units / clusters,
+                              (double)(units * team) / ctx->num_sms, (cache->head_dim / 8) % team == 0);
+    const double t = (us - kWholeCall) / kTileUs;
+    if (best < 0 || t < best) {
+      best = t;
+      pl.team = team;
+      pl.grid = (int)units * team;
     }
   }
   return best;
@@ -1422,23 +1567,28 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
 
 // Row chunks of 256 (two M tiles sharing every K/V tile) read K/V once per KV head and cost little more per key tile than
 // chunks of 128; those double the units that can be spread over the SMs and halve every partial result, the second read of
-// K/V coming from L2.  Chunks of 64, half an M tile, halve the partial results once more: for teams only, whose exchange is
-// half of a short call.  Whichever schedule of any has the least estimated cost, from the caller's cache length hint.
-Plan make_plan(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int cache_len_hint) {
+// K/V coming from L2.  Teams also come with chunks of 96 and 64, whose partial results are smaller still (one sequence of Dream,
+// 224 rows a KV head, at 1024 cached rows: 9.3 us in chunks of 128, 8.7 of 96, 8.5 of 64, all in teams of 4; at 4096: 15.7, 12.5, 13.2 in
+// the best teams that fit).  Whichever schedule of any has the least estimated cost, from the caller's cache length hint.
+Plan make_plan(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int cache_len_hint) {
   const int len = (cache_len_hint > 0 && cache_len_hint < cache->capacity) ? cache_len_hint : cache->capacity;
-  Plan pl, narrow;
+  Plan pl, other;
   double cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 256, pl);
   if (pl.n_mt == 2) {
-    const double narrow_cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 128, narrow);
-    // (a forced team schedule counts as the better one)
-    const bool forced_apart = ctx->attn_team_force && (narrow.team > 1) != (pl.team > 1);
-    if (forced_apart ? narrow.team > 1 : narrow_cost < cost) { pl = narrow; cost = narrow_cost; }
+    const double c = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 128, other);
+    if (c < cost) { pl = other; cost = c; }
   }
-  if (pl.rows > 64) {
-    const double slim_cost = plan_chunked(ctx, cache, nl, n_q_heads, q_cap, len, 64, narrow);
-    if (narrow.team > 1 && slim_cost < cost && !ctx->attn_team_force) pl = narrow;
+  pl.single = pl.whole_units && (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc <= pl.grid;
+  if (pl.whole_units) {   // against teams, which deal a unit's tiles, a ragged tile counts for what it is
+    const UnitTiles tiles(len, q_cap);
+    cost *= tiles.cost(0, tiles.n) / (double)tiles.n;
   }
-  pl.single = pl.whole_units && (pl.team > 1 || (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc <= pl.grid);
+  bool forced = ctx->attn_team_force;
+  for (int chunk : {256, 128, 96, 64}) {
+    if (chunk < 256 && pl.rows_total <= chunk) continue;   // all rows in one chunk: as with 256
+    const double c = plan_teams(ctx, cache, nl, n_q_heads, q_cap, len, chunk, other);
+    if (c >= 0 && (c < cost || forced)) { pl = other; cost = c; forced = false; }
+  }
   const WorkspaceSize ws = workspace_size(ctx, cache, nl, n_q_heads, q_cap);
   pl.ws_o_bytes = ws.o_bytes;
   pl.ws_ml_bytes = ws.ml_bytes;
@@ -1463,7 +1613,8 @@ extern "C" int dlm_selftest_attn_schedule(const dlm_ctx* ctx, const dlm_kv_cache
   if (n_layers_in_call <= 0 || n_q_heads <= 0 || q_cap <= 0 || cache->n_kv_heads <= 0 || cache->batch <= 0 ||
       cache->capacity <= 0 || n_q_heads % cache->n_kv_heads != 0)
     return DLM_ERR_SHAPE;
-  const Plan pl = make_plan(ctx, cache, n_layers_in_call, n_q_heads, q_cap, cache_len_hint);
+  // (a plan may ask the device, once, how many clusters fit)
+  const Plan pl = make_plan(const_cast<dlm_ctx*>(ctx), cache, n_layers_in_call, n_q_heads, q_cap, cache_len_hint);
   *grid = pl.grid;
   *team = pl.team;
   *whole_units = pl.whole_units;
@@ -1544,6 +1695,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   p.by_kv_heads = make_fast_div(p.n_kv_heads);
   p.by_q_cap = make_fast_div(q_cap);
   p.by_team = make_fast_div(pl.team);
+  p.by_live = make_fast_div((pl.rows + 31) & ~31);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.status = &ctx->words->status;
   p.tickets = ctx->words->attn_unit_tickets;
@@ -1560,7 +1712,7 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   if (rc != DLM_OK) return rc;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DLM_CUDA_TRY(dlm_launch(kernel_of(kernel_index(D, pl, nw)), dim3(pl.grid), dim3(kThreads),
-                          (size_t)p.smem_bytes, s, tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
+  DLM_CUDA_TRY(dlm_launch_cluster(kernel_of(kernel_index(D, pl, nw)), dim3(pl.grid), dim3(kThreads), (size_t)p.smem_bytes, s,
+                                  (unsigned int)pl.team, tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
   return dlm_launch_ok(ctx, 1);
 }

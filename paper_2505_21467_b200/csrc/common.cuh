@@ -61,7 +61,8 @@ struct dlm_ctx {
   bool attn_team_force;         // tests: take the team schedule wherever it is possible, whatever the cost estimate says
   dlm_attn_plan_key attn_plan_key;   // of the last call's plan (nl = 0: none yet)
   dlm_attn_plan attn_plan;
-  int attn_smem_limit[20];      // dynamic shared memory the attention kernels may use on this device (0 = not set up yet)
+  int attn_clusters[17];        // clusters of so many attention blocks that the device runs at a time (0 = not asked yet, -1 = none)
+  int attn_smem_limit[24];      // dynamic shared memory the attention kernels may use on this device (0 = not set up yet)
 };
 
 // Writes the descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle,

@@ -436,3 +436,19 @@ def test_teams_of_half_m_tiles(dev, oracle, B, Hq, Hkv, D, Lcap, q_cap, cache_le
     assert sch["team"] > 1 and sch["chunk_rows"] == 64, sch
     for _ in range(2):   # and leave the counters clean
         _case(dev, oracle, 2, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len, seed=Hq, layer_begin=1, hint=max(cache_len))
+
+
+# teams whose blocks split the keys: tiles that end in either half of the keys or at its edge, blocks whose second half has nothing, rows
+# that end inside a warp or at its edge, chunks of 96, team sizes that do not divide the columns
+@pytest.mark.parametrize("D,Hq,Hkv,q_cap", [(128, 1, 1, 31), (128, 3, 1, 32), (128, 1, 1, 128), (64, 2, 1, 65), (128, 7, 1, 32), (64, 5, 1, 33)])
+@pytest.mark.parametrize("last", [1, 33, 63, 64, 65, 127])
+def test_teams_that_split_the_keys_at_the_edges(dev, oracle, D, Hq, Hkv, q_cap, last):
+    try:
+        for team in (2, 3, 7):
+            dlm.dlm_selftest_set_attn_team_max(dev.ctx, team, force=True)
+            cache_len, q_len = [640 + last, last], [q_cap, max(1, q_cap - 3)]
+            sch = _schedule(dev, 1, 2, Hq, Hkv, D, 1000, q_cap, 1, 640 + last)
+            assert sch["team"] == team or team == 7 and sch["team"] > 3, sch
+            _case(dev, oracle, 1, 2, Hq, Hkv, D, 1000, q_cap, cache_len, q_len, seed=last + team, hint=640 + last)
+    finally:
+        dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)

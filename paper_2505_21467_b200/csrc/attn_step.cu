@@ -91,6 +91,7 @@ struct AttnParams {
                    // every block then reduces its share of the unit's outputs over all the team's pieces
   int smem_bytes;           // dynamic shared memory of the launch
   FastDiv by_batch, by_rc, by_kv_heads, by_q_cap, by_team, by_live;
+  int hint_len;             // cached rows to expect (only a guess)
   float scale_log2;
   int* status;
   unsigned int* tickets;   // one zero-initialised counter per unit: pieces finished
@@ -656,6 +657,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t bar_pub = bar_pv_done + 32;                   // partial result of a segment stored by every softmax thread
   const uint32_t bar_team = bar_pub + 8;                         // team schedule: the other blocks' pieces are there
   const uint32_t bar_fold = bar_team + 8;                        // keys split: both halves' O, maxima and sums are there
+  const uint32_t bar_guess = bar_fold + 8;                       // K and V tile copied before the lengths were known [2]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -669,6 +671,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     mbar_init(bar_drain + 8, 1);
     mbar_init(bar_pub, (uint32_t)(kSingle ? n_live / 32 * (kKeys ? 2 : 1) : n_live));   // teams: one arrival per warp
     mbar_init(bar_team, 1);
+    mbar_init(bar_guess, 1);
+    mbar_init(bar_guess + 8, 1);
     mbar_init(bar_fold, (uint32_t)n_live / 16);     // one arrival per live warp of either half
     for (int i = 0; i < KS; ++i) {
       mbar_init(bar_k_full + 8 * i, 1);
@@ -701,8 +705,29 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     prefetch_tensormap(&tm_kn);
     prefetch_tensormap(&tm_vn);
   }
+  // Blocks of a single unit: the key tile that the block has first if the lengths are as expected is copied before they are read.  (Their
+  // chain -- a round trip, the share, the copy's issue -- stood before a call's first scores: K was asked for 2300 cycles after the
+  // wait for the kernel before, now 200.  One-layer calls: one sequence 8.55 -> 8.3 us, 32 KV heads 10.75 -> 10.25, an LLaDA layer 27.9 -> 27.6; 28
+  // layers in one call 25.65 -> 24.95; every 400 cycles that the copy comes later cost 0.15 - 0.2 us.)  That copy has barriers of its own;
+  // where the lengths are others, which all roles see alike, its data is dropped and the rings start as if it had not been.
   Segment one;
-  if (kSingle) decode_single(p, one);
+  int guess_first = 0, guess_n_ct = 0;
+  bool ahead = false, hit = false;   // there is such a copy; it is what the block needs first
+  if (kSingle) {
+    decode_single(p, one);
+    Segment guess = one;
+    set_single_lengths(p, guess, p.hint_len, p.q_cap);
+    ahead = guess.t_end > guess.t_begin;
+    guess_first = guess.t_begin;
+    guess_n_ct = guess.n_ct;
+    if (tid == 0) {   // for the translation of their addresses, not their values
+      prefetch_l2(p.cache_len + one.b);
+      if (p.q_len) prefetch_l2(p.q_len + one.b);
+    }
+  }
+  // barrier "full" of the i-th tile of a ring, and its phase: a copy made ahead takes the place of the first stage's first
+  auto full_bar = [&](uint32_t ring, uint32_t guess, uint32_t i, uint32_t stages) { return kSingle && hit && i == 0 ? guess : ring + 8 * (i % stages); };
+  auto full_parity = [&](uint32_t i, uint32_t stages) { return (i / stages - (kSingle && hit && i >= stages && i % stages == 0 ? 1u : 0u)) & 1u; };
   __syncwarp();
   tc_fence_before_sync();
   // the barriers exist and TMEM is there; in a team, so do the other blocks' barriers
@@ -733,6 +758,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       Lq = max(0, min(Lq, p.q_cap));
     }
     set_single_lengths(p, one, Lc, Lq);
+    const bool same = one.t_begin < one.t_end && one.t_begin == guess_first && (guess_first < guess_n_ct ? guess_first < one.n_ct : guess_n_ct == one.n_ct);
+    hit = ahead && same;
   };
   auto team_shape = [&]() {
     TeamShape a;
@@ -807,12 +834,36 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     setmaxnreg_dec<kRegsOther>();
     if (warp == 8) {
       // ================================================================= TMA producer
+      auto tile_bytes = [&](bool cache) { return (uint32_t)(cache ? min(kTileKeys, p.capacity) : p.fresh_box) * 128u * G::kPanels; };
+      auto copy_tile = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int z) {
+        for (int pn = 0; pn < G::kPanels; ++pn) tma_load_3d(dst + pn * kPanelBytes, map, bar, pn * 64, row, z);
+      };
       if (kSingle) {
         const int zq = (one.lc_layer * p.batch + one.b) * p.n_kv_heads + one.kvh;
-        if (lane == 0) expect_q();
+        const bool cache = guess_first < guess_n_ct;
+        const int row = cache ? guess_first * kTileKeys : (guess_first - guess_n_ct) * p.fresh_box;
+        const int z = cache ? zq + p.layer_begin * p.batch * p.n_kv_heads : zq;
+        if (lane == 0) {
+          expect_q();
+          if (ahead) {
+            mbar_expect_tx(bar_guess, tile_bytes(cache));
+            mbar_expect_tx(bar_guess + 8, tile_bytes(cache));
+          }
+        }
         wait_for_inputs();
-        if (lane == 0) copy_q(zq, one.rc);
+        if (lane == 0) {
+          copy_q(zq, one.rc);
+          if (ahead) {
+            copy_tile(sm_k, cache ? &tm_kc : &tm_kn, bar_guess, row, z);
+            copy_tile(sm_v, cache ? &tm_vc : &tm_vn, bar_guess + 8, row, z);
+          }
+        }
+        __syncwarp();
         read_lengths();
+        if (lane == 0 && ahead && !hit) {   // others go to the same shared memory, so not before these have landed
+          mbar_wait(bar_guess, 0, never_ptr);
+          mbar_wait(bar_guess + 8, 0, never_ptr);
+        }
       }
       if (lane == 0 && has_work) {
         SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
@@ -840,15 +891,18 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             const bool cache = t < g.n_ct;
             const int row = cache ? t * kTileKeys : (t - g.n_ct) * p.fresh_box;
             const int z = cache ? zc : zq;
-            const uint32_t bytes = (uint32_t)(cache ? min(kTileKeys, p.capacity) : p.fresh_box) * 128u * G::kPanels;
+            const uint32_t bytes = tile_bytes(cache);
+            if (kSingle && kt == 0 && hit) {   // on its way already
+              ++kt;
+              ++vt;
+              continue;
+            }
             {
               const uint32_t s = kt % KS;
               if (kt >= (uint32_t)KS) ok = mbar_wait_limit(bar_k_empty + 8 * s, ((kt / KS) - 1) & 1, abort_ptr, kLimit);
               if (!ok) break;
               mbar_expect_tx(bar_k_full + 8 * s, bytes);
-              for (int pn = 0; pn < G::kPanels; ++pn)
-                tma_load_3d(sm_k + s * G::kTileBytes + pn * kPanelBytes, cache ? &tm_kc : &tm_kn, bar_k_full + 8 * s,
-                            pn * 64, row, z);
+              copy_tile(sm_k + s * G::kTileBytes, cache ? &tm_kc : &tm_kn, bar_k_full + 8 * s, row, z);
               ++kt;
             }
             {
@@ -856,9 +910,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               if (vt >= (uint32_t)VS) ok = mbar_wait_limit(bar_v_empty + 8 * s, ((vt / VS) - 1) & 1, abort_ptr, kLimit);
               if (!ok) break;
               mbar_expect_tx(bar_v_full + 8 * s, bytes);
-              for (int pn = 0; pn < G::kPanels; ++pn)
-                tma_load_3d(sm_v + s * G::kTileBytes + pn * kPanelBytes, cache ? &tm_vc : &tm_vn, bar_v_full + 8 * s,
-                            pn * 64, row, z);
+              copy_tile(sm_v + s * G::kTileBytes, cache ? &tm_vc : &tm_vn, bar_v_full + 8 * s, row, z);
               ++vt;
             }
           }
@@ -868,9 +920,9 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         // this lane itself never had to give up (its last copies were issued before another role did, or a unit without key
         // tiles has its Q on the way).  They have landed long since unless the block is unwinding.
         for (uint32_t i = (kt > (uint32_t)KS ? kt - KS : 0); i < kt; ++i)
-          mbar_wait(bar_k_full + 8 * (i % KS), (i / KS) & 1, never_ptr);
+          mbar_wait(full_bar(bar_k_full, bar_guess, i, KS), full_parity(i, KS), never_ptr);
         for (uint32_t i = (vt > (uint32_t)VS ? vt - VS : 0); i < vt; ++i)
-          mbar_wait(bar_v_full + 8 * (i % VS), (i / VS) & 1, never_ptr);
+          mbar_wait(full_bar(bar_v_full, bar_guess + 8, i, VS), full_parity(i, VS), never_ptr);
         if (q_issued > 0) mbar_wait(bar_q_full, (q_issued - 1) & 1, never_ptr);
       }
     } else if (warp == 9 || warp == 10) {
@@ -943,13 +995,13 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           auto issue_next_s = [&]() -> bool {
             HalfStep hs;
             for (; si.skips(); ++si.t, ++kt) {   // (behind the copy, so that the arrival counts for this use of the buffer)
-              if (!wait(bar_k_full + 8 * (kt % KS), (kt / KS) & 1)) return false;
+              if (!wait(full_bar(bar_k_full, bar_guess, kt, KS), full_parity(kt, KS))) return false;
               mbar_arrive(bar_k_empty + 8 * (kt % KS));
             }
             if (!si.get(hs)) return true;
             const uint32_t ks = kt % KS;
             if (hs.first_of_tile) {
-              if (!wait(bar_k_full + 8 * ks, (kt / KS) & 1)) return false;
+              if (!wait(full_bar(bar_k_full, bar_guess, kt, KS), full_parity(kt, KS))) return false;
               tc_fence_after_sync();
             }
             issue_s(ks, hs.k0, (hs.nkeys + 15) & ~15, js & 1);
@@ -968,7 +1020,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           HalfStep hs;
           auto skip_v = [&]() -> bool {
             for (; pi.skips(); ++pi.t, ++vt) {
-              if (!wait(bar_v_full + 8 * (vt % VS), (vt / VS) & 1)) return false;
+              if (!wait(full_bar(bar_v_full, bar_guess + 8, vt, VS), full_parity(vt, VS))) return false;
               mbar_arrive(bar_v_empty + 8 * (vt % VS));
             }
             return true;
@@ -976,7 +1028,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           while (ok && (ok = skip_v()) && pi.get(hs)) {
             const uint32_t vs = vt % VS;
             if (hs.first_of_tile) {
-              ok = wait(bar_v_full + 8 * vs, (vt / VS) & 1);
+              ok = wait(full_bar(bar_v_full, bar_guess + 8, vt, VS), full_parity(vt, VS));
               if (!ok) break;
             }
             ok = wait(bar_p_ready + 16 * mt + 8 * (gt & 1), (gt >> 1) & 1);
@@ -1136,7 +1188,11 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
               // announce the P of the tile's first half-step, so it precedes that tile's P V
               // products (the two M tiles write the same zeros; with the keys split, the half that has them).
               const uint32_t vs = vt % VS;
-              ok = wait_warp(bar_v_full + 8 * vs, (vt / VS) & 1);
+              // (with the keys split, S of this tile does not show that the tile before the one before, whose V had the stage, is
+              // through; a wait for a phase works only when the one before it is over)
+              if (kKeys && gt > 0) ok = wait_warp(bar_pv_done + 16 * mt + 8 * ((gt - 1) & 1), ((gt - 1) >> 1) & 1);
+              if (!ok) break;
+              ok = wait_warp(full_bar(bar_v_full, bar_guess + 8, vt, VS), full_parity(vt, VS));
               if (!ok) break;
               const int per_row = G::kPanels * 8;
               for (int idx = row; idx < (n16 - valid) * per_row; idx += n_live_mt) {
@@ -1696,6 +1752,8 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
   p.by_q_cap = make_fast_div(q_cap);
   p.by_team = make_fast_div(pl.team);
   p.by_live = make_fast_div((pl.rows + 31) & ~31);
+  // a hint of 1 is how a caller says that nothing is cached yet (0 leaves the length open)
+  p.hint_len = cache_len_hint == 1 ? 0 : cache_len_hint > 0 && cache_len_hint < cache->capacity ? cache_len_hint : cache->capacity;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.status = &ctx->words->status;
   p.tickets = ctx->words->attn_unit_tickets;

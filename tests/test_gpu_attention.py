@@ -452,3 +452,12 @@ def test_teams_that_split_the_keys_at_the_edges(dev, oracle, D, Hq, Hkv, q_cap, 
             _case(dev, oracle, 1, 2, Hq, Hkv, D, 1000, q_cap, cache_len, q_len, seed=last + team, hint=640 + last)
     finally:
         dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)
+
+
+# blocks of a single unit ask for the key tile that the hint lets them expect before they read the lengths: hints below, at and beyond the lengths,
+# sequences without cached rows or without active ones, whole units and teams
+@pytest.mark.parametrize("D,Hq,Hkv,q_cap,nl", [(128, 4, 2, 24, 1), (64, 4, 2, 24, 1), (128, 28, 4, 32, 1), (64, 8, 8, 40, 3)])
+@pytest.mark.parametrize("hint", [1, 130, 640, 1100, 0])
+def test_lengths_other_than_the_hint(dev, oracle, D, Hq, Hkv, q_cap, nl, hint):
+    for seed, (cache_len, q_len) in enumerate([([0, 640, 17], [q_cap, 1, q_cap]), ([1100, 128, 129], [q_cap, 0, 7]), ([641, 0, 700], None)]):
+        _case(dev, oracle, nl, 3, Hq, Hkv, D, 1140, q_cap, cache_len, q_len, seed=seed + hint, hint=hint, layers=[nl - 1])

@@ -656,7 +656,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                                                                  // barriers: a parity wait cannot tell phases two apart
   const uint32_t bar_pub = bar_pv_done + 32;                   // partial result of a segment stored by every softmax thread
   const uint32_t bar_team = bar_pub + 8;                         // team schedule: the other blocks' pieces are there
-  const uint32_t bar_fold = bar_team + 8;                        // keys split: both halves' O, maxima and sums are there
+  const uint32_t bar_fold = bar_team + 8;                        // teams: both chains are through (keys split: maxima and sums there too)
   const uint32_t bar_guess = bar_fold + 8;                       // K and V tile copied before the lengths were known [2]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -673,7 +673,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     mbar_init(bar_team, 1);
     mbar_init(bar_guess, 1);
     mbar_init(bar_guess + 8, 1);
-    mbar_init(bar_fold, (uint32_t)n_live / 16);     // one arrival per live warp of either half
+    mbar_init(bar_fold, (uint32_t)n_live / (kKeys ? 16 : 32));     // one arrival per live warp (keys split: of either half)
     for (int i = 0; i < KS; ++i) {
       mbar_init(bar_k_full + 8 * i, 1);
       mbar_init(bar_k_empty + 8 * i, (uint32_t)n_chains);
@@ -1230,6 +1230,11 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           if (!kKeys || gt > 0) ok = wait_warp(bar_pv_done + 16 * mt + 8 * ((gt - 1) & 1), ((gt - 1) >> 1) & 1);
           if (!ok) break;
           tc_fence_after_sync();
+          if (kTeam && !kKeys) {   // the piece is laid out over K tiles, which the other M tile's products may still read
+            if (lane == 0) mbar_arrive(bar_fold);
+            ok = wait_warp(bar_fold, 0);
+            if (!ok) break;
+          }
           float w[2] = {1.f, 0.f};                               // of the key halves' O, at t_first and t_second
           uint32_t t_first = t_o, t_second = t_o;
           if (kKeys) {

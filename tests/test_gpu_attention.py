@@ -461,3 +461,27 @@ def test_teams_that_split_the_keys_at_the_edges(dev, oracle, D, Hq, Hkv, q_cap, 
 def test_lengths_other_than_the_hint(dev, oracle, D, Hq, Hkv, q_cap, nl, hint):
     for seed, (cache_len, q_len) in enumerate([([0, 640, 17], [q_cap, 1, q_cap]), ([1100, 128, 129], [q_cap, 0, 7]), ([641, 0, 700], None)]):
         _case(dev, oracle, nl, 3, Hq, Hkv, D, 1140, q_cap, cache_len, q_len, seed=seed + hint, hint=hint, layers=[nl - 1])
+
+
+# teams of two M tiles: the chain that is through first lays its rows out over the K tiles, which the other one may still read.  Launches back to
+# back with other lengths in between, every one the same
+@pytest.mark.parametrize("B,Hq,Hkv,q_cap", [(6, 16, 8, 128), (8, 8, 8, 250), (6, 16, 8, 65)])
+def test_teams_of_two_m_tiles(dev, oracle, B, Hq, Hkv, q_cap):
+    cap = 1000
+    try:
+        dlm.dlm_selftest_set_attn_team_max(dev.ctx, 2, force=True)
+        sch = _schedule(dev, 1, B, Hq, Hkv, 64, cap, q_cap, 1, 300)
+        assert sch["team"] == 2 and sch["chunk_rows"] == 256, sch
+        rng = np.random.default_rng(q_cap)
+        ck, cv = make_cache(1, B, Hkv, cap, 64, 5, device="cuda")
+        q, kn, vn = make_attn_inputs(1, B, Hq, Hkv, q_cap, 64, 6, device="cuda")
+        calls = [(_i32(rng.integers(0, 700, B)), _i32(rng.integers(1, q_cap + 1, B))) for _ in range(3)]
+        refs = [oracle_attn_layers(oracle, ck, cv, cl, q, kn, vn, ql)[0] for cl, ql in calls]
+        got = [[gpu_attn_step(dev, ck, cv, cl, q, kn, vn, ql, hint=300) for cl, ql in calls] for _ in range(20)]
+        assert dev.status() == 0
+        for i, ref in enumerate(refs):
+            assert_attn_close(got[0][i][0], got[0][i][1], ref, 0)
+            for launch in got[1:]:
+                assert torch.equal(launch[i][0], got[0][i][0]) and torch.equal(launch[i][1], got[0][i][1])
+    finally:
+        dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)

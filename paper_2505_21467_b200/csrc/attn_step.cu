@@ -628,7 +628,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t sm_bar = sm_v + VS * G::kTileBytes;             // barriers, 8 bytes each
   int* const flags = reinterpret_cast<int*>(smem_raw + smem_pad + (size_t)(p.n_mt + KS + VS) * G::kTileBytes + kBarrierBytes);
   volatile int* const abort_ptr = flags;        // raised by the first wait that gives up
-  volatile int* const never_ptr = flags + 1;    // stays 0: for waits that must not be cut short by an abort
+  volatile int* const never_ptr = flags + 1;    // for waits that must not be cut short by an abort; raised by one that runs out
   uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(flags + 2);
   volatile int* const merge_ok = flags + 3;
   volatile int* const any_empty = flags + 4;    // some batch element has no key tile at all
@@ -1406,9 +1406,10 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (kTeam && tid == 0 && *abort_ptr && one.T > 0) mbar_wait(bar_team, 0, never_ptr);
   __syncwarp();
   if (kTeam) cluster_arrive();
-  if (tid == 0 && *abort_ptr) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
   tc_fence_before_sync();
   __syncthreads();
+  // behind the barrier: another role may give up after this thread has come this far, and then its rows are not written
+  if (tid == 0 && (*abort_ptr || *never_ptr)) dlm_set_status(p.status, DLM_ERR_TIMEOUT);
   if (warp == 9) {
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);

@@ -485,3 +485,26 @@ def test_teams_of_two_m_tiles(dev, oracle, B, Hq, Hkv, q_cap):
                 assert torch.equal(launch[i][0], got[0][i][0]) and torch.equal(launch[i][1], got[0][i][1])
     finally:
         dlm.dlm_selftest_set_attn_team_max(dev.ctx, 1 << 20)
+
+
+# a block reports a give-up of any of its roles, also one that comes after the rows of its other M tile are done: units whole (of one segment and
+# of several), split, teams of one and of two M tiles; whichever waits happen to give up, a launch without an error status has every row right
+@pytest.mark.parametrize("name,B,Hq,Hkv,D,q_cap", [("whole", 37, 8, 4, 64, 80), ("whole", 80, 16, 2, 128, 17), ("split", 2, 28, 4, 128, 32),
+                                                   ("team", 1, 28, 4, 128, 32), ("team", 6, 16, 8, 64, 128)])
+def test_no_launch_that_gave_up_passes_for_good(dev, oracle, name, B, Hq, Hkv, D, q_cap):
+    cap = 300 if name == "whole" else 1400
+    ck, cv = make_cache(1, B, Hkv, cap, D, 5, device="cuda")
+    q, kn, vn = make_attn_inputs(1, B, Hq, Hkv, q_cap, D, 6, device="cuda")
+    cl = _i32(np.random.default_rng(B).integers(0, cap - q_cap, B))
+    try:
+        for hint in _each_schedule(dev, [name], 1, B, Hq, Hkv, D, cap, q_cap):
+            ref = oracle_attn_layers(oracle, ck, cv, cl, q, kn, vn)[0]
+            for limit in (0, 0, 0, 2_000_000_000):
+                dlm.dlm_selftest_set_wait_limit(dev.ctx, limit)
+                out, lse = gpu_attn_step(dev, ck, cv, cl, q, kn, vn, hint=hint)
+                status = dev.status()
+                assert status == 0 or limit == 0 and status == dlm.DLM_ERR_TIMEOUT
+                if status == 0:
+                    assert_attn_close(out, lse, ref, 0)
+    finally:
+        dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)

@@ -37,7 +37,8 @@ def test_chunk_edges(dev, oracle, B, L, V, kind):
 
 @pytest.mark.parametrize("L", [31, 32, 33, 64, 1024])
 def test_ranking_of_short_and_long_blocks(dev, oracle, L):
-    """The ranking by one warp (up to 32 positions) and by the block, k beyond and below the number of masked positions."""
+    """Blocks whose rows are merged by eight lanes each (up to 32 positions) and by four, all ranked by eight lanes a position; k beyond and
+    below the number of masked positions."""
     for k, n_masked in ((1, L), (7, L - 1), (L + 3, L // 2)) if L <= 64 else ((1, L), (L + 3, L // 2)):
         for seed in range(12):
             if _compare_scored(dev, oracle, make_logits(2, L, 513, (0.5, 6.0), 10 * L + seed), make_mask(2, L, n_masked, seed).numpy(), k, 0):
@@ -63,5 +64,20 @@ def test_tickets_of_few_masked_rows(dev, oracle, L):
 def test_merge_of_long_blocks(dev, oracle, L, V, kind):
     masked0 = make_mask(1, L, L - 3, V).numpy()
     masked0[0, :5] = 1
-    assert any(_compare_scored(dev, oracle, _inputs(1, L, V, L + V + seed), masked0, k, kind) for k in (0, 3) for seed in range(6))
+    # (ranked: plain rows, since those of _inputs share their top logit, so that their scores are near ties in every draw)
     assert _compare_scored(dev, oracle, _inputs(1, L, V, L + V), masked0, 0, kind)
+    for k in (3, L + 3):
+        assert any(_compare_scored(dev, oracle, make_logits(1, L, V, (0.5, 6.0), L + V + seed), masked0, k, kind) for seed in range(12))
+
+
+# rows of the same logits, hence the same score to the bit: the earlier position goes first, also when the two are eight positions or more
+# apart (another lane's or another round's) and in different words of the set of chosen ones
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("L,pair", [(32, (3, 11)), (32, (0, 31)), (40, (7, 39)), (130, (31, 32)), (130, (2, 129)), (1024, (100, 900))])
+def test_identical_rows_far_apart(dev, oracle, L, pair, kind):
+    z = make_logits(1, L, 513, (0.5, 2.0), L)
+    z[0, pair[0]] = make_logits(1, 1, 513, (1.0, 1.0), 1)[0, 0]
+    z[0, pair[0], 77] = 12.0                                      # 0.99 of the probability: the best row by every score
+    z[0, pair[1]] = z[0, pair[0]]
+    masked0 = np.ones((1, L), np.uint8)
+    assert _compare_scored(dev, oracle, z, masked0, 1, kind) and _compare_scored(dev, oracle, z, masked0, 2, kind)

@@ -508,3 +508,27 @@ def test_no_launch_that_gave_up_passes_for_good(dev, oracle, name, B, Hq, Hkv, D
                     assert_attn_close(out, lse, ref, 0)
     finally:
         dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
+
+
+# a key of NaN or +-inf reaches every row that it makes undefined, whichever block or key half it falls to, and no other row
+@pytest.mark.parametrize("name", ["whole", "split", "team"])
+@pytest.mark.parametrize("D,Hq,Hkv", [(128, 28, 4), (64, 12, 2)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("at", [3, 70, 1111, 1300])
+def test_a_key_that_is_not_finite(dev, name, D, Hq, Hkv, bad, at):
+    B, cap, q_cap, cl = 2, 1400, 32, [1301, 1200]
+    ck, cv = make_cache(1, B, Hkv, cap, D, 31, device="cuda")
+    q, kn, vn = make_attn_inputs(1, B, Hq, Hkv, q_cap, D, 32, device="cuda")
+    for hint in _each_schedule(dev, [name], 1, B, Hq, Hkv, D, cap, q_cap):
+        good, good_lse = gpu_attn_step(dev, ck, cv, _i32(cl), q, kn, vn, hint=hint)
+        ck[0, 0, 1, at, 5] = bad
+        out, lse = gpu_attn_step(dev, ck, cv, _i32(cl), q, kn, vn, hint=hint)
+        assert dev.status() == 0
+    undefined = torch.zeros(lse.shape, dtype=torch.bool, device="cuda")
+    group = Hq // Hkv
+    rows = q[0, 0, group:2 * group, :, 5].float()
+    undefined[0, 0, group:2 * group] = True if bad != bad else rows > 0     # a score of -inf only takes the key out
+    untouched = torch.ones_like(undefined)
+    untouched[0, 0, group:2 * group] = False
+    assert torch.equal(out.isnan().all(-1), undefined) and torch.equal(out.isnan().any(-1), undefined) and torch.equal(lse.isnan(), undefined)
+    assert torch.equal(out[untouched], good[untouched]) and torch.equal(lse[untouched], good_lse[untouched])

@@ -90,8 +90,16 @@ def test_out_projection_tiles(dev, oracle, B, q_cap, dm, Hq, D):
     _close(y, oracle.out_project(widen(o), widen(wo), None), "y")
 
 
-# K of one stage, of two (a stage holds 256 elements of K, or 128 with more than 64 rows), of one more, and of more than the ring holds
+# K of one stage, of two (a stage holds 256 elements of K, 128 with more than 64 rows, 64 where tiles are wide), of one more, and of more than the
+# ring holds
 @pytest.mark.parametrize("dm", [128, 256, 512, 576, 2304])
 @pytest.mark.parametrize("q_cap", [17, 100, 200])
 def test_qkv_projection_stages_of_k(dev, oracle, q_cap, dm):
     _qkv_case(dev, oracle, 1, q_cap, dm, 4, 1, 128, True, q_cap + dm)
+
+
+# the same for stages of 64 elements: 256-feature pair tiles of 64 rows, 192 and 256 of 128 rows, 384
+@pytest.mark.parametrize("dm", [64, 128, 192, 1024])
+@pytest.mark.parametrize("B,q_cap,Hq,Hkv,D", [(1, 100, 128, 16, 64), (1, 250, 72, 4, 128), (1, 130, 104, 4, 128), (2, 640, 28, 4, 128)])
+def test_qkv_projection_stages_of_one_panel(dev, oracle, B, q_cap, Hq, Hkv, D, dm):
+    _qkv_case(dev, oracle, B, q_cap, dm, Hq, Hkv, D, B * q_cap < 1000, q_cap + dm)

@@ -394,11 +394,6 @@ __device__ __forceinline__ bool elect_one_sync() {
   return pred != 0;
 }
 
-// Named barrier among `count` threads (a multiple of 32) of the block; id 0 is __syncthreads.
-__device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 // ---- packed pairs of floats (each operation rounds like its scalar form)
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
   uint64_t r;

@@ -83,7 +83,7 @@ struct AttnParams {
   int rows_total;  // group * q_cap: query rows per (layer, batch element, KV head)
   int n_rc;        // row chunks: rows_total cut into units of up to 256 rows (each re-reads the K/V tiles)
   int rows;        // query rows per unit = min(chunk_rows, rows_total)
-  int chunk_rows;  // 256 (two M tiles share every K/V tile), 128 (one M tile per unit) or 64 (half an M tile; teams)
+  int chunk_rows;  // 256 (two M tiles share every K/V tile), 128 (one M tile per unit), or 96 or 64 (less than one; teams)
   int n_mt;        // M tiles per unit (1 or 2)
   int fresh_box;   // rows per TMA box of the fresh K/V tensors = min(128, q_cap)
   int whole_units; // 1: deal whole units round-robin, no partials
@@ -127,7 +127,7 @@ __device__ __forceinline__ int tiles_of(int Lc, int Lq, int fresh_box) {
 // They are kernels of their own because what stands in front of the first copies is code that is not in the instruction
 // cache (another kernel has run in between): with all schedules in one kernel and the tables, a one-layer call of Dream issued
 // its first K copy 5360 cycles after that wait, now 2260.  Us a call, before -> now: one sequence 10.6 -> 9.3, window of 256
-// rows 18.2 -> 16.8, 8 sequences 19.2 -> 17.2, an LLaDA layer (whole units) 29.5 -> 28.0, 28 layers in one call 26.7 -> 25.3.
+// rows 18.2 -> 16.8, 8 sequences 19.2 -> 17.2, an LLaDA layer (whole units) 29.5 -> 28.0, 28 layers in one call 26.1 -> 25.4 back to back.
 __device__ __forceinline__ void decode_single(const AttnParams& p, Segment& g) {
   const int unit = p.team > 1 ? p.by_team.div(blockIdx.x) : (int)blockIdx.x;
   const int grp = p.by_batch.divmod(unit, g.b);
@@ -1488,8 +1488,8 @@ bool plan_shared_memory(int smem_limit, int head_dim, int batch, Plan& pl) {
   return pl.smem_bytes <= smem_limit;
 }
 
-// Device scratch of a call: room for the partial results of the split and team schedules whenever one of them is possible
-// at all, whichever the hint and the cost estimate then pick.
+// Device scratch of a call: room for the partial results of the split schedule whenever it is possible at all, whichever the hint
+// and the cost estimate then pick.
 struct WorkspaceSize {
   size_t o_bytes, ml_bytes;
 };
@@ -1501,7 +1501,8 @@ WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int 
 }
 
 // Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer), fitted to measurements of one-layer
-// calls: units split across all SMs take 23.4 us with 256 active rows of Dream at 1024 cached ones, 23.8 with 8 sequences of 32.
+// calls: units split across all SMs take 23.4 us with 256 active rows of Dream at 1024 cached ones, 23.8 with 8 sequences of 32.  (Taken when
+// the issuers' loop and the blocks of a single unit were slower than now; the teams' costs below are of the present form.)
 // Heads of 64, which were not in that fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule, the choice
 // was the fastest or within 2 % of it.
 constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer

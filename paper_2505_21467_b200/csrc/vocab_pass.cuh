@@ -376,8 +376,9 @@ __device__ __forceinline__ void select_batch(const Args& a, int score_kind, int 
   if (tid < kMaxBlockLen / 32) sc.sel[tid] = 0;
   if (tid == 0) sc.n_on = 0;
   // Up to 32 positions are one pass of eight lanes a row, one round trip to L2; more (WIDE) take four lanes a row, 64 rows a pass
-  // (4 x 64 positions of 6 chunks, a block's life with two passes of eight lanes: 346 us, now 313).  Which one is the kernel's, not a
-  // branch: this code runs once, and what it holds beside what it needs costs fetches and the streaming loop registers.
+  // (4 x 64 positions of 6 chunks, a block's life with two passes of eight lanes and the ranking of before: 352 us, now 320).  Which one
+  // is the kernel's, not a branch: this code runs once, and what it holds beside what it needs costs fetches and the streaming loop
+  // registers.
   if (!WIDE) merge_rows<KIND, 8, 3>(a, score_kind, p0, sc); else merge_rows<KIND, 4, 5>(a, score_kind, p0, sc);
   if (k <= 0) return;
   __syncthreads();

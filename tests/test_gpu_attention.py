@@ -364,8 +364,8 @@ def test_team_schedule_against_the_oracle_at_every_team_size(dev, oracle, NL, B,
 
 
 def test_team_schedule_repeated_launches_leave_the_counters_clean(dev, oracle):
-    """The team's arrival and departure counters are cleared by the last block to leave: many launches in a row on
-    the same units (also of different team sizes) stay correct, and so does a split-schedule call afterwards."""
+    """Teams meet on barriers of their own launch and count nothing in memory: many launches in a row on the same units (also of
+    different team sizes) stay correct, and so does a split-schedule call, which does count, afterwards."""
     shape = dict(NL=1, B=1, Hq=28, Hkv=4, D=128, Lcap=2200, q_cap=32)
     try:
         for i, tmax in enumerate((1 << 20, 5, 1 << 20, 2, 9)):
@@ -379,8 +379,8 @@ def test_team_schedule_repeated_launches_leave_the_counters_clean(dev, oracle):
 
 
 def test_team_members_without_key_tiles(dev, oracle):
-    """Sequences much shorter than the hint: most blocks of a team have no key tile and are done before the Q they were sent
-    has landed in the shared memory that the others' pieces go to.  Many launches back to back, every one the same."""
+    """Sequences much shorter than the hint: most blocks of a team have no key tile, send their rows' (m, l) only and are done while the Q and
+    the key tile they asked for may still be on their way.  Many launches back to back, every one the same."""
     B, Lcap, q_cap = 2, 2200, 32
     assert _schedule(dev, 1, B, 28, 4, 128, Lcap, q_cap, 1)["team"] > 2
     out, lse, _ = _case(dev, oracle, 1, B, 28, 4, 128, Lcap, q_cap, [0, 60], [1, 32], seed=811)
@@ -395,8 +395,7 @@ def test_team_members_without_key_tiles(dev, oracle):
 
 def test_team_schedule_gives_up_cleanly_when_its_waits_may_not_wait(dev, oracle):
     """The give-up path under the team schedule: with the wait limit at 0 every wait, the one for the team's other
-    blocks included, gives up at once.  The kernel ends normally with DLM_ERR_TIMEOUT, reading the status clears
-    the half-counted team counters, and the next call is correct."""
+    blocks included, gives up at once.  The kernel ends normally with DLM_ERR_TIMEOUT and the next call is correct."""
     shape = dict(NL=1, B=1, Hq=28, Hkv=4, D=128, Lcap=2200, q_cap=32)
     assert _schedule(dev, nl=1, **shape)["team"] > 1
     dlm.dlm_selftest_set_wait_limit(dev.ctx, 0)
@@ -434,7 +433,7 @@ def test_whole_units_as_many_as_sms_and_more(dev, oracle, B, Hkv, group, D, q_ca
 def test_teams_of_half_m_tiles(dev, oracle, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len):
     sch = _schedule(dev, 2, B, Hq, Hkv, D, Lcap, q_cap, 1, max(cache_len))
     assert sch["team"] > 1 and sch["chunk_rows"] == 64, sch
-    for _ in range(2):   # and leave the counters clean
+    for _ in range(2):
         _case(dev, oracle, 2, B, Hq, Hkv, D, Lcap, q_cap, cache_len, q_len, seed=Hq, layer_begin=1, hint=max(cache_len))
 
 

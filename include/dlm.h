@@ -93,11 +93,11 @@ int dlm_selftest_set_wait_limit(dlm_ctx* ctx, uint64_t limit_ns);
 
 /* Diagnostic: the most blocks (>= 1, else DLM_ERR_SHAPE; unlimited by default, the schedule's own maximum is 16)
  * that dlm_freecache_attn_step may give one unit in its team schedule, in the calls that follow.  That schedule
- * serves calls with few (layer, batch element, KV head, row chunk) units: a team of blocks (a thread-block cluster)
+ * serves calls with few (layer, batch element, KV head, row chunk) units: a team of blocks (mostly a thread-block cluster)
  * per unit, the unit's key tiles dealt among them, every block reducing its share of the unit's outputs over all the
  * team's partial results.  It is chosen when a cost estimate prefers it to the other schedules; force = 1 (0 by default; other
  * values DLM_ERR_SHAPE) takes it wherever it is possible at all: no more units than teams that the device runs
- * at a time and more than one key tile per unit.  max_blocks = 1 switches the schedule off, so that the same call can be run through the
+ * at a time, or at most half as many units as SMs, and more than one key tile per unit.  max_blocks = 1 switches the schedule off, so that the same call can be run through the
  * other schedules and the results compared; they agree to rounding, not bit for bit (the order of the merge
  * differs). */
 int dlm_selftest_set_attn_team_max(dlm_ctx* ctx, int max_blocks, int force);

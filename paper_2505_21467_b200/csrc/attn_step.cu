@@ -32,7 +32,8 @@
 // its own O, which is still in TMEM, in block order: the result is deterministic.  When the split
 // would cost more than it saves (the host estimates both) units are dealt whole, round-robin.
 // Calls with few units give each unit a team: a thread-block cluster that deals the unit's key tiles among its blocks and
-// exchanges the partial results through the blocks' shared memory (team_share and below).  A team's block with one M tile
+// exchanges the partial results through the blocks' shared memory (team_share and below), or, where no such clusters fit and a unit's
+// keys are many, a team that is no cluster and exchanges through L2 (WideArgs and below).  A cluster's block with one M tile
 // has a chain of warps to spare, so it splits the keys: warps 0-3 and issuer 9 take the first 64 keys of every tile, warps 4-7
 // and issuer 10 the others, each half with an O, maximum and sum of its own.
 #include <cuda_bf16.h>
@@ -405,6 +406,174 @@ __device__ __forceinline__ void team_reduce(const TeamShape& p, int row, int gro
   }
 }
 
+// Teams that are no cluster: the exchange goes through L2.  The device runs 33 clusters of 4 blocks at a time, 15 of 9, 7 of 16, on 148
+// SMs, and a cluster's blocks start together, once all of its SMs are free; two M tiles of heads of 128 have no room for the pieces
+// in shared memory.  Where units are few and long, more blocks a unit are worth more than the shorter exchange.  Us between
+// projections, the best other schedule -> this one: 2 layers of 3 sequences of 8 heads (2 KV heads) at 10000 cached rows 29.0 -> 24.5, 200 active
+// rows of 2 sequences of Dream at 4000 46.8 -> 40.9, 8 layers of one sequence at 10000 58.2 -> 55.9.
+// What a block of such a team works on after its share of the key tiles.  The team's pieces lie
+// in the workspace as [rank][M tile][head_dim / 4][R rows] 16-byte vectors (4 columns of a row) and
+// [rank][M tile][R rows] (m, l) pairs, R the unit's rows in an M tile rounded up to 32, 64 or 128; the unit's n_mt * head_dim / 4 * R
+// output vectors are dealt to the ranks in that storage order, rank r reducing vectors [lo, hi) over all pieces.
+// Everything the exchange needs, decoded by the caller and handed over by value.
+struct WideArgs {
+  __nv_bfloat16* out;
+  float* lse;
+  float* ws_o;
+  float* ws_ml;
+  unsigned int* arrive;        // the unit's two counters: blocks that have stored their piece ...
+  unsigned int* depart;        // ... and blocks that are past their wait for the first
+  size_t piece0;               // index of the team's first piece
+  size_t qrow0;                // output row of the KV head's first query row
+  FastDiv by_q_cap;
+  int team, n_mt, rows, rows_total, rank, Lq;
+  bool has_keys;
+  int r0, lo, hi;              // r0: the row chunk's first row among the KV head's rows
+  int r_shift;                 // log2 R
+  __device__ __forceinline__ WideArgs(const AttnParams& p, const Segment& g, int D)
+      : out(p.out), lse(p.lse), ws_o(p.ws_o), ws_ml(p.ws_ml), by_q_cap(p.by_q_cap), team(p.team), n_mt(p.n_mt), rows(p.rows),
+        rows_total(p.rows_total), Lq(g.Lq), has_keys(g.T > 0) {
+    const int unit = p.by_team.divmod(blockIdx.x, rank);
+    r0 = g.rc * p.chunk_rows;
+    qrow0 = (((size_t)g.lc_layer * p.batch + g.b) * p.n_q_heads + (size_t)g.kvh * p.group) * p.q_cap;
+    arrive = p.tickets + unit;
+    depart = arrive + kDlmMaxSplitUnits / 2;
+    r_shift = p.rows > 64 ? 7 : p.rows > 32 ? 6 : 5;
+    const int n_vec = (p.n_mt * (D / 4)) << r_shift;
+    lo = p.by_team.div(n_vec * rank);          // n_vec <= 8192, team <= 16
+    hi = p.by_team.div(n_vec * (rank + 1));
+    piece0 = (size_t)unit * p.team * p.n_mt;
+  }
+};
+
+// The two halves of the team schedule's exchange are functions of their own, not inlined: they run once per
+// launch, and inlined they changed the register allocation of the kernel's main loops (measured: 2 - 3 % on the
+// layer-batched calls, when all schedules were one kernel).
+//
+// Publisher warp, one thread: once every softmax thread of this block has stored its row of the block's piece
+// (bar_pub), count the block in the unit's arrival counter; when the whole team has arrived, let the softmax threads go on
+// (bar_team = bar_pub + 8).
+template <bool kNoWait>
+__device__ __noinline__ void wide_publish(const WideArgs p, uint32_t bar_pub, volatile int* abort_ptr) {
+  constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
+  if (!p.has_keys || !mbar_wait_limit(bar_pub, 0, abort_ptr, kLimit)) return;
+  __threadfence();
+  atomicAdd(p.arrive, 1u);
+  if (!wait_counter(p.arrive, (unsigned int)p.team, abort_ptr, kLimit)) return;
+  mbar_arrive(bar_pub + 8);
+  // every block of the team is past its wait on the arrival counter when the last one gets here: the last
+  // one clears both counters for the next launch
+  if (atomicAdd(p.depart, 1u) == (unsigned int)p.team - 1u) {
+    *p.arrive = 0;
+    *p.depart = 0;
+  }
+}
+
+// Softmax threads (all 256 of the block, whole warps).  Live ones store their row of the block's piece --
+// unnormalised O from TMEM at t_o if the block had key tiles, and (m, l), which is (-inf, 0) if it had none
+// (that piece's O is then never read).  Then all wait for the team and reduce this block's share of
+// the unit's output vectors over the C pieces, in rank order.  A thread's vectors lie in one row of an M tile, whose weights it takes
+// once, and what it needs of up to kMax pieces it asks L2 for at once: one round trip for the weights and the first vectors, one
+// for each further pair or single vector.  (Bulk copies of the shares into shared memory, 2 C of them issued by one lane, took 2400 -
+// 2900 cycles until they had landed, and the reduction from there 1400 - 6000.)  Returns false when a wait was given up.
+template <int D, int kMax>
+__device__ __forceinline__ void wide_reduce(const WideArgs& p) {
+  constexpr int kVec = 16 / kMax;             // vectors in flight
+  const int kVecs = (D / 4) << p.r_shift, R = 1 << p.r_shift;   // vectors of one M tile's piece
+  const int tid = threadIdx.x, C = p.team;
+  const int row = (p.lo + tid) & (R - 1);     // 256 is a multiple of R
+  const float4* const o = reinterpret_cast<const float4*>(p.ws_o) + ((p.piece0 * (D / 4)) << p.r_shift);
+  const size_t piece = (size_t)kVecs * p.n_mt;
+  int mt = -1;
+  bool real = false, active = false;
+  float w[kMax], m_all = 0.f, l_all = 0.f, inv = 0.f;
+  size_t qrow = 0;
+  for (int i = p.lo + tid; i < p.hi; i += 256 * kVec) {
+    float4 x[kVec][kMax];
+#pragma unroll
+    for (int u = 0; u < kVec; ++u)
+#pragma unroll
+      for (int c = 0; c < kMax; ++c)
+        if (c < C && i + 256 * u < p.hi) x[u][c] = __ldcg(o + c * piece + i + 256 * u);
+#pragma unroll
+    for (int u = 0; u < kVec; ++u) {
+      const int iu = i + 256 * u, mt_i = iu >= kVecs ? 1 : 0, qd = (iu - mt_i * kVecs) >> p.r_shift;
+      if (iu >= p.hi) break;
+      if (mt_i != mt) {
+        mt = mt_i;
+        const int r_unit = mt * 128 + row, r_kv = p.r0 + r_unit;
+        real = r_unit < ((p.rows + 31) & ~31) && r_kv < p.rows_total;
+        qrow = p.qrow0 + r_kv;                // rows of a KV head's query heads lie one after the other
+        int ir;
+        p.by_q_cap.divmod(r_kv, ir);
+        active = ir < p.Lq;
+        const float2* const a_ml = reinterpret_cast<const float2*>(p.ws_ml) + ((p.piece0 + mt) << p.r_shift) + row;
+        float2 ml[kMax];
+#pragma unroll
+        for (int c = 0; c < kMax; ++c) ml[c] = c < C && real ? __ldcg(a_ml + (((size_t)c * p.n_mt) << p.r_shift)) : make_float2(-CUDART_INF_F, 0.f);
+        m_all = -CUDART_INF_F;
+#pragma unroll
+        for (int c = 0; c < kMax; ++c)
+          m_all = fmaxf(m_all, ml[c].x);
+        l_all = 0.f;
+#pragma unroll
+        for (int c = 0; c < kMax; ++c) {
+          w[c] = ml[c].y != 0.f ? ex2_approx(ml[c].x - m_all) : 0.f;
+          l_all = fmaf(w[c], ml[c].y, l_all);
+        }
+        inv = active ? 1.f / l_all : 0.f;
+      }
+      if (!real) continue;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < kMax; ++c) {
+        if (c < C && w[c] != 0.f) {           // a piece without keys holds no O
+          acc.x = fmaf(w[c], x[u][c].x, acc.x);
+          acc.y = fmaf(w[c], x[u][c].y, acc.y);
+          acc.z = fmaf(w[c], x[u][c].z, acc.z);
+          acc.w = fmaf(w[c], x[u][c].w, acc.w);
+        }
+      }
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(active ? acc.x * inv : 0.f, active ? acc.y * inv : 0.f);
+      const __nv_bfloat162 h1 = __floats2bfloat162_rn(active ? acc.z * inv : 0.f, active ? acc.w * inv : 0.f);
+      *reinterpret_cast<uint2*>(p.out + qrow * D + qd * 4) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+      if (qd == 0 && p.lse) p.lse[qrow] = active ? (m_all + lg2_approx(l_all)) * 0.6931471805599453f : -CUDART_INF_F;
+    }
+  }
+}
+
+template <int D, bool kNoWait>
+__device__ __noinline__ bool wide_exchange(const WideArgs p, uint32_t bar_pub, volatile int* abort_ptr, bool live, uint32_t t_o,
+                                           bool has_tiles, float m_used, float l_run) {
+  constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
+  const int tid = threadIdx.x, mt = tid >> 7, row = tid & 127;
+  if (live) {
+    const size_t mine = p.piece0 + (size_t)p.rank * p.n_mt + mt;
+    if (has_tiles) {
+      float4* po = reinterpret_cast<float4*>(p.ws_o) + ((mine * (D / 4)) << p.r_shift) + row;
+      uint32_t v[32];
+#pragma unroll 1
+      for (int c = 0; c < D / 32; ++c) {
+        tmem_ld32(t_o + c * 32, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          __stcg(po + ((c * 8 + j) << p.r_shift), make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                              __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
+      }
+    }
+    __stcg(reinterpret_cast<float2*>(p.ws_ml) + (mine << p.r_shift) + row, make_float2(m_used, l_run));
+    // no fence here: the arrival below orders the stores before the publisher's wait (block scope), and the
+    // publisher's fence before it counts the block in carries them to device scope
+    mbar_arrive(bar_pub);
+  }
+  if (!mbar_wait_warp(bar_pub + 8, 0, abort_ptr, kLimit)) return false;
+  if (p.team <= 8) wide_reduce<D, 8>(p); else wide_reduce<D, 16>(p);
+  __syncwarp();
+  return true;
+}
+
 // A key tile is processed in half-steps of up to 64 keys.  Each M tile has two 64-column score
 // buffers in TMEM used alternately, so the scores of the half-step after next are computed by the
 // tensor pipe while the softmax warps work on the current one: they never wait for scores in the
@@ -594,7 +763,7 @@ __device__ __noinline__ bool softmax_half_ragged(uint32_t t_s, uint32_t t_o, int
   return true;
 }
 
-enum BlockWork { kManySegments, kOneUnit, kPartOfTeam };   // what a block of a launch has
+enum BlockWork { kManySegments, kOneUnit, kPartOfTeam, kPartOfWideTeam };   // what a block of a launch has
 
 // kNoWait = true is the instantiation a test selects to run the give-up path: every wait on work still to come tests
 // its barrier once and gives up if the data is not there yet (waits that let issued copies and MMAs finish keep the
@@ -609,7 +778,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   constexpr uint64_t kLimit = kNoWait ? 0ull : kWaitLimitNs;
   // One M tile per block: the two chains of warps that otherwise have an M tile each share it and split the keys, chain h taking
   // keys 64 h .. 64 h + 63 of every tile into an O, maximum and sum of its own, folded at the end.
-  constexpr bool kSingle = kWork != kManySegments, kTeam = kWork == kPartOfTeam, kKeys = kTeam && kChunk <= 128;
+  constexpr bool kSingle = kWork != kManySegments, kTeam = kWork == kPartOfTeam, kWide = kWork == kPartOfWideTeam, kKeys = kTeam && kChunk <= 128;
   const int n_chains = kKeys ? 2 : p.n_mt;
   // softmax threads that own a real query row, rounded up to whole warps (tid 0 .. n_live-1; keys split: of either half)
   const int n_live = (p.rows + 31) & ~31;
@@ -669,7 +838,7 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     mbar_init(bar_q_empty, (uint32_t)n_chains);     // one commit per MMA issuer
     mbar_init(bar_drain, 1);
     mbar_init(bar_drain + 8, 1);
-    mbar_init(bar_pub, (uint32_t)(kSingle ? n_live / 32 * (kKeys ? 2 : 1) : n_live));   // teams: one arrival per warp
+    mbar_init(bar_pub, (uint32_t)(kTeam ? n_live / 32 * (kKeys ? 2 : 1) : n_live));   // clusters: one arrival per warp
     mbar_init(bar_team, 1);
     mbar_init(bar_guess, 1);
     mbar_init(bar_guess + 8, 1);
@@ -1062,6 +1231,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       }
       if (kTeam && lane == 0 && one.T > 0) {
         team_expect<D>(team_shape(), bar_team, one.T, one.t_end > one.t_begin);
+      } else if (kWide && lane == 0) {
+        wide_publish<kNoWait>(WideArgs(p, one, D), bar_pub, abort_ptr);
       } else if (!kSingle && lane == 0 && has_work && !p.whole_units) {
         SegmentWalker<kSingle> walk(p, sched, blockIdx.x);
         Segment g = one;
@@ -1172,6 +1343,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             } else if (kTeam) {   // a piece without key tiles
               const float none[2] = {0.f, 0.f};
               lay_out_piece(false, 0, 0, none, -CUDART_INF_F, 0.f);
+            } else if (kWide) {
+              ok = wide_exchange<D, kNoWait>(WideArgs(p, g, D), bar_pub, abort_ptr, true, t_o, false, -CUDART_INF_F, 0.f);
             }
             continue;
           }
@@ -1263,6 +1436,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           uint32_t v[32];
           if (kTeam) {
             lay_out_piece(true, t_first, t_second, w, m_used, l_run);
+          } else if (kWide) {
+            ok = wide_exchange<D, kNoWait>(WideArgs(p, g, D), bar_pub, abort_ptr, true, t_o, true, m_used, l_run);
           } else if (kSingle || g.slot < 0) {
             const float inv = active ? 1.f / l_run : 0.f;
             constexpr int kChunks = kKeys ? D / 64 : D / 32;
@@ -1394,6 +1569,8 @@ attn_step_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         }
       }
     }
+    if (kWide && tid >= n_live && one.T > 0)   // warps without a row of their own help with the reduction
+      wide_exchange<D, kNoWait>(WideArgs(p, one, D), bar_pub, abort_ptr, false, 0, false, 0.f, 0.f);
     if (kTeam && one.T > 0) {
       // teams: the columns that this block finishes, by all softmax threads
       if (mbar_wait_warp(bar_pub, 0, abort_ptr, kLimit) && mbar_wait_warp(bar_team, 0, abort_ptr, kLimit)) {
@@ -1437,9 +1614,10 @@ bool register_budget_ok(const cudaFuncAttributes& a) {
 // tiles) / 128 (one; in teams with the keys split); normal / no-wait (test) waits.
 using AttnKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                             const AttnParams);
+constexpr int kKernels = 16;
 inline int kernel_index(int head_dim, const dlm_attn_plan& pl, bool no_wait) {
   const bool narrow = pl.single ? pl.n_mt == 1 : pl.chunk_rows == 128;
-  return (head_dim == 128 ? 0 : 1) + (narrow ? 2 : 0) + (pl.team > 1 ? 8 : pl.single ? 4 : 0) + (no_wait ? 12 : 0);
+  return (head_dim == 128 ? 0 : 1) + (narrow ? 2 : 0) + (pl.wide ? 12 : pl.team > 1 ? 8 : pl.single ? 4 : 0) + (no_wait ? kKernels : 0);
 }
 template <bool kNoWait>
 AttnKernel kernel_of_waits(int which) {
@@ -1455,10 +1633,14 @@ AttnKernel kernel_of_waits(int which) {
     case 9: return attn_step_sm100_kernel<64, 256, kPartOfTeam, kNoWait>;
     case 10: return attn_step_sm100_kernel<128, 128, kPartOfTeam, kNoWait>;
     case 11: return attn_step_sm100_kernel<64, 128, kPartOfTeam, kNoWait>;
+    case 12: return attn_step_sm100_kernel<128, 256, kPartOfWideTeam, kNoWait>;
+    case 13: return attn_step_sm100_kernel<64, 256, kPartOfWideTeam, kNoWait>;
+    case 14: return attn_step_sm100_kernel<128, 128, kPartOfWideTeam, kNoWait>;
+    case 15: return attn_step_sm100_kernel<64, 128, kPartOfWideTeam, kNoWait>;
     default: return nullptr;   // teams on two M tiles of heads of 128: their pieces have no room in shared memory
   }
 }
-AttnKernel kernel_of(int which) { return which >= 12 ? kernel_of_waits<true>(which - 12) : kernel_of_waits<false>(which); }
+AttnKernel kernel_of(int which) { return which >= kKernels ? kernel_of_waits<true>(which - kKernels) : kernel_of_waits<false>(which); }
 
 // First use of an attention kernel on a context's device: checks the register budget and opts in to
 // all the dynamic shared memory the device allows a block (less the kernel's static part).
@@ -1470,7 +1652,7 @@ int configure_kernel(dlm_ctx* ctx, int which, const void* kern) {
   const int limit = ctx->max_smem_optin - (int)a.sharedSizeBytes;
   if (limit <= 0) return DLM_ERR_UNSUPPORTED;
   DLM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  if (which % 12 >= 8) DLM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  if (which % kKernels >= 8 && which % kKernels < 12) DLM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   ctx->attn_smem_limit[which] = limit;
   return DLM_OK;
 }
@@ -1484,12 +1666,12 @@ bool plan_shared_memory(int smem_limit, int head_dim, int batch, Plan& pl) {
   const int tile = head_dim / 64 * kPanelBytes;
   const int stages = head_dim == 128 ? Geometry<128>::kStages : Geometry<64>::kStages;
   pl.smem_bytes = 1024 + (pl.n_mt + 2 * stages) * tile + kBarrierBytes + kFlagBytes +
-                  (pl.team > 1 ? kFoldBytes + team_bytes(head_dim, pl.team, (pl.rows + 31) & ~31) : pl.single ? 0 : 4 * sched_ints(batch));
+                  (pl.team > 1 && !pl.wide ? kFoldBytes + team_bytes(head_dim, pl.team, (pl.rows + 31) & ~31) : pl.single ? 0 : 4 * sched_ints(batch));
   return pl.smem_bytes <= smem_limit;
 }
 
-// Device scratch of a call: room for the partial results of the split schedule whenever it is possible at all, whichever the hint
-// and the cost estimate then pick.
+// Device scratch of a call: room for the partial results of the split schedule and of teams through L2 whenever one of them is possible
+// at all, whichever the hint and the cost estimate then pick.
 struct WorkspaceSize {
   size_t o_bytes, ml_bytes;
 };
@@ -1500,11 +1682,8 @@ WorkspaceSize workspace_size(const dlm_ctx* ctx, const dlm_kv_cache* cache, int 
   return {slots * n_mt * 128 * cache->head_dim * sizeof(float), slots * n_mt * 128 * 2 * sizeof(float)};
 }
 
-// Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer), fitted to measurements of one-layer
-// calls: units split across all SMs take 23.4 us with 256 active rows of Dream at 1024 cached ones, 23.8 with 8 sequences of 32.  (Taken when
-// the issuers' loop and the blocks of a single unit were slower than now; the teams' costs below are of the present form.)
-// Heads of 64, which were not in that fit: 15 calls (1 - 28 layers, 2 - 1280 units, 3 - 25 key tiles) timed under every schedule, the choice
-// was the fastest or within 2 % of it.
+// Costs of a block's work in key tiles of two M tiles (2.2 us on a Dream-shaped layer): between units dealt whole and split, and between
+// chunks of 256 and 128.
 constexpr double kTileCost[2] = {0.86, 1.0};     // one key tile, for one / two M tiles: the softmax chain hardly gets longer
 constexpr double kSplitCost[2] = {2.5, 4.0};     // the split schedule's partial store, wait and merge of one further piece ...
 constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond that
@@ -1514,33 +1693,56 @@ constexpr double kSplitPiece = 0.7;              // ... and of each piece beyond
 // 2 - 4 us slower at one and two, equal at three, 1 - 2 us faster at four.
 constexpr double kSplitManyCost[2] = {3.2, 2.7};
 
-// The team schedule's call in us, fitted to 190 one-layer calls (28 shapes of six models' heads, 1 - 256 active and 0 - 4096 cached rows, 1 -
-// 8 sequences, every team size that fits, rows in chunks of 64, 96 and 128; rms error 6 %).  t: the key tiles of the block with the most;
-// r: rows of a piece / 128; d: head_dim / 128; full: the teams' part of the clusters that the device runs at a time; g: blocks per SM;
-// even: all blocks finish equally many columns.  Of the teams timed it takes the fastest or one within 5 % for every shape but one (11 %).
-// In the unit above a call of whole units takes (us - kWholeCall) / kTileUs.
-constexpr double kWholeCall = 3.2, kTileUs = 2.2;
-double team_us(double t, double r, double d, int team, double full, double g, bool even) {
-  return 4.9 + t * (0.55 + 0.45 * d) + 1.6 * r + 0.2 * team * full + 0.5 * t * d * g * g + (even ? 0.0 : 0.25);
+// A call of at most as many units as SMs in us, for each schedule, fitted to 515 calls (1 - 16 layers, 1 - 8 sequences, five models' heads of 128
+// and 64, 8 - 200 active and 100 - 10000 cached rows) timed under every schedule, row chunk and team size that is possible, back to
+// back and between projections (weighted 1 : 2, since most calls stand in a layer).  The teams' terms for rows and ragged tiles are rounded
+// towards smaller chunks.  Between projections 28 of these calls were 3 - 34 % slower than before there were clusters, with costs that took heads
+// of 64 for as dear as those of 128 and without teams through L2; now 10 are, by 3 - 7 %.  Back to back it was 79, now 18, most by 3 - 10 %;
+// 8 active rows of 8 - 32 KV heads at 4000 cached rows, where a cluster waits for all of its SMs, by 18 - 25 % (faster between projections).
+struct CallShape {
+  double t;      // key tiles of the block with the most, ragged ones by UnitTiles::cost
+  double two;    // 1 with two M tiles a block, else 0
+  double r;      // rows of a unit, in whole warps, / 128
+  double d;      // head_dim / 128
+  double g;      // blocks per SM
+  double beyond; // 1 with more blocks than half of the SMs: the next call's cannot set themselves up beside them
+};
+double whole_us(const CallShape& c) { return 3.64 + c.t * (0.92 + 0.64 * c.two + 0.31 * c.d + 0.58 * c.g * c.d) + 0.73 * c.r; }
+// full: the teams' part of the clusters that the device runs at a time; even: all blocks finish equally many columns
+double team_us(const CallShape& c, int team, double full, bool even) {
+  const double t = c.t * (1 + c.two);
+  return 4.2 + t * (0.74 + 0.23 * c.d + 0.47 * c.d * c.g * c.g) + c.r * (1.2 + 0.9 * c.d) + 0.19 * team * full + (even ? 0.0 : 0.24) + 0.6 * c.beyond;
 }
+double wide_us(const CallShape& c) { return 5.08 + c.t * (1.16 + 0.62 * c.two + 0.4 * c.g * c.d) + 2.59 * c.r * c.d + 1.58 * c.beyond; }
+// c.t: key tiles of a share, each counted in full; pieces: shares per unit
+double split_us(const CallShape& c, double pieces) {
+  return 8.42 + c.t * (1.04 + 0.59 * c.two - 0.36 * c.d + 1.11 * c.g * c.d) + 2.07 * c.two + 1.14 * pieces;
+}
+constexpr double kWholeCall = 3.2, kTileUs = 2.2;   // us of a call of more units than SMs: kWholeCall + kTileUs * its cost in key tiles
 
-// A unit's key tiles: the cache's, then the fresh rows'.
+// A unit's key tiles: the cache's, then the fresh rows'.  (Where the keys are split over a block's two chains, half a tile takes nearly as long as
+// a whole one.)
+constexpr double kRagged = 0.5, kRaggedSplitKeys = 0.6;
 struct UnitTiles {
   long long len, q_cap, box, n_cache, n;
   UnitTiles(long long len_, long long q_cap_) : len(len_), q_cap(q_cap_), box(q_cap_ < 128 ? q_cap_ : 128), n_cache((len_ + 127) / 128),
                                                 n(n_cache + (q_cap_ + 127) / 128) {}
-  // what tiles [from, to) cost: a ragged one 0.3 and 0.7 of its share
-  double cost(long long from, long long to) const {
+  // what tiles [from, to) cost: a ragged one `ragged` and the rest by its keys
+  double cost(long long from, long long to, double ragged) const {
     double sum = 0;
     for (long long i = from; i < to; ++i) {
       const long long left = i < n_cache ? len - i * 128 : q_cap - (i - n_cache) * box, most = i < n_cache ? 128 : box;
-      sum += 0.3 + 0.7 / 128 * (double)(left < most ? left : most);
+      sum += ragged + (1.0 - ragged) / 128 * (double)(left < most ? left : most);
     }
     return sum;
   }
 };
 
-// The best plan with row chunks of `chunk_rows`, and its estimated cost.
+CallShape call_shape(const dlm_ctx* ctx, const Plan& pl, int head_dim, double tiles) {
+  return {tiles, pl.n_mt == 2 ? 1.0 : 0.0, ((pl.rows + 31) & ~31) / 128.0, head_dim / 128.0, (double)pl.grid / ctx->num_sms, pl.grid * 2 > ctx->num_sms ? 1.0 : 0.0};
+}
+
+// The best plan of whole or split units with row chunks of `chunk_rows`, and its estimated cost.
 double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
   pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
   pl.chunk_rows = chunk_rows;
@@ -1556,6 +1758,7 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
   double best = (double)(((units + sms - 1) / sms) * tiles_unit) * tile;
   pl.whole_units = 1;
   pl.team = 1;
+  pl.wide = 0;
   pl.grid = (int)(units < sms ? units : sms);
   if (!may_split) return best;
   // units split across blocks: equal shares, but a partial store per block and a merge per unit
@@ -1569,6 +1772,15 @@ double plan_chunked(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n
     if (t < best) { best = t; pl.whole_units = 0; pl.grid = sms; }
   }
   return best;
+}
+
+// The us of a plan of whole or split units of that cost.
+double chunked_us(const dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int q_cap, int len, double cost, const Plan& pl) {
+  const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
+  const UnitTiles tiles(len, q_cap);
+  if (units > ctx->num_sms) return kWholeCall + kTileUs * cost;
+  if (pl.whole_units) return whole_us(call_shape(ctx, pl, cache->head_dim, tiles.cost(0, tiles.n, kRagged)));
+  return split_us(call_shape(ctx, pl, cache->head_dim, (double)((units * tiles.n + pl.grid - 1) / pl.grid)), (double)pl.grid / (double)units);
 }
 
 // How many clusters of `team` blocks, one block per SM, the device runs at a time (0: none).  It depends on which SMs a die has: 74 of 2,
@@ -1598,7 +1810,7 @@ int team_clusters(dlm_ctx* ctx, int team) {
   return known > 0 ? known : 0;
 }
 
-// The best plan with teams on row chunks of `chunk_rows`, and its estimated cost (negative: there is none).
+// The best plan with teams on row chunks of `chunk_rows`, and its estimated us (negative: there is none).
 double plan_teams(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
   pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
   pl.chunk_rows = chunk_rows;
@@ -1606,6 +1818,7 @@ double plan_teams(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads
   pl.rows = pl.rows_total < chunk_rows ? pl.rows_total : chunk_rows;
   pl.n_mt = (pl.rows + 127) / 128;
   pl.whole_units = pl.single = 1;
+  pl.wide = 0;
   const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
   const UnitTiles tiles(len, q_cap);
   Plan at = pl;
@@ -1615,10 +1828,10 @@ double plan_teams(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads
     const int clusters = team_clusters(ctx, team);
     if (!plan_shared_memory(ctx->max_smem_optin, cache->head_dim, cache->batch, at) || units > clusters) continue;
     double most = 0;
-    for (int r = 0; r < team; ++r) most = fmax(most, tiles.cost(tiles.n * r / team, tiles.n * (r + 1) / team));
-    const double us = team_us(most * pl.n_mt, ((pl.rows + 31) & ~31) / 128.0, cache->head_dim / 128.0, team, (double)units / clusters,
-                              (double)(units * team) / ctx->num_sms, (cache->head_dim / 8) % team == 0);
-    const double t = (us - kWholeCall) / kTileUs;
+    for (int r = 0; r < team; ++r)
+      most = fmax(most, tiles.cost(tiles.n * r / team, tiles.n * (r + 1) / team, pl.n_mt == 1 ? kRaggedSplitKeys : kRagged));
+    at.grid = (int)units * team;
+    const double t = team_us(call_shape(ctx, at, cache->head_dim, most), team, (double)units / clusters, (cache->head_dim / 8) % team == 0);
     if (best < 0 || t < best) {
       best = t;
       pl.team = team;
@@ -1626,6 +1839,33 @@ double plan_teams(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads
     }
   }
   return best;
+}
+
+// The best plan with teams that exchange through L2, and its estimated us (negative: there is none): the smallest team that reaches the
+// fewest key tiles per block.  They meet in memory, so all blocks have to run at a time: one per SM.
+double plan_wide(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, int q_cap, int len, int chunk_rows, Plan& pl) {
+  pl.rows_total = (n_q_heads / cache->n_kv_heads) * q_cap;
+  pl.chunk_rows = chunk_rows;
+  pl.n_rc = (pl.rows_total + chunk_rows - 1) / chunk_rows;
+  pl.rows = pl.rows_total < chunk_rows ? pl.rows_total : chunk_rows;
+  pl.n_mt = (pl.rows + 127) / 128;
+  pl.whole_units = pl.single = pl.wide = 1;
+  const int sms = ctx->num_sms < kMaxGrid ? ctx->num_sms : kMaxGrid;
+  const long long units = (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc;
+  const UnitTiles tiles(len, q_cap);
+  if (units * 2 > sms) return -1;
+  long long team = ctx->attn_team_max < kTeamMax ? ctx->attn_team_max : kTeamMax;
+  if (team > sms / units) team = sms / units;
+  if (team > tiles.n) team = tiles.n;
+  if (team <= 1) return -1;
+  const long long per_block = (tiles.n + team - 1) / team;
+  team = (tiles.n + per_block - 1) / per_block;
+  if (team <= 1) return -1;
+  pl.team = (int)team;
+  pl.grid = (int)(units * team);
+  double most = 0;
+  for (int r = 0; r < team; ++r) most = fmax(most, tiles.cost(tiles.n * r / team, tiles.n * (r + 1) / team, kRagged));
+  return wide_us(call_shape(ctx, pl, cache->head_dim, most));
 }
 
 // Row chunks of 256 (two M tiles sharing every K/V tile) read K/V once per KV head and cost little more per key tile than
@@ -1642,14 +1882,16 @@ Plan make_plan(dlm_ctx* ctx, const dlm_kv_cache* cache, int nl, int n_q_heads, i
     if (c < cost) { pl = other; cost = c; }
   }
   pl.single = pl.whole_units && (long long)nl * cache->batch * cache->n_kv_heads * pl.n_rc <= pl.grid;
-  if (pl.whole_units) {   // against teams, which deal a unit's tiles, a ragged tile counts for what it is
-    const UnitTiles tiles(len, q_cap);
-    cost *= tiles.cost(0, tiles.n) / (double)tiles.n;
-  }
+  cost = chunked_us(ctx, cache, nl, q_cap, len, cost, pl);
   bool forced = ctx->attn_team_force;
   for (int chunk : {256, 128, 96, 64}) {
     if (chunk < 256 && pl.rows_total <= chunk) continue;   // all rows in one chunk: as with 256
     const double c = plan_teams(ctx, cache, nl, n_q_heads, q_cap, len, chunk, other);
+    if (c >= 0 && (c < cost || forced)) { pl = other; cost = c; forced = false; }
+  }
+  for (int chunk : {256, 128}) {
+    if (chunk < 256 && pl.rows_total <= chunk) continue;
+    const double c = plan_wide(ctx, cache, nl, n_q_heads, q_cap, len, chunk, other);
     if (c >= 0 && (c < cost || forced)) { pl = other; cost = c; forced = false; }
   }
   const WorkspaceSize ws = workspace_size(ctx, cache, nl, n_q_heads, q_cap);
@@ -1778,6 +2020,6 @@ extern "C" int dlm_freecache_attn_step(dlm_ctx* ctx, const dlm_kv_cache* cache, 
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DLM_CUDA_TRY(dlm_launch_cluster(kernel_of(kernel_index(D, pl, nw)), dim3(pl.grid), dim3(kThreads), (size_t)p.smem_bytes, s,
-                                  (unsigned int)pl.team, tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
+                                  (unsigned int)(pl.wide ? 1 : pl.team), tm_q, tm_kc, tm_vc, tm_kn, tm_vn, p));
   return dlm_launch_ok(ctx, 1);
 }

@@ -38,6 +38,7 @@ struct dlm_map_cache {
 struct dlm_attn_plan {
   int n_mt, rows, rows_total, n_rc, grid, whole_units, chunk_rows, team;
   int single;      // whole units or teams, and no block has more than one unit (or piece of one)
+  int wide;        // teams that are no cluster: they exchange through L2
   int smem_bytes;
   size_t ws_o_bytes, ws_ml_bytes;
 };
@@ -62,7 +63,7 @@ struct dlm_ctx {
   dlm_attn_plan_key attn_plan_key;   // of the last call's plan (nl = 0: none yet)
   dlm_attn_plan attn_plan;
   int attn_clusters[17];        // clusters of so many attention blocks that the device runs at a time (0 = not asked yet, -1 = none)
-  int attn_smem_limit[24];      // dynamic shared memory the attention kernels may use on this device (0 = not set up yet)
+  int attn_smem_limit[32];      // dynamic shared memory the attention kernels may use on this device (0 = not set up yet)
 };
 
 // Writes the descriptor of a bf16 tensor of `rank` dimensions (sizes, byte strides of dimensions 1 .., box), 128-byte swizzle,

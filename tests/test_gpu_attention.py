@@ -531,3 +531,29 @@ def test_a_key_that_is_not_finite(dev, name, D, Hq, Hkv, bad, at):
     untouched[0, 0, group:2 * group] = False
     assert torch.equal(out.isnan().all(-1), undefined) and torch.equal(out.isnan().any(-1), undefined) and torch.equal(lse.isnan(), undefined)
     assert torch.equal(out[untouched], good[untouched]) and torch.equal(lse[untouched], good_lse[untouched])
+
+
+# teams that are no cluster: two M tiles of heads of 128, whose pieces have no room in shared memory, and more blocks a unit than clusters of that
+# size fit the device; ragged rows, an inactive element, blocks without a key tile; many launches, which leave the counters clean, and one that gives up
+@pytest.mark.parametrize("NL,B,Hq,Hkv,D,q_cap,lc", [(1, 2, 28, 4, 128, 200, 2000), (2, 3, 8, 2, 128, 32, 5000), (8, 1, 28, 4, 128, 32, 5000), (2, 2, 8, 2, 64, 32, 10000)])
+def test_teams_that_exchange_through_l2(dev, oracle, NL, B, Hq, Hkv, D, q_cap, lc):
+    cap = lc + q_cap
+    sch = _schedule(dev, NL, B, Hq, Hkv, D, cap, q_cap, NL, lc)
+    # (of clusters of 10 and more the device runs 7 at a time)
+    assert sch["team"] > 1 and sch["chunk_rows"] == 256 and (Hq // Hkv * q_cap > 128 and D == 128 or sch["team"] > 9 and sch["grid"] > 7 * sch["team"]), sch
+    cl, ql = [lc, lc // 2 + 3, 0][:B], [q_cap, q_cap // 2, 1][:B]
+    out, lse, _ = _case(dev, oracle, NL, B, Hq, Hkv, D, cap, q_cap, cl, ql, seed=NL, hint=lc, layers=[NL - 1])
+    _case(dev, oracle, NL, B, Hq, Hkv, D, cap, q_cap, [0, lc, 17][:B], [1, 0, q_cap][:B], seed=NL + 1, hint=lc, layers=[0])
+    ck, cv = make_cache(NL, B, Hkv, cap, D, NL)
+    q, kn, vn = make_attn_inputs(NL, B, Hq, Hkv, q_cap, D, NL + 1)
+    args = [t.cuda() for t in (ck, cv)] + [_i32(cl)] + [t.cuda() for t in (q, kn, vn)] + [_i32(ql)]
+    dlm.dlm_selftest_set_wait_limit(dev.ctx, 0)
+    try:
+        gpu_attn_step(dev, *args, hint=lc)
+        assert dev.status() == dlm.DLM_ERR_TIMEOUT
+    finally:
+        dlm.dlm_selftest_set_wait_limit(dev.ctx, 2_000_000_000)
+    again = [gpu_attn_step(dev, *args, hint=lc) for _ in range(20)]
+    assert dev.status() == 0
+    for o, l in again:
+        assert torch.equal(o, out) and torch.equal(l, lse)

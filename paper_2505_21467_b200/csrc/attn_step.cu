@@ -1698,7 +1698,7 @@ constexpr double kSplitManyCost[2] = {3.2, 2.7};
 // back and between projections (weighted 1 : 2, since most calls stand in a layer).  The teams' terms for rows and ragged tiles are rounded
 // towards smaller chunks.  Between projections 28 of these calls were 3 - 34 % slower than before there were clusters, with costs that took heads
 // of 64 for as dear as those of 128 and without teams through L2; now 10 are, by 3 - 7 %.  Back to back it was 79, now 18, most by 3 - 10 %;
-// 8 active rows of 8 - 32 KV heads at 4000 cached rows, where a cluster waits for all of its SMs, by 18 - 25 % (faster between projections).
+// 8 - 32 units of 8 active rows at 4000 cached ones by 18 - 25 % (probably since a cluster waits for all of its SMs; not between projections).
 struct CallShape {
   double t;      // key tiles of the block with the most, ragged ones by UnitTiles::cost
   double two;    // 1 with two M tiles a block, else 0

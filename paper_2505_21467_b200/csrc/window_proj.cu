@@ -538,9 +538,9 @@ bool make_proj_plan(const dlm_ctx* ctx, int rows, int n_out, int k_total, int he
   // per cycle and SM; a block costs some fixed time on top.  It ranks widths and is not a time: HBM, latencies, the producers'
   // loop and the power cap are not in it, and calls take 1.3 to 3 times as long (32 x 3584 -> 4608: 4.0 us against 8.5
   // measured, 256 x 3584 -> 4608 9.2 against 12.4, 1280 x 3584 -> 4608 24.7 against 36.1, 256 x 4096 -> 12288 15.0 against 28.6,
-  // and 28.5 with the weights in L2: it is not HBM that is missing there).  Of 125 calls with every width timed (both
-  // projections of five models' widths, 1 - 3000 rows) it picks the fastest or one within 2 % in 123; the two are 800 rows of
-  // 12288 features (384: 96.5 us, 256: 93.0) and 2000 (192: 210, 512: 189), both under the power cap.
+  // and 28.5 with the weights in L2: it is not HBM that is missing there).  Of 98 calls with every width timed (seven
+  // widths of five models, 1 - 3000 rows) it picks the fastest or one within 2 % in 92; the others are 2000 rows of 4096 -> 12288
+  // (192: 203 us, 512: 174, under the power cap), 3000 of 256 -> 512 and 8 of 3584 -> 3584 (7 %), and three small ones (2 - 4 %).
   double best = 0;
   pl.variant = -1;
   for (int v = 0; v < (int)(sizeof(kVariants) / sizeof(kVariants[0])); ++v) {
